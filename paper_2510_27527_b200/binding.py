@@ -7,7 +7,9 @@ shared library has not been built (``python -m paper_2510_27527_b200.build``).
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
+import threading
 from dataclasses import dataclass
 
 import numpy as np
@@ -154,7 +156,8 @@ def _check(status: int, where: str):
 
 
 def _stream_ptr() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # the handle of the current device's current stream, without building a torch.cuda.Stream object around it (3 us a call)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t) -> int:
@@ -204,11 +207,27 @@ def alloc_operand(R: int, K: int, gs_mode: int, sf_layout: int = SF_TILED128x4, 
     return Operand(codes, sf, gs, R, K, gs_mode, sf_layout)
 
 
+@functools.lru_cache(maxsize=4096)
+def _operand_sizes(R: int, K: int, gs_mode: int, sf_layout: int) -> tuple:
+    """(bytes of codes, bytes of scales, floats of global scales), at least 1 each. Sizes only: no memory is kept."""
+    return (max(_lib.nvfp4_operand_codes_bytes(R, K), 1), max(_lib.nvfp4_operand_sf_bytes(R, K, sf_layout), 1),
+            max(_lib.nvfp4_operand_gscale_count(R, K, gs_mode), 1))
+
+
+def _new_operand(R: int, K: int, gs_mode: int, sf_layout: int, device) -> Operand:
+    """An operand for a library call to fill: the quantizers write every byte, padding included, so nothing is cleared here."""
+    if R <= 0 or K <= 0:
+        return alloc_operand(R, K, gs_mode, sf_layout, device)
+    n_codes, n_sf, n_gs = _operand_sizes(R, K, gs_mode, sf_layout)
+    mk = lambda n, dt: torch.empty(n, dtype=dt, device=device)
+    return Operand(mk(n_codes, torch.uint8), mk(n_sf, torch.uint8), mk(n_gs, torch.float32), R, K, gs_mode, sf_layout)
+
+
 def _matrix(rows: int, cols: int, dtype_code: int, device) -> torch.Tensor:
     """Row-major output whose rows start on 16-byte boundaries (leading dimension padded to 8 elements)."""
     ld = (cols + 7) // 8 * 8
     buf = torch.empty((rows, ld), dtype=torch.float32 if dtype_code == DT_F32 else torch.bfloat16, device=device)
-    return buf[:, :cols]
+    return buf if ld == cols else buf[:, :cols]
 
 
 def upload_bf16(x: np.ndarray, device="cuda") -> torch.Tensor:
@@ -233,7 +252,7 @@ def nvfp4_quantize(src: torch.Tensor, axis: int = AXIS_ROW, rounding: int = ROUN
     kept = cols if keep_cols is None else int(keep_cols.numel())
     R, K = (rows, kept) if axis == AXIS_ROW else (kept, rows)
     if out is None:
-        out = alloc_operand(R, K, gs_mode, sf_layout, src.device)
+        out = _new_operand(R, K, gs_mode, sf_layout, src.device)
     ws = workspace if workspace is not None else _workspace(_lib.nvfp4_quantize_workspace_bytes(R, gs_mode), src.device)
     co = out.c()
     _check(_lib.nvfp4_quantize(_ptr(src), rows, cols, src.stride(0), axis, rounding, seed, stream_id, rht_stream_id,
@@ -251,7 +270,7 @@ def nvfp4_quantize_static(src: torch.Tensor, axis: int = AXIS_ROW, rounding: int
     kept = cols if keep_cols is None else int(keep_cols.numel())
     R, K = (rows, kept) if axis == AXIS_ROW else (kept, rows)
     if out is None:
-        out = alloc_operand(R, K, gs_mode, sf_layout, src.device)
+        out = _new_operand(R, K, gs_mode, sf_layout, src.device)
     co = out.c()
     _check(_lib.nvfp4_quantize_static(_ptr(src), rows, cols, src.stride(0), axis, rounding, seed, stream_id, _ptr(keep_cols),
                                       kept, ctypes.byref(co), _stream_ptr()), "nvfp4_quantize_static")
@@ -264,7 +283,7 @@ def nvfp4_requantize_t(inp: Operand, rounding: int = ROUND_SR, seed: int = 0, st
     gs_mode = inp.gs_mode if gs_mode is None else gs_mode
     D = inp.K if row_map is None else int(row_map.numel())
     if out is None:
-        out = alloc_operand(D, inp.R, gs_mode, sf_layout, inp.codes.device)
+        out = _new_operand(D, inp.R, gs_mode, sf_layout, inp.codes.device)
     ws = workspace if workspace is not None else _workspace(_lib.nvfp4_quantize_workspace_bytes(D, gs_mode), inp.codes.device)
     ci, co = inp.c(), out.c()
     _check(_lib.nvfp4_requantize_t(ctypes.byref(ci), _ptr(hp), 0 if hp is None else hp.stride(0), _ptr(row_map), D, rounding,
@@ -278,7 +297,7 @@ def nvfp4_quantize_w16x16(W: torch.Tensor, sf_layout: int = SF_TILED128x4, out: 
     """Q2 of the 16x16 weight-block recipe: one E4M3 scale per 16x16 square, per-tensor global scale, round to nearest."""
     C, D = W.shape
     if out is None:
-        out = alloc_operand(C, D, GS_TENSOR, sf_layout, W.device)
+        out = _new_operand(C, D, GS_TENSOR, sf_layout, W.device)
     ws = workspace if workspace is not None else _workspace(_lib.nvfp4_quantize_workspace_bytes(C, GS_TENSOR), W.device)
     co = out.c()
     _check(_lib.nvfp4_quantize_w16x16(_ptr(W), C, D, W.stride(0), ctypes.byref(co), _ptr(ws), ws.numel(), _stream_ptr()),
@@ -289,7 +308,7 @@ def nvfp4_quantize_w16x16(W: torch.Tensor, sf_layout: int = SF_TILED128x4, out: 
 def nvfp4_transpose_operand16(inp: Operand, sf_layout: int = SF_TILED128x4, out: Operand | None = None) -> Operand:
     """Operand of W-hat^T from the 16x16-block operand of W (codes transposed, scales re-indexed; no arithmetic)."""
     if out is None:
-        out = alloc_operand(inp.K, inp.R, GS_TENSOR, sf_layout, inp.codes.device)
+        out = _new_operand(inp.K, inp.R, GS_TENSOR, sf_layout, inp.codes.device)
     ci, co = inp.c(), out.c()
     _check(_lib.nvfp4_transpose_operand16(ctypes.byref(ci), ctypes.byref(co), _stream_ptr()), "nvfp4_transpose_operand16")
     return out
@@ -450,48 +469,98 @@ class LayerConfig:
     _outl: torch.Tensor | None = None
     _keep: torch.Tensor | None = None
     _map: torch.Tensor | None = None
-    _D: int = -1
+    _of: tuple | None = None  # (hidden size, device, outlier channels, the three arrays made for them)
     _side: tuple | None = None
 
     def side(self, device):
         """(stream, fork, join, aux) of the second stream for `device`, created on first use; None when not concurrent."""
         if not self.concurrent:
             return None
-        dev = torch.device(device)
-        dev = torch.device("cuda", torch.cuda.current_device()) if dev.index is None else dev
+        dev = _device_of(device)
         if self._side is None or self._side[0] != dev:
-            with torch.cuda.device(dev):
-                self._side = (dev, torch.cuda.Stream(device=dev), torch.cuda.Event(), torch.cuda.Event(), torch.cuda.Event())
-                for ev in self._side[2:]:
-                    ev.record(self._side[1])  # forces creation of the underlying CUDA events (torch makes them lazily)
+            self._side = (dev, *_make_side(dev))
         return self._side[1:]
 
     def prepare(self, D: int, device="cuda"):
         """Uploads the OutControl index arrays for hidden size D (index bookkeeping only)."""
         self.side(device)
-        if self.outliers is None or len(self.outliers) == 0 or self._D == D:
-            return
-        outl = np.asarray(self.outliers, dtype=np.int64)
+        self.index(D, device)
+
+    def index(self, D: int, device="cuda"):
+        """(outlier channels, kept channels, channel map) on the device, or None without outlier channels. What is there already
+        is kept while hidden size, device and the channels themselves (their values, not the array's identity) are the same."""
+        if self.outliers is None or len(self.outliers) == 0:
+            return None
+        outl = np.array(self.outliers, dtype=np.int64)
+        dev = _device_of(device)
+        of = self._of
+        if of is not None and of[0] == D and of[1] == dev and np.array_equal(of[2], outl):
+            return of[3]
         mask = np.ones(D, dtype=bool)
         mask[outl] = False
         keep = np.nonzero(mask)[0]
         cmap = np.full(D, -1, dtype=np.int32)
         cmap[keep] = np.arange(len(keep), dtype=np.int32)
-        self._outl = torch.from_numpy(outl.astype(np.int32)).to(device)
-        self._keep = torch.from_numpy(keep.astype(np.int32)).to(device)
-        self._map = torch.from_numpy(cmap).to(device)
-        self._D = D
+        held = tuple(torch.from_numpy(a.astype(np.int32)).to(dev) for a in (outl, keep, cmap))
+        self._of = (D, dev, outl, held)
+        self._outl, self._keep, self._map = held
+        return held
 
     @property
     def n_out(self) -> int:
         return 0 if self.outliers is None else len(self.outliers)
 
-    def c(self) -> CLayerCfg:
-        side = self._side[1:] if (self.concurrent and self._side is not None) else None
-        sp = (side[0].cuda_stream, side[1].cuda_event, side[2].cuda_event, side[3].cuda_event) if side else (0, 0, 0, 0)
-        return CLayerCfg(self.gs_mode, (c_i32 * 6)(*self.rounding), self.seed, self.y_dtype, self.dx_dtype, self.dw_dtype,
-                         self.n_out, _ptr(self._outl), _ptr(self._keep), _ptr(self._map), _ptr(self.dev_status), int(self.rht),
-                         int(self.outlier_fp8), int(self.w_block16), *sp)
+    def c(self, seed: int | None = None, dtypes: tuple | None = None, index: tuple | None = None, side: tuple | None = None) -> CLayerCfg:
+        """The C structure. Seed, output types, index arrays and second stream are the configuration's own unless `dtypes` is given."""
+        if dtypes is None:
+            dtypes = (self.y_dtype, self.dx_dtype, self.dw_dtype)
+            side = self._side[1:] if (self.concurrent and self._side is not None) else None
+            index = (self._outl, self._keep, self._map)
+        outl, keep, cmap = index if index is not None else (None, None, None)
+        c = CLayerCfg(self.gs_mode, (c_i32 * 6)(*self.rounding), self.seed if seed is None else seed, *dtypes, self.n_out, _ptr(outl),
+                      _ptr(keep), _ptr(cmap), _ptr(self.dev_status), int(self.rht), int(self.outlier_fp8), int(self.w_block16))
+        if side is not None:
+            set_side(c, side)
+        return c
+
+
+def set_side(c: CLayerCfg, side: tuple) -> None:
+    c.side_stream, c.ev_fork, c.ev_join, c.ev_aux = side[0].cuda_stream, side[1].cuda_event, side[2].cuda_event, side[3].cuda_event
+
+
+def _device_of(device) -> torch.device:
+    """`device` with its index filled in."""
+    dev = torch.device(device)
+    return torch.device("cuda", torch.cuda.current_device()) if dev.index is None else dev
+
+
+def _make_side(dev: torch.device) -> tuple:
+    """(stream, fork, join, aux) on `dev`."""
+    with torch.cuda.device(dev):
+        side = (torch.cuda.Stream(device=dev), torch.cuda.Event(), torch.cuda.Event(), torch.cuda.Event())
+        for ev in side[1:]:
+            ev.record(side[0])  # forces creation of the underlying CUDA events (torch makes them lazily)
+    return side
+
+
+_thread = threading.local()
+_THREAD_SIDES = 8
+
+
+def thread_side(dev: torch.device, stream: int) -> tuple:
+    """The calling thread's second stream and events for calls on `stream` of `dev`, made on first use. A thread enqueues its
+    calls on one stream one after another, so they can share a set: a call's waits refer to the records before them in host
+    order, and re-recording an event does not change what was already waited for. A thread holds the sets of the
+    _THREAD_SIDES streams it used last and gives them back when it ends."""
+    sides = _thread.__dict__.setdefault("sides", {})
+    key = (dev.index, stream)
+    side = sides.pop(key, None)
+    if side is None:
+        side = _make_side(dev)
+        if len(sides) >= _THREAD_SIDES:
+            sides.pop(next(iter(sides)))  # the one used longest ago
+    sides[key] = side
+    return side
 
 
 @dataclass
@@ -516,12 +585,15 @@ def alloc_saved(X: torch.Tensor, W: torch.Tensor, cfg: "LayerConfig") -> "Saved"
     Kh = _lib.nvfp4_outlier_pad(cfg.n_out)
     xo = torch.empty((N_tok, Kh), dtype=torch.bfloat16, device=X.device) if Kh else None
     wo = torch.empty((C, Kh), dtype=torch.bfloat16, device=X.device) if Kh else None
-    return Saved(alloc_operand(N_tok, Dk, cfg.gs_mode, SF_TILED128x4, X.device), alloc_operand(C, Dk, cfg.gs_mode, SF_TILED128x4, X.device),
+    return Saved(_new_operand(N_tok, Dk, cfg.gs_mode, SF_TILED128x4, X.device), _new_operand(C, Dk, cfg.gs_mode, SF_TILED128x4, X.device),
                  X, W, xo, wo)
 
 
+_linear_workspace_bytes = functools.lru_cache(maxsize=4096)(_lib.nvfp4_linear_workspace_bytes)
+
+
 def linear_workspace(op_kind: int, N_tok: int, D: int, C: int, cfg: LayerConfig, device="cuda") -> torch.Tensor:
-    return _workspace(_lib.nvfp4_linear_workspace_bytes(op_kind, N_tok, D, C, cfg.n_out, cfg.gs_mode), device)
+    return _workspace(_linear_workspace_bytes(op_kind, N_tok, D, C, cfg.n_out, cfg.gs_mode), device)
 
 
 def nvfp4_linear_bwd_operand(op_kind: int, which: int, N_tok: int, D: int, C: int, cfg: LayerConfig, workspace: torch.Tensor) -> Operand:
@@ -629,12 +701,20 @@ def alloc_dense(R: int, K: int, device="cuda", poison: bool = False) -> DenseOpe
     return DenseOperand(vals, torch.zeros(1, dtype=torch.float32, device=device), R, K)
 
 
+def _new_dense(R: int, K: int, device) -> DenseOperand:
+    """A dense operand for a library call to fill (the kernels write every column, the padding ones included)."""
+    if R <= 0 or K <= 0:
+        return alloc_dense(R, K, device)
+    return DenseOperand(torch.empty((R, _lib.nvfp4_dense_ld(K)), dtype=torch.bfloat16, device=device),
+                        torch.empty(1, dtype=torch.float32, device=device), R, K)
+
+
 def nvfp4_fp6_quantize(src: torch.Tensor, rounding: int = ROUND_RTN, seed: int = 0, stream_id: int = 0,
                        out: DenseOperand | None = None, workspace: torch.Tensor | None = None) -> DenseOperand:
     assert src.dtype == torch.bfloat16 and src.dim() == 2 and src.stride(1) == 1
     rows, cols = src.shape
     if out is None:
-        out = alloc_dense(rows, cols, src.device)
+        out = _new_dense(rows, cols, src.device)
     ws = workspace if workspace is not None else _workspace(_lib.nvfp4_fp6_workspace_bytes(), src.device)
     co = out.c()
     _check(_lib.nvfp4_fp6_quantize(_ptr(src), rows, cols, src.stride(0), rounding, seed, stream_id, ctypes.byref(co), _ptr(ws),
@@ -645,7 +725,7 @@ def nvfp4_fp6_quantize(src: torch.Tensor, rounding: int = ROUND_RTN, seed: int =
 def nvfp4_fp6_requantize_t(inp: DenseOperand, rounding: int = ROUND_SR, seed: int = 0, stream_id: int = 0,
                            out: DenseOperand | None = None, workspace: torch.Tensor | None = None) -> DenseOperand:
     if out is None:
-        out = alloc_dense(inp.K, inp.R, inp.vals.device)
+        out = _new_dense(inp.K, inp.R, inp.vals.device)
     ws = workspace if workspace is not None else _workspace(_lib.nvfp4_fp6_workspace_bytes(), inp.vals.device)
     ci, co = inp.c(), out.c()
     _check(_lib.nvfp4_fp6_requantize_t(ctypes.byref(ci), rounding, seed, stream_id, ctypes.byref(co), _ptr(ws), ws.numel(),
@@ -655,7 +735,7 @@ def nvfp4_fp6_requantize_t(inp: DenseOperand, rounding: int = ROUND_SR, seed: in
 
 def nvfp4_expand_operand(inp: Operand, out: DenseOperand | None = None) -> DenseOperand:
     if out is None:
-        out = alloc_dense(inp.R, inp.K, inp.codes.device)
+        out = _new_dense(inp.R, inp.K, inp.codes.device)
     ci, co = inp.c(), out.c()
     _check(_lib.nvfp4_expand_operand(ctypes.byref(ci), ctypes.byref(co), _stream_ptr()), "nvfp4_expand_operand")
     return out

@@ -7,7 +7,8 @@ from the same configuration share their draws.
 """
 from __future__ import annotations
 
-import dataclasses
+import ctypes
+import functools
 
 import torch
 
@@ -27,20 +28,81 @@ def call_seed(base_seed: int, layer_id: int, call: int) -> int:
     return z ^ (z >> 31)
 
 
+def _up(n: int) -> int:
+    return (n + 255) // 256 * 256
+
+
+@functools.lru_cache(maxsize=1024)
+def _layout(N_tok: int, D: int, C: int, n_out: int, gs_mode: int):
+    """Where a call keeps what forward leaves for backward, inside one buffer: the byte offsets of codes, scales and global
+    scales of qx and qw and of the two compact outlier matrices (-1: none), the offset and size of forward's workspace, the
+    buffer's total, and the size of backward's workspace. Sizes only: no memory is kept."""
+    Dk, Kh, at, offs = D - n_out, B.lib.nvfp4_outlier_pad(n_out), 0, []
+    for R in (N_tok, C):
+        for n in (B.lib.nvfp4_operand_codes_bytes(R, Dk), B.lib.nvfp4_operand_sf_bytes(R, Dk, B.SF_TILED128x4),
+                  4 * B.lib.nvfp4_operand_gscale_count(R, Dk, gs_mode)):
+            offs.append(at)
+            at = _up(at + n)
+    for R in (N_tok, C):
+        offs.append(at if Kh else -1)
+        at = _up(at + R * Kh * 2)
+    ws_fwd = B.lib.nvfp4_linear_workspace_bytes(B.OP_FWD, N_tok, D, C, n_out, gs_mode)
+    return tuple(offs), at, ws_fwd, at + ws_fwd, B.lib.nvfp4_linear_workspace_bytes(B.OP_BWD, N_tok, D, C, n_out, gs_mode)
+
+
+class _Call:
+    """One forward call and, later, its backward. The calls go to the library directly, with one buffer for everything that is
+    saved: a layer step of a few hundred tokens is bound by what the host does around its dozen kernels (fwd + bwd of a
+    512-wide layer on 256 tokens took 390 us with a tensor per saved array and a configuration object, a stream and three
+    events made per call; its kernels take 58 us)."""
+
+    __slots__ = ("buf", "saved", "ccfg", "keeps", "concurrent", "shape", "ws_bwd")
+
+    def forward(self, x: torch.Tensor, weight: torch.Tensor, cfg: B.LayerConfig, seed: int) -> torch.Tensor:
+        (N_tok, D), C, dev = x.shape, weight.shape[0], x.device
+        index = cfg.index(D, dev)
+        n_out, gs = cfg.n_out, cfg.gs_mode
+        offs, ws_at, ws_fwd, total, self.ws_bwd = _layout(N_tok, D, C, n_out, gs)
+        buf = torch.empty(total, dtype=torch.uint8, device=dev)
+        y = B._matrix(N_tok, C, B.DT_BF16, dev)
+        p, stream = buf.data_ptr(), B._stream_ptr()
+        at = [p + o if o >= 0 else 0 for o in offs]
+        saved = B.CSaved(B.COperand(at[0], at[1], at[2], N_tok, D - n_out, gs, B.SF_TILED128x4),
+                         B.COperand(at[3], at[4], at[5], C, D - n_out, gs, B.SF_TILED128x4), X_out=at[6], W_out=at[7])
+        # the configuration as it is now: what the caller changes later belongs to later calls
+        ccfg = cfg.c(seed=seed, dtypes=(B.DT_BF16, B.DT_BF16, B.DT_BF16), index=index,
+                     side=B.thread_side(dev, stream) if cfg.concurrent else None)
+        B._check(B.lib.nvfp4_linear_fwd(x.data_ptr(), x.stride(0), weight.data_ptr(), weight.stride(0), N_tok, D, C, ctypes.byref(ccfg),
+                                        y.data_ptr(), y.stride(0), ctypes.byref(saved), p + ws_at, ws_fwd, stream), "nvfp4_linear_fwd")
+        self.buf, self.saved, self.ccfg, self.shape = buf, saved, ccfg, (N_tok, D, C)
+        self.keeps, self.concurrent = (index, cfg.dev_status), cfg.concurrent
+        return y
+
+    def backward(self, dy: torch.Tensor):
+        (N_tok, D, C), dev = self.shape, dy.device
+        dx, dw = B._matrix(N_tok, D, B.DT_BF16, dev), B._matrix(C, D, B.DT_BF16, dev)
+        ws, stream = torch.empty(self.ws_bwd, dtype=torch.uint8, device=dev), B._stream_ptr()
+        ccfg = B.CLayerCfg.from_buffer_copy(self.ccfg)
+        if self.concurrent:  # autograd runs backward on a thread of its own, which has its own second stream and events
+            B.set_side(ccfg, B.thread_side(dev, stream))
+        B._check(B.lib.nvfp4_linear_bwd(dy.data_ptr(), dy.stride(0), ctypes.byref(self.saved), ctypes.byref(ccfg), dx.data_ptr(), dx.stride(0),
+                                        dw.data_ptr(), dw.stride(0), ws.data_ptr(), self.ws_bwd, stream), "nvfp4_linear_bwd")
+        return dx, dw
+
+
 class _NVFP4LinearFn(torch.autograd.Function):
     @staticmethod
-    def forward(ctx, x2d: torch.Tensor, weight: torch.Tensor, cfg: B.LayerConfig):
-        y, saved = B.nvfp4_linear_fwd(x2d, weight, cfg)
-        ctx.saved_ops, ctx.cfg = saved, cfg
-        return y
+    def forward(ctx, x2d: torch.Tensor, weight: torch.Tensor, cfg: B.LayerConfig, seed: int):
+        ctx.call = _Call()
+        return ctx.call.forward(x2d, weight, cfg, seed)
 
     @staticmethod
     def backward(ctx, dy: torch.Tensor):
         dy = dy.contiguous()
         if dy.dtype != torch.bfloat16:
             dy = dy.to(torch.bfloat16)
-        dx, dw = B.nvfp4_linear_bwd(dy, ctx.saved_ops, ctx.cfg)
-        return dx, dw, None
+        dx, dw = ctx.call.backward(dy)
+        return dx, dw, None, None
 
 
 class NVFP4Linear(torch.nn.Module):
@@ -60,15 +122,17 @@ class NVFP4Linear(torch.nn.Module):
         NVFP4Linear._instances += 1
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
-        lead = x.shape[:-1]
-        x2d = x.reshape(-1, self.in_features)
+        x2d = x if x.dim() == 2 else x.reshape(-1, self.in_features)
         if x2d.dtype != torch.bfloat16:
             x2d = x2d.to(torch.bfloat16)
         x2d = x2d.contiguous()
-        # a fresh configuration per call: same options and index arrays, this layer's key of this call
-        cfg = dataclasses.replace(self.cfg, seed=call_seed(self.cfg.seed, self.layer_id, self._calls), y_dtype=B.DT_BF16, dx_dtype=B.DT_BF16, dw_dtype=B.DT_BF16)
+        # this layer's key of this call
+        seed = call_seed(self.cfg.seed, self.layer_id, self._calls)
         self._calls += 1
-        y = _NVFP4LinearFn.apply(x2d, self.weight, cfg)
+        if torch.is_grad_enabled() and (x2d.requires_grad or self.weight.requires_grad):
+            y = _NVFP4LinearFn.apply(x2d, self.weight, self.cfg, seed)
+        else:
+            y = _Call().forward(x2d, self.weight, self.cfg, seed)
         if self.bias is not None:
             y = y + self.bias
-        return y.reshape(*lead, self.out_features)
+        return y if x.dim() == 2 else y.reshape(*x.shape[:-1], self.out_features)

@@ -31,3 +31,67 @@ def test_module_forward_backward_match_the_oracle():
         assert np.all(bf16_ulp_close(x.grad.reshape(N_tok, D).float().cpu().numpy(), dXo, 1.0, 1e-4 * np.abs(dXo).mean()))
         assert np.all(bf16_ulp_close(lin.weight.grad.float().cpu().numpy(), dWo, 1.0, 1e-4 * np.abs(dWo).mean()))
         lin.weight.grad = None
+
+
+@pytest.mark.parametrize("tokens", [1, 77, 300])  # one saved buffer per call: its pieces at ragged sizes
+@pytest.mark.parametrize("gs_mode,n_out", [(0, 0), (1, 0), (2, 5)])
+def test_module_matches_the_binding_on_every_stream_and_thread(tokens, gs_mode, n_out):
+    """The same calls through nvfp4_linear_fwd / nvfp4_linear_bwd with a buffer per array, and the module's on two streams from
+    two threads at once: identical bytes everywhere."""
+    import threading
+
+    from paper_2510_27527_b200 import binding as b
+    from paper_2510_27527_b200.module import NVFP4Linear, call_seed
+
+    D, C = 200, 136
+    X, W, dY, _ = synth.layer_inputs(3, tokens, D, C, n_outlier=3, factor=30.0, grad_scale=1e-3)
+    outl = synth.outlier_channels(D, n_out, 5) if n_out else None
+    x, w, dy = to_dev_bf16(X), to_dev_bf16(W), to_dev_bf16(dY)
+    want = []
+    for call in range(3):
+        cfg = b.LayerConfig(gs_mode=gs_mode, seed=call_seed(7, 3, call), outliers=outl, dw_dtype=b.DT_BF16)
+        y, saved = b.nvfp4_linear_fwd(x, w, cfg)
+        want.append((y, *b.nvfp4_linear_bwd(dy, saved, cfg)))
+    torch.cuda.synchronize()
+    got, errors = {}, []
+
+    def work(name):
+        try:
+            layer = NVFP4Linear(D, C, cfg=b.LayerConfig(gs_mode=gs_mode, seed=7, outliers=outl))
+            layer.layer_id = 3
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                with torch.no_grad():
+                    layer.weight.copy_(w)
+                xi = x.clone().requires_grad_(True)
+                out = []
+                for _ in range(3):
+                    y = layer(xi)
+                    out.append((y, *torch.autograd.grad(y, (xi, layer.weight), dy)))
+            s.synchronize()
+            got[name] = out
+        except Exception as e:  # noqa: BLE001 - reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for i in range(2):
+        for a, bb in zip(got[i], want):
+            for g, r in zip(a, bb):
+                assert torch.equal(g, r)
+
+
+def test_index_arrays_follow_the_outlier_channels():
+    from paper_2510_27527_b200 import binding as b
+
+    cfg = b.LayerConfig(outliers=np.array([1, 5]))
+    first = cfg.index(16)
+    assert cfg.index(16) is first
+    cfg.outliers[1] = 7  # the same array with other contents
+    outl, keep, cmap = cfg.index(16)
+    assert outl.tolist() == [1, 7] and 5 in keep.tolist() and cmap.tolist()[5] == 4
+    assert cfg.index(24)[1].numel() == 22
