@@ -17,6 +17,40 @@ __device__ __forceinline__ void pdl_prologue() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// The two halves on their own. A kernel that waits first and then calls pdl_launch_next() lets its successor's CTAs start only
+// when everything before itself is complete and visible; that successor may then load what this kernel only reads before its
+// own pdl_wait() (load_cg below), i.e. under this kernel.
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Loads through L2 that stay where they are written (an ordinary load of read-only memory may be moved across the waits).
+__device__ __forceinline__ float4 load_cg4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void load_cg8(const float* p, float* v) {  // 32-byte aligned
+  asm volatile("ld.global.cg.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void store8(float* p, const float* v) {  // 32-byte aligned
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+               "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+__device__ __forceinline__ float load_cg(const float* p) {
+  float v;
+  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t load_cg(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 constexpr int kRoundRTN = 0;
 constexpr int kRoundSR = 1;
 constexpr int kGsTensor = 0;
@@ -51,6 +85,58 @@ __device__ __forceinline__ float bf16_bits_to_float(uint32_t b16) { return __uin
 __device__ __forceinline__ uint16_t f32_to_bf16_bits(float v) {
   const uint32_t b = __float_as_uint(v);
   return (uint16_t)((b + 0x7FFFu + ((b >> 16) & 1u)) >> 16);
+}
+
+// ---------------------------------------------------------------------------------------------------------
+// Maximum of a tensor without a cleared cell: an amax kernel writes N words (N = 32 or 64), one per CTA or per cluster of CTAs
+// and zeros in the rest, and its readers take their maximum. An atomic maximum into one word needs that word cleared first,
+// i.e. one launch more (about 3 us of host time, and a serial point of about 2 us on the device).
+// ---------------------------------------------------------------------------------------------------------
+template <int N>
+__device__ __forceinline__ uint32_t cells_max(const uint32_t* __restrict__ cells) {  // every lane of the warp calls this
+  const int lane = threadIdx.x & 31;
+  uint32_t v = load_cg(cells + lane);
+  if (N == 64) v = max(v, load_cg(cells + 32 + lane));
+  return __reduce_max_sync(0xFFFFFFFFu, v);
+}
+// Word of this thread's cluster <- maximum of the cluster's values m. Every thread of every CTA calls it; blockDim.x is a
+// multiple of 32 and at most 1024, the cluster (cluster_x, 1, 1) has at most 8 CTAs and there are at most N clusters.
+template <int N>
+__device__ __forceinline__ void cells_write(uint32_t m, uint32_t* cells) {
+  __shared__ uint32_t warp_max[32];
+  __shared__ uint32_t cta_max[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+  uint32_t rank, n_rank;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n_rank));
+  m = __reduce_max_sync(0xFFFFFFFFu, m);
+  if (lane == 0) warp_max[wid] = m;
+  __syncthreads();
+  if (wid == 0) {
+    m = __reduce_max_sync(0xFFFFFFFFu, lane < n_warps ? warp_max[lane] : 0u);
+    if (lane == 0) {
+      if (n_rank == 1) {
+        cta_max[0] = m;
+      } else {
+        uint32_t dst;
+        asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(&cta_max[rank])));
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(dst), "r"(m) : "memory");
+      }
+    }
+  }
+  if (n_rank > 1) {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+  if (rank == 0 && wid == 0) {
+    const uint32_t cluster = blockIdx.x / n_rank, n_clusters = gridDim.x / n_rank;
+    m = __reduce_max_sync(0xFFFFFFFFu, lane < (int)n_rank ? cta_max[lane] : 0u);
+    if (lane == 0) cells[cluster] = m;
+    if (cluster == 0)
+      for (uint32_t i = n_clusters + lane; i < (uint32_t)N; i += 32) cells[i] = 0u;
+  }
 }
 
 // ---------------------------------------------------------------------------------------------------------

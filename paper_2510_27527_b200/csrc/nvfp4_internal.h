@@ -97,6 +97,34 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
+// The same with thread-block clusters of `cluster_x` CTAs along x (a divisor of grid.x).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_kernel_cluster(void (*kernel)(KArgs...), dim3 grid, unsigned cluster_x, dim3 block, cudaStream_t st, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster_x;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  g_launch_count.fetch_add(1, std::memory_order_relaxed);
+  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+// Shape of an amax launch that writes at most n_words words (cells_write): CTAs along x and CTAs per cluster.
+struct AmaxGrid {
+  unsigned ctas, cluster;
+};
+inline AmaxGrid amax_grid(int64_t wanted_ctas, int n_words) {
+  const int64_t n = std::max<int64_t>(1, wanted_ctas);
+  if (n <= n_words) return {(unsigned)n, 1u};
+  return {(unsigned)(std::min<int64_t>((n + 7) / 8, n_words) * 8), 8u};
+}
+
 cudaError_t launch_quantize_rows(const QuantRowsArgs& a, cudaStream_t st);
 cudaError_t launch_quantize_transpose(const QuantTransposeArgs& a, cudaStream_t st);
 // amax of a contiguous-row BF16 matrix folded into cells[0] (atomic max; the cell must already hold a valid value)

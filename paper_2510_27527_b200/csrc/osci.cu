@@ -15,21 +15,33 @@ namespace nvfp4 {
 
 namespace {
 
-// 16 floats of row r starting at column k0 (zero beyond K); vector loads when the row is 16-byte aligned
-__device__ __forceinline__ void load16f(const float* __restrict__ row, int64_t k0, int64_t K, bool vec, float (&v)[16]) {
-  if (vec && k0 + 16 <= K) {
+// How rows of a matrix may be read: 2 = 32-byte pieces, 1 = 16-byte pieces, 0 = single floats.
+__device__ __forceinline__ int row_vec(const float* p, int64_t ld) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(p) | (uintptr_t)(ld * 4);
+  return (a & 31) == 0 ? 2 : (a & 15) == 0 ? 1 : 0;
+}
+// 16 floats of a row starting at column k0 (zero beyond K). A thread reads 64 bytes that no other thread needs, so the loads go
+// past L1 in whole 32-byte sectors (16-byte pieces past L1 fetch every sector twice: 8 - 10 % slower on 4096 x 4096).
+__device__ __forceinline__ void load16f(const float* __restrict__ row, int64_t k0, int64_t K, int vec, float (&v)[16]) {
+  if (vec == 2 && k0 + 16 <= K) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) load_cg8(row + k0 + 8 * q, &v[8 * q]);
+  } else if (vec && k0 + 16 <= K) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const float4 t = *reinterpret_cast<const float4*>(row + k0 + 4 * q);
+      const float4 t = load_cg4(row + k0 + 4 * q);
       v[4 * q] = t.x; v[4 * q + 1] = t.y; v[4 * q + 2] = t.z; v[4 * q + 3] = t.w;
     }
   } else {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = (k0 + i < K) ? row[k0 + i] : 0.0f;
+    for (int i = 0; i < 16; ++i) v[i] = (k0 + i < K) ? load_cg(row + k0 + i) : 0.0f;
   }
 }
-__device__ __forceinline__ void store16f(float* __restrict__ row, int64_t k0, int64_t K, bool vec, const float (&v)[16]) {
-  if (vec && k0 + 16 <= K) {
+__device__ __forceinline__ void store16f(float* __restrict__ row, int64_t k0, int64_t K, int vec, const float (&v)[16]) {
+  if (vec == 2 && k0 + 16 <= K) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) store8(row + k0 + 8 * q, &v[8 * q]);
+  } else if (vec && k0 + 16 <= K) {
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       *reinterpret_cast<float4*>(row + k0 + 4 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
@@ -99,56 +111,70 @@ __device__ __forceinline__ void quant_block_with(float (&w)[16], float m, float 
   }
 }
 
-// max |w| per row (cells[r]) or over the matrix (cells[0]); cells are zero before the launch
-__global__ void __launch_bounds__(256) amax_f32_kernel(const float* __restrict__ W, int64_t ld, int64_t C, int64_t D, uint32_t* cells,
-                                                      int per_row) {
-  pdl_prologue();
-  const int64_t chunks = (D + 3) >> 2;
-  const bool vec = (ld & 3) == 0;
+// Words of a matrix's maximum (cells_max): two matrices fit the 256 bytes that the workspace has in the TENSOR mode.
+constexpr int kOsciWords = 32;
+
+__device__ __forceinline__ float amax4(float m, const float4& v) {
+  return fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+}
+// max |w| of columns lane * 4, lane * 4 + 128, ... of a row
+__device__ __forceinline__ float amax_row(const float* __restrict__ p, int64_t D, bool vec, int lane, float m) {
+  int64_t c = lane * 4;
+  if (vec) {
+    for (; c + 384 + 4 <= D; c += 512) {  // four 16-byte loads in flight
+      float4 v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = *reinterpret_cast<const float4*>(p + c + 128 * i);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) m = amax4(m, v[i]);
+    }
+  }
+  for (; c < D; c += 128) {
+    if (vec && c + 4 <= D)
+      m = amax4(m, *reinterpret_cast<const float4*>(p + c));
+    else
+      for (int64_t j = c; j < min(D, c + 4); ++j) m = fmaxf(m, fabsf(p[j]));
+  }
+  return m;
+}
+
+// max |w| over one (gridDim.y = 1) or two matrices, kOsciWords words each. Bound by memory: both matrices of a statistics step
+// are read by one launch, which needs no cleared cells, instead of three. Statistics and reset of the five weight matrices of a
+// 1024 / 2816 wide block, with the loads below under this kernel: 189 -> 138 us; 4096 x 4096: 163 -> 153 us; 256 x 264: 32 -> 17.
+__global__ void __launch_bounds__(512) amax_f32_kernel(const float* __restrict__ W0, int64_t ld0, const float* __restrict__ W1, int64_t ld1,
+                                                      int64_t C, int64_t D, uint32_t* cells) {
+  pdl_wait();
+  pdl_launch_next();  // (its loads of the weights run under this kernel)
+  const float* __restrict__ W = blockIdx.y ? W1 : W0;
+  const int64_t ld = blockIdx.y ? ld1 : ld0;
   float m = 0.0f;
-  for (int64_t r = blockIdx.x; r < C; r += gridDim.x) {
-    const float* p = W + r * ld;
-    float mr = 0.0f;
-    int64_t c = threadIdx.x;
-    if (vec) {
-      for (; ((c + 768) << 2) + 4 <= D; c += 1024) {  // four 16-byte loads in flight
-        const float4 v0 = *reinterpret_cast<const float4*>(p + (c << 2));
-        const float4 v1 = *reinterpret_cast<const float4*>(p + ((c + 256) << 2));
-        const float4 v2 = *reinterpret_cast<const float4*>(p + ((c + 512) << 2));
-        const float4 v3 = *reinterpret_cast<const float4*>(p + ((c + 768) << 2));
-        mr = fmaxf(mr, fmaxf(fmaxf(fabsf(v0.x), fabsf(v0.y)), fmaxf(fabsf(v0.z), fabsf(v0.w))));
-        mr = fmaxf(mr, fmaxf(fmaxf(fabsf(v1.x), fabsf(v1.y)), fmaxf(fabsf(v1.z), fabsf(v1.w))));
-        mr = fmaxf(mr, fmaxf(fmaxf(fabsf(v2.x), fabsf(v2.y)), fmaxf(fabsf(v2.z), fabsf(v2.w))));
-        mr = fmaxf(mr, fmaxf(fmaxf(fabsf(v3.x), fabsf(v3.y)), fmaxf(fabsf(v3.z), fabsf(v3.w))));
-      }
+  if (ld == D && (D & 3) == 0) {  // one run of memory
+    const float4* __restrict__ p = reinterpret_cast<const float4*>(W);
+    const int64_t n = C * (D >> 2), step = (int64_t)gridDim.x * 512;
+    int64_t i = (int64_t)blockIdx.x * 512 + threadIdx.x;
+    for (; i + 3 * step < n; i += 4 * step) {
+      const float4 v0 = p[i], v1 = p[i + step], v2 = p[i + 2 * step], v3 = p[i + 3 * step];
+      m = amax4(amax4(amax4(amax4(m, v0), v1), v2), v3);
     }
-    for (; c < chunks; c += 256) {
-      if (vec && (c << 2) + 4 <= D) {
-        const float4 v = *reinterpret_cast<const float4*>(p + (c << 2));
-        mr = fmaxf(mr, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-      } else {
-        for (int64_t j = c << 2; j < min(D, (c << 2) + 4); ++j) mr = fmaxf(mr, fabsf(p[j]));
-      }
-    }
-    if (per_row) {
-#pragma unroll
-      for (int o = 16; o; o >>= 1) mr = fmaxf(mr, __shfl_xor_sync(0xFFFFFFFFu, mr, o));
-      if ((threadIdx.x & 31) == 0 && mr > 0.0f) atomicMax(cells + r, __float_as_uint(mr));
-    } else {
-      m = fmaxf(m, mr);
-    }
+    for (; i < n; i += step) m = amax4(m, p[i]);
+  } else {  // a warp per row
+    for (int64_t r = (int64_t)blockIdx.x * 16 + (threadIdx.x >> 5); r < C; r += (int64_t)gridDim.x * 16)
+      m = amax_row(W + r * ld, D, (ld & 3) == 0, threadIdx.x & 31, m);
   }
-  if (!per_row) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    __shared__ float wm[8];
-    if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < 8; ++w) m = fmaxf(m, wm[w]);
-      if (m > 0.0f) atomicMax(cells, __float_as_uint(m));
-    }
-  }
+  cells_write<kOsciWords>(__float_as_uint(m), cells + blockIdx.y * kOsciWords);
+}
+
+// max |w| of every row of one or two matrices, a warp per row: cells[r], cells[C + r].
+__global__ void __launch_bounds__(256) amax_rows_f32_kernel(const float* __restrict__ W0, int64_t ld0, const float* __restrict__ W1,
+                                                           int64_t ld1, int64_t C, int64_t D, uint32_t* cells) {
+  pdl_wait();
+  pdl_launch_next();  // (its loads of the weights run under this kernel)
+  const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), ld = blockIdx.y ? ld1 : ld0;
+  const int lane = threadIdx.x & 31;
+  if (r >= C) return;
+  const float m = amax_row((blockIdx.y ? W1 : W0) + r * ld, D, (ld & 3) == 0, lane, 0.0f);
+  const uint32_t u = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));
+  if (lane == 0) cells[blockIdx.y * C + r] = u;
 }
 
 // Algorithm 2, t0 = 0: clear the statistics, take the snapshot
@@ -159,7 +185,7 @@ __global__ void __launch_bounds__(256) osci_init_kernel(const float* __restrict_
   const int64_t gid = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (gid >= C * nb) return;
   const int64_t r = gid / nb, k0 = (gid - r * nb) << 4;
-  const bool vw = (ldw & 3) == 0, vs = (D & 3) == 0;
+  const int vw = row_vec(W, ldw), vs = min(row_vec(Wp, D), min(row_vec(DM, D), row_vec(DQ, D)));
   float v[16], z[16];
   load16f(W + r * ldw, k0, D, vw, v);
 #pragma unroll
@@ -174,13 +200,14 @@ template <int GS>
 __global__ void __launch_bounds__(256) osci_update_kernel(const float* __restrict__ W, int64_t ldw, int64_t C, int64_t D,
                                                          float* __restrict__ Wp, float* __restrict__ DM, float* __restrict__ DQ,
                                                          const uint32_t* __restrict__ cells) {
-  pdl_prologue();
+  pdl_launch_next();
+  if (GS == kGsBlock128) pdl_wait();  // else the kernel before this one is the amax pass of the same call: it writes the cells only
   const int64_t nb = ((D + 127) & ~(int64_t)127) >> 4;  // blocks per row, padded so that 8 lanes share a 128-group
   const int64_t gid = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const bool active = gid < C * nb;
   const int64_t r = active ? gid / nb : 0;
   const int64_t k0 = active ? (gid - r * nb) << 4 : D;  // inactive lanes read nothing and still take part in shuffles
-  const bool vw = (ldw & 3) == 0, vs = (D & 3) == 0;
+  const int vw = row_vec(W, ldw), vs = min(row_vec(Wp, D), min(row_vec(DM, D), row_vec(DQ, D)));
   float w[16], p[16];
   load16f(W + r * ldw, k0, D, vw, w);
   load16f(Wp + r * D, k0, D, vs, p);
@@ -190,9 +217,10 @@ __global__ void __launch_bounds__(256) osci_update_kernel(const float* __restric
   float dm[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) dm[i] = fabsf(__fsub_rn(w[i], p[i]));
+  if (GS != kGsBlock128) pdl_wait();
   if (active && k0 < D) store16f(Wp + r * D, k0, D, vs, w);
-  const uint32_t cw = GS == kGsTensor ? cells[0] : GS == kGsRow ? cells[r] : 0u;
-  const uint32_t cp = GS == kGsTensor ? cells[1] : GS == kGsRow ? cells[C + r] : 0u;
+  const uint32_t cw = GS == kGsTensor ? cells_max<kOsciWords>(cells) : GS == kGsRow ? load_cg(cells + r) : 0u;
+  const uint32_t cp = GS == kGsTensor ? cells_max<kOsciWords>(cells + kOsciWords) : GS == kGsRow ? load_cg(cells + C + r) : 0u;
   quant_dequant16<GS>(w, cw);
   quant_dequant16<GS>(p, cp);
   if (!(active && k0 < D)) return;
@@ -209,13 +237,14 @@ template <int GS>
 __global__ void __launch_bounds__(256, 3) osci_suppress_kernel(float* __restrict__ W, int64_t ldw, int64_t C, int64_t D,
                                                            const float* __restrict__ DM, const float* __restrict__ DQ, float tau,
                                                            const uint32_t* __restrict__ cells, unsigned long long* n_reset) {
-  pdl_prologue();
+  pdl_launch_next();
+  if (GS == kGsBlock128) pdl_wait();  // (as in osci_update_kernel)
   const int64_t nb = ((D + 127) & ~(int64_t)127) >> 4;
   const int64_t gid = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const bool active = gid < C * nb;
   const int64_t r = active ? gid / nb : 0;
   const int64_t k0 = active ? (gid - r * nb) << 4 : D;
-  const bool vw = (ldw & 3) == 0, vs = (D & 3) == 0;
+  const int vw = row_vec(W, ldw), vs = min(row_vec(DM, D), row_vec(DQ, D));
   float w[16], q[16];
   uint32_t hits = 0;
   {
@@ -232,7 +261,8 @@ __global__ void __launch_bounds__(256, 3) osci_suppress_kernel(float* __restrict
   }
 #pragma unroll
   for (int i = 0; i < 16; ++i) q[i] = w[i];
-  quant_dequant16<GS>(q, GS == kGsTensor ? cells[0] : GS == kGsRow ? cells[r] : 0u);
+  if (GS != kGsBlock128) pdl_wait();
+  quant_dequant16<GS>(q, GS == kGsTensor ? cells_max<kOsciWords>(cells) : GS == kGsRow ? load_cg(cells + r) : 0u);
   const int n = __popc(hits);
   if (active && n) {
 #pragma unroll
@@ -265,7 +295,7 @@ __global__ void __launch_bounds__(256, 3) osci_score_kernel(const float* __restr
   const int64_t r = active ? gid / nb : 0;
   const int64_t k0 = active ? (gid - r * nb) << 4 : D;
   float w[16], x[16];
-  load16f(W + r * ldw, k0, D, (ldw & 3) == 0, w);
+  load16f(W + r * ldw, k0, D, row_vec(W, ldw), w);
   float m = 0.0f;
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
@@ -280,7 +310,7 @@ __global__ void __launch_bounds__(256, 3) osci_score_kernel(const float* __restr
     g = max(g, __shfl_xor_sync(0xFFFFFFFFu, g, 4));
     Sg = global_scale_from_amax(__uint_as_float(g));
   } else {
-    const uint32_t cell = GS == kGsTensor ? cells[0] : cells[r];
+    const uint32_t cell = GS == kGsTensor ? cells_max<kOsciWords>(cells) : load_cg(cells + r);
     Sg = global_scale_from_amax(bf16_bits_to_float(f32_to_bf16_bits(__uint_as_float(cell))));
   }
   float rcp;
@@ -508,7 +538,7 @@ __global__ void __launch_bounds__(256) amax_groups_f32_kernel(const float* __res
   const int64_t r = active ? gid / nb : 0;
   const int64_t b = active ? gid - r * nb : 0;
   float w[16];
-  load16f(W + r * ldw, active ? b << 4 : D, D, (ldw & 3) == 0, w);
+  load16f(W + r * ldw, active ? b << 4 : D, D, row_vec(W, ldw), w);
   float m = 0.0f;
 #pragma unroll
   for (int i = 0; i < 16; ++i) m = fmaxf(m, fabsf(w[i]));
@@ -530,12 +560,12 @@ __device__ __forceinline__ void tracked_values(const float* __restrict__ W, int6
   const int64_t k0 = valid ? (int64_t)(c & ~15u) : D;
   mine = valid;
   float w[16], q[16];
-  load16f(W + (int64_t)r * ldw, k0, D, (ldw & 3) == 0, w);
+  load16f(W + (int64_t)r * ldw, k0, D, row_vec(W, ldw), w);
 #pragma unroll
   for (int i = 0; i < 16; ++i) q[i] = w[i];
   const float m = round_block_bf16(q);
   const int64_t G = (D + 127) >> 7;
-  const uint32_t cell = GS == kGsTensor ? cells[0] : GS == kGsRow ? cells[r] : cells[(int64_t)r * G + (c >> 7)];
+  const uint32_t cell = GS == kGsTensor ? cells_max<kOsciWords>(cells) : GS == kGsRow ? load_cg(cells + r) : load_cg(cells + (int64_t)r * G + (c >> 7));
   const float Sg = group_scale<kGsTensor>(m, cell);  // the lookup form (no shuffles) in every mode
   quant_block_with(q, m, Sg);
   wm = 0.0f;
@@ -618,13 +648,22 @@ __global__ void __launch_bounds__(256) osci_sparse_apply_kernel(float* __restric
   }
 }
 
+// (the callers round up to 256 bytes: room for 2 * kOsciWords words in the TENSOR mode)
 size_t osci_cells(int64_t C, int32_t gs_mode) { return gs_mode == kGsRow ? (size_t)(2 * std::max<int64_t>(C, 1)) : 2; }
+static_assert(2 * kOsciWords * 4 <= 256, "workspace of the TENSOR mode");
 
 bool bad_f32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
 
-cudaError_t run_amax(const float* W, int64_t ld, int64_t C, int64_t D, uint32_t* cells, int per_row, cudaStream_t st) {
-  const unsigned grid = (unsigned)std::min<int64_t>(C, device_sm_count() * 8);
-  launch_kernel(amax_f32_kernel, dim3(grid), dim3(256), 0, st, W, ld, C, D, cells, per_row);
+// amax cells of W0 and, unless null, W1
+cudaError_t run_amax(const float* W0, int64_t ld0, const float* W1, int64_t ld1, int64_t C, int64_t D, uint32_t* cells, int per_row,
+                     cudaStream_t st) {
+  const unsigned n = W1 ? 2 : 1;
+  if (per_row) {
+    launch_kernel(amax_rows_f32_kernel, dim3((unsigned)((C + 7) / 8), n), dim3(256), 0, st, W0, ld0, W1, ld1, C, D, cells);
+  } else {  // eight 16-byte loads per thread, until every SM has its share
+    const AmaxGrid g = amax_grid((C * D + 16383) / 16384, kOsciWords);
+    launch_kernel_cluster(amax_f32_kernel, dim3(g.ctas, n), g.cluster, dim3(512), st, W0, ld0, W1, ld1, C, D, cells);
+  }
   return cudaGetLastError();
 }
 
@@ -656,9 +695,7 @@ nvfp4_status nvfp4_osci_update(const float* W, int64_t ldw, int64_t C, int64_t D
   uint32_t* cells = static_cast<uint32_t*>(workspace);
   if (gs_mode != kGsBlock128) {
     const int per_row = gs_mode == kGsRow;
-    if (launch_zero_words(cells, (int64_t)osci_cells(C, gs_mode), st) != cudaSuccess) return NVFP4_ERR_CUDA;
-    if (run_amax(W, ldw, C, D, cells, per_row, st) != cudaSuccess) return NVFP4_ERR_CUDA;
-    if (run_amax(W_prev, D, C, D, cells + (per_row ? C : 1), per_row, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+    if (run_amax(W, ldw, W_prev, D, C, D, cells, per_row, st) != cudaSuccess) return NVFP4_ERR_CUDA;
   }
   const int64_t nb = ((D + 127) & ~(int64_t)127) >> 4;
   const dim3 grid((unsigned)((C * nb + 255) / 256));
@@ -684,9 +721,7 @@ nvfp4_status nvfp4_osci_suppress(float* W, int64_t ldw, int64_t C, int64_t D, in
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint32_t* cells = static_cast<uint32_t*>(workspace);
   if (gs_mode != kGsBlock128) {
-    const int per_row = gs_mode == kGsRow;
-    if (launch_zero_words(cells, (int64_t)osci_cells(C, gs_mode), st) != cudaSuccess) return NVFP4_ERR_CUDA;
-    if (run_amax(W, ldw, C, D, cells, per_row, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+    if (run_amax(W, ldw, nullptr, 0, C, D, cells, gs_mode == kGsRow, st) != cudaSuccess) return NVFP4_ERR_CUDA;
   }
   const int64_t nb = ((D + 127) & ~(int64_t)127) >> 4;
   const dim3 grid((unsigned)((C * nb + 255) / 256));
@@ -741,9 +776,7 @@ nvfp4_status sparse_amax(const float* W, int64_t ldw, int64_t C, int64_t D, int3
     launch_kernel(amax_groups_f32_kernel, dim3((unsigned)((C * nb + 255) / 256)), dim3(256), 0, st, W, ldw, C, D, cells);
     return cudaGetLastError() == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
   }
-  const int per_row = gs_mode == kGsRow;
-  if (launch_zero_words(cells, per_row ? C : 1, st) != cudaSuccess) return NVFP4_ERR_CUDA;
-  return run_amax(W, ldw, C, D, cells, per_row, st) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  return run_amax(W, ldw, nullptr, 0, C, D, cells, gs_mode == kGsRow, st) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 }  // namespace
 

@@ -139,3 +139,25 @@ def test_selection_with_massive_ties_and_extreme_counts():
         b.nvfp4_osci_sparse_update(dev(W), state, 0, b.GS_TENSOR)
         torch.cuda.synchronize()
         assert np.array_equal(state.idx.cpu().numpy().astype(np.int64), ref.idx), n_track
+
+
+# one CTA, as many CTAs as there are words, one more (clusters of eight, the last one part idle), the most; the maximum in the
+# first and in the last element, contiguous rows and padded ones
+@pytest.mark.parametrize("shape", [(3, 20), (512, 1024), (513, 1024), (520, 2056), (4100, 1028)])
+@pytest.mark.parametrize("pad", [0, 4])
+@pytest.mark.parametrize("where", [0, -1])
+def test_tensor_maximum_is_found_wherever_it_is(shape, pad, where):
+    b = B()
+    C, D = shape
+    rng = np.random.default_rng(C + D)
+    W0 = (rng.standard_normal((C, D), dtype=np.float32) * np.float32(0.02)).astype(np.float32)
+    W1 = W0 + rng.standard_normal((C, D), dtype=np.float32) * np.float32(1e-3)
+    W0.reshape(-1)[where] = 3.0
+    W1.reshape(-1)[where] = -5.0
+    ref = osc.Stats((C, D))
+    state = b.alloc_osci_state(dev(W0))
+    for t, W in enumerate((W0, W1)):
+        osc.update_stats(W, ref, t, orc.GS_TENSOR)
+        b.nvfp4_osci_update(dev(W, pad=pad), state, t, orc.GS_TENSOR)
+    torch.cuda.synchronize()
+    assert np.array_equal(bits(state.D_Q.cpu().numpy()), bits(ref.D_Q))
