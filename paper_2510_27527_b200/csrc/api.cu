@@ -162,41 +162,48 @@ static bool side_stream_of(const nvfp4_layer_cfg* cfg, SideStream* out) {
   return true;
 }
 
-nvfp4_status do_quantize_rows(const uint16_t* src, int64_t rows, int64_t cols, int64_t ld, int32_t rounding,
-                              uint64_t seed, uint32_t stream_id, const int32_t* keep, int64_t n_keep,
-                              const nvfp4_operand* out, uint32_t* cells, cudaStream_t st, int cells_zeroed = 0,
-                              const int32_t* excluded = nullptr, uint32_t rht_stream = 0, int compute_amax = 1,
-                              uint16_t* excl_out = nullptr, int64_t ld_excl_out = 0) {
-  if (clear_sf_padding(out, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+int rounding_of(int32_t r) { return r == NVFP4_ROUND_SR ? 1 : r == NVFP4_ROUND_SR_SCALE_UP ? 2 : 0; }
+
+QuantRowsArgs rows_args(const uint16_t* src, int64_t rows, int64_t cols, int64_t ld, int32_t rounding, uint64_t seed, uint32_t stream_id,
+                        const int32_t* keep, int64_t n_keep, const nvfp4_operand* out, uint32_t* cells, uint32_t rht_stream) {
   QuantRowsArgs a{};
-  a.excl_out = keep && excluded ? excl_out : nullptr;
-  a.ld_excl_out = ld_excl_out;
   a.src = src;
   a.rows = rows;
   a.K = keep ? n_keep : cols;
   a.cols_src = cols;
   a.ld = ld;
   a.keep = keep;
-  a.excluded = keep ? excluded : nullptr;
   a.seed = seed;
   a.stream_id = stream_id;
   a.rht_stream = rht_stream;
   a.gs_mode = out->gs_mode;
-  a.sr = rounding == NVFP4_ROUND_SR ? 1 : rounding == NVFP4_ROUND_SR_SCALE_UP ? 2 : 0;
+  a.sr = rounding_of(rounding);
   a.sf_tiled = out->sf_layout == NVFP4_SF_TILED128x4;
-  a.compute_amax = compute_amax;
-  a.cells_zeroed = cells_zeroed;
   a.gs_cells = cells;
+  a.gs_words = kTensorAmaxWords;  // (without an amax pass of its own)
   a.codes = out->codes;
   a.sf = out->sf;
   a.gscale = out->gscale;
+  return a;
+}
+
+nvfp4_status do_quantize_rows(const uint16_t* src, int64_t rows, int64_t cols, int64_t ld, int32_t rounding,
+                              uint64_t seed, uint32_t stream_id, const int32_t* keep, int64_t n_keep,
+                              const nvfp4_operand* out, uint32_t* cells, cudaStream_t st, int cells_zeroed = 0,
+                              const int32_t* excluded = nullptr, uint32_t rht_stream = 0, int compute_amax = 1,
+                              uint16_t* excl_out = nullptr, int64_t ld_excl_out = 0) {
+  if (clear_sf_padding(out, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+  QuantRowsArgs a = rows_args(src, rows, cols, ld, rounding, seed, stream_id, keep, n_keep, out, cells, rht_stream);
+  a.excl_out = keep && excluded ? excl_out : nullptr;
+  a.ld_excl_out = ld_excl_out;
+  a.excluded = keep ? excluded : nullptr;
+  a.compute_amax = compute_amax;
+  a.cells_zeroed = cells_zeroed;
   return launch_quantize_rows(a, st) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
-nvfp4_status do_quantize_transpose(const TransposeSrc& src, int from_codes, int64_t rowsK, int64_t D, int32_t rounding,
-                                   uint64_t seed, uint32_t stream_id, const nvfp4_operand* out, uint32_t* cells,
-                                   cudaStream_t st, int cells_zeroed = 0, uint32_t rht_stream = 0, int compute_amax = 1) {
-  if (clear_sf_padding(out, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+QuantTransposeArgs transpose_args(const TransposeSrc& src, int from_codes, int64_t rowsK, int64_t D, int32_t rounding, uint64_t seed,
+                                  uint32_t stream_id, const nvfp4_operand* out, uint32_t* cells, uint32_t rht_stream) {
   QuantTransposeArgs a{};
   a.from_codes = from_codes;
   a.rowsK = rowsK;
@@ -206,15 +213,36 @@ nvfp4_status do_quantize_transpose(const TransposeSrc& src, int from_codes, int6
   a.stream_id = stream_id;
   a.rht_stream = rht_stream;
   a.gs_mode = out->gs_mode;
-  a.sr = rounding == NVFP4_ROUND_SR ? 1 : rounding == NVFP4_ROUND_SR_SCALE_UP ? 2 : 0;
+  a.sr = rounding_of(rounding);
   a.sf_tiled = out->sf_layout == NVFP4_SF_TILED128x4;
-  a.compute_amax = compute_amax;
-  a.cells_zeroed = cells_zeroed;
   a.gs_cells = cells;
+  a.gs_words = kTensorAmaxWords;
   a.codes = out->codes;
   a.sf = out->sf;
   a.gscale = out->gscale;
+  return a;
+}
+
+nvfp4_status do_quantize_transpose(const TransposeSrc& src, int from_codes, int64_t rowsK, int64_t D, int32_t rounding,
+                                   uint64_t seed, uint32_t stream_id, const nvfp4_operand* out, uint32_t* cells,
+                                   cudaStream_t st, int cells_zeroed = 0, uint32_t rht_stream = 0, int compute_amax = 1) {
+  if (clear_sf_padding(out, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+  QuantTransposeArgs a = transpose_args(src, from_codes, rowsK, D, rounding, seed, stream_id, out, cells, rht_stream);
+  a.compute_amax = compute_amax;
+  a.cells_zeroed = cells_zeroed;
   return launch_quantize_transpose(a, st) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+}
+
+// The source of a re-quantization: a forward operand's codes and scales.
+TransposeSrc codes_src(const nvfp4_operand& o) {
+  TransposeSrc t{};
+  t.in_codes = o.codes;
+  t.in_sf = o.sf;
+  t.in_gscale = o.gscale;
+  t.in_K = o.K;
+  t.in_gs_mode = o.gs_mode;
+  t.in_sf_tiled = o.sf_layout == NVFP4_SF_TILED128x4;
+  return t;
 }
 
 nvfp4_status do_gemm(const nvfp4_operand* A, const nvfp4_operand* B, void* C, int32_t c_dtype, int64_t ldc,
@@ -369,8 +397,7 @@ nvfp4_status nvfp4_quantize_w16x16(const void* W_bf16, int64_t C, int64_t D, int
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint32_t* cell = static_cast<uint32_t*>(workspace);
   if (clear_sf_padding(out, st) != cudaSuccess) return NVFP4_ERR_CUDA;
-  if (launch_zero_words(cell, 1, st) != cudaSuccess) return NVFP4_ERR_CUDA;
-  if (launch_amax_tensor(static_cast<const uint16_t*>(W_bf16), C, D, ldw, cell, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+  if (launch_amax_tensor_words(static_cast<const uint16_t*>(W_bf16), C, D, ldw, cell, st) != cudaSuccess) return NVFP4_ERR_CUDA;
   return launch_quantize_w16(static_cast<const uint16_t*>(W_bf16), C, D, ldw, cell, out->codes, out->sf, out->gscale,
                              out->sf_layout == NVFP4_SF_TILED128x4, st) == cudaSuccess
              ? NVFP4_OK
@@ -413,13 +440,7 @@ nvfp4_status nvfp4_requantize_t(const nvfp4_operand* in, const void* hp_bf16, in
   if (!workspace || ws_bytes < nvfp4_quantize_workspace_bytes(D, out->gs_mode)) return NVFP4_ERR_WORKSPACE;
   if ((s = check_arch()) != NVFP4_OK) return s;
   if (D == 0 || in->R == 0) return NVFP4_OK;
-  TransposeSrc ts{};
-  ts.in_codes = in->codes;
-  ts.in_sf = in->sf;
-  ts.in_gscale = in->gscale;
-  ts.in_K = in->K;
-  ts.in_gs_mode = in->gs_mode;
-  ts.in_sf_tiled = in->sf_layout == NVFP4_SF_TILED128x4;
+  TransposeSrc ts = codes_src(*in);
   ts.row_map = row_map;
   ts.hp = static_cast<const uint16_t*>(hp_bf16);
   ts.hp_ld = hp_ld;
@@ -612,38 +633,46 @@ nvfp4_status nvfp4_linear_fwd(const void* X, int64_t ldx, const void* W, int64_t
   const uint16_t* Xp = static_cast<const uint16_t*>(X);
   const uint16_t* Wp = static_cast<const uint16_t*>(W);
   const int32_t* keep = n_out > 0 ? cfg->keep_cols : nullptr;
-  // (the 1x128 outer-block mode has no amax cells: its scales come out of the quantizers' own pass)
-  if (cfg->gs_mode != NVFP4_GS_BLOCK128 && !zero_cells(cells_x, cells_w, cells_bytes(C, cfg->gs_mode), st)) return NVFP4_ERR_CUDA;
+  // (only the masked amax pass of OutControl folds into a cell; the others write theirs)
+  if (cfg->gs_mode == NVFP4_GS_TENSOR && keep && !zero_cells(cells_x, cells_w, cells_bytes(C, cfg->gs_mode), st)) return NVFP4_ERR_CUDA;
   int amax_pass = 1;
   if (cfg->gs_mode == NVFP4_GS_TENSOR && !keep) {  // the two per-tensor maxima in one launch
-    if (launch_amax_tensor_pair(Xp, N_tok, D, ldx, cells_x, Wp, C, D, ldw, cells_w, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+    if (launch_amax_tensor_words(Xp, N_tok, D, ldx, cells_x, st, Wp, C, D, ldw, cells_w) != cudaSuccess) return NVFP4_ERR_CUDA;
     amax_pass = 0;
   }
   // with outlier channels, the quantizers also write the BF16 side operands X[:, outliers] and W[:, outliers]
   const int64_t Kh = n_out > 0 ? nvfp4_outlier_pad(n_out) : 0;
   if (n_out > 0 && (!saved->X_out || !saved->W_out)) return NVFP4_ERR_NULL;
-  // Q1 and Q2 (each with its own amax pass where it has one) are independent: the weight side runs on the side stream
-  SideStream side_store;
-  SideStream* side = side_stream_of(cfg, &side_store) ? &side_store : nullptr;
-  if (side && (cudaEventRecord(side->fork, st) != cudaSuccess || cudaStreamWaitEvent(side->stream, side->fork, 0) != cudaSuccess))
-    return NVFP4_ERR_CUDA;
-  const nvfp4_status s_x = do_quantize_rows(Xp, N_tok, D, ldx, cfg->rounding[0], cfg->seed, 1, keep, Dk, &saved->qx, cells_x, st, 1,
-                                            cfg->outlier_cols, 0, amax_pass, static_cast<uint16_t*>(saved->X_out), Kh);
-  nvfp4_status s_w;
-  if (cfg->weight_block == 1) {  // 16x16 scale squares (TENSOR mode: amax(W) is already in cells_w)
-    cudaStream_t sw = side ? side->stream : st;
-    s_w = clear_sf_padding(&saved->qw, sw) == cudaSuccess &&
-                  launch_quantize_w16(Wp, C, D, ldw, cells_w, saved->qw.codes, saved->qw.sf, saved->qw.gscale, 1, sw) == cudaSuccess
-              ? NVFP4_OK
-              : NVFP4_ERR_CUDA;
+  const QuantRowsArgs q1 = rows_args(Xp, N_tok, D, ldx, cfg->rounding[0], cfg->seed, 1, nullptr, 0, &saved->qx, cells_x, 0);
+  const QuantRowsArgs q2 = rows_args(Wp, C, D, ldw, cfg->rounding[1], cfg->seed, 2, nullptr, 0, &saved->qw, cells_w, 0);
+  if (n_out == 0 && cfg->weight_block == 0 && quantize_rows_pair_fits(q1, q2)) {
+    // Q1 and Q2 in one launch: nothing to fork. A launch, two event records and two waits cheaper on the host, and no slower on
+    // the device than a kernel on each of two streams (8192 x 1024 -> 3072: 33 against 35.5 us a call).
+    if (launch_quantize_rows_pair(q1, q2, st) != cudaSuccess) return NVFP4_ERR_CUDA;
   } else {
-    s_w = do_quantize_rows(Wp, C, D, ldw, cfg->rounding[1], cfg->seed, 2, keep, Dk, &saved->qw, cells_w, side ? side->stream : st, 1,
-                           cfg->outlier_cols, 0, amax_pass, static_cast<uint16_t*>(saved->W_out), Kh);
+    // Q1 and Q2 (each with its own amax pass where it has one) are independent: the weight side runs on the side stream
+    SideStream side_store;
+    SideStream* side = side_stream_of(cfg, &side_store) ? &side_store : nullptr;
+    if (side && (cudaEventRecord(side->fork, st) != cudaSuccess || cudaStreamWaitEvent(side->stream, side->fork, 0) != cudaSuccess))
+      return NVFP4_ERR_CUDA;
+    const nvfp4_status s_x = do_quantize_rows(Xp, N_tok, D, ldx, cfg->rounding[0], cfg->seed, 1, keep, Dk, &saved->qx, cells_x, st, 1,
+                                              cfg->outlier_cols, 0, amax_pass, static_cast<uint16_t*>(saved->X_out), Kh);
+    nvfp4_status s_w;
+    if (cfg->weight_block == 1) {  // 16x16 scale squares (TENSOR mode: amax(W) is already in cells_w)
+      cudaStream_t sw = side ? side->stream : st;
+      s_w = clear_sf_padding(&saved->qw, sw) == cudaSuccess &&
+                    launch_quantize_w16(Wp, C, D, ldw, cells_w, saved->qw.codes, saved->qw.sf, saved->qw.gscale, 1, sw) == cudaSuccess
+                ? NVFP4_OK
+                : NVFP4_ERR_CUDA;
+    } else {
+      s_w = do_quantize_rows(Wp, C, D, ldw, cfg->rounding[1], cfg->seed, 2, keep, Dk, &saved->qw, cells_w, side ? side->stream : st, 1,
+                             cfg->outlier_cols, 0, amax_pass, static_cast<uint16_t*>(saved->W_out), Kh);
+    }
+    if (side && (cudaEventRecord(side->join, side->stream) != cudaSuccess || cudaStreamWaitEvent(st, side->join, 0) != cudaSuccess))
+      return NVFP4_ERR_CUDA;
+    if (s_x != NVFP4_OK) return s_x;
+    if (s_w != NVFP4_OK) return s_w;
   }
-  if (side && (cudaEventRecord(side->join, side->stream) != cudaSuccess || cudaStreamWaitEvent(st, side->join, 0) != cudaSuccess))
-    return NVFP4_ERR_CUDA;
-  if (s_x != NVFP4_OK) return s_x;
-  if (s_w != NVFP4_OK) return s_w;
   if (n_out > 0 && cfg->outlier_format == 1) {  // outlier channels on their scaled E4M3 grids from here on
     uint32_t* cells_fp8 = static_cast<uint32_t*>(cv.take(16));
     if (!cells_fp8) return NVFP4_ERR_WORKSPACE;
@@ -680,9 +709,9 @@ static nvfp4_status bwd_dx_impl(const void* dY, int64_t lddy, const nvfp4_saved*
   uint32_t *cells3, *cells4;
   nvfp4_operand q3, q4;
   if (!carve_bwd_dx(cv, N_tok, D, C, cfg->gs_mode, &cells3, &cells4, &q3, &q4)) return NVFP4_ERR_WORKSPACE;
-  // with a shared dY amax and a TENSOR -> TENSOR re-quantization (closed-form maximum) no cell of this call is read
+  // the amax pass of dY clears nothing and a TENSOR -> TENSOR re-quantization (closed-form maximum) reads no cell
   const bool cells_unused = cfg->gs_mode == NVFP4_GS_BLOCK128 ||
-                            (dy_amax && n_out == 0 && cfg->gs_mode == NVFP4_GS_TENSOR && saved->qw.gs_mode == NVFP4_GS_TENSOR && !cfg->rht);
+                            (n_out == 0 && cfg->gs_mode == NVFP4_GS_TENSOR && saved->qw.gs_mode == NVFP4_GS_TENSOR && !cfg->rht);
   if (!cells_unused && !zero_cells(cells3, cells4, cells_bytes(D, cfg->gs_mode), st)) return NVFP4_ERR_CUDA;
   // (16x16 weight squares: W-hat^T is the forward operand transposed as it is, so this product takes no Hadamard factor)
   const uint32_t rht = cfg->rht && cfg->weight_block == 0 ? kRhtStreamDx : 0u;
@@ -693,13 +722,7 @@ static nvfp4_status bwd_dx_impl(const void* dY, int64_t lddy, const nvfp4_saved*
     if ((s = do_transpose_operand16(&saved->qw, &q4, st)) != NVFP4_OK) return s;
     return do_gemm(&q3, &q4, dX, cfg->dx_dtype, lddx, 0, cfg->dev_status, st);
   }
-  TransposeSrc ts{};
-  ts.in_codes = saved->qw.codes;
-  ts.in_sf = saved->qw.sf;
-  ts.in_gscale = saved->qw.gscale;
-  ts.in_K = saved->qw.K;
-  ts.in_gs_mode = saved->qw.gs_mode;
-  ts.in_sf_tiled = saved->qw.sf_layout == NVFP4_SF_TILED128x4;
+  TransposeSrc ts = codes_src(saved->qw);
   if (n_out == 0) {
     if ((s = do_quantize_transpose(ts, 1, C, D, cfg->rounding[3], cfg->seed, 4, &q4, cells4, st, 1, rht)) != NVFP4_OK) return s;
   } else {
@@ -722,10 +745,11 @@ static nvfp4_status bwd_dx_impl(const void* dY, int64_t lddy, const nvfp4_saved*
     qa.stream_id = 4;
     qa.rht_stream = rht;
     qa.gs_mode = cfg->gs_mode;
-    qa.sr = cfg->rounding[3] == NVFP4_ROUND_SR ? 1 : cfg->rounding[3] == NVFP4_ROUND_SR_SCALE_UP ? 2 : 0;
+    qa.sr = rounding_of(cfg->rounding[3]);
     qa.sf_tiled = 1;
     qa.cells_zeroed = 1;
     qa.gs_cells = cells4;
+    qa.gs_words = 1;
     qa.codes = q4.codes;
     qa.sf = q4.sf;
     qa.gscale = q4.gscale;
@@ -797,17 +821,11 @@ static nvfp4_status bwd_dw_impl(const void* dY, int64_t lddy, const nvfp4_saved*
   t5.bf16 = static_cast<const uint16_t*>(dY);
   t5.ld = lddy;
   const bool cells_unused = cfg->gs_mode == NVFP4_GS_BLOCK128 ||
-                            (dy_amax && cfg->gs_mode == NVFP4_GS_TENSOR && saved->qx.gs_mode == NVFP4_GS_TENSOR && !cfg->rht);
+                            (cfg->gs_mode == NVFP4_GS_TENSOR && saved->qx.gs_mode == NVFP4_GS_TENSOR && !cfg->rht);
   if (!cells_unused && !zero_cells(cells5, cells6, cells_bytes(Dk, cfg->gs_mode), st)) return NVFP4_ERR_CUDA;
   const uint32_t rht = cfg->rht ? kRhtStreamDw : 0u;
   // Q6 first: it needs nothing of dY, so it can run while another stream still computes the shared amax of dY
-  TransposeSrc t6{};
-  t6.in_codes = saved->qx.codes;
-  t6.in_sf = saved->qx.sf;
-  t6.in_gscale = saved->qx.gscale;
-  t6.in_K = saved->qx.K;
-  t6.in_gs_mode = saved->qx.gs_mode;
-  t6.in_sf_tiled = saved->qx.sf_layout == NVFP4_SF_TILED128x4;
+  TransposeSrc t6 = codes_src(saved->qx);
   if ((s = do_quantize_transpose(t6, 1, N_tok, Dk, cfg->rounding[5], cfg->seed, 6, &q6, cells6, st, 1, rht)) != NVFP4_OK) return s;
   if (dy_amax_ready && cudaStreamWaitEvent(st, dy_amax_ready, 0) != cudaSuccess) return NVFP4_ERR_CUDA;
   if ((s = do_quantize_transpose(t5, 0, N_tok, C, cfg->rounding[4], cfg->seed, 5, &q5, dy_amax ? dy_amax : cells5, st, 1, rht,
@@ -835,6 +853,40 @@ nvfp4_status nvfp4_linear_bwd_dw(const void* dY, int64_t lddy, const nvfp4_saved
   return bwd_dw_impl(dY, lddy, saved, cfg, dW, lddw, workspace, ws_bytes, stream, nullptr);
 }
 
+// Both backward products of a small call on one stream: Q3 .. Q6 in one launch. *done = false (and nothing launched) where the call
+// is too large for that or not of that kind; the caller then goes the general way. Called after the checks of nvfp4_linear_bwd.
+static nvfp4_status bwd_fused(const void* dY, int64_t lddy, const nvfp4_saved* saved, const nvfp4_layer_cfg* cfg, void* dX, int64_t lddx,
+                              void* dW, int64_t lddw, uint8_t* base, size_t need_dx, size_t need_dw, cudaStream_t st, bool* done) {
+  const int64_t N_tok = saved->N_tok, D = saved->D, C = saved->C;
+  nvfp4_status s;
+  if ((s = check_cfg(cfg, D)) != NVFP4_OK) return s;
+  if ((s = check_operand_ptrs(&saved->qw)) != NVFP4_OK || (s = check_operand_ptrs(&saved->qx)) != NVFP4_OK) return s;
+  if (saved->qw.R != C || saved->qw.K != D || saved->qx.R != N_tok || saved->qx.K != D) return NVFP4_ERR_SHAPE;
+  if (bad_matrix(dX, lddx, D, cfg->dx_dtype == NVFP4_DT_F32 ? 4 : 2) || bad_matrix(dW, lddw, D, cfg->dw_dtype == NVFP4_DT_F32 ? 4 : 2))
+    return NVFP4_ERR_ALIGN;
+  Carver cx(base, need_dx), cw(base + need_dx, need_dw);
+  uint32_t *cells3, *cells4, *cells5, *cells6;
+  nvfp4_operand q3, q4, q5, q6;
+  if (!carve_bwd_dx(cx, N_tok, D, C, cfg->gs_mode, &cells3, &cells4, &q3, &q4) ||
+      !carve_bwd_dw(cw, N_tok, D, C, cfg->gs_mode, &cells5, &cells6, &q5, &q6))
+    return NVFP4_ERR_WORKSPACE;
+  const uint16_t* dy = static_cast<const uint16_t*>(dY);
+  TransposeSrc t5{};
+  t5.bf16 = dy;
+  t5.ld = lddy;
+  const uint32_t rht_dx = cfg->rht ? kRhtStreamDx : 0u, rht_dw = cfg->rht ? kRhtStreamDw : 0u;
+  const QuantRowsArgs a3 = rows_args(dy, N_tok, C, lddy, cfg->rounding[2], cfg->seed, 3, nullptr, 0, &q3, cells3, rht_dx);
+  const QuantTransposeArgs a4 = transpose_args(codes_src(saved->qw), 1, C, D, cfg->rounding[3], cfg->seed, 4, &q4, cells4, rht_dx);
+  const QuantTransposeArgs a5 = transpose_args(t5, 0, N_tok, C, cfg->rounding[4], cfg->seed, 5, &q5, cells3, rht_dw);
+  const QuantTransposeArgs a6 = transpose_args(codes_src(saved->qx), 1, N_tok, D, cfg->rounding[5], cfg->seed, 6, &q6, cells6, rht_dw);
+  if (!quantize_bwd_fits(a3, a4, a5, a6)) return NVFP4_OK;
+  *done = true;
+  if (cfg->gs_mode == NVFP4_GS_TENSOR && launch_amax_tensor_words(dy, N_tok, C, lddy, cells3, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+  if (launch_quantize_bwd(a3, a4, a5, a6, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+  if ((s = do_gemm(&q5, &q6, dW, cfg->dw_dtype, lddw, 0, cfg->dev_status, st)) != NVFP4_OK) return s;
+  return do_gemm(&q3, &q4, dX, cfg->dx_dtype, lddx, 0, cfg->dev_status, st);
+}
+
 nvfp4_status nvfp4_linear_bwd(const void* dY, int64_t lddy, const nvfp4_saved* saved, const nvfp4_layer_cfg* cfg, void* dX,
                               int64_t lddx, void* dW, int64_t lddw, void* workspace, size_t ws_bytes, void* stream) {
   if (!dY || !saved || !cfg || !dX || !dW) return NVFP4_ERR_NULL;
@@ -860,6 +912,10 @@ nvfp4_status nvfp4_linear_bwd(const void* dY, int64_t lddy, const nvfp4_saved* s
   if (cfg->side_stream && (!cfg->ev_fork || !cfg->ev_join || !cfg->ev_aux)) return NVFP4_ERR_NULL;
   SideStream side_store;
   SideStream* side = side_stream_of(cfg, &side_store) ? &side_store : nullptr;
+  if (cfg->n_out == 0 && cfg->weight_block == 0) {
+    bool fused = false;
+    if ((s = bwd_fused(dY, lddy, saved, cfg, dX, lddx, dW, lddw, base, need_dx, need_dw, st, &fused)) != NVFP4_OK || fused) return s;
+  }
   // Q3 and Q5 quantize the same tensor with the same per-tensor scale: one amax pass serves both. Without OutControl it
   // runs before the fork. With OutControl it runs at the head of the dX chain, and the dW chain, which starts with Q6 (no
   // dY involved), waits for it only before Q5: the bandwidth-bound amax pass and the arithmetic-bound Q6 overlap.
@@ -868,8 +924,7 @@ nvfp4_status nvfp4_linear_bwd(const void* dY, int64_t lddy, const nvfp4_saved* s
   const bool amax_early = shared_amax && cfg->n_out == 0;
   if (amax_early) {
     shared = reinterpret_cast<uint32_t*>(base + need_dx + need_dw);
-    if (launch_zero_words(shared, 1, st) != cudaSuccess) return NVFP4_ERR_CUDA;
-    if (launch_amax_tensor(static_cast<const uint16_t*>(dY), N_tok, C, lddy, shared, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+    if (launch_amax_tensor_words(static_cast<const uint16_t*>(dY), N_tok, C, lddy, shared, st) != cudaSuccess) return NVFP4_ERR_CUDA;
   }
   if (side && (cudaEventRecord(side->fork, st) != cudaSuccess || cudaStreamWaitEvent(side->stream, side->fork, 0) != cudaSuccess))
     return NVFP4_ERR_CUDA;
@@ -877,8 +932,7 @@ nvfp4_status nvfp4_linear_bwd(const void* dY, int64_t lddy, const nvfp4_saved* s
   cudaEvent_t amax_ready = nullptr;
   if (shared_amax && !amax_early) {
     shared = reinterpret_cast<uint32_t*>(base + need_dx + need_dw);
-    if (launch_zero_words(shared, 1, st_dx) != cudaSuccess) return NVFP4_ERR_CUDA;
-    if (launch_amax_tensor(static_cast<const uint16_t*>(dY), N_tok, C, lddy, shared, st_dx) != cudaSuccess) return NVFP4_ERR_CUDA;
+    if (launch_amax_tensor_words(static_cast<const uint16_t*>(dY), N_tok, C, lddy, shared, st_dx) != cudaSuccess) return NVFP4_ERR_CUDA;
     if (side) {
       if (cudaEventRecord(side->amax, st_dx) != cudaSuccess) return NVFP4_ERR_CUDA;
       amax_ready = side->amax;

@@ -99,10 +99,15 @@ __device__ __forceinline__ uint32_t cells_max(const uint32_t* __restrict__ cells
   if (N == 64) v = max(v, load_cg(cells + 32 + lane));
   return __reduce_max_sync(0xFFFFFFFFu, v);
 }
+// The maximum as its readers see it: one word (folded into by atomics) or 64.
+__device__ __forceinline__ uint32_t tensor_amax_bits(const uint32_t* __restrict__ cells, int words) {
+  return words == 1 ? cells[0] : cells_max<64>(cells);
+}
 // Word of this thread's cluster <- maximum of the cluster's values m. Every thread of every CTA calls it; blockDim.x is a
-// multiple of 32 and at most 1024, the cluster (cluster_x, 1, 1) has at most 8 CTAs and there are at most N clusters.
+// multiple of 32 and at most 1024, the cluster (cluster_x, 1, 1) has at most 8 CTAs. CTA `block` of the n_blocks (whole
+// clusters, at most N of them) that share the N words.
 template <int N>
-__device__ __forceinline__ void cells_write(uint32_t m, uint32_t* cells) {
+__device__ __forceinline__ void cells_write(uint32_t m, uint32_t* cells, uint32_t block, uint32_t n_blocks) {
   __shared__ uint32_t warp_max[32];
   __shared__ uint32_t cta_max[8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
@@ -131,7 +136,7 @@ __device__ __forceinline__ void cells_write(uint32_t m, uint32_t* cells) {
     __syncthreads();
   }
   if (rank == 0 && wid == 0) {
-    const uint32_t cluster = blockIdx.x / n_rank, n_clusters = gridDim.x / n_rank;
+    const uint32_t cluster = block / n_rank, n_clusters = n_blocks / n_rank;
     m = __reduce_max_sync(0xFFFFFFFFu, lane < (int)n_rank ? cta_max[lane] : 0u);
     if (lane == 0) cells[cluster] = m;
     if (cluster == 0)

@@ -19,6 +19,9 @@ int device_sm_count();
 // kernel, so the attribute call is made once per pair.
 cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes);
 
+// Words of a tensor's maximum (cells_write / tensor_amax_bits): the 256 bytes that a workspace has for it in the TENSOR mode.
+constexpr int kTensorAmaxWords = 64;
+
 struct QuantRowsArgs {
   const uint16_t* src;  // BF16 [rows, cols_src], leading dimension ld
   int64_t rows, K, cols_src, ld;
@@ -34,7 +37,8 @@ struct QuantRowsArgs {
   int gs_mode, sr, sf_tiled;  // sr: 0 round to nearest, 1 stochastic, 2 stochastic with the block scale rounded up
   int compute_amax;    // TENSOR mode: run the amax pre-pass (0: gs_cells[0] already holds the amax bits)
   int cells_zeroed;    // the caller has already cleared gs_cells on this stream
-  uint32_t* gs_cells;  // workspace: 1 cell (TENSOR) or `rows` cells (ROW)
+  uint32_t* gs_cells;  // workspace: gs_words cells (TENSOR) or `rows` cells (ROW)
+  int gs_words;        // TENSOR without an amax pre-pass: how many words of gs_cells hold the maximum, 1 or kTensorAmaxWords
   uint8_t* codes;
   uint8_t* sf;
   float* gscale;
@@ -71,7 +75,8 @@ struct QuantTransposeArgs {
   int compute_amax;
   int cells_zeroed;        // the caller has already cleared gs_cells on this stream
   int tensor_closed_form;  // set by the launcher
-  uint32_t* gs_cells;  // 1 cell (TENSOR) or D cells (ROW)
+  uint32_t* gs_cells;  // gs_words cells (TENSOR) or D cells (ROW)
+  int gs_words;        // as in QuantRowsArgs
   uint8_t* codes;
   uint8_t* sf;
   float* gscale;
@@ -127,6 +132,15 @@ inline AmaxGrid amax_grid(int64_t wanted_ctas, int n_words) {
 
 cudaError_t launch_quantize_rows(const QuantRowsArgs& a, cudaStream_t st);
 cudaError_t launch_quantize_transpose(const QuantTransposeArgs& a, cudaStream_t st);
+// Q1 and Q2 in one launch (round to nearest, no column lists, tiled scales; TENSOR: the cells hold the maxima already). The
+// padding of the tiled scales is cleared as well.
+bool quantize_rows_pair_fits(const QuantRowsArgs& a, const QuantRowsArgs& b);
+cudaError_t launch_quantize_rows_pair(const QuantRowsArgs& a, const QuantRowsArgs& b, cudaStream_t st);
+// Q3 .. Q6 in one launch, likewise (TENSOR: the cells of q3 and q5 hold the maximum of dY), for calls small enough that launches
+// and waits between them cost more than the most economical kernel for each.
+bool quantize_bwd_fits(const QuantRowsArgs& q3, const QuantTransposeArgs& q4, const QuantTransposeArgs& q5, const QuantTransposeArgs& q6);
+cudaError_t launch_quantize_bwd(const QuantRowsArgs& q3, const QuantTransposeArgs& q4, const QuantTransposeArgs& q5,
+                                const QuantTransposeArgs& q6, cudaStream_t st);
 // amax of a contiguous-row BF16 matrix folded into cells[0] (atomic max; the cell must already hold a valid value)
 cudaError_t launch_amax_tensor(const uint16_t* src, int64_t rows, int64_t cols, int64_t ld, uint32_t* cell, cudaStream_t st);
 // p[0 .. n) = 0 by a kernel (keeps the programmatic launch chain intact where a memset node would break it)
@@ -134,6 +148,10 @@ cudaError_t launch_zero_words(uint32_t* p, int64_t n, cudaStream_t st);
 // the same for two matrices in one launch
 cudaError_t launch_amax_tensor_pair(const uint16_t* a, int64_t rows_a, int64_t cols_a, int64_t ld_a, uint32_t* cell_a, const uint16_t* b,
                                     int64_t rows_b, int64_t cols_b, int64_t ld_b, uint32_t* cell_b, cudaStream_t st);
+// amax of one or two such matrices as kTensorAmaxWords words each, written without a cleared cell
+cudaError_t launch_amax_tensor_words(const uint16_t* a, int64_t rows_a, int64_t cols_a, int64_t ld_a, uint32_t* cells_a, cudaStream_t st,
+                                     const uint16_t* b = nullptr, int64_t rows_b = 0, int64_t cols_b = 0, int64_t ld_b = 0,
+                                     uint32_t* cells_b = nullptr);
 // amax of a transposing quantizer's source (from codes or BF16) folded into cells[0]; with a non-zero rht_stream, of the
 // source after the random Hadamard transformation along its rows (the operand's K)
 cudaError_t launch_amax_transpose_src(const TransposeSrc& s, int from_codes, int64_t rowsK, int64_t D, uint32_t* cell, cudaStream_t st,
@@ -183,9 +201,9 @@ cudaError_t launch_expand_operand(const uint8_t* codes, const uint8_t* sf, int s
 cudaError_t launch_gather_cols(const uint16_t* src, int64_t ld_src, int64_t rows, const int32_t* cols, int64_t n, uint16_t* dst,
                                int64_t ld_dst, cudaStream_t st);
 
-// 16x16 weight-block recipe: Q2 with one E4M3 scale per 16x16 square (per-tensor global scale from amax_cell, round to
+// 16x16 weight-block recipe: Q2 with one E4M3 scale per 16x16 square (per-tensor global scale from kTensorAmaxWords words, round to
 // nearest), and the transposition of such an operand (codes transposed, scales re-indexed) that replaces Q4.
-cudaError_t launch_quantize_w16(const uint16_t* src, int64_t C, int64_t D, int64_t ld, const uint32_t* amax_cell, uint8_t* codes,
+cudaError_t launch_quantize_w16(const uint16_t* src, int64_t C, int64_t D, int64_t ld, const uint32_t* amax_words, uint8_t* codes,
                                 uint8_t* sf, float* gscale, int tiled, cudaStream_t st);
 cudaError_t launch_transpose_operand(const uint8_t* in_codes, const uint8_t* in_sf, int in_tiled, const float* in_gscale, int64_t C, int64_t D,
                                      uint8_t* out_codes, uint8_t* out_sf, int out_tiled, float* out_gscale, cudaStream_t st);

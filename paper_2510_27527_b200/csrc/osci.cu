@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(512) amax_f32_kernel(const float* __restrict__
     for (int64_t r = (int64_t)blockIdx.x * 16 + (threadIdx.x >> 5); r < C; r += (int64_t)gridDim.x * 16)
       m = amax_row(W + r * ld, D, (ld & 3) == 0, threadIdx.x & 31, m);
   }
-  cells_write<kOsciWords>(__float_as_uint(m), cells + blockIdx.y * kOsciWords);
+  cells_write<kOsciWords>(__float_as_uint(m), cells + blockIdx.y * kOsciWords, blockIdx.x, gridDim.x);
 }
 
 // max |w| of every row of one or two matrices, a warp per row: cells[r], cells[C + r].

@@ -17,8 +17,9 @@ namespace nvfp4 {
 // amax pre-passes. Results are bit patterns of non-negative floats combined with atomicMax (order-free, hence
 // deterministic). The cells must be zero before the launch.
 // =========================================================================================================
-__device__ __forceinline__ void amax_tensor_bf16_body(const uint16_t* __restrict__ src, int64_t rows, int64_t cols, int64_t ld,
-                                                      uint32_t* amax_bits, unsigned block, unsigned n_blocks) {
+// A thread's maximum (binary32 pattern) over its share of the tensor.
+__device__ __forceinline__ uint32_t amax_tensor_bf16_body(const uint16_t* __restrict__ src, int64_t rows, int64_t cols, int64_t ld,
+                                                          unsigned block, unsigned n_blocks) {
   // One 16-byte chunk (8 BF16) per thread per step; rows are walked through a flattened chunk index.
   const int64_t chunks_per_row = (cols + 7) >> 3;
   const int64_t total = rows * chunks_per_row;
@@ -50,33 +51,39 @@ __device__ __forceinline__ void amax_tensor_bf16_body(const uint16_t* __restrict
       for (int64_t j = c; j < cols; ++j) m = amax16x2(m, (uint32_t)p[j - c]);
     }
   }
-  uint32_t a = hmax_of_pair(bf16x2_abs_bits(m));
-#pragma unroll
-  for (int o = 16; o; o >>= 1) a = max(a, __shfl_xor_sync(0xFFFFFFFFu, a, o));
-  __shared__ uint32_t warp_max[8];
-  if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = a;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) a = max(a, warp_max[w]);
-    if (a) atomicMax(amax_bits, a << 16);  // BF16 pattern -> FP32 pattern
-  }
+  return hmax_of_pair(bf16x2_abs_bits(m)) << 16;  // BF16 pattern -> FP32 pattern
 }
 
-__global__ void __launch_bounds__(256) amax_tensor_bf16_kernel(const uint16_t* __restrict__ src, int64_t rows,
-                                                              int64_t cols, int64_t ld, uint32_t* amax_bits) {
-  pdl_prologue();
-  amax_tensor_bf16_body(src, rows, cols, ld, amax_bits, blockIdx.x, gridDim.x);
-}
-
-// Two tensors in one launch (the forward pass's X and W): the first grid_a CTAs take A, the rest take B.
-__global__ void __launch_bounds__(256) amax_tensor_pair_kernel(const uint16_t* __restrict__ a, int64_t rows_a, int64_t cols_a, int64_t ld_a,
+// max |x| of one or two tensors folded into one word each by an atomic maximum (the words are cleared before the launch): where
+// the workspace has no room for more words. The first grid_a CTAs take A, the rest take B.
+__global__ void __launch_bounds__(256) amax_tensor_bf16_kernel(const uint16_t* __restrict__ a, int64_t rows_a, int64_t cols_a, int64_t ld_a,
                                                               uint32_t* cell_a, unsigned grid_a, const uint16_t* __restrict__ b,
                                                               int64_t rows_b, int64_t cols_b, int64_t ld_b, uint32_t* cell_b) {
   pdl_prologue();
-  if (blockIdx.x < grid_a)
-    amax_tensor_bf16_body(a, rows_a, cols_a, ld_a, cell_a, blockIdx.x, grid_a);
-  else
-    amax_tensor_bf16_body(b, rows_b, cols_b, ld_b, cell_b, blockIdx.x - grid_a, gridDim.x - grid_a);
+  const bool first = blockIdx.x < grid_a;
+  uint32_t m = first ? amax_tensor_bf16_body(a, rows_a, cols_a, ld_a, blockIdx.x, grid_a)
+                     : amax_tensor_bf16_body(b, rows_b, cols_b, ld_b, blockIdx.x - grid_a, gridDim.x - grid_a);
+  m = __reduce_max_sync(0xFFFFFFFFu, m);
+  __shared__ uint32_t warp_max[8];
+  if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) m = max(m, warp_max[w]);
+    if (m) atomicMax(first ? cell_a : cell_b, m);
+  }
+}
+
+// max |x| of one or two tensors (X and W in forward) as kTensorAmaxWords words each, which need no clearing (cells_write): the
+// first grid_a CTAs take A, the rest take B. Bound by memory; for a small layer by launches, of which this saves one.
+__global__ void __launch_bounds__(512) amax_tensor_words_kernel(const uint16_t* __restrict__ a, int64_t rows_a, int64_t cols_a, int64_t ld_a,
+                                                               uint32_t* cells_a, unsigned grid_a, const uint16_t* __restrict__ b,
+                                                               int64_t rows_b, int64_t cols_b, int64_t ld_b, uint32_t* cells_b) {
+  pdl_prologue();
+  const bool first = blockIdx.x < grid_a;
+  const unsigned block = first ? blockIdx.x : blockIdx.x - grid_a, n_blocks = first ? grid_a : gridDim.x - grid_a;
+  const uint32_t m = first ? amax_tensor_bf16_body(a, rows_a, cols_a, ld_a, block, n_blocks)
+                           : amax_tensor_bf16_body(b, rows_b, cols_b, ld_b, block, n_blocks);
+  cells_write<kTensorAmaxWords>(m, first ? cells_a : cells_b, block, n_blocks);
 }
 
 // amax of a BF16 matrix over all columns EXCEPT a sorted list of excluded ones (OutControl: the outlier channels do not
@@ -352,25 +359,23 @@ __global__ void __launch_bounds__(256) amax_rows_rht_kernel(const uint16_t* __re
 //   RHT     each block is replaced by (x S) H_16 before anything else looks at it (never together with GATHER).
 // =========================================================================================================
 template <int GS, bool SR, bool TILED, bool GATHER, bool RHT>
-__global__ void __launch_bounds__(256, 4)
-quantize_rows_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld,
+__device__ __forceinline__ void quantize_rows_body(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld,
                      const int32_t* __restrict__ keep, uint64_t seed, uint32_t stream_id,
-                     const uint32_t* __restrict__ gs_cells, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
+                     const uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
                      float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, int64_t cols_src,
-                     int64_t stage_cols8, uint32_t rht_stream, int sb_up, const __grid_constant__ PhiloxKeys pk) {
-  pdl_prologue();
+                     int64_t stage_cols8, uint32_t rht_stream, int sb_up, const PhiloxKeys& pk, uint32_t bx) {
   constexpr int NB = 4;  // inner blocks per thread; all loads are issued before any arithmetic
   extern __shared__ uint16_t row_stage[];  // GATHER only: the source rows this CTA touches, [n_rows][cols_src8]
   const int64_t Kp = (K + 127) & ~(int64_t)127;
   const int64_t K16 = (K + 15) & ~(int64_t)15;
   const int64_t nb = Kp >> 4;  // inner blocks per operand row (multiple of 8)
   const int64_t total = rows * nb;
-  const int64_t cta_base = (int64_t)blockIdx.x * (256 * NB) + threadIdx.x;
+  const int64_t cta_base = (int64_t)bx * (256 * NB) + threadIdx.x;
   // GATHER (OutControl compaction): the CTA's blocks cover a few whole or partial source rows; copy those rows to
   // shared memory with coalesced 16-byte loads, then pick the kept columns from there.
   int64_t stage_row0 = 0;
   if (GATHER && stage_cols8 > 0) {
-    const int64_t first = (int64_t)blockIdx.x * (256 * NB);
+    const int64_t first = (int64_t)bx * (256 * NB);
     const int64_t last = min(first + 256 * NB, total) - 1;
     stage_row0 = first / nb;
     const int64_t n_rows = last / nb - stage_row0 + 1;
@@ -478,8 +483,8 @@ quantize_rows_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, 
 
     float Sg_t = 1.0f;
     if (GS == kGsTensor) {
-      Sg_t = global_scale_from_amax(__uint_as_float(gs_cells[0]));
-      if (blockIdx.x == 0 && threadIdx.x == 0) gscale[0] = Sg_t;
+      Sg_t = global_scale_from_amax(__uint_as_float(tensor_amax_bits(gs_cells, gs_words)));
+      if (bx == 0 && threadIdx.x == 0) gscale[0] = Sg_t;
     }
 
   #pragma unroll
@@ -557,12 +562,24 @@ quantize_rows_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, 
       }
     }
   };
-  const bool full = !GATHER && K32 == (uint32_t)Kp && (int64_t)blockIdx.x * (256 * NB) + 256 * NB <= total;  // CTA-uniform
+  const bool full = !GATHER && K32 == (uint32_t)Kp && (int64_t)bx * (256 * NB) + 256 * NB <= total;  // CTA-uniform
   if (full)
     body(std::true_type{});
   else
     body(std::false_type{});
 }
+
+template <int GS, bool SR, bool TILED, bool GATHER, bool RHT>
+__global__ void __launch_bounds__(256, 4)
+quantize_rows_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld,
+                     const int32_t* __restrict__ keep, uint64_t seed, uint32_t stream_id,
+                     const uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
+                     float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, int64_t cols_src,
+                     int64_t stage_cols8, uint32_t rht_stream, int sb_up, const __grid_constant__ PhiloxKeys pk) {
+  pdl_prologue();
+  quantize_rows_body<GS, SR, TILED, GATHER, RHT>(src, rows, K, ld, keep, seed, stream_id, gs_cells, gs_words, codes, sf, gscale, div_mul, div_shift, wide_loads, cols_src, stage_cols8, rht_stream, sb_up, pk, blockIdx.x);
+}
+
 
 // =========================================================================================================
 // Row-axis quantize from BF16, four ADJACENT inner blocks per thread (64 consecutive k of one operand row).
@@ -577,20 +594,18 @@ quantize_rows_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, 
 // No column list (OutControl's compaction keeps the kernel above).
 // =========================================================================================================
 template <int GS, int RMODE, bool TILED, bool RHT>
-__global__ void __launch_bounds__(256, 3)
-quantize_rows4_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld, uint64_t seed, uint32_t stream_id,
-                      const uint32_t* __restrict__ gs_cells, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
+__device__ __forceinline__ void quantize_rows4_body(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld, uint64_t seed, uint32_t stream_id,
+                      const uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
                       float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, uint32_t rht_stream,
-                      const __grid_constant__ PhiloxKeys pk) {
-  pdl_prologue();
+                      const PhiloxKeys& pk, uint32_t bx) {
   constexpr bool SR = RMODE != 0;
   const uint32_t K32 = (uint32_t)K;
   const uint32_t Kp = (K32 + 127u) & ~127u;
   const uint32_t K16 = (K32 + 15u) & ~15u;
   const uint32_t nu = Kp >> 6;  // units (four inner blocks) per operand row: even, as rows are padded to 128
   const int64_t total = rows * (int64_t)nu;
-  const int64_t unit = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  const bool full = K32 == Kp && (int64_t)blockIdx.x * 256 + 256 <= total;  // CTA-uniform: every block exists and is whole
+  const int64_t unit = (int64_t)bx * 256 + threadIdx.x;
+  const bool full = K32 == Kp && (int64_t)bx * 256 + 256 <= total;  // CTA-uniform: every block exists and is whole
 
   auto body = [&](auto full_tag) {
     constexpr bool FULL = decltype(full_tag)::value;
@@ -680,7 +695,7 @@ quantize_rows4_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K,
       Sg = global_scale_from_amax(__uint_as_float(gs_cells[r]));
       if (active && q == 0) gscale[r] = Sg;
     } else {
-      Sg = global_scale_from_amax(__uint_as_float(gs_cells[0]));
+      Sg = global_scale_from_amax(__uint_as_float(tensor_amax_bits(gs_cells, gs_words)));
       if (unit == 0) gscale[0] = Sg;
     }
 
@@ -727,6 +742,17 @@ quantize_rows4_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K,
   else
     body(std::false_type{});
 }
+
+template <int GS, int RMODE, bool TILED, bool RHT>
+__global__ void __launch_bounds__(256, 3)
+quantize_rows4_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld, uint64_t seed, uint32_t stream_id,
+                      const uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
+                      float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, uint32_t rht_stream,
+                      const __grid_constant__ PhiloxKeys pk) {
+  pdl_prologue();
+  quantize_rows4_body<GS, RMODE, TILED, RHT>(src, rows, K, ld, seed, stream_id, gs_cells, gs_words, codes, sf, gscale, div_mul, div_shift, wide_loads, rht_stream, pk, blockIdx.x);
+}
+
 
 // =========================================================================================================
 // Transposing quantizers. Operand element (d, k) = source element (row k, column d).
@@ -1002,12 +1028,10 @@ quantize_transpose_generic_kernel(TransposeSrc s, int64_t rowsK, int64_t D, uint
 //   RMODE  0 round to nearest, 1 stochastic rounding, 2 stochastic rounding with the block scale rounded up.
 // =========================================================================================================
 template <int SRC, int GS, int RMODE, bool TILED, bool RHT, bool AMAX_ONLY>
-__global__ void __launch_bounds__(256, 3)
-quantize_transpose_kernel(TransposeSrc s, int64_t rowsK, int64_t D, uint64_t seed, uint32_t stream_id,
-                          uint32_t* __restrict__ gs_cells, int tensor_closed_form, uint8_t* __restrict__ codes,
+__device__ __forceinline__ void quantize_transpose_body(TransposeSrc s, int64_t rowsK, int64_t D, uint64_t seed, uint32_t stream_id,
+                          uint32_t* __restrict__ gs_cells, int gs_words, int tensor_closed_form, uint8_t* __restrict__ codes,
                           uint8_t* __restrict__ sf, float* __restrict__ gscale, uint32_t rht_stream,
-                          const __grid_constant__ PhiloxKeys pk) {
-  pdl_prologue();
+                          const PhiloxKeys& pk, uint32_t bx, uint32_t by) {
   constexpr bool SR = RMODE != 0;
   __shared__ __align__(16) uint32_t tile[128 * 32];
   __shared__ float sg_row[128];
@@ -1021,12 +1045,12 @@ quantize_transpose_kernel(TransposeSrc s, int64_t rowsK, int64_t D, uint64_t see
   const uint32_t Kp = (K + 127u) & ~127u;
   const uint32_t nb = Kp >> 4;
   const uint32_t nbp4 = ((nb + 15u) & ~15u) >> 2;  // 512-byte scale tiles per 128-row tile of the output operand
-  const uint32_t k_base = blockIdx.x * 128u;
-  const uint32_t d_base = blockIdx.y * 64u;
+  const uint32_t k_base = bx * 128u;
+  const uint32_t d_base = by * 64u;
   const int tid = threadIdx.x;
   uint4 sw = make_uint4(0, 0, 0, 0);  // the tile's 128 sign bits (k_base is a multiple of 128)
   if (RHT) {
-    sw = rht_sign_words(seed, rht_stream, (uint64_t)blockIdx.x);
+    sw = rht_sign_words(seed, rht_stream, (uint64_t)bx);
     // rows past K rounded up to 16 are layout padding: no signs there, so that they stay +0 and encode as zero bytes
     const int32_t live = (int32_t)((K + 15u) & ~15u) - (int32_t)k_base;
     if (live < 128) {
@@ -1186,23 +1210,23 @@ quantize_transpose_kernel(TransposeSrc s, int64_t rowsK, int64_t D, uint64_t see
 #pragma unroll
       for (int j = 0; j < 8; ++j) g = fmaxf(g, blk_amax[j][2 * dp + c]);
       Sg[c] = global_scale_from_amax(g);
-      if (d0 + c < D32 && kb == 0 && k_base < K) gscale[(size_t)o[c] * (Kp >> 7) + blockIdx.x] = Sg[c];
+      if (d0 + c < D32 && kb == 0 && k_base < K) gscale[(size_t)o[c] * (Kp >> 7) + bx] = Sg[c];
     }
   } else if (GS == kGsRow) {
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       Sg[c] = global_scale_from_amax(d0 + c < D32 ? __uint_as_float(gs_cells[o[c]]) : 0.0f);
-      if (d0 + c < D32 && kb == 0 && blockIdx.x == 0) gscale[o[c]] = Sg[c];
+      if (d0 + c < D32 && kb == 0 && bx == 0) gscale[o[c]] = Sg[c];
     }
   } else {
     // (tensor_closed_form == 2: the cell carries nothing and may be uninitialised)
-    float amax = tensor_closed_form == 2 ? 0.0f : __uint_as_float(gs_cells[0]);
+    float amax = tensor_closed_form == 2 ? 0.0f : __uint_as_float(tensor_amax_bits(gs_cells, gs_words));
     // TENSOR -> TENSOR re-quantization: the aligned tensor's maximum is float32(2688 * S_global) of the forward
     // operand (its largest block has scale 448 and a magnitude-6 element); gs_cells[0] then only covers BF16 rows.
     if (SRC == 1 && tensor_closed_form) amax = fmaxf(amax, __fmul_rn(2688.0f, s.in_gscale[0]));
     if (s.closed_form_sg) amax = fmaxf(amax, __fmul_rn(2688.0f, s.closed_form_sg[0]));
     Sg[0] = Sg[1] = global_scale_from_amax(amax);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) gscale[0] = Sg[0];
+    if (bx == 0 && by == 0 && tid == 0) gscale[0] = Sg[0];
   }
   const uint32_t K16 = (K + 15u) & ~15u;
   const uint32_t k0 = k_base + kb * 16u;
@@ -1238,6 +1262,17 @@ quantize_transpose_kernel(TransposeSrc s, int64_t rowsK, int64_t D, uint64_t see
   }
 }
 
+template <int SRC, int GS, int RMODE, bool TILED, bool RHT, bool AMAX_ONLY>
+__global__ void __launch_bounds__(256, 3)
+quantize_transpose_kernel(TransposeSrc s, int64_t rowsK, int64_t D, uint64_t seed, uint32_t stream_id,
+                          uint32_t* __restrict__ gs_cells, int gs_words, int tensor_closed_form, uint8_t* __restrict__ codes,
+                          uint8_t* __restrict__ sf, float* __restrict__ gscale, uint32_t rht_stream,
+                          const __grid_constant__ PhiloxKeys pk) {
+  pdl_prologue();
+  quantize_transpose_body<SRC, GS, RMODE, TILED, RHT, AMAX_ONLY>(s, rowsK, D, seed, stream_id, gs_cells, gs_words, tensor_closed_form, codes, sf, gscale, rht_stream, pk, blockIdx.x, blockIdx.y);
+}
+
+
 // =========================================================================================================
 // Column-axis quantize from BF16 without a shared-memory transposition (Q5 of Sec. 2.3: the operand is dY^T, its blocks
 // run along the tokens), for the TENSOR and ROW scale modes. A lane owns FOUR neighbouring source columns (= operand rows)
@@ -1262,19 +1297,17 @@ __device__ __forceinline__ uint2 ld_nc_8(const uint16_t* p) {
 }
 
 template <int GS, int RMODE, bool TILED, bool RHT, bool AMAX_ONLY>
-__global__ void __launch_bounds__(128, 4)
-quantize_cols4_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, uint32_t ld, uint64_t seed, uint32_t stream_id,
-                      uint32_t rht_stream, uint32_t* __restrict__ gs_cells, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
-                      float* __restrict__ gscale, const __grid_constant__ PhiloxKeys pk) {
+__device__ __forceinline__ void quantize_cols4_body(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, uint32_t ld, uint64_t seed, uint32_t stream_id,
+                      uint32_t rht_stream, uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes,
+                      uint8_t* __restrict__ sf, float* __restrict__ gscale, const PhiloxKeys& pk, uint32_t bx, uint32_t by, uint32_t tid) {
   static_assert(GS != kGsBlock128, "the outer-block mode has a kernel of its own");
-  pdl_prologue();
   constexpr bool SR = RMODE != 0;
   const uint32_t Kp = (K + 127u) & ~127u;
   const uint32_t K16 = (K + 15u) & ~15u;
   const uint32_t nb = Kp >> 4;
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint32_t d0 = blockIdx.y * 64u + (lane & 15u) * 4u;                          // first of this lane's operand rows
-  const uint32_t k_start = blockIdx.x * 512u + warp * 128u + (lane >> 4) * 64u;      // first of its 64 k
+  const uint32_t lane = tid & 31u, warp = tid >> 5;
+  const uint32_t d0 = by * 64u + (lane & 15u) * 4u;                          // first of this lane's operand rows
+  const uint32_t k_start = bx * 512u + warp * 128u + (lane >> 4) * 64u;      // first of its 64 k
   const bool live = d0 < D && k_start < Kp;  // (all four rows exist or none: D is a multiple of 4)
   const uint16_t* p = src + (size_t)k_start * ld + d0;
 
@@ -1287,8 +1320,8 @@ quantize_cols4_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, 
         if (live && k_start == 0) gscale[d0 + c] = Sg[c];
       }
     } else {
-      Sg[0] = Sg[1] = Sg[2] = Sg[3] = global_scale_from_amax(__uint_as_float(gs_cells[0]));
-      if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) gscale[0] = Sg[0];
+      Sg[0] = Sg[1] = Sg[2] = Sg[3] = global_scale_from_amax(__uint_as_float(tensor_amax_bits(gs_cells, gs_words)));
+      if (bx == 0 && by == 0 && tid == 0) gscale[0] = Sg[0];
     }
   }
   // the 64 sign bits of this lane's k range (one half of a 128-group's generator block)
@@ -1385,6 +1418,16 @@ quantize_cols4_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, 
   }
 }
 
+template <int GS, int RMODE, bool TILED, bool RHT, bool AMAX_ONLY>
+__global__ void __launch_bounds__(128, 4)
+quantize_cols4_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, uint32_t ld, uint64_t seed, uint32_t stream_id,
+                      uint32_t rht_stream, uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes,
+                      uint8_t* __restrict__ sf, float* __restrict__ gscale, const __grid_constant__ PhiloxKeys pk) {
+  pdl_prologue();
+  quantize_cols4_body<GS, RMODE, TILED, RHT, AMAX_ONLY>(src, K, D, ld, seed, stream_id, rht_stream, gs_cells, gs_words, codes, sf, gscale, pk, blockIdx.x, blockIdx.y, threadIdx.x);
+}
+
+
 // The same for the 1 x 128 outer block (BLOCK128), where the scale of a block depends on all 128 k of its group: a lane owns
 // TWO neighbouring source columns and keeps its 64 source rows in registers (one 32-bit word per row), so the data is read
 // once; the two lanes of a group exchange the group maximum with one shuffle. A warp instruction covers two source rows of
@@ -1392,18 +1435,16 @@ quantize_cols4_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, 
 // for their maxima and once more when they are quantized (80 floating-point operations per block and pass; holding the 128
 // transformed values beside the 64 raw words does not fit the register file at a useful occupancy).
 template <int RMODE, bool TILED, bool RHT>
-__global__ void __launch_bounds__(128, 3)
-quantize_cols2_block128_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, uint32_t ld, uint64_t seed, uint32_t stream_id,
+__device__ __forceinline__ void quantize_cols2_block128_body(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, uint32_t ld, uint64_t seed, uint32_t stream_id,
                                uint32_t rht_stream, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf, float* __restrict__ gscale,
-                               const __grid_constant__ PhiloxKeys pk) {
-  pdl_prologue();
+                               const PhiloxKeys& pk, uint32_t bx, uint32_t by, uint32_t tid) {
   constexpr bool SR = RMODE != 0;
   const uint32_t Kp = (K + 127u) & ~127u;
   const uint32_t K16 = (K + 15u) & ~15u;
   const uint32_t nb = Kp >> 4;
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint32_t d0 = blockIdx.y * 32u + (lane & 15u) * 2u;
-  const uint32_t k_start = blockIdx.x * 512u + warp * 128u + (lane >> 4) * 64u;
+  const uint32_t lane = tid & 31u, warp = tid >> 5;
+  const uint32_t d0 = by * 32u + (lane & 15u) * 2u;
+  const uint32_t k_start = bx * 512u + warp * 128u + (lane >> 4) * 64u;
   const bool live = d0 < D && k_start < Kp;  // (both rows exist or none: D is even)
   const uint16_t* p = src + (size_t)k_start * ld + d0;
 
@@ -1501,6 +1542,16 @@ quantize_cols2_block128_kernel(const uint16_t* __restrict__ src, uint32_t K, uin
     *reinterpret_cast<uint32_t*>(sf + off) = sfw[c];
   }
 }
+
+template <int RMODE, bool TILED, bool RHT>
+__global__ void __launch_bounds__(128, 3)
+quantize_cols2_block128_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, uint32_t ld, uint64_t seed, uint32_t stream_id,
+                               uint32_t rht_stream, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf, float* __restrict__ gscale,
+                               const __grid_constant__ PhiloxKeys pk) {
+  pdl_prologue();
+  quantize_cols2_block128_body<RMODE, TILED, RHT>(src, K, D, ld, seed, stream_id, rht_stream, codes, sf, gscale, pk, blockIdx.x, blockIdx.y, threadIdx.x);
+}
+
 
 // Transposing re-quantize of a forward operand (Q4, Q6 of Sec. 2.3) without a shared-memory transposition, for the TENSOR
 // and ROW scale modes of the output. A lane owns EIGHT neighbouring source columns (one 32-bit word of codes per source row,
@@ -1646,29 +1697,121 @@ requantize_cols8_kernel(const TransposeSrc s, uint32_t K, uint32_t D, uint32_t s
 }
 
 // =========================================================================================================
+// Several quantizers of one layer call in one launch. A launch costs the host about 3 us and the stream a serial point; up to a
+// few thousand tokens that is more than the quantizers themselves take. The CTAs of the jobs are numbered one after another and
+// run the bodies above; they also clear the padding of the tiled scales (rows to 128, k blocks to 16), which separate launches
+// leave to a memset before each. Forward of a layer (both quantizers), us before and after, kept buffers: 256 x 512 -> 512 33 / 18,
+// 1000 x 1000 -> 1416 34 / 18, 8192 x 1024 -> 3072 35.5 / 33, with 1x128 groups 60 / 58.
+// =========================================================================================================
+struct RowsJob {
+  const uint16_t* src;
+  int64_t rows, K, ld;
+  const uint32_t* gs_cells;
+  uint8_t *codes, *sf;
+  float* gscale;
+  int gs_words, wide_loads;
+  uint32_t stream_id, rht_stream, div_mul, div_shift, blocks;
+};
+struct TransposeJob {
+  TransposeSrc s;
+  int64_t rowsK, D;
+  uint32_t* gs_cells;
+  uint8_t *codes, *sf;
+  float* gscale;
+  int gs_words, closed_form;
+  uint32_t stream_id, rht_stream, grid_x, blocks;
+};
+
+// Zeroes the words of an operand's tiled scales [R, 16 nb] that belong to no row or k block; CTA `block` of n_blocks.
+__device__ __forceinline__ void clear_scale_padding(uint8_t* sf, uint32_t R, uint32_t nb, uint32_t block, uint32_t n_blocks) {
+  if ((R & 127u) == 0 && (nb & 15u) == 0) return;
+  const uint32_t nbp4 = ((nb + 15u) & ~15u) >> 2, tiles = ((R + 127u) >> 7) * nbp4;  // 512-byte tiles of 128 rows x 4 k blocks
+  const uint32_t t = threadIdx.x & 127u, r = (t & 3u) * 32u + (t >> 2);              // the row whose word is the tile's t-th
+  for (uint32_t tile = block * 2u + (threadIdx.x >> 7); tile < tiles; tile += n_blocks * 2u) {
+    const uint32_t rt = tile / nbp4, kt = tile - rt * nbp4;
+    if (rt * 128u + r >= R || kt * 4u >= nb) *reinterpret_cast<uint32_t*>(sf + (size_t)tile * 512u + t * 4u) = 0u;
+  }
+}
+
+// Q1 and Q2 (round to nearest along the rows, tiled scales).
+template <int GS>
+__global__ void __launch_bounds__(256, 4)
+quantize_rows_pair_kernel(const __grid_constant__ RowsJob a, const __grid_constant__ RowsJob b) {
+  pdl_prologue();
+  const bool first = blockIdx.x < a.blocks;
+  const RowsJob& j = first ? a : b;
+  const uint32_t bx = first ? blockIdx.x : blockIdx.x - a.blocks;
+  const PhiloxKeys no_keys{};
+  quantize_rows_body<GS, false, true, false, false>(j.src, j.rows, j.K, j.ld, nullptr, 0ull, j.stream_id, j.gs_cells, j.gs_words, j.codes, j.sf,
+                                                    j.gscale, j.div_mul, j.div_shift, j.wide_loads, 0, 0, 0u, 0, no_keys, bx);
+  clear_scale_padding(j.sf, (uint32_t)j.rows, (((uint32_t)j.K + 127u) & ~127u) >> 4, bx, j.blocks);
+}
+
+// Q3 .. Q6 of the two backward products (stochastic rounding, tiled scales).
+template <int GS, bool RHT>
+__global__ void __launch_bounds__(256, 3)
+quantize_bwd_kernel(const __grid_constant__ RowsJob q3, const __grid_constant__ TransposeJob q4, const __grid_constant__ TransposeJob q5,
+                    const __grid_constant__ TransposeJob q6, uint64_t seed, const __grid_constant__ PhiloxKeys pk) {
+  pdl_prologue();
+  uint32_t bx = blockIdx.x;
+  if (bx < q3.blocks) {
+    quantize_rows4_body<GS, 1, true, RHT>(q3.src, q3.rows, q3.K, q3.ld, seed, q3.stream_id, q3.gs_cells, q3.gs_words, q3.codes, q3.sf, q3.gscale,
+                                          q3.div_mul, q3.div_shift, q3.wide_loads, q3.rht_stream, pk, bx);
+    clear_scale_padding(q3.sf, (uint32_t)q3.rows, (((uint32_t)q3.K + 127u) & ~127u) >> 4, bx, q3.blocks);
+    return;
+  }
+  bx -= q3.blocks;
+  if (bx < q5.blocks) {
+    quantize_transpose_body<0, GS, 1, true, RHT, false>(q5.s, q5.rowsK, q5.D, seed, q5.stream_id, q5.gs_cells, q5.gs_words, q5.closed_form, q5.codes,
+                                                        q5.sf, q5.gscale, q5.rht_stream, pk, bx % q5.grid_x, bx / q5.grid_x);
+    clear_scale_padding(q5.sf, (uint32_t)q5.D, (((uint32_t)q5.rowsK + 127u) & ~127u) >> 4, bx, q5.blocks);
+    return;
+  }
+  bx -= q5.blocks;
+  const bool is6 = bx < q6.blocks;
+  const TransposeJob& q = is6 ? q6 : q4;
+  if (!is6) bx -= q6.blocks;
+  quantize_transpose_body<1, GS, 1, true, RHT, false>(q.s, q.rowsK, q.D, seed, q.stream_id, q.gs_cells, q.gs_words, q.closed_form, q.codes, q.sf,
+                                                      q.gscale, q.rht_stream, pk, bx % q.grid_x, bx / q.grid_x);
+  clear_scale_padding(q.sf, (uint32_t)q.D, (((uint32_t)q.rowsK + 127u) & ~127u) >> 4, bx, q.blocks);
+}
+
+// =========================================================================================================
 // Host-side launchers
 // =========================================================================================================
+// quantize_bwd_kernel up to so many of its CTAs per SM. Backward of a layer, one launch / a kernel per quantizer on two streams, us,
+// kept buffers. TENSOR: 256 x 512 -> 512 (under 1 CTA per SM) 21 / 30, 1024 x 1024 -> 3072 (7.4) 31 / 47, 2048 x 1024 -> 3072
+// (12.1) 42 / 58, 512 x 4096 -> 4096 (18.2) 60 / 76, but 4096 x 1024 -> 3072 (21.6) 68 / 62: from there on the register-transposing
+// kernels and the overlap of one product's quantizers with the other product win. BLOCK128, whose products take longer and so
+// have more to overlap, without / with the Hadamard transformation: 1024 x 1024 -> 1024 (3.0) 24 / 28, 27 / 28; 1000 x 1000 ->
+// 1416 (4.0) 34 / 38, 36 / 48; 1024 x 1024 -> 3072 (7.4) 41 / 38, 45 / 43.
+constexpr int kFusedBwdCtasTensor = 19, kFusedBwdCtasBlock128 = 6;
 static inline unsigned blocks_for(int64_t n, int per) { return (unsigned)((n + per - 1) / per); }
+
+// Constants for n / d without a hardware division, n < total + slack (n / d = (t + ((n - t) >> 1)) >> shift, t = mulhi(mul, n);
+// mul = 0: a shift alone, or with shift = 2^32 - 1 a plain division).
+static void division_constants(int64_t total, int64_t slack, uint64_t d, uint32_t& mul, uint32_t& shift) {
+  mul = 0;
+  shift = 0xFFFFFFFFu;
+  if (total + slack >= (int64_t)1 << 31) return;
+  uint32_t sft = 0;
+  while (((uint64_t)1 << sft) < d) ++sft;
+  if ((d & (d - 1)) == 0) {
+    shift = sft;
+  } else {
+    mul = (uint32_t)((((uint64_t)1 << 32) * (((uint64_t)1 << sft) - d)) / d + 1);
+    shift = sft - 1;
+  }
+}
 
 template <int GS, bool SR, bool TILED>
 static cudaError_t launch_rows_g(const QuantRowsArgs& a, cudaStream_t st) {
   const int64_t Kp = (a.K + 127) & ~(int64_t)127;
   const int64_t total = a.rows * (Kp >> 4);
   const unsigned grid = blocks_for(total, 256 * 4);
-  // constants for gid / nb without a hardware division (n / d = (t + ((n - t) >> 1)) >> (s - 1), t = mulhi(m, n))
-  uint32_t div_mul = 0, div_shift = 0xFFFFFFFFu;
   const uint64_t d = (uint64_t)(Kp >> 4);
-  if (total + 1024 < (int64_t)1 << 31) {
-    if ((d & (d - 1)) == 0) {
-      div_shift = 0;
-      while (((uint64_t)1 << div_shift) < d) ++div_shift;
-    } else {
-      uint32_t sft = 0;
-      while (((uint64_t)1 << sft) < d) ++sft;
-      div_mul = (uint32_t)((((uint64_t)1 << 32) * (((uint64_t)1 << sft) - d)) / d + 1);
-      div_shift = sft - 1;
-    }
-  }
+  uint32_t div_mul, div_shift;
+  division_constants(total, 1024, d, div_mul, div_shift);
   const int wide_loads = ((reinterpret_cast<uintptr_t>(a.src) & 31u) == 0 && (a.ld & 15) == 0) ? 1 : 0;
   if (a.keep) {
     // rows a CTA can touch: its 1024 blocks span at most 1024 / nb + 2 rows; stage them if they fit in shared memory
@@ -1684,13 +1827,13 @@ static cudaError_t launch_rows_g(const QuantRowsArgs& a, cudaStream_t st) {
       if (e != cudaSuccess) return e;
     }
     launch_kernel(quantize_rows_kernel<GS, SR, TILED, true, false>, dim3(grid), dim3(256), smem, st, a.src, a.rows, a.K, a.ld, a.keep, a.seed,
-                  a.stream_id, a.gs_cells, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, stage_cols8, 0u, a.sr == 2, make_philox_keys(a.seed));
+                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, stage_cols8, 0u, a.sr == 2, make_philox_keys(a.seed));
   } else if (a.rht_stream) {
     launch_kernel(quantize_rows_kernel<GS, SR, TILED, false, true>, dim3(grid), dim3(256), 0, st, a.src, a.rows, a.K, a.ld, nullptr, a.seed,
-                  a.stream_id, a.gs_cells, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, (int64_t)0, a.rht_stream, a.sr == 2, make_philox_keys(a.seed));
+                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, (int64_t)0, a.rht_stream, a.sr == 2, make_philox_keys(a.seed));
   } else {
     launch_kernel(quantize_rows_kernel<GS, SR, TILED, false, false>, dim3(grid), dim3(256), 0, st, a.src, a.rows, a.K, a.ld, nullptr, a.seed,
-                  a.stream_id, a.gs_cells, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, (int64_t)0, 0u, a.sr == 2, make_philox_keys(a.seed));
+                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, (int64_t)0, 0u, a.sr == 2, make_philox_keys(a.seed));
   }
   return cudaGetLastError();
 }
@@ -1702,25 +1845,15 @@ static cudaError_t launch_rows4(const QuantRowsArgs& a, cudaStream_t st) {
   const uint64_t d = (uint64_t)(Kp >> 6);  // units per row
   const int64_t total = a.rows * (int64_t)d;
   const unsigned grid = blocks_for(total, 256);
-  uint32_t div_mul = 0, div_shift = 0xFFFFFFFFu;
-  if (total + 256 < (int64_t)1 << 31) {
-    if ((d & (d - 1)) == 0) {
-      div_shift = 0;
-      while (((uint64_t)1 << div_shift) < d) ++div_shift;
-    } else {
-      uint32_t sft = 0;
-      while (((uint64_t)1 << sft) < d) ++sft;
-      div_mul = (uint32_t)((((uint64_t)1 << 32) * (((uint64_t)1 << sft) - d)) / d + 1);
-      div_shift = sft - 1;
-    }
-  }
+  uint32_t div_mul, div_shift;
+  division_constants(total, 256, d, div_mul, div_shift);
   const int wide_loads = ((reinterpret_cast<uintptr_t>(a.src) & 31u) == 0 && (a.ld & 15) == 0) ? 1 : 0;
   if (a.rht_stream)
     launch_kernel(quantize_rows4_kernel<GS, RMODE, TILED, true>, dim3(grid), dim3(256), 0, st, a.src, a.rows, a.K, a.ld, a.seed, a.stream_id,
-                  a.gs_cells, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.rht_stream, make_philox_keys(a.seed));
+                  a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.rht_stream, make_philox_keys(a.seed));
   else
     launch_kernel(quantize_rows4_kernel<GS, RMODE, TILED, false>, dim3(grid), dim3(256), 0, st, a.src, a.rows, a.K, a.ld, a.seed, a.stream_id,
-                  a.gs_cells, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, 0u, make_philox_keys(a.seed));
+                  a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, 0u, make_philox_keys(a.seed));
   return cudaGetLastError();
 }
 
@@ -1740,7 +1873,9 @@ static cudaError_t launch_rows_r(const QuantRowsArgs& a, cudaStream_t st) {
   return a.sr ? launch_rows_t<GS, true>(a, st) : launch_rows_t<GS, false>(a, st);
 }
 
-static cudaError_t launch_quantize_rows_impl(const QuantRowsArgs& a, cudaStream_t st, bool& side_copy_done) {
+static cudaError_t launch_quantize_rows_impl(const QuantRowsArgs& a0, cudaStream_t st, bool& side_copy_done) {
+  QuantRowsArgs a = a0;
+  if (a.compute_amax) a.gs_words = 1;
   if (a.rows == 0 || a.K == 0) return cudaSuccess;
   if (a.rows >= ((int64_t)1 << 31) || a.cols_src >= ((int64_t)1 << 31) || a.ld >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
   cudaError_t e;
@@ -1760,8 +1895,13 @@ static cudaError_t launch_quantize_rows_impl(const QuantRowsArgs& a, cudaStream_
   }
   if (a.gs_mode == kGsTensor) {
     if (a.compute_amax) {
+      if (!a.keep) {
+        if ((e = launch_amax_tensor_words(a.src, a.rows, a.cols_src, a.ld, a.gs_cells, st)) != cudaSuccess) return e;
+        a.gs_words = kTensorAmaxWords;
+        return launch_rows_r<kGsTensor>(a, st);
+      }
       if (!a.cells_zeroed && (e = launch_zero_words(a.gs_cells, 1, st)) != cudaSuccess) return e;
-      if (a.keep && a.excluded && (a.ld & 7) == 0 && a.cols_src <= 20 * 1024) {
+      if (a.excluded && (a.ld & 7) == 0 && a.cols_src <= 20 * 1024) {
         // amax over the kept columns only: full-width vector loads with the excluded (outlier) columns masked out
         const size_t smem = (size_t)((a.cols_src + 7) >> 3) * 16;  // one 16-byte mask per chunk (at most 40 KB)
         // a contiguous slab of rows per CTA. The side copy divides item numbers by the side operand's width through a
@@ -1777,14 +1917,8 @@ static cudaError_t launch_quantize_rows_impl(const QuantRowsArgs& a, cudaStream_
         side_copy_done = a.excl_out != nullptr;
         return launch_rows_r<kGsTensor>(a, st);
       }
-      if (a.keep) {  // amax over the kept columns only: one row per CTA, one atomic per row
-        launch_kernel(amax_rows_bf16_kernel, dim3((unsigned)a.rows), dim3(256), 0, st, a.src, a.rows, a.cols_src, a.ld, a.keep, a.K, a.gs_cells, 1);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        return launch_rows_r<kGsTensor>(a, st);
-      }
-      const int64_t chunks = a.rows * ((a.cols_src + 7) >> 3);
-      const unsigned grid = (unsigned)std::min<int64_t>((chunks + 255) / 256, device_sm_count() * 8);
-      launch_kernel(amax_tensor_bf16_kernel, dim3(grid), dim3(256), 0, st, a.src, a.rows, a.cols_src, a.ld, a.gs_cells);
+      // amax over the kept columns only: one row per CTA, one atomic per row
+      launch_kernel(amax_rows_bf16_kernel, dim3((unsigned)a.rows), dim3(256), 0, st, a.src, a.rows, a.cols_src, a.ld, a.keep, a.K, a.gs_cells, 1);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return launch_rows_r<kGsTensor>(a, st);
@@ -1870,8 +2004,8 @@ static cudaError_t launch_tr_t(const QuantTransposeArgs& a, cudaStream_t st) {
                   dim3(128), 0, st, a.src.bf16, K32, D32, ld32, a.seed, a.stream_id, a.rht_stream, a.codes, a.sf, a.gscale, keys);  \
   else                                                                                                                              \
     launch_kernel(quantize_cols4_kernel<GS, RMODE, TILED_, RHT_, false>, dim3(blocks_for(a.rowsK, 512), blocks_for(a.D, 64)),       \
-                  dim3(128), 0, st, a.src.bf16, K32, D32, ld32, a.seed, a.stream_id, a.rht_stream, a.gs_cells, a.codes, a.sf,       \
-                  a.gscale, keys)
+                  dim3(128), 0, st, a.src.bf16, K32, D32, ld32, a.seed, a.stream_id, a.rht_stream, a.gs_cells, a.gs_words, a.codes, \
+                  a.sf, a.gscale, keys)
       if (a.sf_tiled) {
         if (a.rht_stream) { NVFP4_LAUNCH_COLS(true, true); } else { NVFP4_LAUNCH_COLS(true, false); }
       } else {
@@ -1884,7 +2018,7 @@ static cudaError_t launch_tr_t(const QuantTransposeArgs& a, cudaStream_t st) {
 #define NVFP4_LAUNCH_TR(TILED_, RHT_)                                                                                                  \
   if (fast)                                                                                                                            \
     launch_kernel(quantize_transpose_kernel<SRC, GS, RMODE, TILED_, RHT_, false>, dim3(grid), dim3(256), 0, st, a.src, a.rowsK, a.D,    \
-                  a.seed, a.stream_id, a.gs_cells, a.tensor_closed_form, a.codes, a.sf, a.gscale, a.rht_stream,                        \
+                  a.seed, a.stream_id, a.gs_cells, a.gs_words, a.tensor_closed_form, a.codes, a.sf, a.gscale, a.rht_stream,            \
                   make_philox_keys(a.seed));                                                                                           \
   else                                                                                                                                 \
     launch_kernel(quantize_transpose_generic_kernel<SRC, GS, RMODE != 0, TILED_, RHT_, false>, dim3(grid), dim3(256), 0, st, a.src,     \
@@ -1913,17 +2047,17 @@ static cudaError_t launch_tr_amax_rht(const TransposeSrc& src, int64_t rowsK, in
     if (rht_stream && !src.out_rows && (D & 3) == 0 && (src.ld & 3) == 0 && (reinterpret_cast<uintptr_t>(src.bf16) & 7u) == 0 &&
         src.ld < ((int64_t)1 << 31) && rowsK < ((int64_t)1 << 31) - 1024 && D < ((int64_t)1 << 31) - 64) {
       launch_kernel(quantize_cols4_kernel<GS, 0, false, true, true>, dim3(blocks_for(rowsK, 512), blocks_for(D, 64)), dim3(128), 0, st,
-                    src.bf16, (uint32_t)rowsK, (uint32_t)D, (uint32_t)src.ld, seed, 0u, rht_stream, cells, no_bytes, no_bytes, no_floats,
+                    src.bf16, (uint32_t)rowsK, (uint32_t)D, (uint32_t)src.ld, seed, 0u, rht_stream, cells, 1, no_bytes, no_bytes, no_floats,
                     make_philox_keys(seed));
       return cudaGetLastError();
     }
   }
   if (transpose_fast_path(src, SRC)) {
     if (rht_stream)
-      launch_kernel(quantize_transpose_kernel<SRC, GS, 0, false, true, true>, dim3(grid), dim3(256), 0, st, src, rowsK, D, seed, 0u, cells, 0,
+      launch_kernel(quantize_transpose_kernel<SRC, GS, 0, false, true, true>, dim3(grid), dim3(256), 0, st, src, rowsK, D, seed, 0u, cells, 1, 0,
                     no_bytes, no_bytes, no_floats, rht_stream, make_philox_keys(seed));
     else
-      launch_kernel(quantize_transpose_kernel<SRC, GS, 0, false, false, true>, dim3(grid), dim3(256), 0, st, src, rowsK, D, seed, 0u, cells, 0,
+      launch_kernel(quantize_transpose_kernel<SRC, GS, 0, false, false, true>, dim3(grid), dim3(256), 0, st, src, rowsK, D, seed, 0u, cells, 1, 0,
                     no_bytes, no_bytes, no_floats, 0u, make_philox_keys(seed));
   } else if (rht_stream) {
     launch_kernel(quantize_transpose_generic_kernel<SRC, GS, false, false, true, true>, dim3(grid), dim3(256), 0, st, src, rowsK, D, seed, 0u, cells,
@@ -1944,6 +2078,7 @@ template <int SRC>
 static cudaError_t launch_tr_s(const QuantTransposeArgs& a0, cudaStream_t st) {
   QuantTransposeArgs a = a0;
   a.tensor_closed_form = 0;
+  if (a.compute_amax) a.gs_words = 1;
   cudaError_t e;
   const dim3 agrid(blocks_for(a.D, 64), blocks_for(a.rowsK, 256));
   if (a.rht_stream && a.gs_mode != kGsBlock128) {
@@ -1958,12 +2093,15 @@ static cudaError_t launch_tr_s(const QuantTransposeArgs& a0, cudaStream_t st) {
   }
   if (a.gs_mode == kGsTensor) {
     if (a.compute_amax) {
+      if (SRC == 0 && transpose_fast_path(a.src, 0)) {
+        if ((e = launch_amax_tensor_words(a.src.bf16, a.rowsK, a.D, a.src.ld, a.gs_cells, st)) != cudaSuccess) return e;
+        a.gs_words = kTensorAmaxWords;
+        return launch_tr_r<SRC, kGsTensor>(a, st);
+      }
       const bool cell_unused = SRC == 1 && a.src.in_gs_mode == kGsTensor && !a.src.row_map;
       if (!cell_unused && !a.cells_zeroed && (e = launch_zero_words(a.gs_cells, 1, st)) != cudaSuccess) return e;
       if (SRC == 0) {
-        const int64_t chunks = a.rowsK * ((a.D + 7) >> 3);
-        const unsigned grid = (unsigned)std::min<int64_t>((chunks + 255) / 256, device_sm_count() * 8);
-        launch_kernel(amax_tensor_bf16_kernel, dim3(grid), dim3(256), 0, st, a.src.bf16, a.rowsK, a.D, a.src.ld, a.gs_cells);
+        if ((e = launch_amax_tensor(a.src.bf16, a.rowsK, a.D, a.src.ld, a.gs_cells, st)) != cudaSuccess) return e;
       } else if (a.src.in_gs_mode == kGsTensor) {
         a.tensor_closed_form = a.src.row_map ? 1 : 2;  // only the BF16 rows (if any) need a pass
         if (a.src.row_map) {
@@ -1995,11 +2133,21 @@ static cudaError_t launch_tr_s(const QuantTransposeArgs& a0, cudaStream_t st) {
   return launch_tr_r<SRC, kGsBlock128>(a, st);
 }
 
+static unsigned amax_tensor_grid(int64_t rows, int64_t cols) {
+  const int64_t chunks = rows * ((cols + 7) >> 3);
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>((chunks + 255) / 256, device_sm_count() * 8));
+}
 cudaError_t launch_amax_tensor(const uint16_t* src, int64_t rows, int64_t cols, int64_t ld, uint32_t* cell, cudaStream_t st) {
   if (rows == 0 || cols == 0) return cudaSuccess;
-  const int64_t chunks = rows * ((cols + 7) >> 3);
-  const unsigned grid = (unsigned)std::min<int64_t>((chunks + 255) / 256, device_sm_count() * 8);
-  launch_kernel(amax_tensor_bf16_kernel, dim3(grid), dim3(256), 0, st, src, rows, cols, ld, cell);
+  const unsigned grid = amax_tensor_grid(rows, cols);
+  launch_kernel(amax_tensor_bf16_kernel, dim3(grid), dim3(256), 0, st, src, rows, cols, ld, cell, grid, nullptr, (int64_t)0, (int64_t)0, (int64_t)0,
+                nullptr);
+  return cudaGetLastError();
+}
+cudaError_t launch_amax_tensor_pair(const uint16_t* a, int64_t rows_a, int64_t cols_a, int64_t ld_a, uint32_t* cell_a, const uint16_t* b,
+                                    int64_t rows_b, int64_t cols_b, int64_t ld_b, uint32_t* cell_b, cudaStream_t st) {
+  const unsigned ga = amax_tensor_grid(rows_a, cols_a), gb = amax_tensor_grid(rows_b, cols_b);
+  launch_kernel(amax_tensor_bf16_kernel, dim3(ga + gb), dim3(256), 0, st, a, rows_a, cols_a, ld_a, cell_a, ga, b, rows_b, cols_b, ld_b, cell_b);
   return cudaGetLastError();
 }
 
@@ -2014,14 +2162,15 @@ cudaError_t launch_zero_words(uint32_t* p, int64_t n, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_amax_tensor_pair(const uint16_t* a, int64_t rows_a, int64_t cols_a, int64_t ld_a, uint32_t* cell_a, const uint16_t* b,
-                                    int64_t rows_b, int64_t cols_b, int64_t ld_b, uint32_t* cell_b, cudaStream_t st) {
-  auto grid_of = [](int64_t rows, int64_t cols) {
-    const int64_t chunks = rows * ((cols + 7) >> 3);
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((chunks + 255) / 256, device_sm_count() * 8));
-  };
-  const unsigned ga = grid_of(rows_a, cols_a), gb = grid_of(rows_b, cols_b);
-  launch_kernel(amax_tensor_pair_kernel, dim3(ga + gb), dim3(256), 0, st, a, rows_a, cols_a, ld_a, cell_a, ga, b, rows_b, cols_b, ld_b, cell_b);
+cudaError_t launch_amax_tensor_words(const uint16_t* a, int64_t rows_a, int64_t cols_a, int64_t ld_a, uint32_t* cells_a, cudaStream_t st,
+                                     const uint16_t* b, int64_t rows_b, int64_t cols_b, int64_t ld_b, uint32_t* cells_b) {
+  // eight 16-byte loads per thread until every SM has about three CTAs of 512 threads; both tensors in clusters if one is
+  auto wanted = [](int64_t rows, int64_t cols) { return (rows * ((cols + 7) >> 3) + 4095) / 4096; };
+  AmaxGrid ga = amax_grid(wanted(rows_a, cols_a), kTensorAmaxWords), gb = b ? amax_grid(wanted(rows_b, cols_b), kTensorAmaxWords) : AmaxGrid{0, ga.cluster};
+  const unsigned cluster = std::max(ga.cluster, gb.cluster);
+  const unsigned na = (ga.ctas + cluster - 1) / cluster * cluster, nb = (gb.ctas + cluster - 1) / cluster * cluster;
+  launch_kernel_cluster(amax_tensor_words_kernel, dim3(na + nb), cluster, dim3(512), st, a, rows_a, cols_a, ld_a, cells_a, na, b, rows_b, cols_b,
+                        ld_b, cells_b);
   return cudaGetLastError();
 }
 
@@ -2036,6 +2185,97 @@ cudaError_t launch_amax_transpose_src(const TransposeSrc& s, int from_codes, int
     launch_kernel(amax_cols_generic_kernel<1>, dim3(agrid), dim3(256), 0, st, s, rowsK, D, cell, 0, 0);
   else
     launch_kernel(amax_cols_generic_kernel<0>, dim3(agrid), dim3(256), 0, st, s, rowsK, D, cell, 0, 0);
+  return cudaGetLastError();
+}
+
+// The job of a row quantizer without a column list: `unit` consecutive elements of a row per step, `units_per_cta` of them per CTA.
+static RowsJob rows_job(const QuantRowsArgs& a, int unit, int units_per_cta, int slack) {
+  const int64_t Kp = (a.K + 127) & ~(int64_t)127, per_row = Kp / unit, total = a.rows * per_row;
+  RowsJob j{};
+  j.src = a.src;
+  j.rows = a.rows;
+  j.K = a.K;
+  j.ld = a.ld;
+  j.gs_cells = a.gs_cells;
+  j.codes = a.codes;
+  j.sf = a.sf;
+  j.gscale = a.gscale;
+  j.gs_words = a.gs_words;
+  j.wide_loads = ((reinterpret_cast<uintptr_t>(a.src) & 31u) == 0 && (a.ld & 15) == 0) ? 1 : 0;
+  j.stream_id = a.stream_id;
+  j.rht_stream = a.rht_stream;
+  division_constants(total, slack, (uint64_t)per_row, j.div_mul, j.div_shift);
+  j.blocks = blocks_for(total, units_per_cta);
+  return j;
+}
+static TransposeJob transpose_job(const QuantTransposeArgs& a) {
+  TransposeJob j{};
+  j.s = a.src;
+  j.rowsK = a.rowsK;
+  j.D = a.D;
+  j.gs_cells = a.gs_cells;
+  j.codes = a.codes;
+  j.sf = a.sf;
+  j.gscale = a.gscale;
+  j.gs_words = a.gs_words;
+  j.closed_form = a.from_codes && a.gs_mode == kGsTensor ? 2 : 0;  // (from a TENSOR operand: its maximum is known in closed form)
+  j.stream_id = a.stream_id;
+  j.rht_stream = a.rht_stream;
+  j.grid_x = blocks_for(a.rowsK, 128);
+  j.blocks = j.grid_x * blocks_for(a.D, 64);
+  return j;
+}
+static bool small_index(int64_t v) { return v > 0 && v < ((int64_t)1 << 31) - 1024; }
+
+bool quantize_rows_pair_fits(const QuantRowsArgs& a, const QuantRowsArgs& b) {
+  auto ok = [](const QuantRowsArgs& q) {
+    return !q.keep && !q.sr && !q.rht_stream && q.sf_tiled && small_index(q.rows) && small_index(q.K) && small_index(q.ld) &&
+           q.rows * ((q.K + 127) / 128) < ((int64_t)1 << 31);
+  };
+  return ok(a) && ok(b) && a.gs_mode == b.gs_mode;
+}
+cudaError_t launch_quantize_rows_pair(const QuantRowsArgs& a, const QuantRowsArgs& b, cudaStream_t st) {
+  if (a.gs_mode == kGsRow) {
+    launch_kernel(amax_rows_warp_kernel, dim3((unsigned)((a.rows + 7) / 8)), dim3(256), 0, st, a.src, a.rows, a.cols_src, a.ld, a.gs_cells);
+    launch_kernel(amax_rows_warp_kernel, dim3((unsigned)((b.rows + 7) / 8)), dim3(256), 0, st, b.src, b.rows, b.cols_src, b.ld, b.gs_cells);
+  }
+  const RowsJob ja = rows_job(a, 16, 1024, 1024), jb = rows_job(b, 16, 1024, 1024);
+  const dim3 grid(ja.blocks + jb.blocks);
+  if (a.gs_mode == kGsTensor)
+    launch_kernel(quantize_rows_pair_kernel<kGsTensor>, grid, dim3(256), 0, st, ja, jb);
+  else if (a.gs_mode == kGsRow)
+    launch_kernel(quantize_rows_pair_kernel<kGsRow>, grid, dim3(256), 0, st, ja, jb);
+  else
+    launch_kernel(quantize_rows_pair_kernel<kGsBlock128>, grid, dim3(256), 0, st, ja, jb);
+  return cudaGetLastError();
+}
+
+bool quantize_bwd_fits(const QuantRowsArgs& q3, const QuantTransposeArgs& q4, const QuantTransposeArgs& q5, const QuantTransposeArgs& q6) {
+  auto ok = [](const QuantTransposeArgs& q) {
+    return q.sr == 1 && q.sf_tiled && small_index(q.rowsK) && small_index(q.D) && !q.src.out_rows && !q.src.closed_form_sg &&
+           transpose_fast_path(q.src, q.from_codes) && (!q.from_codes || q.src.in_gs_mode == q.gs_mode);
+  };
+  if (!(q3.sr == 1 && q3.sf_tiled && !q3.keep && small_index(q3.rows) && small_index(q3.K) && small_index(q3.ld) && ok(q4) && ok(q5) && ok(q6)))
+    return false;
+  const bool rht = q3.rht_stream != 0;
+  if ((q4.rht_stream != 0) != rht || (q5.rht_stream != 0) != rht || (q6.rht_stream != 0) != rht) return false;
+  // the scale modes whose maxima need no pass of their own per quantizer
+  if (!(q3.gs_mode == kGsBlock128 || (q3.gs_mode == kGsTensor && !rht))) return false;
+  const int64_t blocks = rows_job(q3, 64, 256, 256).blocks + (int64_t)transpose_job(q4).blocks + transpose_job(q5).blocks + transpose_job(q6).blocks;
+  return blocks <= (int64_t)(q3.gs_mode == kGsTensor ? kFusedBwdCtasTensor : kFusedBwdCtasBlock128) * device_sm_count();
+}
+cudaError_t launch_quantize_bwd(const QuantRowsArgs& q3, const QuantTransposeArgs& q4, const QuantTransposeArgs& q5,
+                                const QuantTransposeArgs& q6, cudaStream_t st) {
+  const RowsJob j3 = rows_job(q3, 64, 256, 256);
+  const TransposeJob j4 = transpose_job(q4), j5 = transpose_job(q5), j6 = transpose_job(q6);
+  const dim3 grid(j3.blocks + j4.blocks + j5.blocks + j6.blocks);
+  const PhiloxKeys keys = make_philox_keys(q3.seed);
+  if (q3.gs_mode == kGsTensor)
+    launch_kernel(quantize_bwd_kernel<kGsTensor, false>, grid, dim3(256), 0, st, j3, j4, j5, j6, q3.seed, keys);
+  else if (q3.rht_stream)
+    launch_kernel(quantize_bwd_kernel<kGsBlock128, true>, grid, dim3(256), 0, st, j3, j4, j5, j6, q3.seed, keys);
+  else
+    launch_kernel(quantize_bwd_kernel<kGsBlock128, false>, grid, dim3(256), 0, st, j3, j4, j5, j6, q3.seed, keys);
   return cudaGetLastError();
 }
 

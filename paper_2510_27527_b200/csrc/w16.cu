@@ -15,7 +15,7 @@ namespace nvfp4 {
 // CTA = 16 rows x 16 column blocks (256 columns). A warp holds two squares: lane = row in the square + 16 * (which square),
 // so the square's maximum is four xor-shuffles over 16 lanes.
 __global__ void __launch_bounds__(256) quantize_w16_kernel(const uint16_t* __restrict__ src, int64_t C, int64_t D, int64_t ld,
-                                                          const uint32_t* __restrict__ amax_cell, uint8_t* __restrict__ codes,
+                                                          const uint32_t* __restrict__ amax_words, uint8_t* __restrict__ codes,
                                                           uint8_t* __restrict__ sf, float* __restrict__ gscale, int tiled) {
   pdl_prologue();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(256) quantize_w16_kernel(const uint16_t* __res
   for (int i = 0; i < 16; ++i) m = fmaxf(m, fabsf(x[i]));
 #pragma unroll
   for (int o = 1; o < 16; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));  // over the square's 16 rows
-  const float Sg = global_scale_from_amax(__uint_as_float(amax_cell[0]));
+  const float Sg = global_scale_from_amax(__uint_as_float(cells_max<kTensorAmaxWords>(amax_words)));
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) gscale[0] = Sg;
   float rcp;
   const uint32_t sb = block_scale(m, Sg, rcp);
@@ -103,12 +103,12 @@ __global__ void __launch_bounds__(256) transpose_operand_kernel(const uint8_t* _
   if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) out_gscale[0] = in_gscale[0];
 }
 
-cudaError_t launch_quantize_w16(const uint16_t* src, int64_t C, int64_t D, int64_t ld, const uint32_t* amax_cell, uint8_t* codes,
+cudaError_t launch_quantize_w16(const uint16_t* src, int64_t C, int64_t D, int64_t ld, const uint32_t* amax_words, uint8_t* codes,
                                 uint8_t* sf, float* gscale, int tiled, cudaStream_t st) {
   if (C == 0 || D == 0) return cudaSuccess;
   const int64_t nb = ((D + 127) & ~(int64_t)127) >> 4;
   const dim3 grid((unsigned)((nb + 15) / 16), (unsigned)((C + 15) / 16));
-  launch_kernel(quantize_w16_kernel, grid, dim3(256), 0, st, src, C, D, ld, amax_cell, codes, sf, gscale, tiled);
+  launch_kernel(quantize_w16_kernel, grid, dim3(256), 0, st, src, C, D, ld, amax_words, codes, sf, gscale, tiled);
   return cudaGetLastError();
 }
 
