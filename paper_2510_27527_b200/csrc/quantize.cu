@@ -358,6 +358,13 @@ __global__ void __launch_bounds__(256) amax_rows_rht_kernel(const uint16_t* __re
 //   GATHER  columns come from the list `keep` (OutControl compaction) instead of 0..cols-1.
 //   RHT     each block is replaced by (x S) H_16 before anything else looks at it (never together with GATHER).
 // =========================================================================================================
+// CTAs of a TENSOR-mode quantizer take the tensor from its end: the amax pass before them has just read that end, so part of it is
+// still in L2 where the tensor does not fit. us with the amax pass, from the start / from the end: 16384 x 3072 (101 MB) round to
+// nearest 41.6 / 34.6, stochastic 65.9 / 59.8; 16384 x 8192 103 / 94, 164 / 157; no difference up to 8192 x 3072 (50 MB).
+template <int GS>
+__device__ __forceinline__ uint32_t tail_first(uint32_t block) {
+  return GS == kGsTensor ? gridDim.x - 1u - block : block;
+}
 template <int GS, bool SR, bool TILED, bool GATHER, bool RHT>
 __device__ __forceinline__ void quantize_rows_body(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld,
                      const int32_t* __restrict__ keep, uint64_t seed, uint32_t stream_id,
@@ -577,7 +584,7 @@ quantize_rows_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, 
                      float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, int64_t cols_src,
                      int64_t stage_cols8, uint32_t rht_stream, int sb_up, const __grid_constant__ PhiloxKeys pk) {
   pdl_prologue();
-  quantize_rows_body<GS, SR, TILED, GATHER, RHT>(src, rows, K, ld, keep, seed, stream_id, gs_cells, gs_words, codes, sf, gscale, div_mul, div_shift, wide_loads, cols_src, stage_cols8, rht_stream, sb_up, pk, blockIdx.x);
+  quantize_rows_body<GS, SR, TILED, GATHER, RHT>(src, rows, K, ld, keep, seed, stream_id, gs_cells, gs_words, codes, sf, gscale, div_mul, div_shift, wide_loads, cols_src, stage_cols8, rht_stream, sb_up, pk, tail_first<GS>(blockIdx.x));
 }
 
 
@@ -750,7 +757,7 @@ quantize_rows4_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K,
                       float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, uint32_t rht_stream,
                       const __grid_constant__ PhiloxKeys pk) {
   pdl_prologue();
-  quantize_rows4_body<GS, RMODE, TILED, RHT>(src, rows, K, ld, seed, stream_id, gs_cells, gs_words, codes, sf, gscale, div_mul, div_shift, wide_loads, rht_stream, pk, blockIdx.x);
+  quantize_rows4_body<GS, RMODE, TILED, RHT>(src, rows, K, ld, seed, stream_id, gs_cells, gs_words, codes, sf, gscale, div_mul, div_shift, wide_loads, rht_stream, pk, tail_first<GS>(blockIdx.x));
 }
 
 
@@ -1424,7 +1431,13 @@ quantize_cols4_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, 
                       uint32_t rht_stream, uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes,
                       uint8_t* __restrict__ sf, float* __restrict__ gscale, const __grid_constant__ PhiloxKeys pk) {
   pdl_prologue();
-  quantize_cols4_body<GS, RMODE, TILED, RHT, AMAX_ONLY>(src, K, D, ld, seed, stream_id, rht_stream, gs_cells, gs_words, codes, sf, gscale, pk, blockIdx.x, blockIdx.y, threadIdx.x);
+  uint32_t bx = blockIdx.x, by = blockIdx.y;
+  if (GS == kGsTensor && !AMAX_ONLY) {  // from the end, as tail_first: last rows first, all columns of them
+    const uint32_t l = by * gridDim.x + bx, kt = l / gridDim.y;
+    by = l - kt * gridDim.y;
+    bx = gridDim.x - 1u - kt;
+  }
+  quantize_cols4_body<GS, RMODE, TILED, RHT, AMAX_ONLY>(src, K, D, ld, seed, stream_id, rht_stream, gs_cells, gs_words, codes, sf, gscale, pk, bx, by, threadIdx.x);
 }
 
 
@@ -1740,7 +1753,8 @@ quantize_rows_pair_kernel(const __grid_constant__ RowsJob a, const __grid_consta
   pdl_prologue();
   const bool first = blockIdx.x < a.blocks;
   const RowsJob& j = first ? a : b;
-  const uint32_t bx = first ? blockIdx.x : blockIdx.x - a.blocks;
+  uint32_t bx = first ? blockIdx.x : blockIdx.x - a.blocks;
+  if (GS == kGsTensor) bx = j.blocks - 1u - bx;  // (tail_first)
   const PhiloxKeys no_keys{};
   quantize_rows_body<GS, false, true, false, false>(j.src, j.rows, j.K, j.ld, nullptr, 0ull, j.stream_id, j.gs_cells, j.gs_words, j.codes, j.sf,
                                                     j.gscale, j.div_mul, j.div_shift, j.wide_loads, 0, 0, 0u, 0, no_keys, bx);
