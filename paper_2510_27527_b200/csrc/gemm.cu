@@ -191,7 +191,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   __shared__ int abort_flag_s;
   volatile int* abort_flag = &abort_flag_s;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     abort_flag_s = 0;
@@ -556,7 +556,7 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag_s;
   volatile int* abort_flag = &abort_flag_s;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     abort_flag_s = 0;
@@ -1031,7 +1031,7 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag_s;
   volatile int* abort_flag = &abort_flag_s;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
 
   if (threadIdx.x == 0) {
@@ -1254,7 +1254,7 @@ hp_dw_mma_kernel(const __grid_constant__ CUtensorMap tmDY, const __grid_constant
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag_s;
   volatile int* abort_flag = &abort_flag_s;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
   const uint32_t tmem_cols = Kh <= 64 ? 64u : (Kh <= 128 ? 128u : 256u);
 
   if (threadIdx.x == 0) {
@@ -1614,42 +1614,36 @@ cudaError_t launch_dense_gemm(const void* A, const void* B, int64_t M, int64_t N
 size_t gemm_workspace_bytes(int64_t, int64_t, int64_t) { return 0; }
 int64_t gemm_block128_max_k() { return (int64_t)B128_MAX_CHUNKS * 128; }
 
-// Variant choice. All kernels are bound by what the L2 delivers to the SMs (about 13 - 16 TB/s over all SMs): the 128 x 128
-// kernel pulls 36 KB per k tile and SM, a pair on a 256 x 256 tile 38 KB per SM for twice the math. The 128 x 128 kernel has
-// two accumulators (a tile's epilogue overlaps the next tile's MMAs entirely); the 256-wide pair kernel has one and hands it
-// over once its sixteen epilogue warps hold the tile in registers (a few hundred cycles per tile), and 256-wide tiles fill
-// the last wave worse. Pairs therefore run when there are enough tiles: from K = 1024 with five tiles per pair, from
-// K = 2048 with two, and from K = 8192 already when half of the pairs get a tile (the weight gradients of a model: few
-// tiles, K = tokens). Measured, BF16 output, 128 x 128 / 256 x 256 / 256 x 192, us: 16384 x 3072 x 1024 38.9 / 34.8 / 36.9;
-// 16384 x 1024 x 1024 (256 pair tiles) 18.5 / 19.2 / 22.4; 8192 x 3072 x 1024 (384) 24.5 / 22.7 / 22.5; 4096 x 4096 x 1024
-// (256) 18.4 / 18.5 / 20.4; 16384 x 1024 x 2816 31.6 / 28.8 / 32.8; 16384 x 3072 x 2048 61.4 / 51.2 / 55.8; 8192 x 8192 x 3072
-// 100.4 / 77.8 / 87.9; 4096^3 38.9 / 34.8 / 34.8; 16384 x 14336 x 4096 426 / 342 / 387; 4096 x 8192 x 8192 114.8 / 88.1 /
-// 104.4; 16384 x 8192 x 8192 455 / 352 / 408; 3072 x 1024 x 16384 (48 / 72 pair tiles) 38.9 / 30.8 / 30.7, FP32 output 40.9 /
-// 32.7 / 30.7; 1024 x 1024 x 16384 (16 / 24) 22.6 / 30.8 / 28.7; 2048 x 2048 x 16384 (64 / 88) 38.9 / 32.8 / 46.9.
+// Variant choice, by a cost model: rounds of the variant's tiles over the SMs (or SM pairs) x time of a tile, which is a constant and
+// so much per 256-wide k tile, or at short K what writing the tile takes. All kernels are bound by what the L2 delivers to the SMs and by
+// their epilogue: the 128 x 128 kernel pulls 36 KB per k tile and SM, a pair on a 256 x 256 tile 38 KB per SM for twice the math, but
+// it fills the last round worse, holds one accumulator and, with ROW scales, has an epilogue of two more multiplies per element
+// in registers that spill. The constants are fits to measured times (warm L2, BF16 output unless marked), us, 128 x 128 / 256 x 256 /
+// 256 x 192. TENSOR: 16384 x 3072 x 1024 35.0 / 29.8 / 32.1; 16384 x 1024 x 3072 26.9 / 22.8 / 26.1; 16384 x 1024 x 1024 13.0 /
+// 12.8 / 14.4; 8192 x 3072 x 1024 18.6 / 17.0 / 16.7; 8192 x 2816 x 1024 17.0 / 14.8 / 16.4; 8192 x 1024 x 3072 15.9 / 13.5 / 14.9;
+// 4096^3 32.0 / 27.1 / 27.3; 3072 x 1024 x 16384 (FP32) 29.7 / 26.4 / 21.1; 3072 x 1024 x 8192 (FP32) 18.0 / 16.5 / 13.7;
+// 1024 x 1024 x 16384 (FP32) 16.5 / 24.5 / 19.8. ROW: 16384 x 3072 x 1024 49.5 / 53.7 / 58.7; 16384 x 1024 x 3072 37.0 / 32.9 /
+// 38.5; 8192 x 1024 x 3072 18.6 / 16.4 / 18.4; 3072 x 1024 x 16384 (FP32) 44.2 / 40.8 / 31.7; 4096^3 33.9 / 29.8 / 29.8. Short K:
+// 13736 x 2648 x 648 27.4 / 24.6 / 28.9, 8386 x 4680 x 544 (FP32) 37.3 / 33.0 / 35.4, 7084 x 4768 x 760 25.4 / 23.3 / 24.9; ROW 6083 x
+// 6232 x 1320 (FP32) 49.7 / 43.2 / 46.2, 4768 x 2016 x 2616 (FP32) 23.6 / 21.9 / 19.8.
 // A 256-row tile of an operand spans two 128-row scale tiles, and rows are padded to 128 in the scale layout, so any M, N
 // work. The fused high-precision side product and the outer-block scales live in the single-CTA kernels only.
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
   if (a.M == 0 || a.N == 0) return cudaSuccess;
   if (a.gs_mode == kGsBlock128) return a.variant >= 2 ? cudaErrorInvalidValue : launch_block128(a, st);
-  const int64_t tiles256 = ((a.M + 255) / 256) * ((a.N + 255) / 256), n_pairs = sm_count() / 2;
-  // (ROW scales: the pair kernels' epilogue holds a quarter tile in registers and has two more multiplies per element to do,
-  // it spills and becomes the bound at short K -- 16384 x 3072 x 1024, BF16 output: 40.9 / 53.4 / 74.7 us -- so pairs start at
-  // K = 2048 there and the 192-wide kernel, which has the least time per tile to hide it in, is not used.)
+  const int64_t sms = sm_count(), n_pairs = sms / 2, rows256 = (a.M + 255) / 256;
+  const double k_tiles = (double)((a.K + BK - 1) / BK);
   const bool row_scales = a.gs_mode == kGsRow;
-  bool pairs = (!row_scales && a.K >= 1024 && tiles256 >= 5 * n_pairs) || (a.K >= 2048 && tiles256 >= 2 * n_pairs) ||
-               (a.K >= 8192 && 2 * tiles256 >= n_pairs);
-  // Between the two pair kernels, by a cost model in units of one 256-wide k tile: rounds of the pair grid x (k tiles x the
-  // relative cost of a k tile + 1 per tile). A 192-wide k tile costs 0.85 (three quarters of the math, but more operand
-  // traffic per flop); what the 192-wide tiles have is the finer last wave, which decides when tiles are few.
-  bool pairs192 = false;
-  if (pairs) {
-    const int64_t tiles192 = ((a.M + 255) / 256) * ((a.N + 191) / 192);
-    const double k_tiles = (double)((a.K + BK - 1) / BK);
-    const double cost256 = (double)((tiles256 + n_pairs - 1) / n_pairs) * (k_tiles + 1.0);
-    const double cost192 = (double)((tiles192 + n_pairs - 1) / n_pairs) * (0.85 * k_tiles + 1.0);
-    pairs192 = !row_scales && cost192 < cost256;
-  }
-  if (pairs192) pairs = false;
+  auto rounds = [](int64_t tiles, int64_t units) { return (double)((tiles + units - 1) / units); };
+  // us: a tile = max(write, fixed + per_k_tile * k tiles), with TENSOR and with ROW scales
+  auto cost = [&](double n_rounds, double per_k_tile, double fixed, double fixed_row, double write, double write_row) {
+    const double w = (row_scales ? write_row : write) * (a.c_is_f32 ? 1.3 : 1.0);
+    return n_rounds * std::max(w, (row_scales ? fixed_row : fixed) + per_k_tile * k_tiles);
+  };
+  const double cost128 = cost(rounds(((a.M + 127) / 128) * ((a.N + 127) / 128), sms), 0.2275, 0.57, 1.45, 1.40, 2.15);
+  const double cost256 = cost(rounds(rows256 * ((a.N + 255) / 256), n_pairs), 0.300, 1.16, 2.60, 2.35, 4.50);
+  const double cost192 = cost(rounds(rows256 * ((a.N + 191) / 192), n_pairs), 0.250, 0.80, 2.30, 2.15, 3.80);
+  bool pairs = cost256 <= cost192 && cost256 <= cost128, pairs192 = cost192 < cost256 && cost192 < cost128;
   if (a.variant == 1) pairs = pairs192 = false;
   if (a.variant == 2) { pairs = true; pairs192 = false; }
   if (a.variant == 3) { pairs192 = true; pairs = false; }
