@@ -10,8 +10,7 @@
 //               instruction, FP32 accumulators in tensor memory, two accumulator buffers).
 //   warps 2..9  epilogue (two warps per tensor-memory lane quadrant, half of the tile's columns each): tcgen05.ld the
 //               accumulator, apply the FP32 global scales, convert, stage 128-byte row pieces in shared memory and
-//               write them with bulk tensor stores. (The outer-block variant further down keeps four promotion
-//               warps, 2..5.)
+//               write them with bulk tensor stores. (The outer-block variant further down has its own roles.)
 // Every wait on an mbarrier is bounded (Params::wait_limit clock cycles); when a bound is hit the kernel raises a
 // status word, all roles drain and the CTA frees its tensor memory and exits.
 #include <cuda.h>
@@ -24,8 +23,6 @@
 namespace nvfp4 {
 
 namespace {
-
-constexpr int NUM_THREADS = 192;
 
 // Single-CTA kernel: 128 x 128 output tiles.
 constexpr int BN = 128;
@@ -66,7 +63,6 @@ struct Params {
   int32_t m_tiles, n_tiles;
   int32_t c_is_f32, accumulate;
   int32_t hp_k_tiles;     // OutControl: 64-wide BF16 k tiles of the high-precision side product (0 = none)
-  int32_t use_tma_store;  // C is described by a tensor map: stage the epilogue in shared memory and bulk-store it
   int32_t starve;         // test hook: the first stage's "full" barrier expects 16 bytes more than will ever arrive
   long long wait_limit;   // bound of every wait, in clock cycles
   int32_t* dev_status;
@@ -115,55 +111,6 @@ __device__ __forceinline__ void store_ragged(const Params& p, int64_t m, int64_t
     for (int j = 0; j < W; ++j)
       if (n0 + j < p.N) cp[j] = __float2bfloat16_rn(o[j]);
   }
-}
-
-// One output row, 32 consecutive columns starting at n0 (m < M and n0 < N are the caller's business): add the old C when
-// accumulating, convert, store.
-__device__ __forceinline__ void store_row_chunk(const Params& p, int64_t m, int64_t n0, float (&o)[32]) {
-    if (p.c_is_f32) {
-      float* cp = reinterpret_cast<float*>(p.C) + m * p.ldc + n0;
-      if (n0 + 32 <= p.N) {
-#pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-          float4 q = make_float4(o[j], o[j + 1], o[j + 2], o[j + 3]);
-          if (p.accumulate) {
-            const float4 old = *reinterpret_cast<const float4*>(cp + j);
-            q.x += old.x; q.y += old.y; q.z += old.z; q.w += old.w;
-          }
-          *reinterpret_cast<float4*>(cp + j) = q;
-        }
-      } else {
-        for (int j = 0; j < 32 && n0 + j < p.N; ++j) cp[j] = p.accumulate ? cp[j] + o[j] : o[j];
-      }
-    } else {
-      __nv_bfloat16* cp = reinterpret_cast<__nv_bfloat16*>(p.C) + m * p.ldc + n0;
-      if (n0 + 32 <= p.N) {
-#pragma unroll
-        for (int j = 0; j < 32; j += 8) {
-          if (p.accumulate) {
-            const uint4 old = *reinterpret_cast<const uint4*>(cp + j);
-            const uint32_t ow[4] = {old.x, old.y, old.z, old.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              o[j + 2 * q] += bf16_lo(ow[q]);
-              o[j + 2 * q + 1] += bf16_hi(ow[q]);
-            }
-          }
-          uint4 q;
-          __nv_bfloat162 h;
-          h = __floats2bfloat162_rn(o[j], o[j + 1]); q.x = *reinterpret_cast<uint32_t*>(&h);
-          h = __floats2bfloat162_rn(o[j + 2], o[j + 3]); q.y = *reinterpret_cast<uint32_t*>(&h);
-          h = __floats2bfloat162_rn(o[j + 4], o[j + 5]); q.z = *reinterpret_cast<uint32_t*>(&h);
-          h = __floats2bfloat162_rn(o[j + 6], o[j + 7]); q.w = *reinterpret_cast<uint32_t*>(&h);
-          *reinterpret_cast<uint4*>(cp + j) = q;
-        }
-      } else {
-        for (int j = 0; j < 32 && n0 + j < p.N; ++j) {
-          const float prev = p.accumulate ? __bfloat162float(cp[j]) : 0.0f;
-          cp[j] = __float2bfloat16_rn(o[j] + prev);
-        }
-      }
-    }
 }
 
 template <int GS>
@@ -521,38 +468,174 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 }
 
 // =========================================================================================================
-// BLOCK128 variant: the FP32 global scale changes every 128 k (the paper's 1x128 outer block, Sec. 2.2), so a
-// partial product can only be accumulated over 128 k inside tensor memory. The MMA warp writes each 128-k partial
-// (two K = 64 instructions) into one of three tensor-memory buffers; the epilogue warps pull it out and promote it
-// into FP32 register accumulators with the rank-1 scale SgA[m, kc] * SgB[n, kc] (packed f32x2 FMAs). The SgB values
-// of the tile, for all chunks, are staged in shared memory once per tile ([chunk][n] so a warp reads them as
-// broadcasts). 128 x 128 tiles, K <= 16384.
+// BLOCK128 variant: the FP32 global scale changes every 128 k (the paper's 1x128 outer block, Sec. 2.2), so a partial product can
+// only be accumulated over 128 k inside tensor memory. The MMA warp writes each 128-k partial of a 128 x 192 tile (two K = 64
+// instructions) into one of two tensor-memory buffers; twelve promotion warps pull it out, 32 rows x 64 columns each, and promote it
+// into FP32 register accumulators with the rank-1 scale SgA[m, kc] * SgB[n, kc] (packed f32x2 multiply + FMA).
+//
+// What bounds it: the promotion. A packed operation issues every 2.8 cycles at best (measured, from registers, two or more warps
+// per scheduler), which is 540 cycles per partial against 200 of its MMAs; this kernel takes 840 at long K, 1060 at K = 1024.
+//   - Three promotion warps per scheduler: a warp's barrier, tensor-memory load and hand-over latencies (about 400 cycles per
+//     partial) run under the others' arithmetic. With one (a 128 x 128 tile, four warps with 128 columns each) they add up:
+//     760 cycles per 128 columns. 192 columns are what a register file of 128 a thread on average holds (setmaxnreg: 80 for the
+//     four warps that load, issue and fetch scales, 144 for the others) with a buffer to spare in tensor memory.
+//   - Fragments: the 16x256b load gives a thread 2 columns x 8 groups of 2 rows, i.e. 16 column scales and 4 row scales for 64
+//     elements; with a thread per row it would be a column scale per element, read from shared memory by every warp.
+//   - Scales come through shared memory, fetched by two warps in 16-byte pieces (below).
+// us, before (one group of four warps) and now: 8192 x 3072 x 1024 49.0 / 35.7, 8192 x 1024 x 3072 42.5 / 38.9, 3072 x 1024 x 8192
+// (FP32) 55.1 / 33.7, 1999 x 1416 x 1000 14.5 / 10.6, 4096^3 95.7 / 78.5, 16384 x 8192 x 8192 1415 / 1048. K <= 16384.
 // =========================================================================================================
-constexpr int B128_STAGES = 4;
-constexpr int B128_NBUF = 3;
-constexpr int B128_MAX_CHUNKS = 128;
-constexpr uint32_t B128_SGB_BYTES = (B128_MAX_CHUNKS + 1) * 128 * 4 + 512;  // + the high-precision partial; 1024-byte multiple
-constexpr uint32_t B128_STAGING_BYTES = 4 * 4096;  // one 32-row x 128-byte staging buffer per epilogue warp (bulk stores)
-constexpr uint32_t B128_SMEM_BYTES = B128_STAGES * Cfg::STAGE_BYTES + B128_SGB_BYTES + B128_STAGING_BYTES + 1024 + 256;
+constexpr int B128_TN = 192;
+constexpr int B128_STAGES = 3;
+constexpr int B128_NBUF = 2;
+constexpr int64_t B128_MAX_K = 16384;
+constexpr int B128_PROMO_WARPS = 12;                       // warps 4 .. 15: 32 rows x 64 columns each
+constexpr int B128_THREADS = 128 + 32 * B128_PROMO_WARPS;  // warps 0 .. 3: loads, MMA, global scales (two)
+constexpr int B128_SC_SLOTS = 3;                           // ring of global-scale slots, four chunks each
+constexpr uint32_t B128_B_BYTES = B128_TN * 128;
+constexpr uint32_t B128_SFB_BYTES = 4096;                  // the two 128-row scale tiles that the B rows touch
+constexpr uint32_t B128_STAGE_BYTES = A_BYTES + B128_B_BYTES + SFA_BYTES + B128_SFB_BYTES;  // 46 KB
+constexpr uint32_t B128_STAGING_BYTES = B128_PROMO_WARPS * 4096;                            // 32 rows x 128 bytes per promotion warp
+constexpr uint32_t B128_SC_CHUNK = (128 + B128_TN) * 4;                                     // SgA, then SgB of one chunk
+constexpr uint32_t B128_SC_BYTES = 4 * B128_SC_CHUNK;
+constexpr uint32_t B128_SMEM_BYTES = B128_STAGES * B128_STAGE_BYTES + B128_STAGING_BYTES + B128_SC_SLOTS * B128_SC_BYTES + 1024 + 256;
+constexpr uint32_t B128_SF_COLS = 48, B128_SF_SETS = 2;    // tensor-memory columns of a k tile's block scales: 16 of A, 32 of B
+static_assert(B128_NBUF * B128_TN + B128_SF_SETS * B128_SF_COLS <= 512, "tensor memory budget");
+static_assert(B128_SMEM_BYTES <= 227 * 1024, "shared memory budget");
 
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+// 16 rows x 64 columns of a partial: v[4 i + 2 q + e] is row 8 q + lane / 4, column 8 i + 2 (lane % 4) + e. Wait with tc_wait_ld.
+__device__ __forceinline__ void tc_ld_16x256b_x8(uint32_t taddr, uint32_t (&v)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+        "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+        "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr)
+      : "memory");
+}
+// Four global scales of a row from chunk c on (c a multiple of four; 0 past the row's end); vec = floats that a load may take.
+__device__ __forceinline__ float4 load_scales4(const float* row, int32_t c, int32_t chunks, int vec) {
+  if (vec == 4) return __ldg(reinterpret_cast<const float4*>(row + c));
+  float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (vec == 2) {
+    const float2 a = __ldg(reinterpret_cast<const float2*>(row + c));
+    r.x = a.x;
+    r.y = a.y;
+    if (c + 2 < chunks) {
+      const float2 b = __ldg(reinterpret_cast<const float2*>(row + c + 2));
+      r.z = b.x;
+      r.w = b.y;
+    }
+  } else {
+    r.x = __ldg(row + c);
+    if (c + 1 < chunks) r.y = __ldg(row + c + 1);
+    if (c + 2 < chunks) r.z = __ldg(row + c + 2);
+    if (c + 3 < chunks) r.w = __ldg(row + c + 3);
+  }
+  return r;
+}
+__device__ __forceinline__ float4 lds128(uint32_t addr) {
+  float4 r;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "r"(addr));
+  return r;
+}
+
+// A warp's 32 rows x 64 columns of C from accumulator fragments (layout: see tc_ld_16x256b_x8): 128-byte row pieces staged in shared
+// memory with the 128-byte swizzle and written by the bulk-tensor engine as full lines, rows clipped at the edge of C; element
+// stores at the right edge (whose padding columns stay untouched) and when adding to the old C.
+__device__ __forceinline__ void b128_store64(const Params& p, const CUtensorMap& tmC, uint32_t stage, int lane, int64_t m0, int64_t n0,
+                                             const float2 (&acc)[2][2][8]) {
+  const int lr = lane >> 2, lc = lane & 3;
+  if (n0 + 64 <= p.N && !p.accumulate) {
+    if (p.c_is_f32) {
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        if (lane == 0) bulk_wait_read<0>();  // the previous store from this buffer has read it
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 a = acc[r >> 1][r & 1][4 * b + i];
+            const uint32_t dst = stage + (uint32_t)(8 * r + lr) * 128u + (uint32_t)(((2 * i + (lc >> 1)) ^ lr) << 4) + (uint32_t)(lc & 1) * 8u;
+            asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(a.x), "f"(a.y) : "memory");
+          }
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          tma_store_2d(&tmC, stage, (int32_t)n0 + 32 * b, (int32_t)m0);
+          bulk_commit();
+        }
+      }
+    } else {
+      if (lane == 0) bulk_wait_read<0>();
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          uint32_t w[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 a = acc[r >> 1][r & 1][4 * b + i];
+            const __nv_bfloat162 hh = __floats2bfloat162_rn(a.x, a.y);
+            w[i] = *reinterpret_cast<const uint32_t*>(&hh);
+          }
+          // lane l gives the address of row l % 8 of 8 x 8 matrix l / 8, which is column group 4 b + l / 8
+          const uint32_t dst = stage + (uint32_t)(8 * r + (lane & 7)) * 128u + (uint32_t)(((4 * b + (lane >> 3)) ^ (lane & 7)) << 4);
+          asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                       "r"(w[3])
+                       : "memory");
+        }
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        tma_store_2d(&tmC, stage, (int32_t)n0, (int32_t)m0);
+        bulk_commit();
+      }
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int64_t m = m0 + 8 * r + lr, n = n0 + 8 * i + 2 * lc;
+        const float2 a = acc[r >> 1][r & 1][i];
+        if (m < p.M && n < p.N) {
+          if (p.c_is_f32) {
+            float* cp = reinterpret_cast<float*>(p.C) + m * p.ldc + n;
+            cp[0] = p.accumulate ? cp[0] + a.x : a.x;
+            if (n + 1 < p.N) cp[1] = p.accumulate ? cp[1] + a.y : a.y;
+          } else {
+            __nv_bfloat16* cp = reinterpret_cast<__nv_bfloat16*>(p.C) + m * p.ldc + n;
+            cp[0] = __float2bfloat16_rn(p.accumulate ? a.x + __bfloat162float(cp[0]) : a.x);
+            if (n + 1 < p.N) cp[1] = __float2bfloat16_rn(p.accumulate ? a.y + __bfloat162float(cp[1]) : a.y);
+          }
+        }
+      }
+  }
+}
+
+__global__ void __launch_bounds__(B128_THREADS, 1)
 gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                            const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmAh,
                            const __grid_constant__ CUtensorMap tmBh, const Params p) {
-  using C = Cfg;
-  constexpr int BN = 128;
-  constexpr int STAGES = B128_STAGES;
+  constexpr int STAGES = B128_STAGES, SLOTS = B128_SC_SLOTS, TN = B128_TN;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-  float* sgb = reinterpret_cast<float*>(smem_gen + STAGES * C::STAGE_BYTES);
-  const uint32_t staging_base = smem_base + STAGES * C::STAGE_BYTES + B128_SGB_BYTES;  // 1024-byte aligned
-  const uint32_t bar_base = staging_base + B128_STAGING_BYTES;
+  const uint32_t staging_base = smem_base + STAGES * B128_STAGE_BYTES;  // 1024-byte aligned
+  const uint32_t scale_base = staging_base + B128_STAGING_BYTES;
+  const uint32_t bar_base = scale_base + SLOTS * B128_SC_BYTES;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
   auto part_full_bar = [&](int b) { return bar_base + 8u * (2 * STAGES + b); };
   auto part_empty_bar = [&](int b) { return bar_base + 8u * (2 * STAGES + B128_NBUF + b); };
-  const uint32_t drain_bar = bar_base + 8u * (2 * STAGES + 2 * B128_NBUF);
+  auto sc_full_bar = [&](int s) { return bar_base + 8u * (2 * STAGES + 2 * B128_NBUF + s); };
+  auto sc_empty_bar = [&](int s) { return bar_base + 8u * (2 * STAGES + 2 * B128_NBUF + SLOTS + s); };
+  const uint32_t drain_bar = bar_base + 8u * (2 * STAGES + 2 * B128_NBUF + 2 * SLOTS);
+  static_assert(8 * (2 * B128_STAGES + 2 * B128_NBUF + 2 * B128_SC_SLOTS + 1) <= 256, "barrier space");
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag_s;
   volatile int* abort_flag = &abort_flag_s;
@@ -566,7 +649,11 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
     }
     for (int b = 0; b < B128_NBUF; ++b) {
       mbar_init(part_full_bar(b), 1);
-      mbar_init(part_empty_bar(b), 4);
+      mbar_init(part_empty_bar(b), B128_PROMO_WARPS);
+    }
+    for (int s = 0; s < SLOTS; ++s) {
+      mbar_init(sc_full_bar(s), 2);
+      mbar_init(sc_empty_bar(s), B128_PROMO_WARPS);
     }
     mbar_init(drain_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -584,274 +671,252 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
   const int64_t num_tiles = (int64_t)p.m_tiles * p.n_tiles;
   const int32_t chunks = p.k_chunks;  // 128-wide k chunks per tile
 
-  if (warp == 0) {
-    const uint32_t leader = elect_leader();
-    uint32_t it = 0;
-    bool ok = true;
-    for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
-      const int32_t mt = (int32_t)(t / p.n_tiles), nt = (int32_t)(t % p.n_tiles);
-      const uint8_t* sfa_src = p.a_sf + (size_t)mt * p.sf_tiles_a * 512;
-      const uint8_t* sfb_src = p.b_sf + (size_t)nt * p.sf_tiles_b * 512;
-      for (int32_t kt = 0; kt < p.k_tiles; ++kt, ++it) {
-        const int s = it % STAGES;
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.dev_status, p.wait_limit));
-        if (!ok) break;
-        const uint32_t st = smem_base + s * C::STAGE_BYTES;
-        mbar_expect_tx(full_bar(s), C::STAGE_BYTES, leader);
-        tma_load_2d(st, &tmA, kt * (BK / 2), mt * BM, full_bar(s), leader);
-        tma_load_2d(st + A_BYTES, &tmB, kt * (BK / 2), nt * BN, full_bar(s), leader);
-        bulk_load(st + A_BYTES + C::B_BYTES, sfa_src + (size_t)kt * 2048, 2048, full_bar(s), leader);
-        bulk_load(st + A_BYTES + C::B_BYTES + SFA_BYTES, sfb_src + (size_t)kt * 2048, 2048, full_bar(s), leader);
-      }
-      // OutControl: the BF16 outlier channels of both operands, 64 per stage, into the same stage buffers
-      for (int32_t h = 0; h < p.hp_k_tiles && ok; ++h, ++it) {
-        const int s = it % STAGES;
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.dev_status, p.wait_limit));
-        if (!ok) break;
-        const uint32_t st = smem_base + s * C::STAGE_BYTES;
-        mbar_expect_tx(full_bar(s), A_BYTES + C::B_BYTES, leader);
-        tma_load_2d(st, &tmAh, h * 64, mt * BM, full_bar(s), leader);
-        tma_load_2d(st + A_BYTES, &tmBh, h * 64, nt * BN, full_bar(s), leader);
-      }
-    }
-    if (!ok) {
-      const uint32_t n_back = it < (uint32_t)STAGES ? it : (uint32_t)STAGES;
-      for (uint32_t j = 0; j < n_back; ++j) {
-        const uint32_t f = it - 1 - j;
-        const long long t0 = clock64();
-        while (!mbar_try(full_bar(f % STAGES), (f / STAGES) & 1) && clock64() - t0 < p.wait_limit) {
-        }
-      }
-    }
-  } else if (warp == 1) {
-    const uint32_t leader = elect_leader();
-    const uint32_t idesc = instr_desc<BN>();
-    uint32_t it = 0, cit = 0;
-    bool ok = true;
-    for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
-      for (int32_t kt = 0; kt < p.k_tiles && ok; ++kt, ++it) {
-        const int s = it % STAGES;
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(full_bar(s), (it / STAGES) & 1, abort_flag, p.dev_status, p.wait_limit));
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t st = smem_base + s * C::STAGE_BYTES;
-        const uint32_t sf_tmem = tmem_base + B128_NBUF * 128 + (it & 3) * C::SF_COLS;
-#pragma unroll
-        for (int kk = 0; kk < BK / 64; ++kk) {
-          tc_cp_sf(sf_tmem + kk * 4, desc_sf(st + A_BYTES + C::B_BYTES + kk * 512), leader);
-          tc_cp_sf(sf_tmem + 16 + kk * 4, desc_sf(st + A_BYTES + C::B_BYTES + SFA_BYTES + kk * 512), leader);
-        }
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          if (kt * 2 + half >= chunks) break;  // the padded half of the last k tile holds only zeros
-          const uint32_t buf = cit % B128_NBUF;
-          ok = __all_sync(0xFFFFFFFFu, mbar_wait(part_empty_bar(buf), ((cit / B128_NBUF) & 1) ^ 1, abort_flag, p.dev_status, p.wait_limit));
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");  // 128 x 80 + 384 x 144 = 512 x 128 registers
+    if (warp == 0) {
+      // ===================================== TMA producer =====================================================
+      const uint32_t leader = elect_leader();
+      uint32_t it = 0, s = 0, wait_parity = 1;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
+        const int32_t mt = (int32_t)(t / p.n_tiles), nt = (int32_t)(t % p.n_tiles);
+        const uint8_t* sfa_src = p.a_sf + (size_t)mt * p.sf_tiles_a * 512;
+        const int32_t sfb_tile = (nt * TN) >> 7, sfb_last = (int32_t)((p.N + 127) / 128) - 1;
+        const uint8_t* sfb_src = p.b_sf + (size_t)sfb_tile * p.sf_tiles_b * 512;
+        // (a tile may start in the middle of a 128-row scale tile; columns beyond N are computed with whatever scales and not stored)
+        const uint8_t* sfb_src1 = p.b_sf + (size_t)min(sfb_tile + 1, sfb_last) * p.sf_tiles_b * 512;
+        for (int32_t kt = 0; kt < p.k_tiles; ++kt, ++it, s = (s + 1 == (uint32_t)STAGES ? 0u : s + 1), wait_parity ^= (s == 0)) {
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty_bar(s), wait_parity, abort_flag, p.dev_status, p.wait_limit));
           if (!ok) break;
-          tc_fence_after();
-          const uint32_t d_tmem = tmem_base + buf * 128;
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const int kk = 2 * half + q;
-            tc_mma_nvf4(d_tmem, desc_sw128(st + kk * 32), desc_sw128(st + A_BYTES + kk * 32), idesc, sf_tmem + kk * 4,
-                        sf_tmem + 16 + kk * 4, q, leader);
+          const uint32_t st = smem_base + s * B128_STAGE_BYTES;
+          mbar_expect_tx(full_bar(s), B128_STAGE_BYTES, leader);
+          tma_load_2d(st, &tmA, kt * (BK / 2), mt * BM, full_bar(s), leader);
+          tma_load_2d(st + A_BYTES, &tmB, kt * (BK / 2), nt * TN, full_bar(s), leader);
+          bulk_load(st + A_BYTES + B128_B_BYTES, sfa_src + (size_t)kt * 2048, 2048, full_bar(s), leader);
+          bulk_load(st + A_BYTES + B128_B_BYTES + SFA_BYTES, sfb_src + (size_t)kt * 2048, 2048, full_bar(s), leader);
+          bulk_load(st + A_BYTES + B128_B_BYTES + SFA_BYTES + 2048, sfb_src1 + (size_t)kt * 2048, 2048, full_bar(s), leader);
+        }
+        // OutControl: the BF16 outlier channels of both operands, 64 per stage, into the same stage buffers
+        for (int32_t h = 0; h < p.hp_k_tiles && ok; ++h, ++it, s = (s + 1 == (uint32_t)STAGES ? 0u : s + 1), wait_parity ^= (s == 0)) {
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty_bar(s), wait_parity, abort_flag, p.dev_status, p.wait_limit));
+          if (!ok) break;
+          const uint32_t st = smem_base + s * B128_STAGE_BYTES;
+          mbar_expect_tx(full_bar(s), A_BYTES + B128_B_BYTES, leader);
+          tma_load_2d(st, &tmAh, h * 64, mt * BM, full_bar(s), leader);
+          tma_load_2d(st + A_BYTES, &tmBh, h * 64, nt * TN, full_bar(s), leader);
+        }
+      }
+      if (!ok) {
+        const uint32_t n_back = it < (uint32_t)STAGES ? it : (uint32_t)STAGES;
+        for (uint32_t j = 0; j < n_back; ++j) {
+          const uint32_t f = it - 1 - j;
+          const long long t0 = clock64();
+          while (!mbar_try(full_bar(f % STAGES), (f / STAGES) & 1) && clock64() - t0 < p.wait_limit) {
           }
-          tc_commit(part_full_bar(buf), leader);
-          ++cit;
         }
-        tc_commit(empty_bar(s), leader);
       }
-      if (p.hp_k_tiles > 0 && ok) {
-        // high-precision side product: one more partial, handed to the promotion warps like a 128-k chunk (scale 1)
-        const uint32_t buf = cit % B128_NBUF;
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(part_empty_bar(buf), ((cit / B128_NBUF) & 1) ^ 1, abort_flag, p.dev_status, p.wait_limit));
-        if (!ok) break;
+    } else if (warp == 1) {
+      // ===================================== MMA issuer =======================================================
+      const uint32_t leader = elect_leader();
+      const uint32_t idesc = instr_desc<TN>();
+      uint32_t it = 0, stage = 0, phase = 0, buf = 0, buf_parity = 1;
+      bool ok = true;
+      auto take_buffer = [&]() {
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(part_empty_bar(buf), buf_parity, abort_flag, p.dev_status, p.wait_limit));
         tc_fence_after();
-        const uint32_t idesc_bf16 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-        for (int32_t h = 0; h < p.hp_k_tiles; ++h, ++it) {
-          const int s = it % STAGES;
-          ok = __all_sync(0xFFFFFFFFu, mbar_wait(full_bar(s), (it / STAGES) & 1, abort_flag, p.dev_status, p.wait_limit));
+      };
+      auto next_buffer = [&]() {
+        buf = buf + 1 == (uint32_t)B128_NBUF ? 0u : buf + 1;
+        buf_parity ^= (buf == 0);
+      };
+      auto take_stage = [&]() {
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(full_bar(stage), phase, abort_flag, p.dev_status, p.wait_limit));
+        tc_fence_after();
+      };
+      auto give_stage = [&]() {
+        tc_commit(empty_bar(stage), leader);
+        stage = stage + 1 == (uint32_t)STAGES ? 0u : stage + 1;
+        phase ^= (stage == 0);
+      };
+      for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
+        // scales of the B rows: a tile that starts 64 rows into its first scale tile finds its own two columns later
+        const uint32_t sfb_col = (uint32_t)((((int32_t)(t % p.n_tiles) * TN) & 127) >> 5);
+        for (int32_t kt = 0; kt < p.k_tiles && ok; ++kt, ++it) {
+          take_stage();
           if (!ok) break;
-          tc_fence_after();
-          const uint32_t st = smem_base + s * C::STAGE_BYTES;
+          const uint32_t st = smem_base + stage * B128_STAGE_BYTES;
+          const uint32_t sf_tmem = tmem_base + B128_NBUF * TN + (it % B128_SF_SETS) * B128_SF_COLS;
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)  // 64 BF16 = one 128-byte swizzle row = four K = 16 steps of 32 bytes
-            tc_mma_bf16(tmem_base + buf * 128, desc_sw128(st + kk * 32), desc_sw128(st + A_BYTES + kk * 32), idesc_bf16,
-                        (h | kk) != 0, leader);
-          tc_commit(empty_bar(s), leader);
+          for (int kk = 0; kk < BK / 64; ++kk) {
+            tc_cp_sf(sf_tmem + kk * 4, desc_sf(st + A_BYTES + B128_B_BYTES + kk * 512), leader);
+            tc_cp_sf(sf_tmem + 16 + kk * 8, desc_sf(st + A_BYTES + B128_B_BYTES + SFA_BYTES + kk * 512), leader);
+            tc_cp_sf(sf_tmem + 20 + kk * 8, desc_sf(st + A_BYTES + B128_B_BYTES + SFA_BYTES + 2048 + kk * 512), leader);
+          }
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            if (kt * 2 + half >= chunks) break;  // the padded half of the last k tile holds only zeros
+            take_buffer();
+            if (!ok) break;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              const int kk = 2 * half + q;
+              tc_mma_nvf4(tmem_base + buf * TN, desc_sw128(st + kk * 32), desc_sw128(st + A_BYTES + kk * 32), idesc, sf_tmem + kk * 4,
+                          sf_tmem + 16 + kk * 8 + sfb_col, q, leader);
+            }
+            tc_commit(part_full_bar(buf), leader);
+            next_buffer();
+          }
+          if (!ok) break;
+          give_stage();
         }
-        if (!ok) break;
-        tc_commit(part_full_bar(buf), leader);
-        ++cit;
+        if (p.hp_k_tiles > 0 && ok) {
+          // high-precision side product: one more partial, promoted like a 128-k chunk (scale 1)
+          take_buffer();
+          if (!ok) break;
+          const uint32_t idesc_bf16 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+          for (int32_t h = 0; h < p.hp_k_tiles; ++h) {
+            take_stage();
+            if (!ok) break;
+            const uint32_t st = smem_base + stage * B128_STAGE_BYTES;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)  // 64 BF16 = one 128-byte swizzle row = four K = 16 steps of 32 bytes
+              tc_mma_bf16(tmem_base + buf * TN, desc_sw128(st + kk * 32), desc_sw128(st + A_BYTES + kk * 32), idesc_bf16, (h | kk) != 0, leader);
+            give_stage();
+          }
+          if (!ok) break;
+          tc_commit(part_full_bar(buf), leader);
+          next_buffer();
+        }
       }
-    }
-    tc_commit(drain_bar, leader);
-    {
-      const long long t0 = clock64();
-      while (!mbar_try(drain_bar, 0) && clock64() - t0 < p.wait_limit) {
+      tc_commit(drain_bar, leader);
+      {
+        const long long t0 = clock64();
+        while (!mbar_try(drain_bar, 0) && clock64() - t0 < p.wait_limit) {
+        }
+      }
+    } else {
+      // ===================================== global scales (two warps) ========================================
+      // Ring slots of four chunks: per chunk SgA, then SgB. Within 32 rows of A, row r sits at (r & 7) * 4 + (r >> 3): the four rows
+      // of a thread's fragments (lane / 4 + 0, 8, 16, 24) are neighbours. Within 32 columns of B, column n sits at its bits
+      // reordered n4 n2 n1 n3 n0: four of a thread's columns (8 i + 2 (lane % 4) + {0, 1} for an even i and i + 1) are neighbours.
+      // A lane reads four chunks of its five rows at once, a slot ahead (the rows lie 4 G bytes apart: a load per chunk, or an
+      // asynchronous 4-byte copy, is 32 sectors for 128 bytes, and the barriers and reads of the promotion warps queue behind
+      // them: 16384 x 8192 x 8192 took 1454 us with such copies).
+      constexpr int ROWS = (128 + TN) / 64;  // per lane and warp
+      const int64_t G = p.g_per_row;         // global scales per operand row (= padded K / 128)
+      const uint32_t r = (uint32_t)lane;
+      const uint32_t at_a = ((r & 7u) * 4u + (r >> 3)) * 4u, at_b = ((r & 0x11u) | ((r & 6u) << 1) | ((r & 8u) >> 2)) * 4u;
+      const uintptr_t bases = reinterpret_cast<uintptr_t>(p.a_gscale) | reinterpret_cast<uintptr_t>(p.b_gscale);
+      const int vec = (G & 3) == 0 && (bases & 15u) == 0 ? 4 : (G & 1) == 0 && (bases & 7u) == 0 ? 2 : 1;
+      const int32_t slots_per_tile = (chunks + 3) >> 2;
+      uint32_t slot = 0, wait_parity = 1;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
+        const int64_t m0 = (t / p.n_tiles) * BM, n0 = (t % p.n_tiles) * TN;
+        const float* src[ROWS];
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+          const int q = (warp - 2) * ROWS + i;  // group of 32: four of A, then those of B
+          const int64_t row = (q < 4 ? m0 + q * 32 : n0 + (q - 4) * 32) + lane, last = (q < 4 ? p.M : p.N) - 1;
+          src[i] = (q < 4 ? p.a_gscale : p.b_gscale) + min(row, last) * G;  // (rows past the end multiply zeros)
+        }
+        float4 v[ROWS];
+        auto load = [&](int32_t c) {
+#pragma unroll
+          for (int i = 0; i < ROWS; ++i) v[i] = load_scales4(src[i], c, chunks, vec);
+        };
+        load(0);
+        for (int32_t j = 0; j < slots_per_tile; ++j, slot = (slot + 1 == (uint32_t)SLOTS ? 0u : slot + 1), wait_parity ^= (slot == 0)) {
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(sc_empty_bar(slot), wait_parity, abort_flag, p.dev_status, p.wait_limit));
+          if (!ok) break;
+          const uint32_t dst = scale_base + slot * B128_SC_BYTES;
+#pragma unroll
+          for (int i = 0; i < ROWS; ++i) {
+            const int q = (warp - 2) * ROWS + i;
+            const uint32_t d = dst + q * 128 + (q < 4 ? at_a : at_b);
+            const float f[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) asm volatile("st.shared.f32 [%0], %1;" ::"r"(d + c * B128_SC_CHUNK), "f"(f[c]) : "memory");
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(sc_full_bar(slot));
+          if (j + 1 < slots_per_tile) load(4 * (j + 1));
+        }
       }
     }
   } else {
-    // ---- promotion + epilogue: thread = one output row, 128 FP32 accumulators in registers -----------------
-    const int quad = warp & 3;
-    const int epi_tid = (warp - 2) * 32 + lane;  // 0..127
-    const int64_t G = p.g_per_row;               // global scales per operand row (= padded K / 128)
-    uint32_t cit = 0;
+    // ===================================== promotion and epilogue ===============================================
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
+    const int quad = warp & 3, third = (warp - 4) >> 2;  // 32 rows, 64 columns
+    const int lr = lane >> 2, lc = lane & 3;
+    const uint32_t my_part = tmem_base + ((uint32_t)(quad * 32) << 16) + third * 64;
+    const uint32_t my_stage = staging_base + (uint32_t)(warp - 4) * 4096u;
+    const uint32_t my_sa = scale_base + (uint32_t)(quad * 32 + lr * 4) * 4u;
+    const uint32_t my_sb = scale_base + 512u + (uint32_t)(third * 64 + lc * 4) * 4u;
+    uint32_t slot = 0, slot_parity = 0, buf = 0, buf_parity = 0;
     bool ok = true;
+    float2 acc[2][2][8];  // [16-row half][8-row half][8-column group]
+    // one partial: acc += SgA[row] SgB[column] partial. The scales are read under the first tensor-memory load.
+    auto promote = [&](uint32_t sc, bool scaled) {
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(part_full_bar(buf), buf_parity, abort_flag, p.dev_status, p.wait_limit));
+      if (!ok) return;
+      tc_fence_after();
+      float4 sa4 = make_float4(1.0f, 1.0f, 1.0f, 1.0f), sb4[4] = {sa4, sa4, sa4, sa4};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {  // 16 rows
+        uint32_t v[32];
+        tc_ld_16x256b_x8(my_part + buf * TN + ((uint32_t)(16 * h) << 16), v);
+        if (h == 0 && scaled) {
+          sa4 = lds128(my_sa + sc);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) sb4[j] = lds128(my_sb + sc + j * 64u);
+        }
+        tc_wait_ld();
+        if (h == 1) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(part_empty_bar(buf));
+        }
+        const float2 s0 = h ? make_float2(sa4.z, sa4.z) : make_float2(sa4.x, sa4.x);
+        const float2 s1 = h ? make_float2(sa4.w, sa4.w) : make_float2(sa4.y, sa4.y);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float2 sb = (i & 1) ? make_float2(sb4[i >> 1].z, sb4[i >> 1].w) : make_float2(sb4[i >> 1].x, sb4[i >> 1].y);
+          const float2 x0 = __fmul2_rn(make_float2(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1])), s0);
+          const float2 x1 = __fmul2_rn(make_float2(__uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3])), s1);
+          acc[h][0][i] = __ffma2_rn(x0, sb, acc[h][0][i]);
+          acc[h][1][i] = __ffma2_rn(x1, sb, acc[h][1][i]);
+        }
+      }
+      buf = buf + 1 == (uint32_t)B128_NBUF ? 0u : buf + 1;
+      buf_parity ^= (buf == 0);
+    };
     for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
       const int32_t mt = (int32_t)(t / p.n_tiles), nt = (int32_t)(t % p.n_tiles);
-      // stage SgB[n, :] of this tile as sgb[chunk][n]
-      asm volatile("bar.sync 1, 128;" ::: "memory");  // everyone is done with the previous tile's values
-      {
-        const int64_t n = (int64_t)nt * BN + epi_tid;
-        const float* src = p.b_gscale + n * G;
-        if (n < p.N) {
-          int32_t kc = 0;
-          if ((G & 3) == 0) {  // a row's scales as 16-byte loads, sixteen values in flight per thread
-#pragma unroll 4
-            for (; kc + 4 <= chunks; kc += 4) {
-              const float4 q = __ldg(reinterpret_cast<const float4*>(src + kc));
-              sgb[kc * 128 + epi_tid] = q.x;
-              sgb[(kc + 1) * 128 + epi_tid] = q.y;
-              sgb[(kc + 2) * 128 + epi_tid] = q.z;
-              sgb[(kc + 3) * 128 + epi_tid] = q.w;
-            }
-          }
-          for (; kc < chunks; ++kc) sgb[kc * 128 + epi_tid] = __ldg(src + kc);
-        } else {
-          for (int32_t kc = 0; kc < chunks; ++kc) sgb[kc * 128 + epi_tid] = 0.0f;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) acc[j >> 4][(j >> 3) & 1][j & 7] = make_float2(0.0f, 0.0f);
+      for (int32_t kc = 0; kc < chunks; kc += 4) {
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(sc_full_bar(slot), slot_parity, abort_flag, p.dev_status, p.wait_limit));
+        if (!ok) break;
+        const uint32_t sc = slot * B128_SC_BYTES;
+#pragma unroll 1
+        for (int c = 0; c < 4 && kc + c < chunks; ++c) {
+          promote(sc + c * B128_SC_CHUNK, true);
+          if (!ok) break;
         }
-        if (p.hp_k_tiles > 0) sgb[chunks * 128 + epi_tid] = 1.0f;  // the high-precision partial carries no scale
-      }
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      const int64_t m = (int64_t)mt * BM + quad * 32 + lane;
-      const float* sa_row = p.a_gscale + (m < p.M ? m : 0) * G;
-      float2 acc[64];
-#pragma unroll
-      for (int j = 0; j < 64; ++j) acc[j] = make_float2(0.0f, 0.0f);
-      const int32_t parts = chunks + (p.hp_k_tiles > 0 ? 1 : 0);
-      // SgA[m, kc] is fetched two chunks ahead: with one promotion warp per scheduler nothing else would hide the load
-      float sa_0 = chunks > 0 ? __ldg(sa_row) : 1.0f, sa_1 = chunks > 1 ? __ldg(sa_row + 1) : 1.0f;
-      for (int32_t kc = 0; kc < parts && ok; ++kc, ++cit) {
-        const float sa = kc < chunks ? sa_0 : 1.0f;
-        sa_0 = sa_1;
-        if (kc + 2 < chunks) sa_1 = __ldg(sa_row + kc + 2);
-        const uint32_t buf = cit % B128_NBUF;
-        if (!(ok = mbar_wait(part_full_bar(buf), (cit / B128_NBUF) & 1, abort_flag, p.dev_status, p.wait_limit))) break;
-        tc_fence_after();
-        const float2 sa2 = make_float2(sa, sa);
-        const float4* sb4 = reinterpret_cast<const float4*>(sgb + kc * 128);
-#pragma unroll
-        for (int c0 = 0; c0 < 128; c0 += 32) {
-          uint32_t v[32];
-          tc_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + buf * 128 + c0, v);
-          tc_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            const float4 sb = sb4[(c0 + j) >> 2];
-            const float2 t0 = __fmul2_rn(make_float2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), sa2);
-            const float2 t1 = __fmul2_rn(make_float2(__uint_as_float(v[j + 2]), __uint_as_float(v[j + 3])), sa2);
-            acc[(c0 + j) >> 1] = __ffma2_rn(t0, make_float2(sb.x, sb.y), acc[(c0 + j) >> 1]);
-            acc[((c0 + j) >> 1) + 1] = __ffma2_rn(t1, make_float2(sb.z, sb.w), acc[((c0 + j) >> 1) + 1]);
-          }
-        }
-        tc_fence_before();
+        if (!ok) break;
         __syncwarp();
-        if (lane == 0) mbar_arrive(part_empty_bar(buf));
+        if (lane == 0) mbar_arrive(sc_empty_bar(slot));
+        slot = slot + 1 == (uint32_t)SLOTS ? 0u : slot + 1;
+        slot_parity ^= (slot == 0);
       }
-      if (ok && p.use_tma_store && !p.accumulate) {
-        // 128-byte row pieces staged in shared memory with the 128-byte swizzle and written by the bulk-tensor engine:
-        // full lines, clipped at the edges of C (a thread-per-row store from registers took longer than the whole
-        // promotion loop of a K = 1024 tile)
-        const uint32_t buf = staging_base + (uint32_t)(warp - 2) * 4096u;
-        const int64_t m0 = (int64_t)mt * BM + quad * 32;
-        // (both loops are fully unrolled: the accumulators must be addressed with compile-time indices)
-        if (p.c_is_f32) {
-#pragma unroll
-          for (int c0 = 0; c0 < 128; c0 += 32) {
-            const int64_t n0 = (int64_t)nt * BN + c0;
-            if (n0 < p.N && n0 + 32 > p.N) {  // ragged last chunk of the row
-              if (m < p.M) {
-                float o[32];
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                  o[2 * j] = acc[(c0 >> 1) + j].x;
-                  o[2 * j + 1] = acc[(c0 >> 1) + j].y;
-                }
-                store_ragged<32>(p, m, n0, o);
-              }
-            } else if (n0 < p.N) {
-              if (lane == 0) bulk_wait_read<0>();  // the previous store from this buffer has read it
-              __syncwarp();
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const float2 a0 = acc[(c0 >> 1) + 2 * j], a1 = acc[(c0 >> 1) + 2 * j + 1];
-                const uint32_t dst = buf + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) << 4);
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(__float_as_uint(a0.x)),
-                             "r"(__float_as_uint(a0.y)), "r"(__float_as_uint(a1.x)), "r"(__float_as_uint(a1.y))
-                             : "memory");
-              }
-              fence_async_smem();
-              __syncwarp();
-              if (lane == 0) {
-                tma_store_2d(&tmC, buf, (int32_t)n0, (int32_t)m0);
-                bulk_commit();
-              }
-            }
-          }
-        } else {
-#pragma unroll
-          for (int c0 = 0; c0 < 128; c0 += 64) {
-            const int64_t n0 = (int64_t)nt * BN + c0;
-            if (n0 < p.N && n0 + 64 > p.N) {  // ragged last chunk of the row
-              if (m < p.M) {
-                float o[64];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                  o[2 * j] = acc[(c0 >> 1) + j].x;
-                  o[2 * j + 1] = acc[(c0 >> 1) + j].y;
-                }
-                store_ragged<64>(p, m, n0, o);
-              }
-            } else if (n0 < p.N) {
-              if (lane == 0) bulk_wait_read<0>();
-              __syncwarp();
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                uint32_t q[4];
-#pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                  const float2 a = acc[(c0 >> 1) + 4 * j + h];
-                  const __nv_bfloat162 hh = __floats2bfloat162_rn(a.x, a.y);
-                  q[h] = *reinterpret_cast<const uint32_t*>(&hh);
-                }
-                const uint32_t dst = buf + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) << 4);
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(q[0]), "r"(q[1]), "r"(q[2]), "r"(q[3])
-                             : "memory");
-              }
-              fence_async_smem();
-              __syncwarp();
-              if (lane == 0) {
-                tma_store_2d(&tmC, buf, (int32_t)n0, (int32_t)m0);
-                bulk_commit();
-              }
-            }
-          }
-        }
-      } else if (ok && m < p.M) {
-#pragma unroll
-        for (int c0 = 0; c0 < 128; c0 += 32) {
-          const int64_t n0 = (int64_t)nt * BN + c0;
-          if (n0 < p.N) {
-            float o[32];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              o[2 * j] = acc[(c0 >> 1) + j].x;
-              o[2 * j + 1] = acc[(c0 >> 1) + j].y;
-            }
-            store_row_chunk(p, m, n0, o);
-          }
-        }
+      if (!ok) break;
+      if (p.hp_k_tiles > 0) {  // the high-precision partial carries no scale
+        promote(0, false);
+        if (!ok) break;
       }
+      const int64_t m0 = (int64_t)mt * BM + quad * 32, n0 = (int64_t)nt * TN + third * 64;
+      if (m0 < p.M && n0 < p.N) b128_store64(p, tmC, my_stage, lane, m0, n0, acc);
     }
     if (lane == 0) bulk_wait_all();  // this lane's bulk stores are complete before the CTA may exit
   }
@@ -1392,13 +1457,13 @@ bool make_c_map(CUtensorMap* tm, void* Cp, int64_t M, int64_t N, int64_t ldc, bo
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// A compact BF16 side matrix [R, Kh] (Kh a multiple of 64) as a 2-D tensor; box = 64 columns (128 bytes) x 128 rows.
-bool make_hp_map(CUtensorMap* tm, const void* base, int64_t R, int64_t Kh) {
+// A compact BF16 side matrix [R, Kh] (Kh a multiple of 64) as a 2-D tensor; box = 64 columns (128 bytes) x box_rows rows.
+bool make_hp_map(CUtensorMap* tm, const void* base, int64_t R, int64_t Kh, uint32_t box_rows = 128) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)Kh, (cuuint64_t)R};
   const cuuint64_t strides[1] = {(cuuint64_t)Kh * 2};
-  const cuuint32_t box[2] = {64, 128};
+  const cuuint32_t box[2] = {64, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1418,7 +1483,6 @@ cudaError_t launch_tile128(const GemmArgs& a, cudaStream_t st) {
   if (!make_c_map(&tmC, a.C, a.M, a.N, a.ldc, a.c_is_f32 != 0)) return cudaErrorInvalidValue;
   CUtensorMap tmAh = tmA, tmBh = tmB;  // placeholders unless the high-precision side product is requested
   Params p{};
-  p.use_tma_store = 1;
   p.starve = a.starve_first_stage;
   p.wait_limit = wait_limit_of(a);
   if (a.hp_Kh > 0) {
@@ -1503,17 +1567,16 @@ cudaError_t launch_2cta(const GemmArgs& a, cudaStream_t st) {
 
 cudaError_t launch_block128(const GemmArgs& a, cudaStream_t st) {
   const int64_t Kp = (a.K + 127) & ~(int64_t)127;
-  if (Kp / 128 > B128_MAX_CHUNKS) return cudaErrorInvalidValue;
+  if (Kp > B128_MAX_K) return cudaErrorInvalidValue;
   CUtensorMap tmA, tmB, tmC;
-  if (!make_codes_map(&tmA, a.a_codes, a.M, Kp, BM) || !make_codes_map(&tmB, a.b_codes, a.N, Kp, 128)) return cudaErrorInvalidValue;
+  if (!make_codes_map(&tmA, a.a_codes, a.M, Kp, BM) || !make_codes_map(&tmB, a.b_codes, a.N, Kp, B128_TN)) return cudaErrorInvalidValue;
   Params p{};
   CUtensorMap tmAh = tmA, tmBh = tmB;  // placeholders unless the high-precision side product is requested
   if (a.hp_Kh > 0) {
-    if (!make_hp_map(&tmAh, a.hp_a, a.M, a.hp_Kh) || !make_hp_map(&tmBh, a.hp_b, a.N, a.hp_Kh)) return cudaErrorInvalidValue;
+    if (!make_hp_map(&tmAh, a.hp_a, a.M, a.hp_Kh) || !make_hp_map(&tmBh, a.hp_b, a.N, a.hp_Kh, B128_TN)) return cudaErrorInvalidValue;
     p.hp_k_tiles = (int32_t)(a.hp_Kh / 64);
   }
-  p.use_tma_store = make_c_map(&tmC, a.C, a.M, a.N, a.ldc, a.c_is_f32 != 0) ? 1 : 0;
-  if (!p.use_tma_store) tmC = tmA;  // unused by the kernel then
+  if (!make_c_map(&tmC, a.C, a.M, a.N, a.ldc, a.c_is_f32 != 0)) return cudaErrorInvalidValue;
   p.a_sf = a.a_sf;
   p.b_sf = a.b_sf;
   p.a_gscale = a.a_gscale;
@@ -1528,7 +1591,7 @@ cudaError_t launch_block128(const GemmArgs& a, cudaStream_t st) {
   const int64_t kb_padded = ((Kp >> 4) + 15) & ~(int64_t)15;
   p.sf_tiles_a = p.sf_tiles_b = (int32_t)(kb_padded >> 2);
   p.m_tiles = (int32_t)((a.M + BM - 1) / BM);
-  p.n_tiles = (int32_t)((a.N + 127) / 128);
+  p.n_tiles = (int32_t)((a.N + B128_TN - 1) / B128_TN);
   p.c_is_f32 = a.c_is_f32;
   p.accumulate = a.accumulate;
   p.dev_status = a.dev_status;
@@ -1537,7 +1600,7 @@ cudaError_t launch_block128(const GemmArgs& a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   const int64_t tiles = (int64_t)p.m_tiles * p.n_tiles;
   const unsigned grid = (unsigned)std::min<int64_t>(tiles, sm_count());
-  launch_kernel(gemm_nvfp4_block128_kernel, dim3(grid), dim3(NUM_THREADS), B128_SMEM_BYTES, st, tmA, tmB, tmC, tmAh, tmBh, p);
+  launch_kernel(gemm_nvfp4_block128_kernel, dim3(grid), dim3(B128_THREADS), B128_SMEM_BYTES, st, tmA, tmB, tmC, tmAh, tmBh, p);
   return cudaGetLastError();
 }
 
@@ -1589,7 +1652,6 @@ cudaError_t launch_dense_gemm(const void* A, const void* B, int64_t M, int64_t N
   if (!make_hp_map(&tmAh, A, M, ld) || !make_hp_map(&tmBh, B, N, ld) || !make_c_map(&tmC, Cp, M, N, ldc, c_is_f32 != 0))
     return cudaErrorInvalidValue;
   Params p{};
-  p.use_tma_store = 1;
   p.wait_limit = DEFAULT_WAIT_LIMIT_CYCLES;
   p.hp_k_tiles = (int32_t)(ld / 64);
   p.a_gscale = a_gscale;
@@ -1612,7 +1674,7 @@ cudaError_t launch_dense_gemm(const void* A, const void* B, int64_t M, int64_t N
 }
 
 size_t gemm_workspace_bytes(int64_t, int64_t, int64_t) { return 0; }
-int64_t gemm_block128_max_k() { return (int64_t)B128_MAX_CHUNKS * 128; }
+int64_t gemm_block128_max_k() { return B128_MAX_K; }
 
 // Variant choice, by a cost model: rounds of the variant's tiles over the SMs (or SM pairs) x time of a tile, which is a constant and
 // so much per 256-wide k tile, or at short K what writing the tile takes. All kernels are bound by what the L2 delivers to the SMs and by
