@@ -28,7 +28,7 @@ struct QuantRowsArgs {
   const int32_t* keep;  // optional column list of length K
   const int32_t* excluded;  // optional: the sorted complement of `keep` (cols_src - K entries); enables the masked amax
   // optional (with `excluded`): excl_out[r, j] = src[r, excluded[j]], zero for cols_src - K <= j < ld_excl_out. Written by the
-  // masked amax pass where that runs (the matrix is read once for both), else by a separate gather launch.
+  // masked amax pass where that runs, else by the quantizer from the rows that it stages, else by a separate gather launch.
   uint16_t* excl_out;
   int64_t ld_excl_out;
   uint64_t seed;

@@ -370,7 +370,8 @@ __device__ __forceinline__ void quantize_rows_body(const uint16_t* __restrict__ 
                      const int32_t* __restrict__ keep, uint64_t seed, uint32_t stream_id,
                      const uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
                      float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, int64_t cols_src,
-                     int64_t stage_cols8, uint32_t rht_stream, int sb_up, const PhiloxKeys& pk, uint32_t bx) {
+                     int64_t stage_cols8, const int32_t* __restrict__ excluded, uint32_t n_excl, uint16_t* __restrict__ excl_out,
+                     uint32_t ld_excl_out, uint32_t rht_stream, int sb_up, const PhiloxKeys& pk, uint32_t bx) {
   constexpr int NB = 4;  // inner blocks per thread; all loads are issued before any arithmetic
   extern __shared__ uint16_t row_stage[];  // GATHER only: the source rows this CTA touches, [n_rows][cols_src8]
   const int64_t Kp = (K + 127) & ~(int64_t)127;
@@ -418,6 +419,18 @@ __device__ __forceinline__ void quantize_rows_body(const uint16_t* __restrict__ 
         if (off[q] != 0xFFFFFFFFu) *reinterpret_cast<uint4*>(row_stage + off[q]) = v[q];
     }
     __syncthreads();
+    if (excl_out) {
+      // OutControl's BF16 side operand: the excluded columns of the staged rows that begin in this CTA, two per thread and step
+      // (a launch of its own that gathered them read the matrix once more: the MLP at 8192 tokens, 10 % of the channels, 797 / 775 us)
+      const int64_t own0 = (first + nb - 1) / nb;
+      const uint32_t pairs = ld_excl_out >> 1, n_own = (uint32_t)max((int64_t)0, stage_row0 + n_rows - own0);
+      for (uint32_t e = threadIdx.x; e < n_own * pairs; e += 256) {
+        const uint32_t rr = e / pairs, c = (e - rr * pairs) * 2u;
+        const uint16_t* sp = row_stage + (own0 - stage_row0 + rr) * stage_cols8;
+        const uint32_t lo = c < n_excl ? (uint32_t)sp[excluded[c]] : 0u, hi = c + 1 < n_excl ? (uint32_t)sp[excluded[c + 1]] : 0u;
+        *reinterpret_cast<uint32_t*>(excl_out + (own0 + rr) * ld_excl_out + c) = lo | (hi << 16);
+      }
+    }
   }
 
   // Rows, K and the leading dimension are below 2^31 (checked by the launcher): row / block / column indices are 32-bit,
@@ -582,9 +595,10 @@ quantize_rows_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, 
                      const int32_t* __restrict__ keep, uint64_t seed, uint32_t stream_id,
                      const uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
                      float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, int64_t cols_src,
-                     int64_t stage_cols8, uint32_t rht_stream, int sb_up, const __grid_constant__ PhiloxKeys pk) {
+                     int64_t stage_cols8, const int32_t* __restrict__ excluded, uint32_t n_excl, uint16_t* __restrict__ excl_out,
+                     uint32_t ld_excl_out, uint32_t rht_stream, int sb_up, const __grid_constant__ PhiloxKeys pk) {
   pdl_prologue();
-  quantize_rows_body<GS, SR, TILED, GATHER, RHT>(src, rows, K, ld, keep, seed, stream_id, gs_cells, gs_words, codes, sf, gscale, div_mul, div_shift, wide_loads, cols_src, stage_cols8, rht_stream, sb_up, pk, tail_first<GS>(blockIdx.x));
+  quantize_rows_body<GS, SR, TILED, GATHER, RHT>(src, rows, K, ld, keep, seed, stream_id, gs_cells, gs_words, codes, sf, gscale, div_mul, div_shift, wide_loads, cols_src, stage_cols8, excluded, n_excl, excl_out, ld_excl_out, rht_stream, sb_up, pk, tail_first<GS>(blockIdx.x));
 }
 
 
@@ -1757,7 +1771,7 @@ quantize_rows_pair_kernel(const __grid_constant__ RowsJob a, const __grid_consta
   if (GS == kGsTensor) bx = j.blocks - 1u - bx;  // (tail_first)
   const PhiloxKeys no_keys{};
   quantize_rows_body<GS, false, true, false, false>(j.src, j.rows, j.K, j.ld, nullptr, 0ull, j.stream_id, j.gs_cells, j.gs_words, j.codes, j.sf,
-                                                    j.gscale, j.div_mul, j.div_shift, j.wide_loads, 0, 0, 0u, 0, no_keys, bx);
+                                                    j.gscale, j.div_mul, j.div_shift, j.wide_loads, 0, 0, nullptr, 0u, nullptr, 0u, 0u, 0, no_keys, bx);
   clear_scale_padding(j.sf, (uint32_t)j.rows, (((uint32_t)j.K + 127u) & ~127u) >> 4, bx, j.blocks);
 }
 
@@ -1818,6 +1832,14 @@ static void division_constants(int64_t total, int64_t slack, uint64_t d, uint32_
   }
 }
 
+// Shared memory for the source rows that a CTA of the compacting row quantizer touches (its 1024 blocks span at most 1024 / nb + 2
+// rows); 0 if they do not fit or cannot be copied in 16-byte pieces.
+static size_t gather_stage_bytes(const QuantRowsArgs& a) {
+  const int64_t cols8 = (a.cols_src + 7) & ~(int64_t)7, nb = ((a.K + 127) & ~(int64_t)127) >> 4;
+  const size_t smem = (size_t)((1024 / nb + 2) * cols8 * 2);
+  return smem > 160 * 1024 || (reinterpret_cast<uintptr_t>(a.keep) & 15u) != 0 || (a.ld & 7) != 0 ? 0 : smem;
+}
+
 template <int GS, bool SR, bool TILED>
 static cudaError_t launch_rows_g(const QuantRowsArgs& a, cudaStream_t st) {
   const int64_t Kp = (a.K + 127) & ~(int64_t)127;
@@ -1828,26 +1850,21 @@ static cudaError_t launch_rows_g(const QuantRowsArgs& a, cudaStream_t st) {
   division_constants(total, 1024, d, div_mul, div_shift);
   const int wide_loads = ((reinterpret_cast<uintptr_t>(a.src) & 31u) == 0 && (a.ld & 15) == 0) ? 1 : 0;
   if (a.keep) {
-    // rows a CTA can touch: its 1024 blocks span at most 1024 / nb + 2 rows; stage them if they fit in shared memory
-    const int64_t cols8 = (a.cols_src + 7) & ~(int64_t)7;
-    const int64_t max_rows = 1024 / (int64_t)d + 2;
-    size_t smem = (size_t)(max_rows * cols8 * 2);
-    int64_t stage_cols8 = cols8;
-    if (smem > 160 * 1024 || (reinterpret_cast<uintptr_t>(a.keep) & 15u) != 0 || (a.ld & 7) != 0) {
-      smem = 0;
-      stage_cols8 = 0;  // fall back to per-element global loads
-    } else {
+    const size_t smem = gather_stage_bytes(a);
+    const int64_t stage_cols8 = smem ? (a.cols_src + 7) & ~(int64_t)7 : 0;  // (0: per-element global loads)
+    if (smem) {
       cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(quantize_rows_kernel<GS, SR, TILED, true, false>), smem);
       if (e != cudaSuccess) return e;
     }
     launch_kernel(quantize_rows_kernel<GS, SR, TILED, true, false>, dim3(grid), dim3(256), smem, st, a.src, a.rows, a.K, a.ld, a.keep, a.seed,
-                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, stage_cols8, 0u, a.sr == 2, make_philox_keys(a.seed));
+                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, stage_cols8, a.excluded, (uint32_t)(a.cols_src - a.K),
+                  stage_cols8 > 0 ? a.excl_out : nullptr, (uint32_t)a.ld_excl_out, 0u, a.sr == 2, make_philox_keys(a.seed));
   } else if (a.rht_stream) {
     launch_kernel(quantize_rows_kernel<GS, SR, TILED, false, true>, dim3(grid), dim3(256), 0, st, a.src, a.rows, a.K, a.ld, nullptr, a.seed,
-                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, (int64_t)0, a.rht_stream, a.sr == 2, make_philox_keys(a.seed));
+                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, (int64_t)0, nullptr, 0u, nullptr, 0u, a.rht_stream, a.sr == 2, make_philox_keys(a.seed));
   } else {
     launch_kernel(quantize_rows_kernel<GS, SR, TILED, false, false>, dim3(grid), dim3(256), 0, st, a.src, a.rows, a.K, a.ld, nullptr, a.seed,
-                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, (int64_t)0, 0u, a.sr == 2, make_philox_keys(a.seed));
+                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, (int64_t)0, nullptr, 0u, nullptr, 0u, 0u, a.sr == 2, make_philox_keys(a.seed));
   }
   return cudaGetLastError();
 }
@@ -1892,6 +1909,8 @@ static cudaError_t launch_quantize_rows_impl(const QuantRowsArgs& a0, cudaStream
   if (a.compute_amax) a.gs_words = 1;
   if (a.rows == 0 || a.K == 0) return cudaSuccess;
   if (a.rows >= ((int64_t)1 << 31) || a.cols_src >= ((int64_t)1 << 31) || a.ld >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
+  if (!a.excluded || (a.ld_excl_out & 1) || (reinterpret_cast<uintptr_t>(a.excl_out) & 3u)) a.excl_out = nullptr;
+  side_copy_done = a.keep && a.excl_out && gather_stage_bytes(a) != 0;  // the quantizer writes it from the rows that it stages
   cudaError_t e;
   if (a.rht_stream) {  // the scales come from the transformed data; column lists are not combined with the transformation
     if (a.keep) return cudaErrorInvalidValue;
@@ -1929,6 +1948,7 @@ static cudaError_t launch_quantize_rows_impl(const QuantRowsArgs& a0, cudaStream
                       (uint64_t)((1ull << 32) / (uint64_t)std::max<int64_t>(1, a.ld_excl_out) + 1ull));
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         side_copy_done = a.excl_out != nullptr;
+        a.excl_out = nullptr;
         return launch_rows_r<kGsTensor>(a, st);
       }
       // amax over the kept columns only: one row per CTA, one atomic per row
