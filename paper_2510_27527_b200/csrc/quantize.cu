@@ -349,13 +349,89 @@ __global__ void __launch_bounds__(256) amax_rows_rht_kernel(const uint16_t* __re
 }
 
 // =========================================================================================================
-// Shared epilogue of one 16-element inner block: scale, round, pack.
+// Shared epilogue of one 16-element inner block (row r, block b of its row): scales, rounding, packing and stores. The 32 threads
+// of a warp call it together; eight neighbouring ones hold the eight blocks of an outer block. in_k: the block begins below K.
 // =========================================================================================================
+template <int GS, bool SR, bool TILED, bool RHT>
+__device__ __forceinline__ void finish_block16(const uint32_t (&w)[8], uint32_t r, uint32_t b, bool active, bool in_k, uint32_t Kp, uint32_t K16,
+                                               float Sg_t, uint64_t seed, uint32_t stream_id, const uint32_t* __restrict__ gs_cells,
+                                               uint8_t* __restrict__ codes, uint8_t* __restrict__ sf, float* __restrict__ gscale,
+                                               uint32_t rht_stream, int sb_up, const PhiloxKeys& pk) {
+  const uint32_t k0 = b << 4, nb = Kp >> 4;
+  float x[16];
+  uint32_t amax_b_bits;  // binary32 pattern of the block's amax (non-negative, so integer order = float order)
+  if (RHT) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      x[2 * i] = bf16_lo(w[i]);
+      x[2 * i + 1] = bf16_hi(w[i]);
+    }
+    // blocks past K (layout padding up to 128) take no signs, so that they stay +0 and encode as zero bytes
+    rht_scale16(x, in_k ? rht_sign16(seed, rht_stream, (int64_t)k0) : 0u);
+    hadamard16_butterflies(x);
+    float m = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) m = fmaxf(m, fabsf(x[i]));
+    amax_b_bits = __float_as_uint(m);
+  } else {
+    uint32_t m2 = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m2 = amax16x2(m2, w[i]);
+    amax_b_bits = hmax_of_pair(bf16x2_abs_bits(m2)) << 16;
+  }
+
+  // ---- global scale -------------------------------------------------------------------------------------
+  float Sg;
+  if (GS == kGsBlock128) {
+    uint32_t g = amax_b_bits;
+    g = max(g, __shfl_xor_sync(0xFFFFFFFFu, g, 1));
+    g = max(g, __shfl_xor_sync(0xFFFFFFFFu, g, 2));
+    g = max(g, __shfl_xor_sync(0xFFFFFFFFu, g, 4));
+    Sg = global_scale_from_amax(__uint_as_float(g));
+    if (active && (b & 7) == 0) gscale[(size_t)r * (Kp >> 7) + (b >> 3)] = Sg;
+  } else if (GS == kGsRow) {
+    Sg = global_scale_from_amax(__uint_as_float(gs_cells[r]));
+    if (active && b == 0) gscale[r] = Sg;
+  } else {
+    Sg = Sg_t;
+  }
+
+  // ---- block scale, rounding, packing -------------------------------------------------------------------
+  float rcp;
+  const uint32_t sb = block_scale(__uint_as_float(amax_b_bits), Sg, rcp, SR && sb_up);
+  if (!RHT) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      x[2 * i] = bf16_lo(w[i]);
+      x[2 * i + 1] = bf16_hi(w[i]);
+    }
+  }
+  const uint2 packed = quantize_block16<SR>(x, rcp, pk, stream_id, ((uint64_t)r * K16 + k0) >> 3);
+
+  // four neighbouring threads own the four scale bytes of one 32-bit word in either layout
+  uint32_t sf4 = sb << (8 * (b & 3));
+  sf4 |= __shfl_xor_sync(0xFFFFFFFFu, sf4, 1);
+  sf4 |= __shfl_xor_sync(0xFFFFFFFFu, sf4, 2);
+  if (active) {
+    *reinterpret_cast<uint2*>(codes + (size_t)r * (Kp >> 1) + (k0 >> 1)) = packed;
+    if ((b & 3) == 0) {
+      size_t off;
+      if (TILED) {
+        const uint32_t tile = (r >> 7) * (((nb + 15u) & ~15u) >> 2) + (b >> 2);  // 512-byte tiles, k fastest
+        off = (size_t)tile * 512u + ((r & 31u) * 16u + ((r >> 5) & 3u) * 4u);       // b & 3 == 0 here
+      } else {
+        off = (size_t)r * nb + b;
+      }
+      *reinterpret_cast<uint32_t*>(sf + off) = sf4;
+    }
+  }
+}
+
 // =========================================================================================================
 // Row-axis quantize from BF16: one thread per inner block, eight neighbouring threads per 128-wide outer block.
 //   GS      scale mode. TENSOR reads the amax cell gs_cells[0]; ROW reads gs_cells[row]; BLOCK128 reduces the
 //           group amax over the 8 threads of the group with shuffles (single pass over the data).
-//   GATHER  columns come from the list `keep` (OutControl compaction) instead of 0..cols-1.
+//   GATHER  columns come from the list `keep` instead of 0..cols-1, element by element: what quantize_rows_gather_kernel cannot take.
 //   RHT     each block is replaced by (x S) H_16 before anything else looks at it (never together with GATHER).
 // =========================================================================================================
 // CTAs of a TENSOR-mode quantizer take the tensor from its end: the amax pass before them has just read that end, so part of it is
@@ -369,69 +445,14 @@ template <int GS, bool SR, bool TILED, bool GATHER, bool RHT>
 __device__ __forceinline__ void quantize_rows_body(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld,
                      const int32_t* __restrict__ keep, uint64_t seed, uint32_t stream_id,
                      const uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
-                     float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, int64_t cols_src,
-                     int64_t stage_cols8, const int32_t* __restrict__ excluded, uint32_t n_excl, uint16_t* __restrict__ excl_out,
-                     uint32_t ld_excl_out, uint32_t rht_stream, int sb_up, const PhiloxKeys& pk, uint32_t bx) {
+                     float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads,
+                     uint32_t rht_stream, int sb_up, const PhiloxKeys& pk, uint32_t bx) {
   constexpr int NB = 4;  // inner blocks per thread; all loads are issued before any arithmetic
-  extern __shared__ uint16_t row_stage[];  // GATHER only: the source rows this CTA touches, [n_rows][cols_src8]
   const int64_t Kp = (K + 127) & ~(int64_t)127;
   const int64_t K16 = (K + 15) & ~(int64_t)15;
   const int64_t nb = Kp >> 4;  // inner blocks per operand row (multiple of 8)
   const int64_t total = rows * nb;
   const int64_t cta_base = (int64_t)bx * (256 * NB) + threadIdx.x;
-  // GATHER (OutControl compaction): the CTA's blocks cover a few whole or partial source rows; copy those rows to
-  // shared memory with coalesced 16-byte loads, then pick the kept columns from there.
-  int64_t stage_row0 = 0;
-  if (GATHER && stage_cols8 > 0) {
-    const int64_t first = (int64_t)bx * (256 * NB);
-    const int64_t last = min(first + 256 * NB, total) - 1;
-    stage_row0 = first / nb;
-    const int64_t n_rows = last / nb - stage_row0 + 1;
-    const uint32_t chunks_per_row = (uint32_t)(stage_cols8 >> 3);
-    const uint32_t n_chunks = (uint32_t)n_rows * chunks_per_row;
-    // e / chunks_per_row by multiplication (exact while e * chunks_per_row < 2^32, and a CTA stages a few thousand chunks)
-    const uint64_t inv = (1ull << 32) / chunks_per_row + 1ull;
-    // eight chunks per thread and pass, every load issued before the first store: one exposed memory latency per pass
-    for (uint32_t e0 = threadIdx.x; e0 < n_chunks; e0 += 256 * 8) {
-      uint4 v[8];
-      uint32_t off[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const uint32_t e = e0 + q * 256;
-        v[q] = make_uint4(0, 0, 0, 0);
-        off[q] = 0xFFFFFFFFu;
-        if (e < n_chunks) {
-          const uint32_t rr = (uint32_t)(((uint64_t)e * inv) >> 32), ch = (e - rr * chunks_per_row) << 3;
-          off[q] = rr * (uint32_t)stage_cols8 + ch;
-          const uint16_t* p = src + (stage_row0 + rr) * ld + ch;
-          if ((int64_t)ch + 8 <= cols_src) {
-            v[q] = *reinterpret_cast<const uint4*>(p);
-          } else {
-            uint32_t t[4] = {0, 0, 0, 0};
-            for (int i = 0; i < 8; ++i)
-              if ((int64_t)ch + i < cols_src) t[i >> 1] |= (uint32_t)p[i] << (16 * (i & 1));
-            v[q] = make_uint4(t[0], t[1], t[2], t[3]);
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (off[q] != 0xFFFFFFFFu) *reinterpret_cast<uint4*>(row_stage + off[q]) = v[q];
-    }
-    __syncthreads();
-    if (excl_out) {
-      // OutControl's BF16 side operand: the excluded columns of the staged rows that begin in this CTA, two per thread and step
-      // (a launch of its own that gathered them read the matrix once more: the MLP at 8192 tokens, 10 % of the channels, 797 / 775 us)
-      const int64_t own0 = (first + nb - 1) / nb;
-      const uint32_t pairs = ld_excl_out >> 1, n_own = (uint32_t)max((int64_t)0, stage_row0 + n_rows - own0);
-      for (uint32_t e = threadIdx.x; e < n_own * pairs; e += 256) {
-        const uint32_t rr = e / pairs, c = (e - rr * pairs) * 2u;
-        const uint16_t* sp = row_stage + (own0 - stage_row0 + rr) * stage_cols8;
-        const uint32_t lo = c < n_excl ? (uint32_t)sp[excluded[c]] : 0u, hi = c + 1 < n_excl ? (uint32_t)sp[excluded[c + 1]] : 0u;
-        *reinterpret_cast<uint32_t*>(excl_out + (own0 + rr) * ld_excl_out + c) = lo | (hi << 16);
-      }
-    }
-  }
 
   // Rows, K and the leading dimension are below 2^31 (checked by the launcher): row / block / column indices are 32-bit,
   // only the final byte offsets are formed in 64 bits (one widening multiply each).
@@ -481,15 +502,6 @@ __device__ __forceinline__ void quantize_rows_body(const uint16_t* __restrict__ 
             w[j][0] = v0.x; w[j][1] = v0.y; w[j][2] = v0.z; w[j][3] = v0.w;
             w[j][4] = v1.x; w[j][5] = v1.y; w[j][6] = v1.z; w[j][7] = v1.w;
           }
-        } else if (GATHER && stage_cols8 > 0 && k0 + 16 <= K32) {
-          const uint16_t* sp = row_stage + ((int64_t)r - stage_row0) * stage_cols8;
-          const int4* kp = reinterpret_cast<const int4*>(keep + k0);  // keep is 16-byte aligned, k0 a multiple of 16
-  #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int4 id = kp[q];
-            w[j][2 * q] = (uint32_t)sp[id.x] | ((uint32_t)sp[id.y] << 16);
-            w[j][2 * q + 1] = (uint32_t)sp[id.z] | ((uint32_t)sp[id.w] << 16);
-          }
         } else {
           for (int i = 0; i < 16; ++i) {
             if (k0 + i < K32) {
@@ -512,74 +524,8 @@ __device__ __forceinline__ void quantize_rows_body(const uint16_t* __restrict__ 
       const bool active = FULL || row[j] >= 0;
       const uint32_t r = active ? (uint32_t)row[j] : 0u;
       const uint32_t b = blk[j];
-      const uint32_t k0 = b << 4;
-      float x[16];
-      uint32_t amax_b_bits;  // binary32 pattern of the block's amax (non-negative, so integer order = float order)
-      if (RHT) {
-  #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          x[2 * i] = bf16_lo(w[j][i]);
-          x[2 * i + 1] = bf16_hi(w[j][i]);
-        }
-        // blocks past K (layout padding up to 128) take no signs, so that they stay +0 and encode as zero bytes
-        rht_scale16(x, (FULL || k0 < K32) ? rht_sign16(seed, rht_stream, (int64_t)k0) : 0u);
-        hadamard16_butterflies(x);
-        float m = 0.0f;
-  #pragma unroll
-        for (int i = 0; i < 16; ++i) m = fmaxf(m, fabsf(x[i]));
-        amax_b_bits = __float_as_uint(m);
-      } else {
-        uint32_t m2 = 0;
-  #pragma unroll
-        for (int i = 0; i < 8; ++i) m2 = amax16x2(m2, w[j][i]);
-        amax_b_bits = hmax_of_pair(bf16x2_abs_bits(m2)) << 16;
-      }
-
-      // ---- global scale -------------------------------------------------------------------------------------
-      float Sg;
-      if (GS == kGsBlock128) {
-        uint32_t g = amax_b_bits;
-        g = max(g, __shfl_xor_sync(0xFFFFFFFFu, g, 1));
-        g = max(g, __shfl_xor_sync(0xFFFFFFFFu, g, 2));
-        g = max(g, __shfl_xor_sync(0xFFFFFFFFu, g, 4));
-        Sg = global_scale_from_amax(__uint_as_float(g));
-        if (active && (b & 7) == 0) gscale[(size_t)r * (uint32_t)(Kp >> 7) + (b >> 3)] = Sg;
-      } else if (GS == kGsRow) {
-        Sg = global_scale_from_amax(__uint_as_float(gs_cells[r]));
-        if (active && b == 0) gscale[r] = Sg;
-      } else {
-        Sg = Sg_t;
-      }
-
-      // ---- block scale, rounding, packing -------------------------------------------------------------------
-      float rcp;
-      const uint32_t sb = block_scale(__uint_as_float(amax_b_bits), Sg, rcp, SR && sb_up);
-      if (!RHT) {
-  #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          x[2 * i] = bf16_lo(w[j][i]);
-          x[2 * i + 1] = bf16_hi(w[j][i]);
-        }
-      }
-      const uint2 packed = quantize_block16<SR>(x, rcp, pk, stream_id, ((uint64_t)r * (uint32_t)K16 + k0) >> 3);
-
-      // four neighbouring threads own the four scale bytes of one 32-bit word in either layout
-      uint32_t sf4 = sb << (8 * (b & 3));
-      sf4 |= __shfl_xor_sync(0xFFFFFFFFu, sf4, 1);
-      sf4 |= __shfl_xor_sync(0xFFFFFFFFu, sf4, 2);
-      if (active) {
-        *reinterpret_cast<uint2*>(codes + (size_t)r * (uint32_t)(Kp >> 1) + (k0 >> 1)) = packed;
-        if ((b & 3) == 0) {
-          size_t off;
-          if (TILED) {
-            const uint32_t tile = (r >> 7) * (((nb32 + 15u) & ~15u) >> 2) + (b >> 2);  // 512-byte tiles, k fastest
-            off = (size_t)tile * 512u + ((r & 31u) * 16u + ((r >> 5) & 3u) * 4u);       // b & 3 == 0 here
-          } else {
-            off = (size_t)r * nb32 + b;
-          }
-          *reinterpret_cast<uint32_t*>(sf + off) = sf4;
-        }
-      }
+      finish_block16<GS, SR, TILED, RHT>(w[j], r, b, active, FULL || (b << 4) < K32, (uint32_t)Kp, (uint32_t)K16, Sg_t, seed, stream_id, gs_cells, codes, sf,
+                                         gscale, rht_stream, sb_up, pk);
     }
   };
   const bool full = !GATHER && K32 == (uint32_t)Kp && (int64_t)bx * (256 * NB) + 256 * NB <= total;  // CTA-uniform
@@ -589,16 +535,120 @@ __device__ __forceinline__ void quantize_rows_body(const uint16_t* __restrict__ 
     body(std::false_type{});
 }
 
+// =========================================================================================================
+// Row-axis quantize of the columns `keep` (OutControl compaction). A CTA takes R whole rows: it copies them to shared memory as
+// they are (16-byte asynchronous copies, all in flight at once), moves the kept columns together there, two per thread and row, so
+// that neighbouring threads touch neighbouring words, and quantizes the compact rows, a block per thread and step.
+// excl_out, if given, takes the columns `excluded` of the rows: the BF16 side operand, zero up to ld_excl_out.
+// Bound by instruction issue (three quarters of the slots). Picking a block's sixteen elements singly from the copied rows met in the
+// same banks: 8192 x 1024 without 10 % of its columns, BLOCK128, 17.9 / 10.1 us, 8192 x 2816 37 / 23, 2816 x 1024 16.0 / 5.6. Rows
+// interleaved in shared memory by 8-column pieces save address arithmetic and lose more: their copies go out 16 bytes at a time.
+// =========================================================================================================
+struct RowWalk {  // 256 threads over the items of rows of n items each: where a thread starts, and its step, without a division
+  uint32_t n, inv, step_r, step_c;
+  static RowWalk of(int64_t n) { return {(uint32_t)n, (uint32_t)((1u << 20) / n + 1), (uint32_t)(256 / n), (uint32_t)(256 % n)}; }
+  __device__ __forceinline__ void start(uint32_t& r, uint32_t& c) const {
+    r = (threadIdx.x * inv) >> 20;  // threadIdx.x / n: exact, as 255 * n < 2^20 for n <= 255 and the quotient is 0 above that
+    c = threadIdx.x - r * n;
+  }
+  __device__ __forceinline__ void next(uint32_t& r, uint32_t& c) const {
+    r += step_r;
+    c += step_c;
+    if (c >= n) c -= n, ++r;
+  }
+};
+struct GatherArgs {
+  const uint16_t* src;
+  const int32_t *keep, *excluded;
+  const uint32_t* gs_cells;
+  uint8_t *codes, *sf;
+  float* gscale;
+  uint16_t* excl_out;
+  int64_t ld;
+  uint64_t seed;
+  uint32_t rows, K, cols_src, n_excl, ld_excl_out, stream_id;
+  int32_t gs_words, sb_up;
+  RowWalk chunks, blocks;  // 16-byte pieces of a source row, blocks of the operand's row
+};
+
+template <int GS, bool SR, bool TILED, uint32_t R>
+__global__ void __launch_bounds__(256)
+quantize_rows_gather_kernel(const __grid_constant__ GatherArgs a, const __grid_constant__ PhiloxKeys pk) {
+  extern __shared__ __align__(16) uint16_t stage[];  // [R][cols8] as they are, then [R][Kp] compact
+  const uint32_t bx = tail_first<GS>(blockIdx.x);
+  const uint32_t K = a.K, nb = a.blocks.n, Kp = nb << 4, cols8 = a.chunks.n << 3;
+  const uint32_t r0 = bx * R, n_rows = min(R, a.rows - r0);
+  uint16_t* const compact = stage + R * cols8;
+  uint32_t rr, c;
+  pdl_prologue();
+  for (a.chunks.start(rr, c); rr < n_rows; a.chunks.next(rr, c)) {
+    const uint16_t* p = a.src + (size_t)(r0 + rr) * (size_t)a.ld + (c << 3);
+    uint16_t* d = stage + rr * cols8 + (c << 3);
+    if ((c << 3) + 8u <= a.cols_src) {
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(d)), "l"(p) : "memory");
+    } else {
+      for (uint32_t i = 0; (c << 3) + i < a.cols_src; ++i) d[i] = p[i];
+    }
+  }
+  float Sg_t = 1.0f;
+  if (GS == kGsTensor) {
+    Sg_t = global_scale_from_amax(__uint_as_float(tensor_amax_bits(a.gs_cells, a.gs_words)));
+    if (bx == 0 && threadIdx.x == 0) a.gscale[0] = Sg_t;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  for (uint32_t k = threadIdx.x * 2u; k < Kp; k += 512u) {
+    uint16_t* d = compact + k;
+    if (k + 2u <= K) {
+      const int2 id = *reinterpret_cast<const int2*>(a.keep + k);  // keep is 8-byte aligned, k is even
+      const uint16_t *s0 = stage + (uint32_t)id.x, *s1 = stage + (uint32_t)id.y;
+#pragma unroll
+      for (uint32_t r = 0; r < R; ++r)
+        *reinterpret_cast<uint32_t*>(d + r * Kp) = __byte_perm((uint32_t)s0[r * cols8], (uint32_t)s1[r * cols8], 0x5410);
+    } else {
+      const uint16_t* s0 = stage + (k < K ? (uint32_t)a.keep[k] : 0u);
+#pragma unroll
+      for (uint32_t r = 0; r < R; ++r) *reinterpret_cast<uint32_t*>(d + r * Kp) = k < K ? (uint32_t)s0[r * cols8] : 0u;
+    }
+  }
+  if (a.excl_out) {
+    for (uint32_t k = threadIdx.x * 2u; k < a.ld_excl_out; k += 512u) {
+      const uint16_t* s0 = stage + (k < a.n_excl ? (uint32_t)a.excluded[k] : 0u);
+      const uint16_t* s1 = stage + (k + 1u < a.n_excl ? (uint32_t)a.excluded[k + 1u] : 0u);
+      const uint32_t mask = (k < a.n_excl ? 0xFFFFu : 0u) | (k + 1u < a.n_excl ? 0xFFFF0000u : 0u);
+      uint16_t* d = a.excl_out + (size_t)r0 * a.ld_excl_out + k;
+#pragma unroll
+      for (uint32_t r = 0; r < R; ++r, d += a.ld_excl_out)
+        if (r < n_rows) *reinterpret_cast<uint32_t*>(d) = __byte_perm((uint32_t)s0[r * cols8], (uint32_t)s1[r * cols8], 0x5410) & mask;
+    }
+  }
+  __syncthreads();
+  const uint32_t n_blocks = n_rows * nb;
+  uint32_t b;
+  a.blocks.start(rr, b);
+  for (uint32_t e = threadIdx.x; (e & ~31u) < n_blocks; e += 256u, a.blocks.next(rr, b)) {  // a warp's 32 threads leave together
+    const bool active = e < n_blocks;
+    uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (active) {
+      const uint4* p = reinterpret_cast<const uint4*>(compact + rr * Kp + (b << 4));
+      const uint4 v0 = p[0], v1 = p[1];
+      w[0] = v0.x; w[1] = v0.y; w[2] = v0.z; w[3] = v0.w;
+      w[4] = v1.x; w[5] = v1.y; w[6] = v1.z; w[7] = v1.w;
+    }
+    finish_block16<GS, SR, TILED, false>(w, active ? r0 + rr : 0u, b, active, (b << 4) < K, Kp, (K + 15u) & ~15u, Sg_t, a.seed, a.stream_id,
+                                         a.gs_cells, a.codes, a.sf, a.gscale, 0u, a.sb_up, pk);
+  }
+}
+
 template <int GS, bool SR, bool TILED, bool GATHER, bool RHT>
 __global__ void __launch_bounds__(256, 4)
 quantize_rows_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld,
                      const int32_t* __restrict__ keep, uint64_t seed, uint32_t stream_id,
                      const uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
-                     float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, int64_t cols_src,
-                     int64_t stage_cols8, const int32_t* __restrict__ excluded, uint32_t n_excl, uint16_t* __restrict__ excl_out,
-                     uint32_t ld_excl_out, uint32_t rht_stream, int sb_up, const __grid_constant__ PhiloxKeys pk) {
+                     float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads,
+                     uint32_t rht_stream, int sb_up, const __grid_constant__ PhiloxKeys pk) {
   pdl_prologue();
-  quantize_rows_body<GS, SR, TILED, GATHER, RHT>(src, rows, K, ld, keep, seed, stream_id, gs_cells, gs_words, codes, sf, gscale, div_mul, div_shift, wide_loads, cols_src, stage_cols8, excluded, n_excl, excl_out, ld_excl_out, rht_stream, sb_up, pk, tail_first<GS>(blockIdx.x));
+  quantize_rows_body<GS, SR, TILED, GATHER, RHT>(src, rows, K, ld, keep, seed, stream_id, gs_cells, gs_words, codes, sf, gscale, div_mul, div_shift, wide_loads, rht_stream, sb_up, pk, tail_first<GS>(blockIdx.x));
 }
 
 
@@ -1771,7 +1821,7 @@ quantize_rows_pair_kernel(const __grid_constant__ RowsJob a, const __grid_consta
   if (GS == kGsTensor) bx = j.blocks - 1u - bx;  // (tail_first)
   const PhiloxKeys no_keys{};
   quantize_rows_body<GS, false, true, false, false>(j.src, j.rows, j.K, j.ld, nullptr, 0ull, j.stream_id, j.gs_cells, j.gs_words, j.codes, j.sf,
-                                                    j.gscale, j.div_mul, j.div_shift, j.wide_loads, 0, 0, nullptr, 0u, nullptr, 0u, 0u, 0, no_keys, bx);
+                                                    j.gscale, j.div_mul, j.div_shift, j.wide_loads, 0u, 0, no_keys, bx);
   clear_scale_padding(j.sf, (uint32_t)j.rows, (((uint32_t)j.K + 127u) & ~127u) >> 4, bx, j.blocks);
 }
 
@@ -1832,12 +1882,15 @@ static void division_constants(int64_t total, int64_t slack, uint64_t d, uint32_
   }
 }
 
-// Shared memory for the source rows that a CTA of the compacting row quantizer touches (its 1024 blocks span at most 1024 / nb + 2
-// rows); 0 if they do not fit or cannot be copied in 16-byte pieces.
-static size_t gather_stage_bytes(const QuantRowsArgs& a) {
-  const int64_t cols8 = (a.cols_src + 7) & ~(int64_t)7, nb = ((a.K + 127) & ~(int64_t)127) >> 4;
-  const size_t smem = (size_t)((1024 / nb + 2) * cols8 * 2);
-  return smem > 160 * 1024 || (reinterpret_cast<uintptr_t>(a.keep) & 15u) != 0 || (a.ld & 7) != 0 ? 0 : smem;
+// Rows per CTA of the compacting row quantizer; 0 if two do not fit in shared memory or rows cannot be copied in 16-byte pieces.
+// us with 2 / 4 / 8 rows, BLOCK128, 10 % of the columns left out: 8192 x 1024 11.3 / 10.1 / 11.8, 4095 x 1024 8.0 / 7.2 / 8.2,
+// 8192 x 2816 22.8 / 23.4 / 31.4, 1024 x 2816 7.2 / 8.1 / 8.3, 16384 x 4096 62 / 77 / 133: wide rows leave too few CTAs on an SM.
+static int gather_rows_per_cta(const QuantRowsArgs& a, size_t& smem) {
+  const size_t row_bytes = (size_t)((((a.cols_src + 7) & ~(int64_t)7) + ((a.K + 127) & ~(int64_t)127)) * 2);
+  if ((reinterpret_cast<uintptr_t>(a.src) & 15u) != 0 || (a.ld & 7) != 0 || (reinterpret_cast<uintptr_t>(a.keep) & 7u) != 0) return 0;
+  const int r = row_bytes <= 6 * 1024 ? 4 : 2;
+  smem = r * row_bytes;
+  return smem > 200 * 1024 ? 0 : r;
 }
 
 template <int GS, bool SR, bool TILED>
@@ -1850,21 +1903,30 @@ static cudaError_t launch_rows_g(const QuantRowsArgs& a, cudaStream_t st) {
   division_constants(total, 1024, d, div_mul, div_shift);
   const int wide_loads = ((reinterpret_cast<uintptr_t>(a.src) & 31u) == 0 && (a.ld & 15) == 0) ? 1 : 0;
   if (a.keep) {
-    const size_t smem = gather_stage_bytes(a);
-    const int64_t stage_cols8 = smem ? (a.cols_src + 7) & ~(int64_t)7 : 0;  // (0: per-element global loads)
-    if (smem) {
-      cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(quantize_rows_kernel<GS, SR, TILED, true, false>), smem);
+    size_t smem;
+    const int rows_per_cta = gather_rows_per_cta(a, smem);
+    if (rows_per_cta) {
+      const GatherArgs g{a.src, a.keep, a.excluded, a.gs_cells, a.codes, a.sf, a.gscale, a.excl_out, a.ld, a.seed, (uint32_t)a.rows, (uint32_t)a.K,
+                         (uint32_t)a.cols_src, (uint32_t)(a.cols_src - a.K), (uint32_t)a.ld_excl_out, a.stream_id, a.gs_words, a.sr == 2,
+                         RowWalk::of((a.cols_src + 7) >> 3), RowWalk::of(Kp >> 4)};
+      auto launch = [&](auto r) -> cudaError_t {
+        const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(quantize_rows_gather_kernel<GS, SR, TILED, r.value>), smem);
+        if (e == cudaSuccess)
+          launch_kernel(quantize_rows_gather_kernel<GS, SR, TILED, r.value>, dim3(blocks_for(a.rows, r.value)), dim3(256), smem, st, g, make_philox_keys(a.seed));
+        return e;
+      };
+      const cudaError_t e = rows_per_cta == 4 ? launch(std::integral_constant<uint32_t, 4>{}) : launch(std::integral_constant<uint32_t, 2>{});
       if (e != cudaSuccess) return e;
+    } else {
+      launch_kernel(quantize_rows_kernel<GS, SR, TILED, true, false>, dim3(grid), dim3(256), 0, st, a.src, a.rows, a.K, a.ld, a.keep, a.seed,
+                    a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, 0u, a.sr == 2, make_philox_keys(a.seed));
     }
-    launch_kernel(quantize_rows_kernel<GS, SR, TILED, true, false>, dim3(grid), dim3(256), smem, st, a.src, a.rows, a.K, a.ld, a.keep, a.seed,
-                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, stage_cols8, a.excluded, (uint32_t)(a.cols_src - a.K),
-                  stage_cols8 > 0 ? a.excl_out : nullptr, (uint32_t)a.ld_excl_out, 0u, a.sr == 2, make_philox_keys(a.seed));
   } else if (a.rht_stream) {
     launch_kernel(quantize_rows_kernel<GS, SR, TILED, false, true>, dim3(grid), dim3(256), 0, st, a.src, a.rows, a.K, a.ld, nullptr, a.seed,
-                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, (int64_t)0, nullptr, 0u, nullptr, 0u, a.rht_stream, a.sr == 2, make_philox_keys(a.seed));
+                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.rht_stream, a.sr == 2, make_philox_keys(a.seed));
   } else {
     launch_kernel(quantize_rows_kernel<GS, SR, TILED, false, false>, dim3(grid), dim3(256), 0, st, a.src, a.rows, a.K, a.ld, nullptr, a.seed,
-                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, a.cols_src, (int64_t)0, nullptr, 0u, nullptr, 0u, 0u, a.sr == 2, make_philox_keys(a.seed));
+                  a.stream_id, a.gs_cells, a.gs_words, a.codes, a.sf, a.gscale, div_mul, div_shift, wide_loads, 0u, a.sr == 2, make_philox_keys(a.seed));
   }
   return cudaGetLastError();
 }
@@ -1910,7 +1972,8 @@ static cudaError_t launch_quantize_rows_impl(const QuantRowsArgs& a0, cudaStream
   if (a.rows == 0 || a.K == 0) return cudaSuccess;
   if (a.rows >= ((int64_t)1 << 31) || a.cols_src >= ((int64_t)1 << 31) || a.ld >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
   if (!a.excluded || (a.ld_excl_out & 1) || (reinterpret_cast<uintptr_t>(a.excl_out) & 3u)) a.excl_out = nullptr;
-  side_copy_done = a.keep && a.excl_out && gather_stage_bytes(a) != 0;  // the quantizer writes it from the rows that it stages
+  size_t smem;
+  side_copy_done = a.keep && a.excl_out && gather_rows_per_cta(a, smem) != 0;  // the quantizer writes it from the rows that it stages
   cudaError_t e;
   if (a.rht_stream) {  // the scales come from the transformed data; column lists are not combined with the transformation
     if (a.keep) return cudaErrorInvalidValue;
