@@ -1347,17 +1347,17 @@ quantize_transpose_kernel(TransposeSrc s, int64_t rowsK, int64_t D, uint64_t see
 // =========================================================================================================
 // Column-axis quantize from BF16 without a shared-memory transposition (Q5 of Sec. 2.3: the operand is dY^T, its blocks
 // run along the tokens), for the TENSOR and ROW scale modes. A lane owns FOUR neighbouring source columns (= operand rows)
-// and 64 consecutive source rows (= operand k). It reads 8 bytes per source row, so one warp instruction covers two source
-// rows of 128 contiguous bytes (lanes 0..15: rows k .. , lanes 16..31: rows k + 64 ..), and the 16 values of an inner block
-// are the same half of 16 loaded words: the transposition is the choice of that half. Per 16 source rows the lane quantizes
-// four blocks (one per column) and stores 8 code bytes to each of its four operand rows; the four scale bytes of an operand
-// row (64 k) are one aligned word of either scale layout. No barrier, no shared memory, and the index arithmetic is paid
-// once per 256 elements.
+// and 16 consecutive source rows (= operand k), i.e. one inner block of four operand rows. It reads 8 bytes per source row, so one
+// warp instruction covers two source rows of 128 contiguous bytes, and the 16 values of an inner block are the same half of 16
+// loaded words: the transposition is the choice of that half. It stores 8 code bytes and a scale byte to each of its four operand
+// rows. No barrier, no shared memory. Bound by instruction issue (stochastic rounding, 20 instructions per element). Lanes that
+// took 64 source rows, whose four scale bytes are one word, paid the index arithmetic once per 256 elements, but their CTAs ran
+// 16 us each: us with the amax pass, stochastic, 64 / 16 rows per lane: 16384 x 2816 65.5 / 62.5, 8192 x 3072 38.9 / 35.0,
+// 8192 x 1024 23.7 / 14.7, 4095 x 2816 25.4 / 19.0, 1024 x 1024 10.7 / 6.9, 256 x 512 9.9 / 4.9.
 //   RMODE      0 round to nearest, 1 stochastic rounding, 2 stochastic rounding with the block scale rounded up.
-//   RHT        every block is replaced by (x S) H_16 first (Sec. 4.1): the lane's 64 sign bits are half of one generator
-//              block, the butterflies run on the 16 values it holds anyway.
+//   RHT        every block is replaced by (x S) H_16 first (Sec. 4.1): the butterflies run on the 16 values the lane holds anyway.
 //   AMAX_ONLY  the pre-pass of RHT: only the maximum of the transformed values, folded into gs_cells (one cell, or one per
-//              operand row in ROW mode); nothing else is written.
+//              operand row in ROW mode); nothing else is written. 64 source rows per lane there: a quarter of the atomics.
 // Preconditions (the launcher falls back to the staged kernel otherwise): D and ld multiples of 4, src 8-byte aligned,
 // identity row order.
 // =========================================================================================================
@@ -1367,18 +1367,21 @@ __device__ __forceinline__ uint2 ld_nc_8(const uint16_t* p) {
   return v;
 }
 
+template <bool AMAX_ONLY>
+constexpr uint32_t kColsBlocks = AMAX_ONLY ? 4 : 1;  // 16-element blocks per lane and operand row
 template <int GS, int RMODE, bool TILED, bool RHT, bool AMAX_ONLY>
 __device__ __forceinline__ void quantize_cols4_body(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, uint32_t ld, uint64_t seed, uint32_t stream_id,
                       uint32_t rht_stream, uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes,
                       uint8_t* __restrict__ sf, float* __restrict__ gscale, const PhiloxKeys& pk, uint32_t bx, uint32_t by, uint32_t tid) {
   static_assert(GS != kGsBlock128, "the outer-block mode has a kernel of its own");
   constexpr bool SR = RMODE != 0;
+  constexpr uint32_t TBT = kColsBlocks<AMAX_ONLY>;
   const uint32_t Kp = (K + 127u) & ~127u;
   const uint32_t K16 = (K + 15u) & ~15u;
   const uint32_t nb = Kp >> 4;
   const uint32_t lane = tid & 31u, warp = tid >> 5;
   const uint32_t d0 = by * 64u + (lane & 15u) * 4u;                          // first of this lane's operand rows
-  const uint32_t k_start = bx * 512u + warp * 128u + (lane >> 4) * 64u;      // first of its 64 k
+  const uint32_t k_start = (bx * 8u + warp * 2u + (lane >> 4)) * (16u * TBT);  // first of its 16 * TBT k
   const bool live = d0 < D && k_start < Kp;  // (all four rows exist or none: D is a multiple of 4)
   const uint16_t* p = src + (size_t)k_start * ld + d0;
 
@@ -1395,19 +1398,15 @@ __device__ __forceinline__ void quantize_cols4_body(const uint16_t* __restrict__
       if (bx == 0 && by == 0 && tid == 0) gscale[0] = Sg[0];
     }
   }
-  // the 64 sign bits of this lane's k range (one half of a 128-group's generator block)
-  uint32_t sgn_lo = 0, sgn_hi = 0;
-  if (RHT && live) {
-    const uint4 sw = rht_sign_words(seed, rht_stream, (uint64_t)(k_start >> 7));
-    sgn_lo = (k_start & 64u) ? sw.z : sw.x;
-    sgn_hi = (k_start & 64u) ? sw.w : sw.y;
-  }
+  // the sign bits of this lane's k range, which lies in one 128-group
+  uint4 sgn = make_uint4(0u, 0u, 0u, 0u);
+  if (RHT && live) sgn = rht_sign_words(seed, rht_stream, (uint64_t)(k_start >> 7));
   float am_run[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // AMAX_ONLY: running maxima of the four operand rows
 
-  uint32_t sfw[4] = {0u, 0u, 0u, 0u};
+  uint32_t sfw[4] = {0u, 0u, 0u, 0u};  // the four operand rows' block scales
   if (live) {
 #pragma unroll 1
-    for (uint32_t tb = 0; tb < 4; ++tb) {
+    for (uint32_t tb = 0; tb < TBT; ++tb) {
       const uint32_t k0 = k_start + 16u * tb;
       if (AMAX_ONLY && k0 >= K16) break;  // layout padding: zeros
       uint2 w[16];
@@ -1434,7 +1433,7 @@ __device__ __forceinline__ void quantize_cols4_body(const uint16_t* __restrict__
         am[3] = __uint_as_float(my & 0xFFFF0000u);
       }
       // signs of rows k0 .. k0 + 15; rows past K rounded up to 16 are layout padding and take none (they stay +0)
-      const uint32_t s16 = RHT && k0 < K16 ? ((((tb & 2u) ? sgn_hi : sgn_lo) >> (16u * (tb & 1u))) & 0xFFFFu) : 0u;
+      const uint32_t s16 = RHT && k0 < K16 ? ((rht_pick_word(sgn, (k0 >> 5) & 3u) >> (k0 & 16u)) & 0xFFFFu) : 0u;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         float x[16];
@@ -1456,7 +1455,7 @@ __device__ __forceinline__ void quantize_cols4_body(const uint16_t* __restrict__
         } else {
           float rcp;
           const uint32_t sb = block_scale(am[c], Sg[c], rcp, RMODE == 2);
-          sfw[c] |= sb << (8u * tb);
+          sfw[c] = sb;
           const uint2 packed = quantize_block16<SR>(x, rcp, pk, stream_id, ((uint64_t)(d0 + c) * K16 + k0) >> 3);
           *reinterpret_cast<uint2*>(codes + (size_t)(d0 + c) * (Kp >> 1) + (k0 >> 1)) = packed;
         }
@@ -1479,13 +1478,13 @@ __device__ __forceinline__ void quantize_cols4_body(const uint16_t* __restrict__
     return;
   }
   if (!live) return;
-  const uint32_t b = k_start >> 4;  // first of this lane's four k blocks: a multiple of 4
+  const uint32_t b = k_start >> 4;
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const uint32_t o = d0 + c;
-    const size_t off = TILED ? (size_t)((o >> 7) * (((nb + 15u) & ~15u) >> 2) + (b >> 2)) * 512u + ((o & 31u) * 16u + ((o >> 5) & 3u) * 4u)
+    const size_t off = TILED ? (size_t)((o >> 7) * (((nb + 15u) & ~15u) >> 2) + (b >> 2)) * 512u + ((o & 31u) * 16u + ((o >> 5) & 3u) * 4u + (b & 3u))
                              : (size_t)o * nb + b;
-    *reinterpret_cast<uint32_t*>(sf + off) = sfw[c];
+    sf[off] = (uint8_t)sfw[c];
   }
 }
 
@@ -2100,7 +2099,7 @@ static cudaError_t launch_tr_t(const QuantTransposeArgs& a, cudaStream_t st) {
     launch_kernel(quantize_cols2_block128_kernel<RMODE, TILED_, RHT_>, dim3(blocks_for(a.rowsK, 512), blocks_for(a.D, 32)),         \
                   dim3(128), 0, st, a.src.bf16, K32, D32, ld32, a.seed, a.stream_id, a.rht_stream, a.codes, a.sf, a.gscale, keys);  \
   else                                                                                                                              \
-    launch_kernel(quantize_cols4_kernel<GS, RMODE, TILED_, RHT_, false>, dim3(blocks_for(a.rowsK, 512), blocks_for(a.D, 64)),       \
+    launch_kernel(quantize_cols4_kernel<GS, RMODE, TILED_, RHT_, false>, dim3(blocks_for(a.rowsK, 128), blocks_for(a.D, 64)),       \
                   dim3(128), 0, st, a.src.bf16, K32, D32, ld32, a.seed, a.stream_id, a.rht_stream, a.gs_cells, a.gs_words, a.codes, \
                   a.sf, a.gscale, keys)
       if (a.sf_tiled) {
