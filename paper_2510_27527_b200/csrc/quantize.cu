@@ -1503,129 +1503,99 @@ quantize_cols4_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, 
   quantize_cols4_body<GS, RMODE, TILED, RHT, AMAX_ONLY>(src, K, D, ld, seed, stream_id, rht_stream, gs_cells, gs_words, codes, sf, gscale, pk, bx, by, threadIdx.x);
 }
 
-
-// The same for the 1 x 128 outer block (BLOCK128), where the scale of a block depends on all 128 k of its group: a lane owns
-// TWO neighbouring source columns and keeps its 64 source rows in registers (one 32-bit word per row), so the data is read
-// once; the two lanes of a group exchange the group maximum with one shuffle. A warp instruction covers two source rows of
-// 64 contiguous bytes. With RHT the group maximum is that of the transformed values: the eight blocks are transformed once
-// for their maxima and once more when they are quantized (80 floating-point operations per block and pass; holding the 128
-// transformed values beside the 64 raw words does not fit the register file at a useful occupancy).
+// =========================================================================================================
+// The same for the 1x128 outer blocks. A CTA takes 128 source rows (one outer block of k) of 64 columns; a lane owns four neighbouring
+// columns of 16 rows, i.e. one inner block of four operand rows. The eight lanes of a column group hold the eight inner blocks of its
+// outer block, so the group maximum is three shuffles, and a Hadamard-transformed block stays in registers from the maximum to the
+// rounding. Loads are whole 32-byte sectors (four lanes of 8 bytes), code stores 64 contiguous bytes per operand row.
+// Lanes that kept 64 rows of two columns read 64-byte pieces, but transformed every block twice and left small operands to a few long
+// CTAs: us, stochastic rounding, without / with the transformation: 8192 x 2816 28.4 / 34.6, now 25.2 / 30.1; 8192 x 1024 14.5 / 17.2,
+// now 11.5 / 12.6; 2000 x 1400 10.2 / 11.4, now 7.5 / 8.0; 256 x 512 5.5 / 6.9, now 2.9 / 3.3.
+// =========================================================================================================
 template <int RMODE, bool TILED, bool RHT>
-__device__ __forceinline__ void quantize_cols2_block128_body(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, uint32_t ld, uint64_t seed, uint32_t stream_id,
+__global__ void __launch_bounds__(128, 4)
+quantize_cols4_block128_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, uint32_t ld, uint64_t seed, uint32_t stream_id,
                                uint32_t rht_stream, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf, float* __restrict__ gscale,
-                               const PhiloxKeys& pk, uint32_t bx, uint32_t by, uint32_t tid) {
+                               const __grid_constant__ PhiloxKeys pk) {
+  pdl_prologue();
   constexpr bool SR = RMODE != 0;
   const uint32_t Kp = (K + 127u) & ~127u;
   const uint32_t K16 = (K + 15u) & ~15u;
   const uint32_t nb = Kp >> 4;
-  const uint32_t lane = tid & 31u, warp = tid >> 5;
-  const uint32_t d0 = by * 32u + (lane & 15u) * 2u;
-  const uint32_t k_start = bx * 512u + warp * 128u + (lane >> 4) * 64u;
-  const bool live = d0 < D && k_start < Kp;  // (both rows exist or none: D is even)
-  const uint16_t* p = src + (size_t)k_start * ld + d0;
-
-  uint32_t w[64];
-  if (live && k_start + 64u <= K) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t d0 = blockIdx.y * 64u + warp * 16u + (lane & 3u) * 4u;
+  const uint32_t k0 = blockIdx.x * 128u + (lane >> 2) * 16u;
+  const bool live = d0 < D;  // (all four columns exist or none: D is a multiple of 4)
+  const uint16_t* p = src + (size_t)k0 * ld + d0;
+  uint2 w[16];
+  if (live && k0 + 16u <= K) {
 #pragma unroll
-    for (int t = 0; t < 64; ++t) asm volatile("ld.global.nc.L1::no_allocate.b32 %0, [%1];" : "=r"(w[t]) : "l"(p + (size_t)t * ld));
+    for (int t = 0; t < 16; ++t) w[t] = ld_nc_8(p + (size_t)t * ld);
   } else {
 #pragma unroll
-    for (int t = 0; t < 64; ++t) {
-      w[t] = 0u;
-      if (live && k_start + t < K) asm volatile("ld.global.nc.L1::no_allocate.b32 %0, [%1];" : "=r"(w[t]) : "l"(p + (size_t)t * ld));
+    for (int t = 0; t < 16; ++t) w[t] = live && k0 + t < K ? ld_nc_8(p + (size_t)t * ld) : make_uint2(0u, 0u);
+  }
+  auto unpack = [&](int c, float (&x)[16]) {
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+      const uint32_t word = c < 2 ? w[t].x : w[t].y;
+      x[t] = (c & 1) ? bf16_hi(word) : bf16_lo(word);
     }
-  }
-  // the 64 sign bits of this lane's k range; rows past K rounded up to 16 are layout padding and take none (they stay +0)
-  uint32_t sgn[2] = {0u, 0u};
-  if (RHT && live) {
-    const uint4 sw = rht_sign_words(seed, rht_stream, (uint64_t)(k_start >> 7));
-    sgn[0] = (k_start & 64u) ? sw.z : sw.x;
-    sgn[1] = (k_start & 64u) ? sw.w : sw.y;
-  }
-  auto sign16 = [&](int tb) -> uint32_t { return k_start + 16u * tb < K16 ? ((sgn[tb >> 1] >> (16 * (tb & 1))) & 0xFFFFu) : 0u; };
-
-  float Sg[2];
-  float bam[RHT ? 4 : 1][2];  // RHT: block maxima of the transformed values
-  uint32_t bm[4];             // otherwise: packed block maxima (sign bits meaningless until masked)
+  };
+  float xr[RHT ? 4 : 1][16];  // the transformed blocks
+  uint32_t am[4];             // block maxima (binary32 patterns of non-negative values: integer order = float order)
   if (RHT) {
-    float g0 = 0.0f, g1 = 0.0f;
+    // rows past K rounded up to 16 are layout padding and take no signs (they stay +0)
+    const uint32_t s16 = k0 < K16 ? rht_sign16(seed, rht_stream, (int64_t)k0) : 0u;
 #pragma unroll
-    for (int tb = 0; tb < 4; ++tb) {
+    for (int c = 0; c < 4; ++c) {
+      float(&x)[16] = xr[RHT ? c : 0];
+      unpack(c, x);
+      rht_scale16(x, s16);
+      hadamard16_butterflies(x);
+      float m = 0.0f;
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        float x[16];
-#pragma unroll
-        for (int t = 0; t < 16; ++t) x[t] = c ? bf16_hi(w[16 * tb + t]) : bf16_lo(w[16 * tb + t]);
-        rht_scale16(x, sign16(tb));
-        hadamard16_butterflies(x);
-        float m = 0.0f;
-#pragma unroll
-        for (int t = 0; t < 16; ++t) m = fmaxf(m, fabsf(x[t]));
-        bam[RHT ? tb : 0][c] = m;
-        if (c) g1 = fmaxf(g1, m); else g0 = fmaxf(g0, m);
-      }
+      for (int t = 0; t < 16; ++t) m = fmaxf(m, fabsf(x[t]));
+      am[c] = __float_as_uint(m);
     }
-    g0 = fmaxf(g0, __shfl_xor_sync(0xFFFFFFFFu, g0, 16));  // the other half of the 128-wide group
-    g1 = fmaxf(g1, __shfl_xor_sync(0xFFFFFFFFu, g1, 16));
-    Sg[0] = global_scale_from_amax(g0);
-    Sg[1] = global_scale_from_amax(g1);
   } else {
+    uint32_t mx = 0, my = 0;
 #pragma unroll
-    for (int tb = 0; tb < 4; ++tb) {
-      uint32_t m = 0;
-#pragma unroll
-      for (int t = 0; t < 16; ++t) m = amax16x2(m, w[16 * tb + t]);
-      bm[tb] = m;
+    for (int t = 0; t < 16; ++t) {
+      mx = amax16x2(mx, w[t].x);
+      my = amax16x2(my, w[t].y);
     }
-    uint32_t g = amax16x2(amax16x2(bm[0], bm[1]), amax16x2(bm[2], bm[3]));
-    g = bf16x2_abs_bits(amax16x2(g, __shfl_xor_sync(0xFFFFFFFFu, g, 16)));
-    Sg[0] = global_scale_from_amax(__uint_as_float(g << 16));
-    Sg[1] = global_scale_from_amax(__uint_as_float(g & 0xFFFF0000u));
+    mx = bf16x2_abs_bits(mx);
+    my = bf16x2_abs_bits(my);
+    am[0] = mx << 16;
+    am[1] = mx & 0xFFFF0000u;
+    am[2] = my << 16;
+    am[3] = my & 0xFFFF0000u;
+  }
+  float Sg[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    uint32_t g = am[c];
+    g = max(g, __shfl_xor_sync(0xFFFFFFFFu, g, 4));
+    g = max(g, __shfl_xor_sync(0xFFFFFFFFu, g, 8));
+    g = max(g, __shfl_xor_sync(0xFFFFFFFFu, g, 16));
+    Sg[c] = global_scale_from_amax(__uint_as_float(g));
   }
   if (!live) return;
-  if ((lane >> 4) == 0) {
-    gscale[(size_t)d0 * (Kp >> 7) + (k_start >> 7)] = Sg[0];
-    gscale[(size_t)(d0 + 1) * (Kp >> 7) + (k_start >> 7)] = Sg[1];
-  }
-  uint32_t sfw[2] = {0u, 0u};
+  const uint32_t b = k0 >> 4;
 #pragma unroll
-  for (int tb = 0; tb < 4; ++tb) {
-    const uint32_t k0 = k_start + 16u * tb;
-    const uint32_t m = RHT ? 0u : bf16x2_abs_bits(bm[tb]);
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const float am = RHT ? bam[RHT ? tb : 0][c] : __uint_as_float(c ? (m & 0xFFFF0000u) : (m << 16));
-      float rcp;
-      const uint32_t sb = block_scale(am, Sg[c], rcp, RMODE == 2);
-      sfw[c] |= sb << (8 * tb);
-      float x[16];
-#pragma unroll
-      for (int t = 0; t < 16; ++t) x[t] = c ? bf16_hi(w[16 * tb + t]) : bf16_lo(w[16 * tb + t]);
-      if (RHT) {
-        rht_scale16(x, sign16(tb));
-        hadamard16_butterflies(x);
-      }
-      const uint2 packed = quantize_block16<SR>(x, rcp, pk, stream_id, ((uint64_t)(d0 + c) * K16 + k0) >> 3);
-      *reinterpret_cast<uint2*>(codes + (size_t)(d0 + c) * (Kp >> 1) + (k0 >> 1)) = packed;
-    }
-  }
-  const uint32_t b = k_start >> 4;
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
+  for (int c = 0; c < 4; ++c) {
     const uint32_t o = d0 + c;
-    const size_t off = TILED ? (size_t)((o >> 7) * (((nb + 15u) & ~15u) >> 2) + (b >> 2)) * 512u + ((o & 31u) * 16u + ((o >> 5) & 3u) * 4u)
+    if ((lane >> 2) == 0) gscale[(size_t)o * (Kp >> 7) + blockIdx.x] = Sg[c];
+    float rcp;
+    const uint32_t sb = block_scale(__uint_as_float(am[c]), Sg[c], rcp, RMODE == 2);
+    if (!RHT) unpack(c, xr[0]);
+    const uint2 packed = quantize_block16<SR>(xr[RHT ? c : 0], rcp, pk, stream_id, ((uint64_t)o * K16 + k0) >> 3);
+    *reinterpret_cast<uint2*>(codes + (size_t)o * (Kp >> 1) + (k0 >> 1)) = packed;
+    const size_t off = TILED ? (size_t)((o >> 7) * (((nb + 15u) & ~15u) >> 2) + (b >> 2)) * 512u + ((o & 31u) * 16u + ((o >> 5) & 3u) * 4u + (b & 3u))
                              : (size_t)o * nb + b;
-    *reinterpret_cast<uint32_t*>(sf + off) = sfw[c];
+    sf[off] = (uint8_t)sb;
   }
-}
-
-template <int RMODE, bool TILED, bool RHT>
-__global__ void __launch_bounds__(128, 3)
-quantize_cols2_block128_kernel(const uint16_t* __restrict__ src, uint32_t K, uint32_t D, uint32_t ld, uint64_t seed, uint32_t stream_id,
-                               uint32_t rht_stream, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf, float* __restrict__ gscale,
-                               const __grid_constant__ PhiloxKeys pk) {
-  pdl_prologue();
-  quantize_cols2_block128_body<RMODE, TILED, RHT>(src, K, D, ld, seed, stream_id, rht_stream, codes, sf, gscale, pk, blockIdx.x, blockIdx.y, threadIdx.x);
 }
 
 
@@ -2096,7 +2066,7 @@ static cudaError_t launch_tr_t(const QuantTransposeArgs& a, cudaStream_t st) {
       const uint32_t K32 = (uint32_t)a.rowsK, D32 = (uint32_t)a.D, ld32 = (uint32_t)a.src.ld;
 #define NVFP4_LAUNCH_COLS(TILED_, RHT_)                                                                                             \
   if constexpr (GS == kGsBlock128)                                                                                                  \
-    launch_kernel(quantize_cols2_block128_kernel<RMODE, TILED_, RHT_>, dim3(blocks_for(a.rowsK, 512), blocks_for(a.D, 32)),         \
+    launch_kernel(quantize_cols4_block128_kernel<RMODE, TILED_, RHT_>, dim3(blocks_for(a.rowsK, 128), blocks_for(a.D, 64)),         \
                   dim3(128), 0, st, a.src.bf16, K32, D32, ld32, a.seed, a.stream_id, a.rht_stream, a.codes, a.sf, a.gscale, keys);  \
   else                                                                                                                              \
     launch_kernel(quantize_cols4_kernel<GS, RMODE, TILED_, RHT_, false>, dim3(blocks_for(a.rowsK, 128), blocks_for(a.D, 64)),       \
