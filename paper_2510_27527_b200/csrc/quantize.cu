@@ -814,8 +814,10 @@ __device__ __forceinline__ void quantize_rows4_body(const uint16_t* __restrict__
     body(std::false_type{});
 }
 
+// (With the transformation three CTAs per SM spill; two are faster: us, stochastic, 1x128 outer scales, 3 / 2: 16384 x 2816 58.3 / 56.9,
+// 8192 x 2816 30.7 / 29.8, 2000 x 1400 10.5 / 10.1.)
 template <int GS, int RMODE, bool TILED, bool RHT>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(256, RHT ? 2 : 3)
 quantize_rows4_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld, uint64_t seed, uint32_t stream_id,
                       const uint32_t* __restrict__ gs_cells, int gs_words, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
                       float* __restrict__ gscale, uint32_t div_mul, uint32_t div_shift, int wide_loads, uint32_t rht_stream,
@@ -1333,8 +1335,8 @@ __device__ __forceinline__ void quantize_transpose_body(TransposeSrc s, int64_t 
   }
 }
 
-template <int SRC, int GS, int RMODE, bool TILED, bool RHT, bool AMAX_ONLY>
-__global__ void __launch_bounds__(256, 3)
+template <int SRC, int GS, int RMODE, bool TILED, bool RHT, bool AMAX_ONLY, int CTAS = 3>
+__global__ void __launch_bounds__(256, CTAS)
 quantize_transpose_kernel(TransposeSrc s, int64_t rowsK, int64_t D, uint64_t seed, uint32_t stream_id,
                           uint32_t* __restrict__ gs_cells, int gs_words, int tensor_closed_form, uint8_t* __restrict__ codes,
                           uint8_t* __restrict__ sf, float* __restrict__ gscale, uint32_t rht_stream,
@@ -2054,11 +2056,17 @@ static cudaError_t launch_tr_t(const QuantTransposeArgs& a, cudaStream_t st) {
       return cudaGetLastError();
     }
   }
+  // four CTAs per SM (64 registers) for the outer block once the grid fills them: us, stochastic, with the Hadamard transformation,
+  // 3 / 4: 16384 x 2816 74.7 / 70.6, 8192 x 2816 39.0 / 37.0, 8192 x 1024 15.3 / 14.3; smaller grids pile up on some of the SMs:
+  // 3072 x 1024 6.9 / 8.5, 1024 x 1024 6.0 / 7.0
+  constexpr int kMost = SRC == 1 && GS == kGsBlock128 ? 4 : 3;
+  const bool most = kMost == 4 && (int64_t)grid.x * grid.y > 4 * (int64_t)device_sm_count();
 #define NVFP4_LAUNCH_TR(TILED_, RHT_)                                                                                                  \
   if (fast)                                                                                                                            \
-    launch_kernel(quantize_transpose_kernel<SRC, GS, RMODE, TILED_, RHT_, false>, dim3(grid), dim3(256), 0, st, a.src, a.rowsK, a.D,    \
-                  a.seed, a.stream_id, a.gs_cells, a.gs_words, a.tensor_closed_form, a.codes, a.sf, a.gscale, a.rht_stream,            \
-                  make_philox_keys(a.seed));                                                                                           \
+    launch_kernel(most ? quantize_transpose_kernel<SRC, GS, RMODE, TILED_, RHT_, false, kMost>                                         \
+                       : quantize_transpose_kernel<SRC, GS, RMODE, TILED_, RHT_, false>,                                               \
+                  dim3(grid), dim3(256), 0, st, a.src, a.rowsK, a.D, a.seed, a.stream_id, a.gs_cells, a.gs_words, a.tensor_closed_form, \
+                  a.codes, a.sf, a.gscale, a.rht_stream, make_philox_keys(a.seed));                                                    \
   else                                                                                                                                 \
     launch_kernel(quantize_transpose_generic_kernel<SRC, GS, RMODE != 0, TILED_, RHT_, false>, dim3(grid), dim3(256), 0, st, a.src,     \
                   a.rowsK, a.D, a.seed, a.stream_id, a.gs_cells, a.tensor_closed_form, a.codes, a.sf, a.gscale, a.rht_stream,          \

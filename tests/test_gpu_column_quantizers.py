@@ -30,3 +30,19 @@ def test_edges(shape, gs_mode, rounding, rht):
         src = to_dev_bf16(np.pad(x, ((0, 0), (0, -shape[1] % 8))))[:, : shape[1]]
         b.nvfp4_quantize(src, b.AXIS_COL, rounding, 42, 5, gs_mode, layout, out=out, rht_stream_id=rht)
         assert_operand_equal(out, ref, f"{shape} gs{gs_mode} r{rounding} rht{rht} layout{layout}", k_extended=rht != 0)
+
+
+# the largest grid of 128 x 64 tiles that runs three CTAs per SM (592 on 148 SMs), the next one, and a ragged one
+@pytest.mark.parametrize("shape", [(4736, 1024), (4740, 1024), (4999, 1000)])
+@pytest.mark.parametrize("rht", [0, 9])
+def test_requantize_outer_block_large(shape, rht):
+    from paper_2510_27527_b200 import binding as b
+
+    x, _ = synth.activations(shape[0], shape[1], 11, n_outlier=3, factor=50.0)
+    fwd_ref = orc.quantize(x, orc.AXIS_ROW, orc.RTN, orc.GS_BLOCK128)
+    xt = np.ascontiguousarray(orc.rematerialize_f32(fwd_ref).T)
+    ref = orc.quantize(orc.rht16(xt, 5, rht) if rht else xt, orc.AXIS_ROW, orc.SR, orc.GS_BLOCK128, seed=5, stream_id=6)
+    fwd = b.nvfp4_quantize(to_dev_bf16(x), b.AXIS_ROW, b.ROUND_RTN, 0, 1, b.GS_BLOCK128)
+    out = b.alloc_operand(shape[1], shape[0], b.GS_BLOCK128, poison=True)
+    b.nvfp4_requantize_t(fwd, b.ROUND_SR, 5, 6, out=out, rht_stream_id=rht)
+    assert_operand_equal(out, ref, f"{shape} rht{rht}", k_extended=rht != 0)
