@@ -122,6 +122,8 @@ class NVFP4Linear(torch.nn.Module):
         NVFP4Linear._instances += 1
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
+        if x.dim() == 0 or x.shape[-1] != self.in_features:  # the library takes a narrower input with the weights' leading dimension
+            raise RuntimeError(f"NVFP4Linear: input of shape {tuple(x.shape)} for {self.in_features} input features")
         x2d = x if x.dim() == 2 else x.reshape(-1, self.in_features)
         if x2d.dtype != torch.bfloat16:
             x2d = x2d.to(torch.bfloat16)

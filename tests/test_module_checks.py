@@ -1,0 +1,14 @@
+"""What NVFP4Linear refuses before it touches a device."""
+import pytest
+import torch
+
+
+@pytest.mark.parametrize("grad", [False, True])
+@pytest.mark.parametrize("shape", [(64, 128), (64, 512), (128,), (4, 16, 512), (2, 128), (0, 128), ()])
+def test_inputs_of_another_width_are_refused(shape, grad):
+    from paper_2510_27527_b200.module import NVFP4Linear
+
+    layer = NVFP4Linear(256, 64, device="cpu")
+    with torch.set_grad_enabled(grad), pytest.raises(RuntimeError, match="256 input features"):
+        layer(torch.zeros(shape, dtype=torch.bfloat16))
+    assert layer._calls == 0  # no key of the layer's sequence is used up
