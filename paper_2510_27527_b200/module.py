@@ -11,6 +11,7 @@ import ctypes
 import functools
 
 import torch
+from torch.autograd import forward_ad
 
 from . import binding as B
 
@@ -59,7 +60,7 @@ class _Call:
     __slots__ = ("buf", "saved", "ccfg", "keeps", "concurrent", "shape", "ws_bwd")
 
     def forward(self, x: torch.Tensor, weight: torch.Tensor, cfg: B.LayerConfig, seed: int) -> torch.Tensor:
-        (N_tok, D), C, dev = x.shape, weight.shape[0], x.device
+        (N_tok, D), C, dev = map(int, x.shape), int(weight.shape[0]), x.device  # (under jit.trace sizes are tensors)
         index = cfg.index(D, dev)
         n_out, gs = cfg.n_out, cfg.gs_mode
         offs, ws_at, ws_fwd, total, self.ws_bwd = _layout(N_tok, D, C, n_out, gs)
@@ -88,6 +89,13 @@ class _Call:
         B._check(B.lib.nvfp4_linear_bwd(dy.data_ptr(), dy.stride(0), ctypes.byref(self.saved), ctypes.byref(ccfg), dx.data_ptr(), dx.stride(0),
                                         dw.data_ptr(), dw.stride(0), ws.data_ptr(), self.ws_bwd, stream), "nvfp4_linear_bwd")
         return dx, dw
+
+
+def _needs_function(*inputs: torch.Tensor) -> bool:
+    """Whether a call has to go through the autograd function: a gradient can be asked for, a trace is being recorded (which sees the
+    function, but not what the library writes), or an input carries a forward-mode tangent (which the function refuses)."""
+    return (torch.is_grad_enabled() and any(t.requires_grad for t in inputs)) or torch.jit.is_tracing() or any(
+        forward_ad.unpack_dual(t).tangent is not None for t in inputs)
 
 
 class _NVFP4LinearFn(torch.autograd.Function):
@@ -131,7 +139,7 @@ class NVFP4Linear(torch.nn.Module):
         # this layer's key of this call
         seed = call_seed(self.cfg.seed, self.layer_id, self._calls)
         self._calls += 1
-        if torch.is_grad_enabled() and (x2d.requires_grad or self.weight.requires_grad):
+        if _needs_function(x2d, self.weight):
             y = _NVFP4LinearFn.apply(x2d, self.weight, self.cfg, seed)
         else:
             y = _Call().forward(x2d, self.weight, self.cfg, seed)

@@ -95,3 +95,24 @@ def test_index_arrays_follow_the_outlier_channels():
     outl, keep, cmap = cfg.index(16)
     assert outl.tolist() == [1, 7] and 5 in keep.tolist() and cmap.tolist()[5] == 4
     assert cfg.index(24)[1].numel() == 22
+
+
+@pytest.mark.filterwarnings("ignore::torch.jit.TracerWarning", "ignore::DeprecationWarning")
+@pytest.mark.parametrize("grad", [False, True])
+@pytest.mark.parametrize("weight_grad", [False, True])
+def test_traces_and_tangents_do_not_pass_the_autograd_function_by(grad, weight_grad):
+    import torch.autograd.forward_ad as fa
+
+    from paper_2510_27527_b200.module import NVFP4Linear
+
+    layer = NVFP4Linear(256, 136).requires_grad_(weight_grad)
+    x = torch.randn(64, 256, device="cuda").to(torch.bfloat16)
+    with torch.set_grad_enabled(grad):
+        traced = torch.jit.trace(layer, x, check_trace=False)  # a recorded call keeps the key it was recorded with
+        layer._calls = 0
+        want = layer(2 * x)
+        assert torch.equal(traced(2 * x), want)
+        with fa.dual_level(), pytest.raises(NotImplementedError, match="jvp"):
+            layer(fa.make_dual(x, torch.ones_like(x)))
+        with fa.dual_level(), pytest.raises(NotImplementedError, match="jvp"):
+            torch.func.functional_call(layer, {"weight": fa.make_dual(layer.weight.detach(), torch.ones_like(layer.weight))}, (x,))
