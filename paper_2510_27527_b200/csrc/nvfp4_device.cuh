@@ -103,20 +103,31 @@ __device__ __forceinline__ uint32_t cells_max(const uint32_t* __restrict__ cells
 __device__ __forceinline__ uint32_t tensor_amax_bits(const uint32_t* __restrict__ cells, int words) {
   return words == 1 ? cells[0] : cells_max<64>(cells);
 }
-// Word of this thread's cluster <- maximum of the cluster's values m. Every thread of every CTA calls it; blockDim.x is a
-// multiple of 32 and at most 1024, the cluster (cluster_x, 1, 1) has at most 8 CTAs. CTA `block` of the n_blocks (whole
-// clusters, at most N of them) that share the N words.
+__device__ __forceinline__ uint32_t cluster_ctas() {
+  uint32_t n;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+  return n;
+}
+// At the head of a kernel that ends with cells_write: says that this CTA has started. A CTA's shared memory may be written from another
+// one only after that, and a CTA without work gets to its store at once; the wait is in cells_write, under the loads of the others.
+__device__ __forceinline__ void cells_begin() {
+  if (cluster_ctas() > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+// Word of this thread's cluster <- maximum of the cluster's values m. Every thread of every CTA calls it, after cells_begin;
+// blockDim.x is a multiple of 32 and at most 1024, the cluster (cluster_x, 1, 1) has at most 8 CTAs. CTA `block` of the n_blocks
+// (whole clusters, at most N of them) that share the N words.
 template <int N>
 __device__ __forceinline__ void cells_write(uint32_t m, uint32_t* cells, uint32_t block, uint32_t n_blocks) {
   __shared__ uint32_t warp_max[32];
   __shared__ uint32_t cta_max[8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-  uint32_t rank, n_rank;
+  const uint32_t n_rank = cluster_ctas();
+  uint32_t rank;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n_rank));
   m = __reduce_max_sync(0xFFFFFFFFu, m);
   if (lane == 0) warp_max[wid] = m;
   __syncthreads();
+  if (n_rank > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every CTA of the cluster has started (cells_begin)
   if (wid == 0) {
     m = __reduce_max_sync(0xFFFFFFFFu, lane < n_warps ? warp_max[lane] : 0u);
     if (lane == 0) {

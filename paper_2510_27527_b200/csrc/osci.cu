@@ -143,6 +143,7 @@ __device__ __forceinline__ float amax_row(const float* __restrict__ p, int64_t D
 // 1024 / 2816 wide block, with the loads below under this kernel: 189 -> 138 us; 4096 x 4096: 163 -> 153 us; 256 x 264: 32 -> 17.
 __global__ void __launch_bounds__(512) amax_f32_kernel(const float* __restrict__ W0, int64_t ld0, const float* __restrict__ W1, int64_t ld1,
                                                       int64_t C, int64_t D, uint32_t* cells) {
+  cells_begin();
   pdl_wait();
   pdl_launch_next();  // (its loads of the weights run under this kernel)
   const float* __restrict__ W = blockIdx.y ? W1 : W0;

@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(256) amax_tensor_bf16_kernel(const uint16_t* _
 __global__ void __launch_bounds__(512) amax_tensor_words_kernel(const uint16_t* __restrict__ a, int64_t rows_a, int64_t cols_a, int64_t ld_a,
                                                                uint32_t* cells_a, unsigned grid_a, const uint16_t* __restrict__ b,
                                                                int64_t rows_b, int64_t cols_b, int64_t ld_b, uint32_t* cells_b) {
+  cells_begin();
   pdl_prologue();
   const bool first = blockIdx.x < grid_a;
   const unsigned block = first ? blockIdx.x : blockIdx.x - grid_a, n_blocks = first ? grid_a : gridDim.x - grid_a;

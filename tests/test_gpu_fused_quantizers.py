@@ -72,3 +72,21 @@ def test_tensor_maximum(rows, cols, where, pad):
     q = b.nvfp4_quantize(x, gs_mode=b.GS_TENSOR, workspace=poison(torch.empty(256, dtype=torch.uint8, device="cuda")))
     torch.cuda.synchronize()
     assert q.gscale.item() == (torch.tensor(21.0) / torch.tensor(2688.0)).item()
+
+
+@pytest.mark.parametrize("rows", [513, 517, 1025, 4097])  # one row past whole clusters: most CTAs of the last one have nothing to read
+def test_tensor_maximum_with_ctas_that_have_no_work(rows):
+    b = B()
+    xs = [torch.full((rows, 4096), 0.5, dtype=torch.bfloat16, device="cuda") for _ in range(4)]
+    ends = torch.tensor([3.0, -21.0, 5.0, -40.0])
+    for x, v, i in zip(xs, ends.tolist(), (0, rows - 1, rows // 2, rows - 1)):
+        x[i, -1] = v
+    ops = [[b.alloc_operand(rows, 4096, b.GS_TENSOR) for _ in xs] for _ in range(10)]
+    ws = torch.empty(256, dtype=torch.uint8, device="cuda")
+    for row in ops:  # back to back on one workspace
+        for x, q in zip(xs, row):
+            b.nvfp4_quantize(x, gs_mode=b.GS_TENSOR, out=q, workspace=ws)
+    torch.cuda.synchronize()
+    want = (ends.abs() / torch.tensor(2688.0)).tolist()
+    for row in ops:
+        assert [q.gscale.item() for q in row] == want
