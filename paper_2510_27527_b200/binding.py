@@ -449,6 +449,51 @@ def nvfp4_osci_sparse_suppress(W: torch.Tensor, state: OsciSparseState, tau: flo
            "nvfp4_osci_sparse_suppress")
 
 
+class IndexArrays(tuple):
+    """(outlier channels, kept channels, channel map): int32 device arrays that several streams may read."""
+
+    streams: set | None = None  # streams that the allocator knows to read them; None: not on a CUDA device
+
+    def here(self) -> "IndexArrays":
+        """The arrays, for kernels on the current stream: given back, their memory waits for that stream too."""
+        if self.streams is not None and (s := _stream_ptr()) not in self.streams:
+            for a in self:
+                a.record_stream(torch.cuda.current_stream())
+            self.streams.add(s)
+        return self
+
+
+class IndexCache:
+    """The index arrays of the channel lists used last, by hidden size, device and the channels themselves (their values, not the
+    array's identity)."""
+
+    MOST = 8
+
+    def __init__(self):
+        self._of = {}
+
+    def __reduce__(self):  # a copy of a configuration makes its own
+        return IndexCache, ()
+
+    def get(self, outliers, D: int, dev: torch.device) -> IndexArrays:
+        outl = np.asarray(outliers, dtype=np.int64)
+        key = (D, dev, outl.tobytes())
+        held = self._of.pop(key, None)
+        if held is None:
+            mask = np.ones(D, dtype=bool)
+            mask[outl] = False
+            keep = np.nonzero(mask)[0]
+            cmap = np.full(D, -1, dtype=np.int32)
+            cmap[keep] = np.arange(len(keep), dtype=np.int32)
+            held = IndexArrays(torch.from_numpy(a.astype(np.int32)).to(dev) for a in (outl, keep, cmap))
+            if dev.type == "cuda":
+                held.streams = {torch.cuda.current_stream(dev).cuda_stream}
+        self._of[key] = held
+        if len(self._of) > self.MOST:
+            self._of.pop(next(iter(list(self._of))), None)  # the one used longest ago
+        return held.here()
+
+
 @dataclass
 class LayerConfig:
     gs_mode: int = GS_TENSOR
@@ -465,11 +510,11 @@ class LayerConfig:
     # run the independent chains of a call (dX beside dW, the weight quantizer beside the activation quantizer) on a
     # second stream: the stream and its three events are created here, with torch, and handed to the library
     concurrent: bool = True
-    # device index arrays, built by prepare()
+    # the device index arrays that prepare() made last
     _outl: torch.Tensor | None = None
     _keep: torch.Tensor | None = None
     _map: torch.Tensor | None = None
-    _of: tuple | None = None  # (hidden size, device, outlier channels, the three arrays made for them)
+    _arrays: IndexCache | None = None
     _side: tuple | None = None
 
     def side(self, device):
@@ -482,45 +527,35 @@ class LayerConfig:
         return self._side[1:]
 
     def prepare(self, D: int, device="cuda"):
-        """Uploads the OutControl index arrays for hidden size D (index bookkeeping only)."""
+        """Second stream and OutControl index arrays (returned; None without outlier channels) for hidden size D."""
         self.side(device)
-        self.index(D, device)
+        index = self.index(D, device)
+        if index is not None:
+            self._outl, self._keep, self._map = index
+        return index
 
     def index(self, D: int, device="cuda"):
-        """(outlier channels, kept channels, channel map) on the device, or None without outlier channels. What is there already
-        is kept while hidden size, device and the channels themselves (their values, not the array's identity) are the same."""
+        """(outlier channels, kept channels, channel map) on the device, or None without outlier channels. Leaves what prepare() made
+        last alone: layers of other widths may share a configuration."""
         if self.outliers is None or len(self.outliers) == 0:
             return None
-        outl = np.array(self.outliers, dtype=np.int64)
-        dev = _device_of(device)
-        of = self._of
-        if of is not None and of[0] == D and of[1] == dev and np.array_equal(of[2], outl):
-            return of[3]
-        mask = np.ones(D, dtype=bool)
-        mask[outl] = False
-        keep = np.nonzero(mask)[0]
-        cmap = np.full(D, -1, dtype=np.int32)
-        cmap[keep] = np.arange(len(keep), dtype=np.int32)
-        held = tuple(torch.from_numpy(a.astype(np.int32)).to(dev) for a in (outl, keep, cmap))
-        self._of = (D, dev, outl, held)
-        self._outl, self._keep, self._map = held
-        return held
+        if self._arrays is None:
+            self._arrays = IndexCache()
+        return self._arrays.get(self.outliers, D, _device_of(device))
 
     @property
     def n_out(self) -> int:
         return 0 if self.outliers is None else len(self.outliers)
 
-    def c(self, seed: int | None = None, dtypes: tuple | None = None, index: tuple | None = None, side: tuple | None = None) -> CLayerCfg:
-        """The C structure. Seed, output types, index arrays and second stream are the configuration's own unless `dtypes` is given."""
-        if dtypes is None:
-            dtypes = (self.y_dtype, self.dx_dtype, self.dw_dtype)
-            side = self._side[1:] if (self.concurrent and self._side is not None) else None
-            index = (self._outl, self._keep, self._map)
-        outl, keep, cmap = index if index is not None else (None, None, None)
-        c = CLayerCfg(self.gs_mode, (c_i32 * 6)(*self.rounding), self.seed if seed is None else seed, *dtypes, self.n_out, _ptr(outl),
-                      _ptr(keep), _ptr(cmap), _ptr(self.dev_status), int(self.rht), int(self.outlier_fp8), int(self.w_block16))
-        if side is not None:
-            set_side(c, side)
+    def c(self, index: tuple | None = None, seed: int | None = None, dtypes: tuple | None = None, side: tuple | None = None) -> CLayerCfg:
+        """The C structure. What is not given is the configuration's own: the index arrays prepared last, seed, output types (of y, dX
+        and dW) and second stream."""
+        outl, keep, cmap = index if index is not None else (self._outl, self._keep, self._map)
+        c = CLayerCfg(self.gs_mode, (c_i32 * 6)(*self.rounding), self.seed if seed is None else seed,
+                      *(dtypes if dtypes is not None else (self.y_dtype, self.dx_dtype, self.dw_dtype)), self.n_out, _ptr(outl), _ptr(keep),
+                      _ptr(cmap), _ptr(self.dev_status), int(self.rht), int(self.outlier_fp8), int(self.w_block16))
+        if self.concurrent and (side is not None or self._side is not None):
+            set_side(c, side if side is not None else self._side[1:])
         return c
 
 
@@ -529,9 +564,9 @@ def set_side(c: CLayerCfg, side: tuple) -> None:
 
 
 def _device_of(device) -> torch.device:
-    """`device` with its index filled in."""
+    """`device`, a CUDA device with its index filled in."""
     dev = torch.device(device)
-    return torch.device("cuda", torch.cuda.current_device()) if dev.index is None else dev
+    return torch.device("cuda", torch.cuda.current_device()) if dev.type == "cuda" and dev.index is None else dev
 
 
 def _make_side(dev: torch.device) -> tuple:
@@ -571,6 +606,7 @@ class Saved:
     W: torch.Tensor
     X_out: torch.Tensor | None = None  # [N_tok, Kh] bf16, OutControl only
     W_out: torch.Tensor | None = None  # [C, Kh] bf16
+    index: IndexArrays | None = None  # of the forward call, OutControl only
 
     def c(self) -> CSaved:
         return CSaved(self.qx.c(), self.qw.c(), _ptr(self.X), _ptr(self.W), self.X.stride(0), self.W.stride(0),
@@ -618,19 +654,26 @@ def nvfp4_linear_fwd(X: torch.Tensor, W: torch.Tensor, cfg: LayerConfig, Y: torc
                      saved: Saved | None = None, workspace: torch.Tensor | None = None):
     N_tok, D = X.shape
     C = W.shape[0]
-    cfg.prepare(D, X.device)
-    Dk = D - cfg.n_out
+    index = cfg.prepare(D, X.device)
     if saved is None:
         saved = alloc_saved(X, W, cfg)
     else:
         saved.X, saved.W = X, W
+    saved.index = index
     if Y is None:
         Y = _matrix(N_tok, C, cfg.y_dtype, X.device)
     ws = workspace if workspace is not None else linear_workspace(OP_FWD, N_tok, D, C, cfg, X.device)
-    cs, cc = saved.c(), cfg.c()
+    cs, cc = saved.c(), cfg.c(index)
     _check(_lib.nvfp4_linear_fwd(_ptr(X), X.stride(0), _ptr(W), W.stride(0), N_tok, D, C, ctypes.byref(cc), _ptr(Y),
                                  Y.stride(0), ctypes.byref(cs), _ptr(ws), ws.numel(), _stream_ptr()), "nvfp4_linear_fwd")
     return Y, saved
+
+
+def _index_of(saved: Saved, cfg: LayerConfig, device):
+    """The index arrays of the forward call behind `saved`, whatever `cfg` has been used for since."""
+    if cfg.n_out == 0:
+        return None
+    return saved.index.here() if saved.index is not None else cfg.prepare(saved.X.shape[1], device)
 
 
 def nvfp4_linear_bwd_dx(dY: torch.Tensor, saved: Saved, cfg: LayerConfig, dX: torch.Tensor | None = None,
@@ -640,7 +683,7 @@ def nvfp4_linear_bwd_dx(dY: torch.Tensor, saved: Saved, cfg: LayerConfig, dX: to
     if dX is None:
         dX = _matrix(N_tok, D, cfg.dx_dtype, dY.device)
     ws = workspace if workspace is not None else linear_workspace(OP_BWD_DX, N_tok, D, C, cfg, dY.device)
-    cs, cc = saved.c(), cfg.c()
+    cs, cc = saved.c(), cfg.c(_index_of(saved, cfg, dY.device))
     _check(_lib.nvfp4_linear_bwd_dx(_ptr(dY), dY.stride(0), ctypes.byref(cs), ctypes.byref(cc), _ptr(dX), dX.stride(0),
                                     _ptr(ws), ws.numel(), _stream_ptr()), "nvfp4_linear_bwd_dx")
     return dX
@@ -653,7 +696,7 @@ def nvfp4_linear_bwd_dw(dY: torch.Tensor, saved: Saved, cfg: LayerConfig, dW: to
     if dW is None:
         dW = _matrix(C, D, cfg.dw_dtype, dY.device)
     ws = workspace if workspace is not None else linear_workspace(OP_BWD_DW, N_tok, D, C, cfg, dY.device)
-    cs, cc = saved.c(), cfg.c()
+    cs, cc = saved.c(), cfg.c(_index_of(saved, cfg, dY.device))
     _check(_lib.nvfp4_linear_bwd_dw(_ptr(dY), dY.stride(0), ctypes.byref(cs), ctypes.byref(cc), _ptr(dW), dW.stride(0),
                                     _ptr(ws), ws.numel(), _stream_ptr()), "nvfp4_linear_bwd_dw")
     return dW
@@ -664,13 +707,13 @@ def nvfp4_linear_bwd(dY: torch.Tensor, saved: Saved, cfg: LayerConfig, dX: torch
     """Both backward products in one call (dX, dW); the per-tensor amax of dY is computed once where Q3 and Q5 share it."""
     N_tok, D = saved.X.shape
     C = saved.W.shape[0]
-    cfg.prepare(D, dY.device)
+    cfg.side(dY.device)
     if dX is None:
         dX = _matrix(N_tok, D, cfg.dx_dtype, dY.device)
     if dW is None:
         dW = _matrix(C, D, cfg.dw_dtype, dY.device)
     ws = workspace if workspace is not None else linear_workspace(OP_BWD, N_tok, D, C, cfg, dY.device)
-    cs, cc = saved.c(), cfg.c()
+    cs, cc = saved.c(), cfg.c(_index_of(saved, cfg, dY.device))
     _check(_lib.nvfp4_linear_bwd(_ptr(dY), dY.stride(0), ctypes.byref(cs), ctypes.byref(cc), _ptr(dX), dX.stride(0), _ptr(dW),
                                  dW.stride(0), _ptr(ws), ws.numel(), _stream_ptr()), "nvfp4_linear_bwd")
     return dX, dW

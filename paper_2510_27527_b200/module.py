@@ -71,8 +71,7 @@ class _Call:
         saved = B.CSaved(B.COperand(at[0], at[1], at[2], N_tok, D - n_out, gs, B.SF_TILED128x4),
                          B.COperand(at[3], at[4], at[5], C, D - n_out, gs, B.SF_TILED128x4), X_out=at[6], W_out=at[7])
         # the configuration as it is now: what the caller changes later belongs to later calls
-        ccfg = cfg.c(seed=seed, dtypes=(B.DT_BF16, B.DT_BF16, B.DT_BF16), index=index,
-                     side=B.thread_side(dev, stream) if cfg.concurrent else None)
+        ccfg = cfg.c(index, seed, (B.DT_BF16, B.DT_BF16, B.DT_BF16), B.thread_side(dev, stream) if cfg.concurrent else None)
         B._check(B.lib.nvfp4_linear_fwd(x.data_ptr(), x.stride(0), weight.data_ptr(), weight.stride(0), N_tok, D, C, ctypes.byref(ccfg),
                                         y.data_ptr(), y.stride(0), ctypes.byref(saved), p + ws_at, ws_fwd, stream), "nvfp4_linear_fwd")
         self.buf, self.saved, self.ccfg, self.shape = buf, saved, ccfg, (N_tok, D, C)
@@ -84,6 +83,8 @@ class _Call:
         dx, dw = B._matrix(N_tok, D, B.DT_BF16, dev), B._matrix(C, D, B.DT_BF16, dev)
         ws, stream = torch.empty(self.ws_bwd, dtype=torch.uint8, device=dev), B._stream_ptr()
         ccfg = B.CLayerCfg.from_buffer_copy(self.ccfg)
+        if self.keeps[0] is not None:
+            self.keeps[0].here()
         if self.concurrent:  # autograd runs backward on a thread of its own, which has its own second stream and events
             B.set_side(ccfg, B.thread_side(dev, stream))
         B._check(B.lib.nvfp4_linear_bwd(dy.data_ptr(), dy.stride(0), ctypes.byref(self.saved), ctypes.byref(ccfg), dx.data_ptr(), dx.stride(0),

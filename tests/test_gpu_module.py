@@ -97,6 +97,52 @@ def test_index_arrays_follow_the_outlier_channels():
     assert cfg.index(24)[1].numel() == 22
 
 
+def test_layers_of_two_widths_share_a_configuration():
+    """A module's call between a forward call and its separate backward calls changes nothing for them."""
+    from paper_2510_27527_b200 import binding as b
+    from paper_2510_27527_b200.module import NVFP4Linear
+
+    mk = lambda r, c: torch.randn(r, c, device="cuda").to(torch.bfloat16)
+    outl = [3, 40, 41, 199]
+    x, w, dy, wide = mk(96, 200), mk(72, 200), mk(96, 72), mk(50, 1024)
+    want_cfg = b.LayerConfig(seed=5, outliers=outl)
+    _, saved = b.nvfp4_linear_fwd(x, w, want_cfg)
+    want = b.nvfp4_linear_bwd(dy, saved, want_cfg)
+    cfg = b.LayerConfig(seed=5, outliers=outl)
+    layer = NVFP4Linear(1024, 64, cfg=cfg)
+    _, saved = b.nvfp4_linear_fwd(x, w, cfg)
+    with torch.no_grad():
+        layer(wide)
+    b.nvfp4_linear_fwd(wide, layer.weight.detach(), cfg)  # (and a direct call of that width)
+    got = b.nvfp4_linear_bwd_dx(dy, saved, cfg), b.nvfp4_linear_bwd_dw(dy, saved, cfg)
+    both = b.nvfp4_linear_bwd(dy, saved, cfg)
+    for a, c, r in zip(got, both, want):
+        assert torch.equal(a, r) and torch.equal(c, r)
+
+
+def test_index_arrays_outlive_their_readers_on_other_streams():
+    """Arrays uploaded on one stream, read by a call that another stream has yet to run, replaced meanwhile: their memory is not
+    given to anyone before that call is done."""
+    from paper_2510_27527_b200 import binding as b
+    from paper_2510_27527_b200.module import NVFP4Linear
+
+    D, outl = 4096, list(range(0, 4096, 13))
+    layer = NVFP4Linear(D, 64, cfg=b.LayerConfig(outliers=outl))
+    x = torch.randn(64, D, device="cuda").to(torch.bfloat16)
+    side = torch.cuda.Stream()
+    with torch.no_grad():
+        want = layer(x)  # uploads on the current stream
+        layer._calls = 0
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(100_000_000)  # (about 50 ms; the call below waits behind it)
+            got = layer(x)
+        layer.cfg._arrays._of.clear()
+        ids = [torch.arange(n, dtype=torch.int32, device="cuda") for n in (len(outl), D - len(outl), D) for _ in range(8)]  # valid indexes, other ones
+    torch.cuda.synchronize()
+    assert torch.equal(got, want) and len(ids) == 24
+
+
 @pytest.mark.filterwarnings("ignore::torch.jit.TracerWarning", "ignore::DeprecationWarning")
 @pytest.mark.parametrize("grad", [False, True])
 @pytest.mark.parametrize("weight_grad", [False, True])
