@@ -60,7 +60,7 @@ class _Call:
     __slots__ = ("buf", "saved", "ccfg", "keeps", "concurrent", "shape", "ws_bwd")
 
     def forward(self, x: torch.Tensor, weight: torch.Tensor, cfg: B.LayerConfig, seed: int) -> torch.Tensor:
-        (N_tok, D), C, dev = map(int, x.shape), int(weight.shape[0]), x.device  # (under jit.trace sizes are tensors)
+        N_tok, D, C, dev = int(x.shape[0]), int(x.shape[1]), int(weight.shape[0]), x.device  # (under jit.trace sizes are tensors)
         index = cfg.index(D, dev)
         n_out, gs = cfg.n_out, cfg.gs_mode
         offs, ws_at, ws_fwd, total, self.ws_bwd = _layout(N_tok, D, C, n_out, gs)
@@ -92,11 +92,11 @@ class _Call:
         return dx, dw
 
 
-def _needs_function(*inputs: torch.Tensor) -> bool:
-    """Whether a call has to go through the autograd function: a gradient can be asked for, a trace is being recorded (which sees the
-    function, but not what the library writes), or an input carries a forward-mode tangent (which the function refuses)."""
-    return (torch.is_grad_enabled() and any(t.requires_grad for t in inputs)) or torch.jit.is_tracing() or any(
-        forward_ad.unpack_dual(t).tangent is not None for t in inputs)
+def _needs_function(x: torch.Tensor, weight: torch.Tensor) -> bool:
+    """Whether a call has to go through the autograd function: a gradient can be asked for, an input may carry a forward-mode tangent
+    (which the function refuses), or a trace is being recorded (which sees the function, but not what the library writes). (Plain
+    comparisons: unpack_dual and a generator over the two tensors took 2 us of a 32 us call.)"""
+    return (torch.is_grad_enabled() and (x.requires_grad or weight.requires_grad)) or forward_ad._current_level >= 0 or torch.jit.is_tracing()
 
 
 class _NVFP4LinearFn(torch.autograd.Function):
