@@ -141,7 +141,7 @@ nvfp4_status nvfp4_quantize(const void* src_bf16, int64_t rows, int64_t cols, in
  *     and nothing is launched. TENSOR and BLOCK128 have no such limit.
  *   - The first call made with a given device current looks up the array's device address; make that first call
  *     outside any stream capture.
- *   - Every call on a device shares the one array. The cells a call uses are cleared on `stream` before use, so
+ *   - Every call on a device shares the one array. The cells that a call reads are all written or cleared on `stream` before, so
  *     calls that are ordered (same stream, or ordered by events) are independent; calls whose kernels can overlap
  *     on the GPU (different streams, no ordering) race on the cells and give undefined scales.
  * --------------------------------------------------------------------------------------------------------- */

@@ -113,8 +113,9 @@ inline size_t carve_size(size_t& total, size_t bytes) {
   return total;
 }
 
+// Scratch of an amax pass: a cell per operand row (ROW), the words of a tensor's maximum (TENSOR); BLOCK128 has no pass.
 size_t cells_bytes(int64_t rows, int32_t gs_mode) {
-  return gs_mode == NVFP4_GS_ROW ? (size_t)std::max<int64_t>(rows, 1) * 4 : 4;
+  return gs_mode == NVFP4_GS_ROW ? (size_t)std::max<int64_t>(rows, 1) * 4 : gs_mode == NVFP4_GS_TENSOR ? kTensorAmaxWords * 4 : 4;
 }
 
 // Operand carved from a workspace (tiled scales).

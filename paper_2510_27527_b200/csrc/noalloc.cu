@@ -43,13 +43,15 @@ nvfp4_status nvfp4_quantize_static(const void* src_bf16, int64_t rows, int64_t c
                                    int32_t rounding, uint64_t seed, uint32_t stream_id, const int32_t* keep_cols,
                                    int64_t n_keep, const nvfp4_operand* out, void* stream) {
   if (!out) return NVFP4_ERR_NULL;
-  // The ROW scale mode needs one cell per operand row; the other modes need one cell.
+  // The ROW scale mode needs one cell per operand row, TENSOR the words of a maximum, BLOCK128 none.
+  static_assert(kStaticCells >= nvfp4::kTensorAmaxWords, "the words of a tensor's maximum fit");
   if (out->gs_mode == NVFP4_GS_ROW && out->R > kStaticCells) return NVFP4_ERR_LIMIT;
   uint32_t* cells = nullptr;
   const nvfp4_status s = static_cells(&cells);
   if (s != NVFP4_OK) return s;
-  // Same validation, same kernels, same order as nvfp4_quantize; only the scratch differs. The launchers zero the
-  // cells they use on `stream` before the amax pass, so the previous call's contents never leak into this one.
+  // Same validation, same kernels, same order as nvfp4_quantize; only the scratch differs. The amax
+  // pass of a call writes every cell that its quantizer reads (or folds into cells that a launch before it cleared), so the
+  // previous call's contents never leak into this one.
   return nvfp4_quantize(src_bf16, rows, cols, ld, axis, rounding, seed, stream_id, 0u, keep_cols, n_keep, out, cells,
                         (size_t)kStaticCells * sizeof(uint32_t), stream);
 }

@@ -14,8 +14,8 @@
 namespace nvfp4 {
 
 // =========================================================================================================
-// amax pre-passes. Results are bit patterns of non-negative floats combined with atomicMax (order-free, hence
-// deterministic). The cells must be zero before the launch.
+// amax pre-passes. Results are bit patterns of non-negative floats, whose maxima do not depend on an order. A kernel writes its
+// cells (amax_tensor_words, amax_rows*) or folds into cells that are zero before the launch (atomicMax): said at each.
 // =========================================================================================================
 // A thread's maximum (binary32 pattern) over its share of the tensor.
 __device__ __forceinline__ uint32_t amax_tensor_bf16_body(const uint16_t* __restrict__ src, int64_t rows, int64_t cols, int64_t ld,
