@@ -494,39 +494,47 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
 // =========================================================================================================
 // BLOCK128 variant: the FP32 global scale changes every 128 k (the paper's 1x128 outer block, Sec. 2.2), so a partial product can
-// only be accumulated over 128 k inside tensor memory. The MMA warp writes each 128-k partial of a 128 x 192 tile (two K = 64
-// instructions) into one of two tensor-memory buffers; twelve promotion warps pull it out, 32 rows x 64 columns each, and promote it
+// only be accumulated over 128 k inside tensor memory. The MMA warp writes each 128-k partial of a 128 x TN tile (two K = 64
+// instructions) into one of two or three tensor-memory buffers; promotion warps pull it out, 32 rows x CW columns each, and promote it
 // into FP32 register accumulators with the rank-1 scale SgA[m, kc] * SgB[n, kc] (packed f32x2 multiply + FMA).
 //
-// What bounds it: the promotion. A packed operation issues every 2.8 cycles at best (measured, from registers, two or more warps
-// per scheduler), which is 540 cycles per partial against 200 of its MMAs; this kernel takes 840 at long K, 1060 at K = 1024.
-//   - Three promotion warps per scheduler: a warp's barrier, tensor-memory load and hand-over latencies (about 400 cycles per
+// What bounds it: the promotion. A packed operation issues every 2.8 cycles at best (timed in a loop from registers, two or more
+// warps per scheduler), which is 540 cycles per partial of 192 columns against 200 of its MMAs; the kernel takes 790 to 840 there at long
+// K, about 620 with 128 columns and 380 with 64.
+//   - Two or three promotion warps per scheduler: a warp's barrier, tensor-memory load and hand-over latencies (about 400 cycles per
 //     partial) run under the others' arithmetic. With one (a 128 x 128 tile, four warps with 128 columns each) they add up:
 //     760 cycles per 128 columns. 192 columns are what a register file of 128 a thread on average holds (setmaxnreg: 80 for the
-//     four warps that load, issue and fetch scales, 144 for the others) with a buffer to spare in tensor memory.
+//     four warps that load, issue and fetch scales, 144 for the others) with a buffer to spare in tensor memory. With 64 columns a
+//     warp has 32 of them and both of its loads in flight at once.
 //   - Fragments: the 16x256b load gives a thread 2 columns x 8 groups of 2 rows, i.e. 16 column scales and 4 row scales for 64
 //     elements; with a thread per row it would be a column scale per element, read from shared memory by every warp.
 //   - Scales come through shared memory, fetched by two warps in 16-byte pieces (below).
-// us, before (one group of four warps) and now: 8192 x 3072 x 1024 49.0 / 35.7, 8192 x 1024 x 3072 42.5 / 38.9, 3072 x 1024 x 8192
-// (FP32) 55.1 / 33.7, 1999 x 1416 x 1000 14.5 / 10.6, 4096^3 95.7 / 78.5, 16384 x 8192 x 8192 1415 / 1048. K <= 16384.
+// us, with one group of four warps / now (tile width by block128_tile_cols): 8192 x 3072 x 1024 49.1 / 31.9, 8192 x 1024 x 3072 42.6 /
+// 36.0, 3072 x 1024 x 8192 (FP32) 54.8 / 32.7, 1024 x 1024 x 8192 (FP32) 28.3 / 15.9, 4096^3 103.9 / 85.0. K <= 16384.
 // =========================================================================================================
-constexpr int B128_TN = 192;
-constexpr int B128_STAGES = 3;
-constexpr int B128_NBUF = 2;
 constexpr int64_t B128_MAX_K = 16384;
-constexpr int B128_PROMO_WARPS = 12;                       // warps 4 .. 15: 32 rows x 64 columns each
-constexpr int B128_THREADS = 128 + 32 * B128_PROMO_WARPS;  // warps 0 .. 3: loads, MMA, global scales (two)
-constexpr int B128_SC_SLOTS = 3;                           // ring of global-scale slots, four chunks each
-constexpr uint32_t B128_B_BYTES = B128_TN * 128;
-constexpr uint32_t B128_SFB_BYTES = 4096;                  // the two 128-row scale tiles that the B rows touch
-constexpr uint32_t B128_STAGE_BYTES = A_BYTES + B128_B_BYTES + SFA_BYTES + B128_SFB_BYTES;  // 46 KB
-constexpr uint32_t B128_STAGING_BYTES = B128_PROMO_WARPS * 4096;                            // 32 rows x 128 bytes per promotion warp
-constexpr uint32_t B128_SC_CHUNK = (128 + B128_TN) * 4;                                     // SgA, then SgB of one chunk
-constexpr uint32_t B128_SC_BYTES = 4 * B128_SC_CHUNK;
-constexpr uint32_t B128_SMEM_BYTES = B128_STAGES * B128_STAGE_BYTES + B128_STAGING_BYTES + B128_SC_SLOTS * B128_SC_BYTES + 1024 + 256;
-constexpr uint32_t B128_SF_COLS = 48, B128_SF_SETS = 2;    // tensor-memory columns of a k tile's block scales: 16 of A, 32 of B
-static_assert(B128_NBUF * B128_TN + B128_SF_SETS * B128_SF_COLS <= 512, "tensor memory budget");
-static_assert(B128_SMEM_BYTES <= 227 * 1024, "shared memory budget");
+template <int TN_>
+struct B128 {
+  static constexpr int TN = TN_;                             // columns of a tile: 192, 128 or 64
+  static constexpr int CW = TN == 64 ? 32 : 64;              // columns of a promotion warp (32 rows each)
+  static constexpr int PROMO_WARPS = 4 * (TN / CW);          // warps 4 .. : twelve, or eight
+  static constexpr int THREADS = 128 + 32 * PROMO_WARPS;     // warps 0 .. 3: loads, MMA, global scales (two)
+  static constexpr int STAGES = TN == 192 ? 3 : 4;
+  static constexpr int NBUF = TN == 192 ? 2 : 3;             // partials in tensor memory
+  static constexpr int SC_SLOTS = 3;                         // ring of global-scale slots, four chunks each
+  static constexpr int SF_TILES = TN == 192 ? 2 : 1;         // 128-row scale tiles that the B rows touch
+  static constexpr uint32_t B_BYTES = TN * 128;
+  static constexpr uint32_t SFB_BYTES = SF_TILES * 2048;
+  static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES + SFA_BYTES + SFB_BYTES;  // 46, 36 or 28 KB
+  static constexpr uint32_t STAGING_BYTES = PROMO_WARPS * 4096;                       // 32 rows x 128 bytes per promotion warp
+  static constexpr uint32_t SC_CHUNK = (128 + TN) * 4;                                // SgA, then SgB of one chunk
+  static constexpr uint32_t SC_BYTES = 4 * SC_CHUNK;
+  static constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + STAGING_BYTES + SC_SLOTS * SC_BYTES + 1024 + 256;
+  static constexpr uint32_t SF_COLS = 16 + 16 * SF_TILES, SF_SETS = 2;  // tensor-memory columns of a k tile's block scales: of A, of B
+  static_assert(NBUF * TN + SF_SETS * SF_COLS <= 512, "tensor memory budget");
+  static_assert(STAGE_BYTES % 1024 == 0 && SMEM_BYTES <= 227 * 1024, "shared memory budget");
+  static_assert(8 * (2 * STAGES + 2 * NBUF + 2 * SC_SLOTS + 1) <= 256, "barrier space");
+};
 
 // 16 rows x 64 columns of a partial: v[4 i + 2 q + e] is row 8 q + lane / 4, column 8 i + 2 (lane % 4) + e. Wait with tc_wait_ld.
 __device__ __forceinline__ void tc_ld_16x256b_x8(uint32_t taddr, uint32_t (&v)[32]) {
@@ -537,6 +545,14 @@ __device__ __forceinline__ void tc_ld_16x256b_x8(uint32_t taddr, uint32_t (&v)[3
         "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
         "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
         "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tc_ld_16x256b_x4(uint32_t taddr, uint32_t (&v)[16]) {  // (32 columns: i < 4)
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr)
       : "memory");
 }
@@ -625,18 +641,19 @@ __device__ __forceinline__ void b128_store_rows(const Params& p, uint32_t stage,
   }
 }
 
-// A warp's 32 rows x 64 columns of C from accumulator fragments (layout: see tc_ld_16x256b_x8): 128-byte row pieces staged in shared
+// A warp's 32 rows x CW columns of C from accumulator fragments (layout: see tc_ld_16x256b_x8): 128-byte row pieces staged in shared
 // memory with the 128-byte swizzle. Written by the bulk-tensor engine as full lines, rows clipped at the edge of C; at the right edge
 // (whose padding columns stay untouched) and when adding to the old C read back by rows, four columns per lane, eight lanes per row.
 // (Straight from the fragments those accesses are 2 and 4 bytes wide: us, accumulating, from fragments / by rows: 16384 x 1024 x 1024
 // BF16 103 / 48, FP32 122 / 51; 4096^3 FP32 172 / 103; 16384 x 200 x 1024 BF16 58 / 19; 256 x 512 x 512 FP32 20.8 / 8.0.)
-__device__ __forceinline__ void b128_store64(const Params& p, const CUtensorMap& tmC, uint32_t stage, int lane, int64_t m0, int64_t n0,
-                                             const float2 (&acc)[2][2][8]) {
+template <int CW>
+__device__ __forceinline__ void b128_store(const Params& p, const CUtensorMap& tmC, uint32_t stage, int lane, int64_t m0, int64_t n0,
+                                           const float2 (&acc)[2][2][CW / 8]) {
   const int lr = lane >> 2, lc = lane & 3;
-  const bool whole = n0 + 64 <= p.N && !p.accumulate;
+  const bool whole = n0 + CW <= p.N && !p.accumulate && (CW == 64 || p.c_is_f32);  // (32 BF16 columns are half of a bulk store)
   if (p.c_is_f32 || !whole) {
 #pragma unroll
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < CW / 32; ++b) {
       const int64_t nb = n0 + 32 * b;
       if (nb >= p.N) break;
       auto stage_rows = [&]() {
@@ -666,7 +683,7 @@ __device__ __forceinline__ void b128_store64(const Params& p, const CUtensorMap&
         bulk_commit();
       }
     }
-  } else {
+  } else if constexpr (CW == 64) {
     if (lane == 0) bulk_wait_read<0>();
     __syncwarp();
 #pragma unroll
@@ -695,24 +712,25 @@ __device__ __forceinline__ void b128_store64(const Params& p, const CUtensorMap&
   }
 }
 
-__global__ void __launch_bounds__(B128_THREADS, 1)
+template <int TN>
+__global__ void __launch_bounds__(B128<TN>::THREADS, 1)
 gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                            const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmAh,
                            const __grid_constant__ CUtensorMap tmBh, const Params p) {
-  constexpr int STAGES = B128_STAGES, SLOTS = B128_SC_SLOTS, TN = B128_TN;
+  using C = B128<TN>;
+  constexpr int STAGES = C::STAGES, SLOTS = C::SC_SLOTS;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t staging_base = smem_base + STAGES * B128_STAGE_BYTES;  // 1024-byte aligned
-  const uint32_t scale_base = staging_base + B128_STAGING_BYTES;
-  const uint32_t bar_base = scale_base + SLOTS * B128_SC_BYTES;
+  const uint32_t staging_base = smem_base + STAGES * C::STAGE_BYTES;  // 1024-byte aligned
+  const uint32_t scale_base = staging_base + C::STAGING_BYTES;
+  const uint32_t bar_base = scale_base + SLOTS * C::SC_BYTES;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
   auto part_full_bar = [&](int b) { return bar_base + 8u * (2 * STAGES + b); };
-  auto part_empty_bar = [&](int b) { return bar_base + 8u * (2 * STAGES + B128_NBUF + b); };
-  auto sc_full_bar = [&](int s) { return bar_base + 8u * (2 * STAGES + 2 * B128_NBUF + s); };
-  auto sc_empty_bar = [&](int s) { return bar_base + 8u * (2 * STAGES + 2 * B128_NBUF + SLOTS + s); };
-  const uint32_t drain_bar = bar_base + 8u * (2 * STAGES + 2 * B128_NBUF + 2 * SLOTS);
-  static_assert(8 * (2 * B128_STAGES + 2 * B128_NBUF + 2 * B128_SC_SLOTS + 1) <= 256, "barrier space");
+  auto part_empty_bar = [&](int b) { return bar_base + 8u * (2 * STAGES + C::NBUF + b); };
+  auto sc_full_bar = [&](int s) { return bar_base + 8u * (2 * STAGES + 2 * C::NBUF + s); };
+  auto sc_empty_bar = [&](int s) { return bar_base + 8u * (2 * STAGES + 2 * C::NBUF + SLOTS + s); };
+  const uint32_t drain_bar = bar_base + 8u * (2 * STAGES + 2 * C::NBUF + 2 * SLOTS);
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag_s;
   volatile int* abort_flag = &abort_flag_s;
@@ -724,13 +742,13 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
     }
-    for (int b = 0; b < B128_NBUF; ++b) {
+    for (int b = 0; b < C::NBUF; ++b) {
       mbar_init(part_full_bar(b), 1);
-      mbar_init(part_empty_bar(b), B128_PROMO_WARPS);
+      mbar_init(part_empty_bar(b), C::PROMO_WARPS);
     }
     for (int s = 0; s < SLOTS; ++s) {
       mbar_init(sc_full_bar(s), 2);
-      mbar_init(sc_empty_bar(s), B128_PROMO_WARPS);
+      mbar_init(sc_empty_bar(s), C::PROMO_WARPS);
     }
     mbar_init(drain_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -749,7 +767,7 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
   const int32_t chunks = p.k_chunks;  // 128-wide k chunks per tile
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");  // 128 x 80 + 384 x 144 = 512 x 128 registers
+    if (TN == 192) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");  // 128 x 80 + 384 x 144 = 512 x 128 registers
     if (warp == 0) {
       // ===================================== TMA producer =====================================================
       const uint32_t leader = elect_leader();
@@ -765,20 +783,20 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
         for (int32_t kt = 0; kt < p.k_tiles; ++kt, ++it, s = (s + 1 == (uint32_t)STAGES ? 0u : s + 1), wait_parity ^= (s == 0)) {
           ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty_bar(s), wait_parity, abort_flag, p.dev_status, p.wait_limit));
           if (!ok) break;
-          const uint32_t st = smem_base + s * B128_STAGE_BYTES;
-          mbar_expect_tx(full_bar(s), B128_STAGE_BYTES, leader);
+          const uint32_t st = smem_base + s * C::STAGE_BYTES;
+          mbar_expect_tx(full_bar(s), C::STAGE_BYTES, leader);
           tma_load_2d(st, &tmA, kt * (BK / 2), mt * BM, full_bar(s), leader);
           tma_load_2d(st + A_BYTES, &tmB, kt * (BK / 2), nt * TN, full_bar(s), leader);
-          bulk_load(st + A_BYTES + B128_B_BYTES, sfa_src + (size_t)kt * 2048, 2048, full_bar(s), leader);
-          bulk_load(st + A_BYTES + B128_B_BYTES + SFA_BYTES, sfb_src + (size_t)kt * 2048, 2048, full_bar(s), leader);
-          bulk_load(st + A_BYTES + B128_B_BYTES + SFA_BYTES + 2048, sfb_src1 + (size_t)kt * 2048, 2048, full_bar(s), leader);
+          bulk_load(st + A_BYTES + C::B_BYTES, sfa_src + (size_t)kt * 2048, 2048, full_bar(s), leader);
+          bulk_load(st + A_BYTES + C::B_BYTES + SFA_BYTES, sfb_src + (size_t)kt * 2048, 2048, full_bar(s), leader);
+          if (C::SF_TILES == 2) bulk_load(st + A_BYTES + C::B_BYTES + SFA_BYTES + 2048, sfb_src1 + (size_t)kt * 2048, 2048, full_bar(s), leader);
         }
         // OutControl: the BF16 outlier channels of both operands, 64 per stage, into the same stage buffers
         for (int32_t h = 0; h < p.hp_k_tiles && ok; ++h, ++it, s = (s + 1 == (uint32_t)STAGES ? 0u : s + 1), wait_parity ^= (s == 0)) {
           ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty_bar(s), wait_parity, abort_flag, p.dev_status, p.wait_limit));
           if (!ok) break;
-          const uint32_t st = smem_base + s * B128_STAGE_BYTES;
-          mbar_expect_tx(full_bar(s), A_BYTES + B128_B_BYTES, leader);
+          const uint32_t st = smem_base + s * C::STAGE_BYTES;
+          mbar_expect_tx(full_bar(s), A_BYTES + C::B_BYTES, leader);
           tma_load_2d(st, &tmAh, h * 64, mt * BM, full_bar(s), leader);
           tma_load_2d(st + A_BYTES, &tmBh, h * 64, nt * TN, full_bar(s), leader);
         }
@@ -803,7 +821,7 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
         tc_fence_after();
       };
       auto next_buffer = [&]() {
-        buf = buf + 1 == (uint32_t)B128_NBUF ? 0u : buf + 1;
+        buf = buf + 1 == (uint32_t)C::NBUF ? 0u : buf + 1;
         buf_parity ^= (buf == 0);
       };
       auto take_stage = [&]() {
@@ -821,13 +839,13 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
         for (int32_t kt = 0; kt < p.k_tiles && ok; ++kt, ++it) {
           take_stage();
           if (!ok) break;
-          const uint32_t st = smem_base + stage * B128_STAGE_BYTES;
-          const uint32_t sf_tmem = tmem_base + B128_NBUF * TN + (it % B128_SF_SETS) * B128_SF_COLS;
+          const uint32_t st = smem_base + stage * C::STAGE_BYTES;
+          const uint32_t sf_tmem = tmem_base + C::NBUF * TN + (it % C::SF_SETS) * C::SF_COLS;
 #pragma unroll
           for (int kk = 0; kk < BK / 64; ++kk) {
-            tc_cp_sf(sf_tmem + kk * 4, desc_sf(st + A_BYTES + B128_B_BYTES + kk * 512), leader);
-            tc_cp_sf(sf_tmem + 16 + kk * 8, desc_sf(st + A_BYTES + B128_B_BYTES + SFA_BYTES + kk * 512), leader);
-            tc_cp_sf(sf_tmem + 20 + kk * 8, desc_sf(st + A_BYTES + B128_B_BYTES + SFA_BYTES + 2048 + kk * 512), leader);
+            tc_cp_sf(sf_tmem + kk * 4, desc_sf(st + A_BYTES + C::B_BYTES + kk * 512), leader);
+            tc_cp_sf(sf_tmem + 16 + kk * 4 * C::SF_TILES, desc_sf(st + A_BYTES + C::B_BYTES + SFA_BYTES + kk * 512), leader);
+            if (C::SF_TILES == 2) tc_cp_sf(sf_tmem + 20 + kk * 8, desc_sf(st + A_BYTES + C::B_BYTES + SFA_BYTES + 2048 + kk * 512), leader);
           }
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
@@ -838,7 +856,7 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
             for (int q = 0; q < 2; ++q) {
               const int kk = 2 * half + q;
               tc_mma_nvf4(tmem_base + buf * TN, desc_sw128(st + kk * 32), desc_sw128(st + A_BYTES + kk * 32), idesc, sf_tmem + kk * 4,
-                          sf_tmem + 16 + kk * 8 + sfb_col, q, leader);
+                          sf_tmem + 16 + kk * 4 * C::SF_TILES + sfb_col, q, leader);
             }
             tc_commit(part_full_bar(buf), leader);
             next_buffer();
@@ -854,7 +872,7 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
           for (int32_t h = 0; h < p.hp_k_tiles; ++h) {
             take_stage();
             if (!ok) break;
-            const uint32_t st = smem_base + stage * B128_STAGE_BYTES;
+            const uint32_t st = smem_base + stage * C::STAGE_BYTES;
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)  // 64 BF16 = one 128-byte swizzle row = four K = 16 steps of 32 bytes
               tc_mma_bf16(tmem_base + buf * TN, desc_sw128(st + kk * 32), desc_sw128(st + A_BYTES + kk * 32), idesc_bf16, (h | kk) != 0, leader);
@@ -876,7 +894,7 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
       // Ring slots of four chunks: per chunk SgA, then SgB. Within 32 rows of A, row r sits at (r & 7) * 4 + (r >> 3): the four rows
       // of a thread's fragments (lane / 4 + 0, 8, 16, 24) are neighbours. Within 32 columns of B, column n sits at its bits
       // reordered n4 n2 n1 n3 n0: four of a thread's columns (8 i + 2 (lane % 4) + {0, 1} for an even i and i + 1) are neighbours.
-      // A lane reads four chunks of its five rows at once, a slot ahead (the rows lie 4 G bytes apart: a load per chunk, or an
+      // A lane reads four chunks of its (at 192 columns five) rows at once, a slot ahead (the rows lie 4 G bytes apart: a load per chunk, or an
       // asynchronous 4-byte copy, is 32 sectors for 128 bytes, and the barriers and reads of the promotion warps queue behind
       // them: 16384 x 8192 x 8192 took 1454 us with such copies).
       constexpr int ROWS = (128 + TN) / 64;  // per lane and warp
@@ -906,14 +924,14 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
         for (int32_t j = 0; j < slots_per_tile; ++j, slot = (slot + 1 == (uint32_t)SLOTS ? 0u : slot + 1), wait_parity ^= (slot == 0)) {
           ok = __all_sync(0xFFFFFFFFu, mbar_wait(sc_empty_bar(slot), wait_parity, abort_flag, p.dev_status, p.wait_limit));
           if (!ok) break;
-          const uint32_t dst = scale_base + slot * B128_SC_BYTES;
+          const uint32_t dst = scale_base + slot * C::SC_BYTES;
 #pragma unroll
           for (int i = 0; i < ROWS; ++i) {
             const int q = (warp - 2) * ROWS + i;
             const uint32_t d = dst + q * 128 + (q < 4 ? at_a : at_b);
             const float f[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
 #pragma unroll
-            for (int c = 0; c < 4; ++c) asm volatile("st.shared.f32 [%0], %1;" ::"r"(d + c * B128_SC_CHUNK), "f"(f[c]) : "memory");
+            for (int c = 0; c < 4; ++c) asm volatile("st.shared.f32 [%0], %1;" ::"r"(d + c * C::SC_CHUNK), "f"(f[c]) : "memory");
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(sc_full_bar(slot));
@@ -923,62 +941,83 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
     }
   } else {
     // ===================================== promotion and epilogue ===============================================
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
-    const int quad = warp & 3, third = (warp - 4) >> 2;  // 32 rows, 64 columns
+    if (TN == 192) asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
+    constexpr int CW = C::CW, NG = CW / 8;
+    const int quad = warp & 3, part = (warp - 4) >> 2;  // 32 rows, CW columns
     const int lr = lane >> 2, lc = lane & 3;
-    const uint32_t my_part = tmem_base + ((uint32_t)(quad * 32) << 16) + third * 64;
+    const uint32_t my_part = tmem_base + ((uint32_t)(quad * 32) << 16) + part * CW;
     const uint32_t my_stage = staging_base + (uint32_t)(warp - 4) * 4096u;
     const uint32_t my_sa = scale_base + (uint32_t)(quad * 32 + lr * 4) * 4u;
-    const uint32_t my_sb = scale_base + 512u + (uint32_t)(third * 64 + lc * 4) * 4u;
+    const uint32_t my_sb = scale_base + 512u + (uint32_t)(part * CW + lc * 4) * 4u;
     uint32_t slot = 0, slot_parity = 0, buf = 0, buf_parity = 0;
     bool ok = true;
-    float2 acc[2][2][8];  // [16-row half][8-row half][8-column group]
+    float2 acc[2][2][NG];  // [16-row half][8-row half][8-column group]
     // one partial: acc += SgA[row] SgB[column] partial. The scales are read under the first tensor-memory load.
     auto promote = [&](uint32_t sc, bool scaled) {
       ok = __all_sync(0xFFFFFFFFu, mbar_wait(part_full_bar(buf), buf_parity, abort_flag, p.dev_status, p.wait_limit));
       if (!ok) return;
       tc_fence_after();
-      float4 sa4 = make_float4(1.0f, 1.0f, 1.0f, 1.0f), sb4[4] = {sa4, sa4, sa4, sa4};
+      float4 sa4 = make_float4(1.0f, 1.0f, 1.0f, 1.0f), sb4[NG / 2];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {  // 16 rows
-        uint32_t v[32];
-        tc_ld_16x256b_x8(my_part + buf * TN + ((uint32_t)(16 * h) << 16), v);
-        if (h == 0 && scaled) {
-          sa4 = lds128(my_sa + sc);
+      for (int j = 0; j < NG / 2; ++j) sb4[j] = sa4;
+      auto scales = [&]() {
+        if (!scaled) return;
+        sa4 = lds128(my_sa + sc);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) sb4[j] = lds128(my_sb + sc + j * 64u);
-        }
-        tc_wait_ld();
-        if (h == 1) {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(part_empty_bar(buf));
-        }
+        for (int j = 0; j < NG / 2; ++j) sb4[j] = lds128(my_sb + sc + j * 64u);
+      };
+      auto give_back = [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(part_empty_bar(buf));
+      };
+      auto add = [&](int h, const uint32_t(&v)[4 * NG]) {  // 16 rows
         const float2 s0 = h ? make_float2(sa4.z, sa4.z) : make_float2(sa4.x, sa4.x);
         const float2 s1 = h ? make_float2(sa4.w, sa4.w) : make_float2(sa4.y, sa4.y);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < NG; ++i) {
           const float2 sb = (i & 1) ? make_float2(sb4[i >> 1].z, sb4[i >> 1].w) : make_float2(sb4[i >> 1].x, sb4[i >> 1].y);
           const float2 x0 = __fmul2_rn(make_float2(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1])), s0);
           const float2 x1 = __fmul2_rn(make_float2(__uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3])), s1);
           acc[h][0][i] = __ffma2_rn(x0, sb, acc[h][0][i]);
           acc[h][1][i] = __ffma2_rn(x1, sb, acc[h][1][i]);
         }
+      };
+      const uint32_t src = my_part + buf * TN;
+      if constexpr (CW == 32) {  // both halves on their way at once
+        uint32_t v0[16], v1[16];
+        tc_ld_16x256b_x4(src, v0);
+        tc_ld_16x256b_x4(src + (16u << 16), v1);
+        scales();
+        tc_wait_ld();
+        give_back();
+        add(0, v0);
+        add(1, v1);
+      } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t v[32];
+          tc_ld_16x256b_x8(src + ((uint32_t)(16 * h) << 16), v);
+          if (h == 0) scales();
+          tc_wait_ld();
+          if (h == 1) give_back();
+          add(h, v);
+        }
       }
-      buf = buf + 1 == (uint32_t)B128_NBUF ? 0u : buf + 1;
+      buf = buf + 1 == (uint32_t)C::NBUF ? 0u : buf + 1;
       buf_parity ^= (buf == 0);
     };
     for (TileWalk t((uint32_t)blockIdx.x, (uint32_t)gridDim.x, (uint32_t)p.n_tiles); t.index < num_tiles && ok; t.next()) {
       const int32_t mt = (int32_t)t.m, nt = (int32_t)t.n;
 #pragma unroll
-      for (int j = 0; j < 32; ++j) acc[j >> 4][(j >> 3) & 1][j & 7] = make_float2(0.0f, 0.0f);
+      for (int j = 0; j < 4 * NG; ++j) acc[j / (2 * NG)][(j / NG) & 1][j % NG] = make_float2(0.0f, 0.0f);
       for (int32_t kc = 0; kc < chunks; kc += 4) {
         ok = __all_sync(0xFFFFFFFFu, mbar_wait(sc_full_bar(slot), slot_parity, abort_flag, p.dev_status, p.wait_limit));
         if (!ok) break;
-        const uint32_t sc = slot * B128_SC_BYTES;
+        const uint32_t sc = slot * C::SC_BYTES;
 #pragma unroll 1
         for (int c = 0; c < 4 && kc + c < chunks; ++c) {
-          promote(sc + c * B128_SC_CHUNK, true);
+          promote(sc + c * C::SC_CHUNK, true);
           if (!ok) break;
         }
         if (!ok) break;
@@ -992,8 +1031,8 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
         promote(0, false);
         if (!ok) break;
       }
-      const int64_t m0 = (int64_t)mt * BM + quad * 32, n0 = (int64_t)nt * TN + third * 64;
-      if (m0 < p.M && n0 < p.N) b128_store64(p, tmC, my_stage, lane, m0, n0, acc);
+      const int64_t m0 = (int64_t)mt * BM + quad * 32, n0 = (int64_t)nt * TN + part * CW;
+      if (m0 < p.M && n0 < p.N) b128_store<CW>(p, tmC, my_stage, lane, m0, n0, acc);
     }
     if (lane == 0) bulk_wait_all();  // this lane's bulk stores are complete before the CTA may exit
   }
@@ -1642,15 +1681,16 @@ cudaError_t launch_2cta(const GemmArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_block128(const GemmArgs& a, cudaStream_t st) {
+template <int TN>
+cudaError_t launch_block128_tn(const GemmArgs& a, cudaStream_t st) {
   const int64_t Kp = (a.K + 127) & ~(int64_t)127;
   if (Kp > B128_MAX_K) return cudaErrorInvalidValue;
   CUtensorMap tmA, tmB, tmC;
-  if (!make_codes_map(&tmA, a.a_codes, a.M, Kp, BM) || !make_codes_map(&tmB, a.b_codes, a.N, Kp, B128_TN)) return cudaErrorInvalidValue;
+  if (!make_codes_map(&tmA, a.a_codes, a.M, Kp, BM) || !make_codes_map(&tmB, a.b_codes, a.N, Kp, TN)) return cudaErrorInvalidValue;
   Params p{};
   CUtensorMap tmAh = tmA, tmBh = tmB;  // placeholders unless the high-precision side product is requested
   if (a.hp_Kh > 0) {
-    if (!make_hp_map(&tmAh, a.hp_a, a.M, a.hp_Kh) || !make_hp_map(&tmBh, a.hp_b, a.N, a.hp_Kh, B128_TN)) return cudaErrorInvalidValue;
+    if (!make_hp_map(&tmAh, a.hp_a, a.M, a.hp_Kh) || !make_hp_map(&tmBh, a.hp_b, a.N, a.hp_Kh, TN)) return cudaErrorInvalidValue;
     p.hp_k_tiles = (int32_t)(a.hp_Kh / 64);
   }
   if (!make_c_map(&tmC, a.C, a.M, a.N, a.ldc, a.c_is_f32 != 0)) return cudaErrorInvalidValue;
@@ -1668,17 +1708,38 @@ cudaError_t launch_block128(const GemmArgs& a, cudaStream_t st) {
   const int64_t kb_padded = ((Kp >> 4) + 15) & ~(int64_t)15;
   p.sf_tiles_a = p.sf_tiles_b = (int32_t)(kb_padded >> 2);
   p.m_tiles = (int32_t)((a.M + BM - 1) / BM);
-  p.n_tiles = (int32_t)((a.N + B128_TN - 1) / B128_TN);
+  p.n_tiles = (int32_t)((a.N + TN - 1) / TN);
   p.c_is_f32 = a.c_is_f32;
   p.accumulate = a.accumulate;
   p.dev_status = a.dev_status;
   p.wait_limit = wait_limit_of(a);
-  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_nvfp4_block128_kernel), B128_SMEM_BYTES);
+  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_nvfp4_block128_kernel<TN>), B128<TN>::SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const int64_t tiles = (int64_t)p.m_tiles * p.n_tiles;
   const unsigned grid = (unsigned)std::min<int64_t>(tiles, sm_count());
-  launch_kernel(gemm_nvfp4_block128_kernel, dim3(grid), dim3(B128_THREADS), B128_SMEM_BYTES, st, tmA, tmB, tmC, tmAh, tmBh, p);
+  launch_kernel(gemm_nvfp4_block128_kernel<TN>, dim3(grid), dim3(B128<TN>::THREADS), B128<TN>::SMEM_BYTES, st, tmA, tmB, tmC, tmAh, tmBh, p);
   return cudaGetLastError();
+}
+
+// Tile width by a cost model: rounds of the tiles over the SMs x time of a tile, which is a constant (its store, mostly) and so much per
+// 128-wide chunk of K. Wide tiles cost the least per column; narrow ones leave fewer SMs idle where a product has few tiles (a weight
+// gradient: few tiles, K = tokens). us, 192 / 128 / 64 columns: 1024 x 1024 x 8192 31.0 / 24.0 / 16.5 (27.4 with the 128-column tiles of
+// one promotion warp per scheduler), 512 x 512 x 4096 17.3 / 13.4 / 9.8 (15.1), 4096 x 1024 x 3072 25.6 / 20.0 / 26.4 (22.7),
+// 16384 x 1024 x 2816 68.5 / 62.7 / 89.6, 2816 x 1024 x 8192 31.4 / 45.0 / 43.2, 8192 x 3072 x 1024 31.9 / 35.8 / 60.1 (FP32 40.0 / 43.9 /
+// 45.9), 4096^3 85.0 / 90.8 / 124.
+int block128_tile_cols(int64_t M, int64_t N, int64_t K, bool c_is_f32) {
+  const double chunks = (double)((K + 127) / 128);
+  auto cost = [&](int tn, double fixed, double per_chunk) {
+    const int64_t tiles = ((M + BM - 1) / BM) * ((N + tn - 1) / tn), sms = sm_count();
+    return (double)((tiles + sms - 1) / sms) * (fixed + per_chunk * chunks);
+  };
+  const double c192 = cost(192, c_is_f32 ? 1.9 : 0.8, 0.415), c128 = cost(128, c_is_f32 ? 1.2 : 0.48, 0.32), c64 = cost(64, c_is_f32 ? 0.5 : 1.1, 0.195);
+  return c192 <= c128 && c192 <= c64 ? 192 : c128 <= c64 ? 128 : 64;
+}
+
+cudaError_t launch_block128(const GemmArgs& a, cudaStream_t st) {
+  const int tn = block128_tile_cols(a.M, a.N, a.K, a.c_is_f32 != 0);
+  return tn == 192 ? launch_block128_tn<192>(a, st) : tn == 128 ? launch_block128_tn<128>(a, st) : launch_block128_tn<64>(a, st);
 }
 
 // BF16 matrix [T, W] (leading dimension ld elements) as a 2-D tensor; box = 64 columns x 64 rows, 128-byte swizzle.

@@ -1,6 +1,6 @@
-"""The product with 1x128 outer scales at the sizes where its kernel can go wrong: edges of the 128 x 192 tile, tiles that start in the
-middle of a 128-row scale tile, numbers of 128-k chunks around the groups of four (and rows of scales that cannot be read in 16- or
-8-byte pieces), several tiles per CTA."""
+"""The product with 1x128 outer scales at the sizes where its kernel can go wrong: edges of the 128 x 192, 128 and 64 tiles, tiles that
+start in the middle of a 128-row scale tile, numbers of 128-k chunks around the groups of four (and rows of scales that cannot be read
+in 16- or 8-byte pieces), several tiles per CTA."""
 import pytest
 import torch
 
@@ -51,3 +51,25 @@ def test_product(M, N, K, c_dtype, accumulate):
     # result: typical errors add in quadrature, sqrt(130 + G) 2^-24 sqrt(2) < 1.5e-6 of the norm. BF16 adds 2^-9.
     err = ((out.double() - want).norm() / want.norm()).item()
     assert err <= (3e-6 if c_dtype else 2.0**-9 + 3e-6), err
+
+
+# the wide tiles, which products of few tiles do not take: 192 columns (whole and ragged last ones, starting in the middle of a scale
+# tile; three chunks, five) and 128 (whole, ragged; eight chunks, three), in several rounds over the SMs
+@pytest.mark.parametrize("M,N,K", [(2820, 1000, 392), (2700, 1152, 640), (2049, 1345, 136), (3000, 1160, 904), (9000, 1000, 304), (16400, 1024, 1000)])
+@pytest.mark.parametrize("c_dtype", [0, 1])
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_product_of_many_tiles(M, N, K, c_dtype, accumulate):
+    test_product(M, N, K, c_dtype, accumulate)
+
+
+@pytest.mark.parametrize("T,D,C", [(200, 264, 136), (2820, 384, 1000), (3000, 1000, 1160)])  # tiles of 64, 192 and 128 columns
+def test_outlier_channels_ride_along(T, D, C):
+    """The BF16 side product as one more partial: against the operands' product and X_out W_out^T in 64 bits."""
+    b = B()
+    g = torch.Generator(device="cuda").manual_seed(T)
+    x, w = torch.randn(T, D, generator=g, device="cuda").bfloat16(), (torch.randn(C, D, generator=g, device="cuda") * 0.02).bfloat16()
+    outl = list(range(3, D, 11))
+    cfg = b.LayerConfig(gs_mode=b.GS_BLOCK128, outliers=outl, y_dtype=b.DT_F32)
+    y, saved = b.nvfp4_linear_fwd(x, w, cfg)
+    want = dequantize(saved.qx) @ dequantize(saved.qw).T + x[:, outl].double() @ w[:, outl].double().T
+    assert ((y.double() - want).norm() / want.norm()).item() <= 3e-6  # (as above; the side product is one partial more)
