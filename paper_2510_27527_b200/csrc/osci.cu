@@ -117,19 +117,20 @@ constexpr int kOsciWords = 32;
 __device__ __forceinline__ float amax4(float m, const float4& v) {
   return fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
 }
-// max |w| of columns lane * 4, lane * 4 + 128, ... of a row
-__device__ __forceinline__ float amax_row(const float* __restrict__ p, int64_t D, bool vec, int lane, float m) {
-  int64_t c = lane * 4;
+// thread t's share of a row's max |w| among n threads: columns 4 t, 4 (t + n), ...
+__device__ __forceinline__ float amax_row(const float* __restrict__ p, int64_t D, bool vec, int t, int n, float m) {
+  const int64_t step = 4 * n;
+  int64_t c = 4 * t;
   if (vec) {
-    for (; c + 384 + 4 <= D; c += 512) {  // four 16-byte loads in flight
+    for (; c + 3 * step + 4 <= D; c += 4 * step) {  // four 16-byte loads in flight
       float4 v[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] = *reinterpret_cast<const float4*>(p + c + 128 * i);
+      for (int i = 0; i < 4; ++i) v[i] = *reinterpret_cast<const float4*>(p + c + i * step);
 #pragma unroll
       for (int i = 0; i < 4; ++i) m = amax4(m, v[i]);
     }
   }
-  for (; c < D; c += 128) {
+  for (; c < D; c += step) {
     if (vec && c + 4 <= D)
       m = amax4(m, *reinterpret_cast<const float4*>(p + c));
     else
@@ -160,21 +161,30 @@ __global__ void __launch_bounds__(512) amax_f32_kernel(const float* __restrict__
     for (; i < n; i += step) m = amax4(m, p[i]);
   } else {  // a warp per row
     for (int64_t r = (int64_t)blockIdx.x * 16 + (threadIdx.x >> 5); r < C; r += (int64_t)gridDim.x * 16)
-      m = amax_row(W + r * ld, D, (ld & 3) == 0, threadIdx.x & 31, m);
+      m = amax_row(W + r * ld, D, (ld & 3) == 0, threadIdx.x & 31, 32, m);
   }
   cells_write<kOsciWords>(__float_as_uint(m), cells + blockIdx.y * kOsciWords, blockIdx.x, gridDim.x);
 }
 
-// max |w| of every row of one or two matrices, a warp per row: cells[r], cells[C + r].
-__global__ void __launch_bounds__(256) amax_rows_f32_kernel(const float* __restrict__ W0, int64_t ld0, const float* __restrict__ W1,
-                                                           int64_t ld1, int64_t C, int64_t D, uint32_t* cells) {
+// max |w| of every row of one or two matrices: cells[r], cells[C + r]. A warp per row, or a CTA where rows are long and few. us, the
+// statistics step of rows in ROW mode, warp / CTA per row: 3 x 100000 64.7 / 8.3, 40 x 40000 34.8 / 11.6, 300 x 5000 15.2 / 11.9.
+template <bool CTA_PER_ROW>
+__global__ void __launch_bounds__(CTA_PER_ROW ? 1024 : 256) amax_rows_f32_kernel(const float* __restrict__ W0, int64_t ld0, const float* __restrict__ W1,
+                                                                                int64_t ld1, int64_t C, int64_t D, uint32_t* cells) {
   pdl_wait();
   pdl_launch_next();  // (its loads of the weights run under this kernel)
-  const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), ld = blockIdx.y ? ld1 : ld0;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t r = CTA_PER_ROW ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * 8 + wid, ld = blockIdx.y ? ld1 : ld0;
   if (r >= C) return;
-  const float m = amax_row((blockIdx.y ? W1 : W0) + r * ld, D, (ld & 3) == 0, lane, 0.0f);
-  const uint32_t u = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));
+  const float m = amax_row((blockIdx.y ? W1 : W0) + r * ld, D, (ld & 3) == 0, CTA_PER_ROW ? threadIdx.x : lane, CTA_PER_ROW ? blockDim.x : 32, 0.0f);
+  uint32_t u = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));
+  if (CTA_PER_ROW) {
+    __shared__ uint32_t warp_max[32];
+    if (lane == 0) warp_max[wid] = u;
+    __syncthreads();
+    if (wid != 0) return;
+    u = __reduce_max_sync(0xFFFFFFFFu, lane < (int)(blockDim.x >> 5) ? warp_max[lane] : 0u);
+  }
   if (lane == 0) cells[blockIdx.y * C + r] = u;
 }
 
@@ -659,8 +669,10 @@ bool bad_f32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0
 cudaError_t run_amax(const float* W0, int64_t ld0, const float* W1, int64_t ld1, int64_t C, int64_t D, uint32_t* cells, int per_row,
                      cudaStream_t st) {
   const unsigned n = W1 ? 2 : 1;
-  if (per_row) {
-    launch_kernel(amax_rows_f32_kernel, dim3((unsigned)((C + 7) / 8), n), dim3(256), 0, st, W0, ld0, W1, ld1, C, D, cells);
+  if (per_row && D > 1024 && C < 16 * (int64_t)device_sm_count()) {  // a warp per row would leave warps idle that eight loads per lane need
+    launch_kernel(amax_rows_f32_kernel<true>, dim3((unsigned)C, n), dim3(D > 16384 ? 1024 : 256), 0, st, W0, ld0, W1, ld1, C, D, cells);
+  } else if (per_row) {
+    launch_kernel(amax_rows_f32_kernel<false>, dim3((unsigned)((C + 7) / 8), n), dim3(256), 0, st, W0, ld0, W1, ld1, C, D, cells);
   } else {  // eight 16-byte loads per thread, until every SM has its share
     const AmaxGrid g = amax_grid((C * D + 16383) / 16384, kOsciWords);
     launch_kernel_cluster(amax_f32_kernel, dim3(g.ctas, n), g.cluster, dim3(512), st, W0, ld0, W1, ld1, C, D, cells);

@@ -161,3 +161,28 @@ def test_tensor_maximum_is_found_wherever_it_is(shape, pad, where):
         b.nvfp4_osci_update(dev(W, pad=pad), state, t, orc.GS_TENSOR)
     torch.cuda.synchronize()
     assert np.array_equal(bits(state.D_Q.cpu().numpy()), bits(ref.D_Q))
+
+
+# rows long enough for a CTA each (256 and 1024 threads), a warp's rows beside them, rows that cannot be read in 16-byte pieces; the
+# maximum in the last element of every row
+@pytest.mark.parametrize("shape", [(3, 1028), (5, 1025), (40, 5000), (2, 16388), (1, 40001), (9, 1024)])
+@pytest.mark.parametrize("pad", [0, 4])
+def test_row_maxima_of_long_rows(shape, pad):
+    b = B()
+    C, D = shape
+    rng = np.random.default_rng(C + D)
+    W0 = (rng.standard_normal((C, D), dtype=np.float32) * np.float32(0.02)).astype(np.float32)
+    W1 = W0 + rng.standard_normal((C, D), dtype=np.float32) * np.float32(1e-3)
+    W0[:, -1] = np.arange(1, C + 1)
+    W1[:, -1] = -np.arange(2, C + 2)
+    ref = osc.Stats((C, D))
+    state = b.alloc_osci_state(dev(W0))
+    for t, W in enumerate((W0, W1)):
+        osc.update_stats(W, ref, t, orc.GS_ROW)
+        b.nvfp4_osci_update(dev(W, pad=pad), state, t, orc.GS_ROW)
+    want, _ = osc.suppress(W1, ref, 1.0, orc.GS_ROW)
+    Wd = dev(W1, pad=pad)
+    b.nvfp4_osci_suppress(Wd, state, 1.0, orc.GS_ROW)
+    torch.cuda.synchronize()
+    assert np.array_equal(bits(state.D_Q.cpu().numpy()), bits(ref.D_Q))
+    assert np.array_equal(bits(Wd.cpu().numpy()), bits(want))
