@@ -24,6 +24,11 @@ __global__ void __launch_bounds__(256) quantize_w16_kernel(const uint16_t* __res
   const int64_t r = (int64_t)blockIdx.y * 16 + (lane & 15);
   const int64_t b = (int64_t)blockIdx.x * 16 + warp * 2 + (lane >> 4);
   const int64_t k0 = b << 4;
+  // The words of the maximum, through L1 and ahead of the block's loads: a warp has only the one block to its name, so that the reads
+  // of all warps from the same two lines of L2 were what bounded this kernel. us with the amax pass, one word / 64 from L2 / now:
+  // 16384 x 8192 151.7 / 176.4 / 151.1, 5262 x 6704 37.2 / 45.3 / 32.6, 11967 x 2424 29.0 / 39.1 / 26.9.
+  const uint32_t amax_word = max(load_ca(amax_words + lane), load_ca(amax_words + 32 + lane));
+  static_assert(kTensorAmaxWords == 64, "two words per lane");
   float x[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) x[i] = 0.0f;
@@ -47,7 +52,7 @@ __global__ void __launch_bounds__(256) quantize_w16_kernel(const uint16_t* __res
   for (int i = 0; i < 16; ++i) m = fmaxf(m, fabsf(x[i]));
 #pragma unroll
   for (int o = 1; o < 16; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));  // over the square's 16 rows
-  const float Sg = global_scale_from_amax(__uint_as_float(cells_max<kTensorAmaxWords>(amax_words)));
+  const float Sg = global_scale_from_amax(__uint_as_float(__reduce_max_sync(0xFFFFFFFFu, amax_word)));
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) gscale[0] = Sg;
   float rcp;
   const uint32_t sb = block_scale(m, Sg, rcp);
