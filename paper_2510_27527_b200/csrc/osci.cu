@@ -21,7 +21,11 @@ __device__ __forceinline__ int row_vec(const float* p, int64_t ld) {
   return (a & 31) == 0 ? 2 : (a & 15) == 0 ? 1 : 0;
 }
 // 16 floats of a row starting at column k0 (zero beyond K). A thread reads 64 bytes that no other thread needs, so the loads go
-// past L1 in whole 32-byte sectors (16-byte pieces past L1 fetch every sector twice: 8 - 10 % slower on 4096 x 4096).
+// past L1 in whole 32-byte sectors (16-byte pieces past L1 fetch every sector twice: 8 - 10 % slower on 4096 x 4096). Single floats go
+// through L1, which has the rest of the sector for the next ones (us, past L1 / through it, 1000 x 999 in BLOCK128 mode: sparse
+// statistics 15.2 / 8.5, reset 14.9 / 13.9), unless EARLY: loads before the kernel's wait, which only L2 is known to serve with what the
+// kernels before it wrote.
+template <bool EARLY = false>
 __device__ __forceinline__ void load16f(const float* __restrict__ row, int64_t k0, int64_t K, int vec, float (&v)[16]) {
   if (vec == 2 && k0 + 16 <= K) {
 #pragma unroll
@@ -34,7 +38,7 @@ __device__ __forceinline__ void load16f(const float* __restrict__ row, int64_t k
     }
   } else {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = (k0 + i < K) ? load_cg(row + k0 + i) : 0.0f;
+    for (int i = 0; i < 16; ++i) v[i] = (k0 + i < K) ? (EARLY ? load_cg(row + k0 + i) : load_ca(row + k0 + i)) : 0.0f;
   }
 }
 __device__ __forceinline__ void store16f(float* __restrict__ row, int64_t k0, int64_t K, int vec, const float (&v)[16]) {
@@ -117,24 +121,35 @@ constexpr int kOsciWords = 32;
 __device__ __forceinline__ float amax4(float m, const float4& v) {
   return fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
 }
-// thread t's share of a row's max |w| among n threads: columns 4 t, 4 (t + n), ...
+// Thread t's share of a row's max |w| among n threads: every n-th 16-byte piece, or float where rows are not aligned to them
+// (us, four floats of a piece one after another / eight apart and in flight, statistics of 999 x 2001 in TENSOR mode: 57.3 / 49.4).
 __device__ __forceinline__ float amax_row(const float* __restrict__ p, int64_t D, bool vec, int t, int n, float m) {
+  if (!vec) {
+    int64_t c = t;
+    for (; c + 7 * n < D; c += 8 * n) {  // eight loads in flight
+      float v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = p[c + i * n];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) m = fmaxf(m, fabsf(v[i]));
+    }
+    for (; c < D; c += n) m = fmaxf(m, fabsf(p[c]));
+    return m;
+  }
   const int64_t step = 4 * n;
   int64_t c = 4 * t;
-  if (vec) {
-    for (; c + 3 * step + 4 <= D; c += 4 * step) {  // four 16-byte loads in flight
-      float4 v[4];
+  for (; c + 3 * step + 4 <= D; c += 4 * step) {  // four 16-byte loads in flight
+    float4 v[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] = *reinterpret_cast<const float4*>(p + c + i * step);
+    for (int i = 0; i < 4; ++i) v[i] = *reinterpret_cast<const float4*>(p + c + i * step);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) m = amax4(m, v[i]);
-    }
+    for (int i = 0; i < 4; ++i) m = amax4(m, v[i]);
   }
   for (; c < D; c += step) {
-    if (vec && c + 4 <= D)
+    if (c + 4 <= D)
       m = amax4(m, *reinterpret_cast<const float4*>(p + c));
     else
-      for (int64_t j = c; j < min(D, c + 4); ++j) m = fmaxf(m, fabsf(p[j]));
+      for (int64_t j = c; j < D; ++j) m = fmaxf(m, fabsf(p[j]));
   }
   return m;
 }
@@ -220,11 +235,11 @@ __global__ void __launch_bounds__(256) osci_update_kernel(const float* __restric
   const int64_t k0 = active ? (gid - r * nb) << 4 : D;  // inactive lanes read nothing and still take part in shuffles
   const int vw = row_vec(W, ldw), vs = min(row_vec(Wp, D), min(row_vec(DM, D), row_vec(DQ, D)));
   float w[16], p[16];
-  load16f(W + r * ldw, k0, D, vw, w);
-  load16f(Wp + r * D, k0, D, vs, p);
+  load16f<GS != kGsBlock128>(W + r * ldw, k0, D, vw, w);
+  load16f<GS != kGsBlock128>(Wp + r * D, k0, D, vs, p);
   float a[16], aq[16];
-  load16f(DM + r * D, k0, D, vs, a);  // requested before the arithmetic
-  load16f(DQ + r * D, k0, D, vs, aq);
+  load16f<GS != kGsBlock128>(DM + r * D, k0, D, vs, a);  // requested before the arithmetic
+  load16f<GS != kGsBlock128>(DQ + r * D, k0, D, vs, aq);
   float dm[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) dm[i] = fabsf(__fsub_rn(w[i], p[i]));
@@ -260,9 +275,9 @@ __global__ void __launch_bounds__(256, 3) osci_suppress_kernel(float* __restrict
   uint32_t hits = 0;
   {
     float dm[16], dq[16];
-    load16f(W + r * ldw, k0, D, vw, w);  // all three streams are requested before any arithmetic
-    load16f(DM + r * D, k0, D, vs, dm);
-    load16f(DQ + r * D, k0, D, vs, dq);
+    load16f<GS != kGsBlock128>(W + r * ldw, k0, D, vw, w);  // all three streams are requested before any arithmetic
+    load16f<GS != kGsBlock128>(DM + r * D, k0, D, vs, dm);
+    load16f<GS != kGsBlock128>(DQ + r * D, k0, D, vs, dq);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       // NaN (0 / 0) compares false; an element whose quantized value never moved has risk 0 (or 0 / 0): no division

@@ -186,3 +186,10 @@ def test_row_maxima_of_long_rows(shape, pad):
     torch.cuda.synchronize()
     assert np.array_equal(bits(state.D_Q.cpu().numpy()), bits(ref.D_Q))
     assert np.array_equal(bits(Wd.cpu().numpy()), bits(want))
+
+
+@pytest.mark.parametrize("shape", [(37, 1027), (3, 2049)])  # rows that cannot be read in 16-byte pieces
+@pytest.mark.parametrize("gs_mode", MODES)
+def test_unaligned_rows(shape, gs_mode):
+    test_update_and_suppress_bit_exact(shape, gs_mode)
+    test_memory_efficient_statistics_bit_exact(shape, gs_mode)
