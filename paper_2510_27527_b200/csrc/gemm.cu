@@ -69,7 +69,7 @@ struct Params {
 };
 
 // The output tiles of a persistent CTA (or pair), first, first + step, ...: row and column of the tile by additions (the
-// launchers keep the number of tiles below 2^31). Two 64-bit divisions per tile in every role are what this replaces; at short K,
+// number of tiles is below 2^31: that many are 70 TB of C). Two 64-bit divisions per tile in every role are what this replaces; at short K,
 // where a tile is a few k tiles, they showed: 8192 x 3072 x 1024 on 256 x 192 tiles 16.9 -> 16.0 us, with 1x128 scales 35.7 -> 34.9.
 struct TileWalk {
   uint32_t index, m, n;
@@ -1825,7 +1825,10 @@ int64_t gemm_block128_max_k() { return B128_MAX_K; }
 // 1024 x 1024 x 16384 (FP32) 16.5 / 24.5 / 19.8. ROW: 16384 x 3072 x 1024 49.5 / 53.7 / 58.7; 16384 x 1024 x 3072 37.0 / 32.9 /
 // 38.5; 8192 x 1024 x 3072 18.6 / 16.4 / 18.4; 3072 x 1024 x 16384 (FP32) 44.2 / 40.8 / 31.7; 4096^3 33.9 / 29.8 / 29.8. Short K:
 // 13736 x 2648 x 648 27.4 / 24.6 / 28.9, 8386 x 4680 x 544 (FP32) 37.3 / 33.0 / 35.4, 7084 x 4768 x 760 25.4 / 23.3 / 24.9; ROW 6083 x
-// 6232 x 1320 (FP32) 49.7 / 43.2 / 46.2, 4768 x 2016 x 2616 (FP32) 23.6 / 21.9 / 19.8.
+// 6232 x 1320 (FP32) 49.7 / 43.2 / 46.2, 4768 x 2016 x 2616 (FP32) 23.6 / 21.9 / 19.8. Adding to the old C costs the pairs' epilogue more
+// (a lane per row reads it): 16384 x 1024 x 1024 (FP32) 29.2 / 32.3 / 41.3, 4989 x 6232 x 1000 (FP32) 78.7 / 87.8 / 92.1, ROW 3825 x 5496 x
+// 1216 37.8 / 44.4 / 46.2. Over 125 shapes of every kind the choice is 1.3 % off the fastest in the mean; single shapes, mostly those
+// whose rows of C do not start on 128-byte lines, are up to a fifth off.
 // A 256-row tile of an operand spans two 128-row scale tiles, and rows are padded to 128 in the scale layout, so any M, N
 // work. The fused high-precision side product and the outer-block scales live in the single-CTA kernels only.
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
@@ -1835,14 +1838,14 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
   const double k_tiles = (double)((a.K + BK - 1) / BK);
   const bool row_scales = a.gs_mode == kGsRow;
   auto rounds = [](int64_t tiles, int64_t units) { return (double)((tiles + units - 1) / units); };
-  // us: a tile = max(write, fixed + per_k_tile * k tiles), with TENSOR and with ROW scales
-  auto cost = [&](double n_rounds, double per_k_tile, double fixed, double fixed_row, double write, double write_row) {
-    const double w = (row_scales ? write_row : write) * (a.c_is_f32 ? 1.3 : 1.0);
+  // us: a tile = max(write, fixed + per_k_tile * k tiles), with TENSOR and with ROW scales; add: what adding to C makes of a write
+  auto cost = [&](double n_rounds, double per_k_tile, double fixed, double fixed_row, double write, double write_row, double add) {
+    const double w = (row_scales ? write_row : write) * (a.c_is_f32 ? 1.3 : 1.0) * (a.accumulate ? add : 1.0);
     return n_rounds * std::max(w, (row_scales ? fixed_row : fixed) + per_k_tile * k_tiles);
   };
-  const double cost128 = cost(rounds(((a.M + 127) / 128) * ((a.N + 127) / 128), sms), 0.2275, 0.57, 1.45, 1.40, 2.15);
-  const double cost256 = cost(rounds(rows256 * ((a.N + 255) / 256), n_pairs), 0.300, 1.16, 2.60, 2.35, 4.90);
-  const double cost192 = cost(rounds(rows256 * ((a.N + 191) / 192), n_pairs), 0.250, 0.80, 2.30, 2.15, 3.80);
+  const double cost128 = cost(rounds(((a.M + 127) / 128) * ((a.N + 127) / 128), sms), 0.2275, 0.57, 1.45, 1.40, 2.15, 1.2);
+  const double cost256 = cost(rounds(rows256 * ((a.N + 255) / 256), n_pairs), 0.300, 1.16, 2.60, 2.35, 4.90, 1.4);
+  const double cost192 = cost(rounds(rows256 * ((a.N + 191) / 192), n_pairs), 0.250, 0.80, 2.30, 2.15, 3.80, 1.4);
   bool pairs = cost256 <= cost192 && cost256 <= cost128, pairs192 = cost192 < cost256 && cost192 < cost128;
   if (a.variant == 1) pairs = pairs192 = false;
   if (a.variant == 2) { pairs = true; pairs192 = false; }
