@@ -68,9 +68,9 @@ struct Params {
   int32_t* dev_status;
 };
 
-// The output tiles of a persistent CTA (or pair), first, first + step, ...: row and column of the tile by additions (the
-// number of tiles is below 2^31: that many are 70 TB of C). Two 64-bit divisions per tile in every role are what this replaces; at short K,
-// where a tile is a few k tiles, they showed: 8192 x 3072 x 1024 on 256 x 192 tiles 16.9 -> 16.0 us, with 1x128 scales 35.7 -> 34.9.
+// The output tiles of a persistent CTA (or pair), first, first + step, ...: row and column of the tile by additions (there are
+// fewer than 2^31 tiles: that many are 70 TB of C). Two 64-bit divisions per tile in every role are what this replaces; at short K,
+// where a tile is a few k tiles, they showed: 8192 x 3072 x 1024 on 256 x 192 tiles 16.9 -> 16.0 us.
 struct TileWalk {
   uint32_t index, m, n;
   __device__ __forceinline__ TileWalk(uint32_t first, uint32_t step, uint32_t n_tiles) : index(first), step_(step), n_tiles_(n_tiles) {

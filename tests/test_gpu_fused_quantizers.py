@@ -18,9 +18,11 @@ def poison(ws):
 
 
 # one row; less than a tile; one more than a tile in every direction; k blocks that end inside a 256-wide k tile; whole tiles; the
-# first sizes past the limit of the fused backward (TENSOR: 19 CTAs per SM, BLOCK128: 6)
+# last sizes within the limit of the fused backward and the first ones past it on 148 SMs (TENSOR: 19 CTAs per SM, 2812; BLOCK128: 5,
+# 740): 3300 and 3500 x 1024 x 3072 have 2667 and 2833 CTAs (Q3 a CTA per 256 units of 64, the others per 128 x 64 tile), 1900 and
+# 2000 x 1024 x 1024 have 727 and 765
 SHAPES = [(1, 8, 8), (5, 40, 24), (127, 72, 136), (129, 136, 264), (257, 520, 392), (256, 512, 512), (384, 1032, 1288), (3000, 1024, 3072),
-          (1024, 1024, 3080)]
+          (1024, 1024, 3080), (3300, 1024, 3072), (3500, 1024, 3072), (1900, 1024, 1024), (2000, 1024, 1024)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
@@ -57,11 +59,11 @@ def test_layer_equals_separate_calls(shape, gs_mode, rht):
     assert torch.equal(dx, dx1) and torch.equal(dw, dw1)
 
 
-@pytest.mark.parametrize("rows,cols", [(1, 8), (64, 4096), (64, 4104), (65, 4096), (513, 4096), (2049, 4104)])
+@pytest.mark.parametrize("rows,cols", [(1, 8), (64, 4096), (64, 4104), (65, 4096), (513, 4096), (2049, 4104), (4200, 4104)])
 @pytest.mark.parametrize("where", [0, -1])
 @pytest.mark.parametrize("pad", [0, 8])
 def test_tensor_maximum(rows, cols, where, pad):
-    """One CTA, as many CTAs as words, clusters of eight (part idle, and as many clusters as words): the scale is the maximum's."""
+    """One CTA, as many CTAs as words, clusters of eight (part idle; 33; as many clusters as words): the scale is the maximum's."""
     b = B()
     buf = torch.zeros(rows, cols + pad, dtype=torch.bfloat16, device="cuda")
     x = buf[:, :cols]
