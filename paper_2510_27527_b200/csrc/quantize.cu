@@ -543,7 +543,7 @@ __device__ __forceinline__ void quantize_rows_body(const uint16_t* __restrict__ 
 // they are (16-byte asynchronous copies, all in flight at once), moves the kept columns together there, two per thread and row, so
 // that neighbouring threads touch neighbouring words, and quantizes the compact rows, a block per thread and step.
 // excl_out, if given, takes the columns `excluded` of the rows: the BF16 side operand, zero up to ld_excl_out.
-// Bound by instruction issue (three quarters of the slots). Picking a block's sixteen elements singly from the copied rows met in the
+// Bound by instruction issue (two thirds of the slots, with barriers between its phases). Picking a block's sixteen elements singly from the copied rows met in the
 // same banks: 8192 x 1024 without 10 % of its columns, BLOCK128, 17.9 / 10.1 us, 8192 x 2816 37 / 23, 2816 x 1024 16.0 / 5.6. Rows
 // interleaved in shared memory by 8-column pieces save address arithmetic and lose more: their copies go out 16 bytes at a time.
 // =========================================================================================================
@@ -1355,7 +1355,7 @@ quantize_transpose_kernel(TransposeSrc s, int64_t rowsK, int64_t D, uint64_t see
 // and 16 consecutive source rows (= operand k), i.e. one inner block of four operand rows. It reads 8 bytes per source row, so one
 // warp instruction covers two source rows of 128 contiguous bytes, and the 16 values of an inner block are the same half of 16
 // loaded words: the transposition is the choice of that half. It stores 8 code bytes and a scale byte to each of its four operand
-// rows. No barrier, no shared memory. Bound by instruction issue (stochastic rounding, 20 instructions per element). Lanes that
+// rows. No barrier, no shared memory. Bound by instruction issue (stochastic rounding, 23 instructions per element). Lanes that
 // took 64 source rows, whose four scale bytes are one word, paid the index arithmetic once per 256 elements, but their CTAs ran
 // 16 us each: us with the amax pass, stochastic, 64 / 16 rows per lane: 16384 x 2816 65.5 / 62.5, 8192 x 3072 38.9 / 35.0,
 // 8192 x 1024 23.7 / 14.7, 4095 x 2816 25.4 / 19.0, 1024 x 1024 10.7 / 6.9, 256 x 512 9.9 / 4.9.
