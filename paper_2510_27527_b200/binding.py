@@ -457,8 +457,7 @@ class IndexArrays(tuple):
     def here(self) -> "IndexArrays":
         """The arrays, for kernels on the current stream: given back, their memory waits for that stream too."""
         if self.streams is not None and (s := _stream_ptr()) not in self.streams:
-            for a in self:
-                a.record_stream(torch.cuda.current_stream())
+            self[0].record_stream(torch.cuda.current_stream())  # (the three are pieces of one allocation)
             self.streams.add(s)
         return self
 
@@ -483,11 +482,14 @@ class IndexCache:
             mask = np.ones(D, dtype=bool)
             mask[outl] = False
             keep = np.nonzero(mask)[0]
-            cmap = np.full(D, -1, dtype=np.int32)
-            cmap[keep] = np.arange(len(keep), dtype=np.int32)
-            held = IndexArrays(torch.from_numpy(a.astype(np.int32)).to(dev) for a in (outl, keep, cmap))
+            at = (0, (len(outl) + 3) // 4 * 4, (len(outl) + 3) // 4 * 4 + (len(keep) + 3) // 4 * 4)  # on 16-byte boundaries
+            one = np.full(at[2] + D, -1, dtype=np.int32)  # (one upload instead of three)
+            one[: len(outl)], one[at[1]: at[1] + len(keep)] = outl, keep
+            one[at[2]:][keep] = np.arange(len(keep), dtype=np.int32)
+            one = torch.from_numpy(one).to(dev)
+            held = IndexArrays(one[o: o + n] for o, n in zip(at, (len(outl), len(keep), D)))
             if dev.type == "cuda":
-                held.streams = {torch.cuda.current_stream(dev).cuda_stream}
+                held.streams = {torch._C._cuda_getCurrentRawStream(dev.index)}
         self._of[key] = held
         if len(self._of) > self.MOST:
             self._of.pop(next(iter(list(self._of))), None)  # the one used longest ago
@@ -524,7 +526,7 @@ class LayerConfig:
         dev = _device_of(device)
         if self._side is None or self._side[0] != dev:
             self._side = (dev, *_make_side(dev))
-        return self._side[1:]
+        return self._side[1:5]
 
     def prepare(self, D: int, device="cuda"):
         """Second stream and OutControl index arrays (returned; None without outlier channels) for hidden size D."""
@@ -560,7 +562,7 @@ class LayerConfig:
 
 
 def set_side(c: CLayerCfg, side: tuple) -> None:
-    c.side_stream, c.ev_fork, c.ev_join, c.ev_aux = side[0].cuda_stream, side[1].cuda_event, side[2].cuda_event, side[3].cuda_event
+    c.side_stream, c.ev_fork, c.ev_join, c.ev_aux = side[4]
 
 
 def _device_of(device) -> torch.device:
@@ -570,12 +572,12 @@ def _device_of(device) -> torch.device:
 
 
 def _make_side(dev: torch.device) -> tuple:
-    """(stream, fork, join, aux) on `dev`."""
+    """(stream, fork, join, aux, their four handles) on `dev`."""
     with torch.cuda.device(dev):
         side = (torch.cuda.Stream(device=dev), torch.cuda.Event(), torch.cuda.Event(), torch.cuda.Event())
         for ev in side[1:]:
             ev.record(side[0])  # forces creation of the underlying CUDA events (torch makes them lazily)
-    return side
+    return (*side, (side[0].cuda_stream, *(ev.cuda_event for ev in side[1:])))
 
 
 _thread = threading.local()
@@ -583,9 +585,9 @@ _THREAD_SIDES = 8
 
 
 def thread_side(dev: torch.device, stream: int) -> tuple:
-    """The calling thread's second stream and events for calls on `stream` of `dev`, made on first use. A thread enqueues its
-    calls on one stream one after another, so they can share a set: a call's waits refer to the records before them in host
-    order, and re-recording an event does not change what was already waited for. A thread holds the sets of the
+    """The calling thread's second stream and events (as _make_side gives them) for calls on `stream` of `dev`, made on first use. A
+    thread enqueues its calls on one stream one after another, so they can share a set: a call's waits refer to the records before
+    them in host order, and re-recording an event does not change what was already waited for. A thread holds the sets of the
     _THREAD_SIDES streams it used last and gives them back when it ends."""
     sides = _thread.__dict__.setdefault("sides", {})
     key = (dev.index, stream)

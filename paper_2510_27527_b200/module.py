@@ -60,7 +60,9 @@ class _Call:
     __slots__ = ("buf", "saved", "ccfg", "keeps", "concurrent", "shape", "ws_bwd")
 
     def forward(self, x: torch.Tensor, weight: torch.Tensor, cfg: B.LayerConfig, seed: int) -> torch.Tensor:
-        N_tok, D, C, dev = int(x.shape[0]), int(x.shape[1]), int(weight.shape[0]), x.device  # (under jit.trace sizes are tensors)
+        (N_tok, D), C, dev = x.shape, weight.shape[0], x.device
+        if type(N_tok) is not int:  # (under jit.trace sizes are tensors)
+            N_tok, D, C = int(N_tok), int(D), int(C)
         index = cfg.index(D, dev)
         n_out, gs = cfg.n_out, cfg.gs_mode
         offs, ws_at, ws_fwd, total, self.ws_bwd = _layout(N_tok, D, C, n_out, gs)
@@ -131,19 +133,20 @@ class NVFP4Linear(torch.nn.Module):
         NVFP4Linear._instances += 1
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
-        if x.dim() == 0 or x.shape[-1] != self.in_features:  # the library takes a narrower input with the weights' leading dimension
-            raise RuntimeError(f"NVFP4Linear: input of shape {tuple(x.shape)} for {self.in_features} input features")
-        x2d = x if x.dim() == 2 else x.reshape(-1, self.in_features)
+        shape, weight = x.shape, self.weight
+        if len(shape) == 0 or shape[-1] != self.in_features:  # the library takes a narrower input with the weights' leading dimension
+            raise RuntimeError(f"NVFP4Linear: input of shape {tuple(shape)} for {self.in_features} input features")
+        x2d = x if len(shape) == 2 else x.reshape(-1, self.in_features)
         if x2d.dtype != torch.bfloat16:
             x2d = x2d.to(torch.bfloat16)
         x2d = x2d.contiguous()
         # this layer's key of this call
         seed = call_seed(self.cfg.seed, self.layer_id, self._calls)
         self._calls += 1
-        if _needs_function(x2d, self.weight):
-            y = _NVFP4LinearFn.apply(x2d, self.weight, self.cfg, seed)
+        if _needs_function(x2d, weight):
+            y = _NVFP4LinearFn.apply(x2d, weight, self.cfg, seed)
         else:
-            y = _Call().forward(x2d, self.weight, self.cfg, seed)
+            y = _Call().forward(x2d, weight, self.cfg, seed)
         if self.bias is not None:
             y = y + self.bias
-        return y if x.dim() == 2 else y.reshape(*x.shape[:-1], self.out_features)
+        return y if len(shape) == 2 else y.reshape(*shape[:-1], self.out_features)
