@@ -307,21 +307,14 @@ __device__ __forceinline__ void hadamard16_butterflies(float (&v)[16]) {
 // ---------------------------------------------------------------------------------------------------------
 // Element rounding to E2M1 (paper Sec. 2.1). Codes: sign << 3 | magnitude index.
 // ---------------------------------------------------------------------------------------------------------
-// Stochastic rounding. For an element with 16-bit draw u the rule is
-//     round the magnitude up  iff  (u + 0.5) / 65536 < (a - q1) / (q2 - q1),   a = min(|y|, 6) in [q1, q2).
-// It is evaluated exactly with one integer multiply-add on the bits of a float z:
-//   * for a >= 1, z = a: the E2M1 cell of a is (bits >> 22) - 252 and the low 22 mantissa bits are the position inside
-//     the cell in units of 2^-22 of the cell width;
-//   * for a < 1 the cells [0, .5) and [.5, 1) are mapped onto [.5, .75) and [.75, 1) by z = 0.5 + a / 2, computed with
-//     round-up so that the low bits are ceil(position * 2^22) (an integer n is < x iff n < ceil(x); when the ceiling
-//     crosses into the next cell the true position was within 2^-24 of 1, where every draw rounds up);
-//     0.5 + a / 2 >= a exactly when a <= 1, so z = max(a, 0.5 + a / 2) picks the right branch;
-//   * adding r22 = 2^22 - 1 - ((2u + 1) << 5) = ((~u & 0xFFFF) << 6) | 0x1F to the bits carries into the cell index iff
-//     position > (2u + 1) << 5, and adding -(252 << 22) as well leaves the magnitude index 0..7 in bits 22..24 with
-//     nothing above. Both additions and a shift by 6 are one multiply-add modulo 2^32:
-//         v = bits * 64 + c6,   c6 = ((~u & 0xFFFF) << 12) | 0x7C0 | (4 << 28)      (-252 = 4 modulo 16)
-//     has the magnitude index in bits 28..30 and bit 31 clear, i.e. the code's magnitude already sits next to where the
-//     sign bit of y lives: one bit-select gives the nibble in the top four bits (e2m1x8_sr below).
+// a * c and b * c rounded to nearest / up: one packed instruction.
+__device__ __forceinline__ void mul2_rn(float a, float b, float c, float& ra, float& rb) {
+  asm("{.reg .b64 p, q;\nmov.b64 p, {%2, %3};\nmov.b64 q, {%4, %4};\nmul.rn.f32x2 p, p, q;\nmov.b64 {%0, %1}, p;}" : "=f"(ra), "=f"(rb) : "f"(a), "f"(b), "f"(c));
+}
+__device__ __forceinline__ void mul2_up(float a, float b, float c, float& ra, float& rb) {
+  asm("{.reg .b64 p, q;\nmov.b64 p, {%2, %3};\nmov.b64 q, {%4, %4};\nmul.rp.f32x2 p, p, q;\nmov.b64 {%0, %1}, p;}" : "=f"(ra), "=f"(rb) : "f"(a), "f"(b), "f"(c));
+}
+
 // Round-to-nearest (ties to the even code, saturating) of 8 scaled values, packed low nibble first.
 __device__ __forceinline__ uint32_t e2m1x8_rtn(const float (&y)[8]) {
   uint32_t out;
@@ -338,35 +331,45 @@ __device__ __forceinline__ uint32_t e2m1x8_rtn(const float (&y)[8]) {
   return out;
 }
 
-// Stochastic rounding of 8 scaled values with the draws packed in w (two 16-bit draws per word), packed low nibble
-// first. The sign bits are those of y. Elements are taken last to first: a funnel shift moves each code's four top bits
-// in below the ones already collected, so that element 0 ends in the lowest nibble.
+// Stochastic rounding. For an element with 16-bit draw u the rule is
+//     round the magnitude up  iff  (u + 0.5) / 65536 < (a - q1) / (q2 - q1),   a = min(|y|, 6) in [q1, q2).
+// It is evaluated exactly with one integer multiply-add on the bits of a float:
+//   * w = a * 2^-126, rounded up. E2M1 is spaced evenly below 1 and by binades above, as binary32 is below and above 2^-126, so the
+//     cell of a is bits(w) >> 22 (0 .. 7) everywhere, and the low 22 bits are the position inside the cell in units of 2^-22 of its
+//     width. The product is exact for a >= 1; below, it is ceil(a * 2^23) in units of 2^-149 (an integer n is < x iff n < ceil(x);
+//     when the ceiling reaches the next cell the position was within 2^-24 of its end, where every draw rounds up).
+//   * f + ((~u & 0xFFFF) << 6) + 31 reaches 2^22 iff the position f > (2u + 1) << 5. Four times that,
+//         v = 4 * bits + ((~u & 0xFFFF) << 8) + 127 = 4 * bits - c,   c = (u << 8) + 129 - 2^24,
+//     has the magnitude index of the result as its top byte, and c is the draw's two bytes between two constant ones: one byte
+//     permutation per element.
+// The codes' bytes are then collected by byte permutations, even and odd elements apart, and the signs likewise. 13.0 instructions per
+// element with the draws. An earlier form (a second mapping for a < 1, the draw brought to bits 12 .. 27 by multiply-adds, sign and
+// code moved into place element by element) took 17.3. us, 16384 x 8192, before / after: rows 114.6 / 100.1, columns 129.2 / 108.6, from
+// codes 162.5 / 141.5 (1x128 outer scales), and 16384 x 2816 with one scale and the amax pass 63.0 / 57.4, 62.7 / 58.0, 48.2 / 42.1.
+// What bounds it is the ALU pipe (16 lanes a cycle): the generator's logic operations, the permutations, the clamp, and the two cycles
+// of that pipe which each widening multiply takes beside its four of the multiply pipe. Measured and not better: packing by dp4a, the
+// generator's high halves by FP64 FMAs, its first two rounds folded.
+//
+// Stochastic rounding of 8 scaled values with the draws packed in w (two 16-bit draws per word), packed low nibble first. The
+// sign bits are those of the scaled values.
 __device__ __forceinline__ uint32_t e2m1x8_sr(const float (&y)[8], const uint4& w) {
   const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-  uint32_t out = 0, u_odd = 0;
+  uint32_t v[8];
 #pragma unroll
-  for (int e = 7; e >= 0; --e) {
-    // The draw u of element e (the even element is the low half of its word), then c6 = ((0xFFFF - u) << 12) | 0x400007C0
-    // = 0x4FFFF7C0 - u * 4096. Multiply-adds are written as such on purpose: the logic / shift / min-max pipe is the one
-    // this code saturates (half the rate of the multiply-add pipe), so shifts and adds that can be a multiply-add are one.
-    uint32_t c6, v;
-    if (e & 1) {
-      asm("mul.hi.u32 %0, %1, 65536;" : "=r"(u_odd) : "r"(ww[e >> 1]));
-      asm("mad.lo.u32 %0, %1, 0xFFFFF000, 0x4FFFF7C0;" : "=r"(c6) : "r"(u_odd));
-    } else {
-      // the even element's draw is the low half of the same word: w * -4096 = u_even * -4096 - u_odd * 2^28 (mod 2^32),
-      // so adding u_odd * 2^28 back gives its c6 without a mask (two multiply-adds instead of a logic op and one)
-      uint32_t t;
-      asm("mad.lo.u32 %0, %1, 0xFFFFF000, 0x4FFFF7C0;" : "=r"(t) : "r"(ww[e >> 1]));
-      asm("mad.lo.u32 %0, %1, 0x10000000, %2;" : "=r"(c6) : "r"(u_odd), "r"(t));
-    }
-    const float a = fminf(fabsf(y[e]), 6.0f);
-    const float z = fmaxf(a, __fmaf_ru(a, 0.5f, 0.5f));
-    asm("mad.lo.u32 %0, %1, 64, %2;" : "=r"(v) : "r"(__float_as_uint(z)), "r"(c6));
-    // code in bits 28..31 (v has the magnitude index in 28..30 and bit 31 clear); the funnel shift takes those four bits
-    out = __funnelshift_l((__float_as_uint(y[e]) & 0x80000000u) | (v & 0x7FFFFFFFu), out, 4);
+  for (int e = 0; e < 8; e += 2) {
+    float w0, w1;
+    mul2_up(fminf(fabsf(y[e]), 6.0f), fminf(fabsf(y[e + 1]), 6.0f), 0x1p-126f, w0, w1);
+    // bytes of c from the low one: 0x81, the draw's two, 0xFF
+    v[e] = __float_as_uint(w0) * 4u - __byte_perm(ww[e >> 1], 0xFF81u, 0x5104);
+    v[e + 1] = __float_as_uint(w1) * 4u - __byte_perm(ww[e >> 1], 0xFF81u, 0x5324);
   }
-  return out;
+  auto top_bytes = [](uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return __byte_perm(__byte_perm(a, b, 0x0073), __byte_perm(c, d, 0x0073), 0x5410);
+  };
+  auto bits = [&](int e) { return __float_as_uint(y[e]); };
+  const uint32_t code = top_bytes(v[0], v[2], v[4], v[6]) + top_bytes(v[1], v[3], v[5], v[7]) * 16u;
+  const uint32_t even = top_bytes(bits(0), bits(2), bits(4), bits(6)), odd = top_bytes(bits(1), bits(3), bits(5), bits(7));
+  return code | ((even >> 4) & 0x08080808u) | (odd & 0x80808080u);
 }
 
 // E2M1 code -> value, as float.
@@ -433,9 +436,9 @@ __device__ __forceinline__ uint2 quantize_block16(const float (&x)[16], float rc
                                                   uint64_t idx8) {
   float y0[8], y1[8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    y0[i] = __fmul_rn(x[i], rcp);
-    y1[i] = __fmul_rn(x[8 + i], rcp);
+  for (int i = 0; i < 8; i += 2) {
+    mul2_rn(x[i], x[i + 1], rcp, y0[i], y0[i + 1]);
+    mul2_rn(x[8 + i], x[9 + i], rcp, y1[i], y1[i + 1]);
   }
   uint2 out;
   if (SR) {

@@ -1355,7 +1355,7 @@ quantize_transpose_kernel(TransposeSrc s, int64_t rowsK, int64_t D, uint64_t see
 // and 16 consecutive source rows (= operand k), i.e. one inner block of four operand rows. It reads 8 bytes per source row, so one
 // warp instruction covers two source rows of 128 contiguous bytes, and the 16 values of an inner block are the same half of 16
 // loaded words: the transposition is the choice of that half. It stores 8 code bytes and a scale byte to each of its four operand
-// rows. No barrier, no shared memory. Bound by instruction issue (stochastic rounding, 23 instructions per element). Lanes that
+// rows. No barrier, no shared memory. Bound by instruction issue and the ALU pipe (stochastic rounding, 19 instructions per element). Lanes that
 // took 64 source rows, whose four scale bytes are one word, paid the index arithmetic once per 256 elements, but their CTAs ran
 // 16 us each: us with the amax pass, stochastic, 64 / 16 rows per lane: 16384 x 2816 65.5 / 62.5, 8192 x 3072 38.9 / 35.0,
 // 8192 x 1024 23.7 / 14.7, 4095 x 2816 25.4 / 19.0, 1024 x 1024 10.7 / 6.9, 256 x 512 9.9 / 4.9.
