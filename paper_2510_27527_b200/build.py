@@ -1,9 +1,10 @@
-"""Builds the CUDA library (sm_100a only) in-tree with nvcc: ``python -m paper_2510_27527_b200.build``."""
+"""Builds the CUDA libraries (sm_100a only, nvcc) and the autograd node (g++) in-tree: ``python -m paper_2510_27527_b200.build``."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -12,6 +13,9 @@ SOURCES = ["api.cu", "quantize.cu", "gemm.cu", "hp.cu", "noalloc.cu", "calib.cu"
 # measurement aids (the tensor-core issue loop): a library of their own, loaded by the benchmark only
 MEASURE_LIB = os.path.join(HERE, "libnvfp4_measure.so")
 MEASURE_SOURCES = ["probe.cu"]
+# the autograd node of NVFP4Linear: a Python module that calls the library (found beside it) between torch's allocator and engine
+NODE_LIB = os.path.join(HERE, "_node.so")
+NODE_SOURCES = ["torch_node.cpp"]
 HEADERS = ["nvfp4_device.cuh", "nvfp4_internal.h", "nvfp4_tc.cuh", os.path.join("..", "..", "include", "nvfp4.h"),
            os.path.join("..", "..", "include", "nvfp4_measure.h")]
 NVCC_FLAGS = [
@@ -35,10 +39,25 @@ def _compile(lib, sources, verbose):
     os.replace(tmp, lib)
 
 
+def _compile_node(lib, sources):
+    import torch
+
+    at, cuda = os.path.dirname(torch.__file__), os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = lib + f".{os.getpid()}.tmp"
+    subprocess.check_call(
+        [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+        + ["-isystem" + d for d in (f"{at}/include", f"{at}/include/torch/csrc/api/include", f"{cuda}/include", sysconfig.get_paths()["include"])]
+        + [os.path.join(CSRC, f) for f in sources] + ["-o", tmp, f"-L{at}/lib", "-ltorch", "-ltorch_cpu", "-ltorch_python", "-lc10", "-lc10_cuda",
+                                                      f"-L{cuda}/lib64", "-lcudart", f"-L{HERE}", "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, lib)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     for lib, sources in ((LIB, SOURCES), (MEASURE_LIB, MEASURE_SOURCES)):
         if force or _stale(lib, sources):
             _compile(lib, sources, verbose)
+    if force or _stale(NODE_LIB, NODE_SOURCES):
+        _compile_node(NODE_LIB, NODE_SOURCES)
     return LIB
 
 

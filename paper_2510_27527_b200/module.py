@@ -15,6 +15,11 @@ from torch.autograd import forward_ad
 
 from . import binding as B
 
+try:
+    from . import _node
+except ImportError as e:
+    raise ImportError(f"{e}: build it with `python -m paper_2510_27527_b200.build`") from e
+
 
 _MASK64 = (1 << 64) - 1
 
@@ -52,10 +57,8 @@ def _layout(N_tok: int, D: int, C: int, n_out: int, gs_mode: int):
 
 
 class _Call:
-    """One forward call and, later, its backward. The calls go to the library directly, with one buffer for everything that is
-    saved: a layer step of a few hundred tokens is bound by what the host does around its dozen kernels (fwd + bwd of a
-    512-wide layer on 256 tokens took 350 us with a tensor per saved array and a configuration object, a stream and three
-    events made per call, and takes 134 now; its kernels took 58 us then)."""
+    """One forward call and, later, its backward, through the binding: what `_node.linear` does, where it cannot go (`_plain`). Everything
+    that is saved lies in one buffer."""
 
     __slots__ = ("buf", "saved", "ccfg", "keeps", "concurrent", "shape", "ws_bwd")
 
@@ -94,11 +97,11 @@ class _Call:
         return dx, dw
 
 
-def _needs_function(x: torch.Tensor, weight: torch.Tensor) -> bool:
-    """Whether a call has to go through the autograd function: a gradient can be asked for, an input may carry a forward-mode tangent
-    (which the function refuses), or a trace is being recorded (which sees the function, but not what the library writes). (Plain
-    comparisons: unpack_dual and a generator over the two tensors took 2 us of a 32 us call.)"""
-    return (torch.is_grad_enabled() and (x.requires_grad or weight.requires_grad)) or forward_ad._current_level >= 0 or torch.jit.is_tracing()
+def _plain(x: torch.Tensor, weight: torch.Tensor) -> bool:
+    """Whether a call can go to the native node. Not while a trace is recorded or compiled (it would not see what the library writes), under
+    forward-mode differentiation or a function transform (which the autograd function refuses), or with tensor subclasses."""
+    return (type(x) is torch.Tensor and type(weight) is torch.nn.Parameter and forward_ad._current_level < 0 and not torch._C._is_tracing()
+            and not torch._C._are_functorch_transforms_active() and not torch.compiler.is_compiling())
 
 
 class _NVFP4LinearFn(torch.autograd.Function):
@@ -143,10 +146,12 @@ class NVFP4Linear(torch.nn.Module):
         # this layer's key of this call
         seed = call_seed(self.cfg.seed, self.layer_id, self._calls)
         self._calls += 1
-        if _needs_function(x2d, weight):
-            y = _NVFP4LinearFn.apply(x2d, weight, self.cfg, seed)
+        if _plain(x2d, weight):
+            cfg = self.cfg
+            index = None if cfg.outliers is None else cfg.index(self.in_features, x2d.device)
+            y = _node.linear(x2d, weight, cfg, index, seed, torch.is_grad_enabled() and (x2d.requires_grad or weight.requires_grad))
         else:
-            y = _Call().forward(x2d, weight, self.cfg, seed)
+            y = _NVFP4LinearFn.apply(x2d, weight, self.cfg, seed)
         if self.bias is not None:
             y = y + self.bias
         return y if len(shape) == 2 else y.reshape(*shape[:-1], self.out_features)
