@@ -2,6 +2,8 @@
 // product runs on the tensor cores inside the FP4 GEMM kernels and dW[:, outliers] = dY^T X_out in a BF16 tensor-core
 // kernel of its own (gemm.cu); here are the copy that builds a compact side operand, the FP8 snap of the side operands,
 // and the pass that assembles dW from the compact FP4 product and the side product's token splits.
+#include <type_traits>
+
 #include "nvfp4_device.cuh"
 #include "nvfp4_internal.h"
 
@@ -13,75 +15,83 @@ constexpr int kHpDwSplit = 16;
 
 // dW[c, d] for whole output rows (OutControl's weight gradient): a kept channel takes its value from the compact FP4
 // product, an outlier channel the sum of the high-precision side product's token splits. One coalesced pass over dW
-// instead of a column scatter plus a scattered reduce. Each CTA first builds, in shared memory, where every channel comes
-// from: src_of[d] = position in the compact product (>= 0) or -(1 + rank among the outliers). Rows are then taken four at a
-// time: all threads first reduce the splits of the group's outlier channels into shared memory (fixed order), then all
-// threads assemble and store the four rows.
+// instead of a column scatter plus a scattered reduce. A CTA takes kAsmRows rows. It builds, in shared memory, where every channel comes
+// from: src_of[d] = position in the compact product (>= 0) or -(1 + rank among the outliers); sums the splits of its outlier channels
+// there (four channels per thread, fixed order); and (STAGED) copies its rows of the compact product there as they are. All three start
+// at once and meet at one barrier, after which the rows are put together from shared memory and stored.
+// What bounds it is the latency of those loads: the rows of one CTA take a microsecond, a wave of CTAs is one or two of them. Reading the
+// compact product only once src_of is known, and the sums a channel per thread, was a second round of latency: us of a layer's backward with it,
+// before / now: 8192 x 1024 -> 2816 with 102 outlier channels 155 / 149, 8192 x 2816 -> 1024 with 282 161 / 150, 4095 x 1024 -> 2816 with
+// 102 (BF16) 82 / 77, 1000 x 9000 -> 256 with 180 (two rows per CTA) 85 / 61. More registers for more splits in flight: the same.
 constexpr int kAsmRows = 4;
-template <bool F32>
-__global__ void __launch_bounds__(256) dw_assemble_kernel(HpDwArgs a, int n_split, const float* __restrict__ compact, int64_t ld_compact,
-                                                         const int32_t* __restrict__ col_map, int64_t D, int vec) {
+template <bool F32, int ROWS, bool STAGED>
+__global__ void __launch_bounds__(256) dw_assemble_kernel(const __grid_constant__ HpDwArgs a, int n_split, int vec) {
   pdl_prologue();
-  extern __shared__ int32_t src_of[];                                       // [D]
-  float* osum = reinterpret_cast<float*>(src_of + ((D + 3) & ~(int64_t)3));  // [kAsmRows][n_out]
-  for (int64_t d = threadIdx.x; d < D; d += 256) src_of[d] = col_map[d];
-  __syncthreads();
-  for (int64_t j = threadIdx.x; j < a.n_out; j += 256) src_of[a.outl[j]] = -(int32_t)(1 + j);
-  __syncthreads();
-  const uint32_t n_out = (uint32_t)a.n_out, D32 = (uint32_t)D;
-  const uint32_t chunks = (D32 + 3) >> 2;
-  for (int64_t c0 = (int64_t)blockIdx.x * kAsmRows; c0 < a.C; c0 += (int64_t)gridDim.x * kAsmRows) {
-    const uint32_t nr = (uint32_t)min((int64_t)kAsmRows, a.C - c0);
-    for (uint32_t e = threadIdx.x; e < nr * n_out; e += 256) {
-      const uint32_t rr = e / n_out, j = e - rr * n_out;
-      const float* p = a.partial + (c0 + rr) * a.Kh + j;
-      float v = 0.0f;
-      for (int sp = 0; sp < n_split; ++sp) v += p[(int64_t)sp * a.C * a.Kh];  // fixed order
-      osum[rr * n_out + j] = v;
-    }
-    __syncthreads();
-    if (vec) {  // four channels per item, one 16-byte (FP32) or 8-byte (BF16) store
-      for (uint32_t e = threadIdx.x; e < nr * chunks; e += 256) {
-        const uint32_t rr = e / chunks, d = (e - rr * chunks) << 2;
-        const int64_t c = c0 + rr;
-        float v[4];
+  extern __shared__ __align__(16) float asm_smem[];
+  const uint32_t D = (uint32_t)a.D, n_out = (uint32_t)a.n_out, n_out4 = (n_out + 3u) >> 2, ldc = (uint32_t)a.ld_compact;
+  float* const osum = asm_smem;                                          // [ROWS][4 n_out4]
+  float* const rows = osum + ROWS * n_out4 * 4;                          // [ROWS][ldc] if STAGED
+  int32_t* const src_of = reinterpret_cast<int32_t*>(rows + (STAGED ? ROWS * ldc : 0u));  // [D]
+  const int64_t c0 = (int64_t)blockIdx.x * ROWS;
+  const uint32_t nr = (uint32_t)min((int64_t)ROWS, a.C - c0);
+  if (STAGED) {  // (rows of 16-byte pieces, one after another)
+    const float* p = a.compact + c0 * ldc;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(rows), pieces = nr * (ldc >> 2);
+    for (uint32_t e = threadIdx.x; e < pieces; e += 256)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + e * 16u), "l"(p + (size_t)e * 4u) : "memory");
+  }
+  const int64_t split_stride = a.C * a.Kh;
+  for (uint32_t e = threadIdx.x; e < nr * n_out4; e += 256) {
+    const uint32_t rr = e / n_out4, j = (e - rr * n_out4) * 4u;  // (Kh is a multiple of 64: the columns past n_out exist)
+    const float* p = a.partial + (c0 + rr) * a.Kh + j;
+    float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int s0 = 0; s0 < n_split; s0 += 8) {
+      float4 t[8];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          v[i] = 0.0f;
-          if (d + i < D32) {
-            const int32_t m = src_of[d + i];
-            v[i] = m >= 0 ? compact[c * ld_compact + m] : osum[rr * n_out + (uint32_t)(-m - 1)];
-          }
-        }
-        if (d + 4 <= D32) {
+      for (int i = 0; i < 8; ++i)
+        t[i] = s0 + i < n_split ? __ldg(reinterpret_cast<const float4*>(p + (s0 + i) * split_stride)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (s0 + i < n_split) v = make_float4(v.x + t[i].x, v.y + t[i].y, v.z + t[i].z, v.w + t[i].w);
+    }
+    *reinterpret_cast<float4*>(osum + rr * n_out4 * 4u + j) = v;
+  }
+  for (uint32_t d = threadIdx.x; d < D; d += 256) {
+    const int32_t m = __ldg(a.col_map + d);
+    if (m >= 0) src_of[d] = m;
+  }
+  for (uint32_t j = threadIdx.x; j < n_out; j += 256) src_of[__ldg(a.outl + j)] = -(int32_t)(1 + j);
+  if (STAGED) asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  for (uint32_t rr = 0; rr < nr; ++rr) {
+    const float* const kept = STAGED ? rows + rr * ldc : a.compact + (c0 + rr) * ldc;
+    const float* const sums = osum + rr * n_out4 * 4u - 1;
+    float* const df = reinterpret_cast<float*>(a.dW) + (c0 + rr) * a.lddw;
+    uint16_t* const dh = reinterpret_cast<uint16_t*>(a.dW) + (c0 + rr) * a.lddw;
+    auto value = [&](int32_t m) { return m >= 0 ? kept[m] : sums[-m]; };
+    auto store1 = [&](uint32_t d, float v) {
+      if (F32)
+        df[d] = v;
+      else
+        dh[d] = f32_to_bf16_bits(v);
+    };
+    if (vec) {  // four channels per item, one 16-byte (FP32) or 8-byte (BF16) store
+      for (uint32_t d = threadIdx.x * 4u; d < D; d += 1024u) {
+        if (d + 4u <= D) {
+          const int4 m = *reinterpret_cast<const int4*>(src_of + d);
+          const float4 v = make_float4(value(m.x), value(m.y), value(m.z), value(m.w));
           if (F32)
-            *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.dW) + c * a.lddw + d) = make_float4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<float4*>(df + d) = v;
           else
-            *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(a.dW) + c * a.lddw + d) =
-                make_uint2((uint32_t)f32_to_bf16_bits(v[0]) | ((uint32_t)f32_to_bf16_bits(v[1]) << 16),
-                           (uint32_t)f32_to_bf16_bits(v[2]) | ((uint32_t)f32_to_bf16_bits(v[3]) << 16));
+            *reinterpret_cast<uint2*>(dh + d) = make_uint2((uint32_t)f32_to_bf16_bits(v.x) | ((uint32_t)f32_to_bf16_bits(v.y) << 16),
+                                                           (uint32_t)f32_to_bf16_bits(v.z) | ((uint32_t)f32_to_bf16_bits(v.w) << 16));
         } else {
-          for (int i = 0; d + i < D32; ++i) {
-            if (F32)
-              reinterpret_cast<float*>(a.dW)[c * a.lddw + d + i] = v[i];
-            else
-              reinterpret_cast<uint16_t*>(a.dW)[c * a.lddw + d + i] = f32_to_bf16_bits(v[i]);
-          }
+          for (; d < D; ++d) store1(d, value(src_of[d]));
         }
       }
     } else {
-      for (uint32_t e = threadIdx.x; e < nr * D32; e += 256) {
-        const uint32_t rr = e / D32, d = e - rr * D32;
-        const int64_t c = c0 + rr;
-        const int32_t m = src_of[d];
-        const float v = m >= 0 ? compact[c * ld_compact + m] : osum[rr * n_out + (uint32_t)(-m - 1)];
-        if (F32)
-          reinterpret_cast<float*>(a.dW)[c * a.lddw + d] = v;
-        else
-          reinterpret_cast<uint16_t*>(a.dW)[c * a.lddw + d] = f32_to_bf16_bits(v);
-      }
+      for (uint32_t d = threadIdx.x; d < D; d += 256u) store1(d, value(src_of[d]));
     }
-    __syncthreads();  // osum is rewritten by the next group
   }
 }
 
@@ -169,20 +179,28 @@ cudaError_t launch_hp_dw_finish(const HpDwArgs& a, cudaStream_t st) {
   int n_split;
   hp_dw_splits(a, t_per_split, n_split);
   if (!a.compact || !a.col_map || !hp_dw_assemble_fits(a.D, a.n_out)) return cudaErrorInvalidValue;
-  // kept and outlier channels written together, row by row
-  const size_t smem = (size_t)(((a.D + 3) & ~(int64_t)3) + kAsmRows * a.n_out) * 4;
-  const int f32 = a.dw_is_f32;
-  const int elt = f32 ? 4 : 2;
+  // kept and outlier channels written together, row by row; the compact rows go through shared memory where two CTAs of four rows fit an
+  // SM, else one of two rows, else they are read as they are needed
+  const int64_t n4 = (a.n_out + 3) & ~(int64_t)3;
+  auto smem_of = [&](int64_t rows, bool staged) { return (size_t)((rows * n4 + (staged ? rows * a.ld_compact : 0) + a.D) * 4); };
+  const bool aligned = (a.ld_compact & 3) == 0 && (reinterpret_cast<uintptr_t>(a.compact) & 15u) == 0;
+  const int elt = a.dw_is_f32 ? 4 : 2;
   const int vec = (a.lddw & 3) == 0 && (reinterpret_cast<uintptr_t>(a.dW) & (size_t)(4 * elt - 1)) == 0;
-  const cudaError_t e = ensure_dynamic_smem(f32 ? reinterpret_cast<const void*>(dw_assemble_kernel<true>)
-                                                : reinterpret_cast<const void*>(dw_assemble_kernel<false>), smem);
-  if (e != cudaSuccess) return e;
-  const dim3 grid((unsigned)std::min<int64_t>((a.C + kAsmRows - 1) / kAsmRows, (int64_t)device_sm_count() * 8));
-  if (f32)
-    launch_kernel(dw_assemble_kernel<true>, grid, dim3(256), smem, st, a, n_split, a.compact, a.ld_compact, a.col_map, a.D, vec);
-  else
-    launch_kernel(dw_assemble_kernel<false>, grid, dim3(256), smem, st, a, n_split, a.compact, a.ld_compact, a.col_map, a.D, vec);
-  return cudaGetLastError();
+  auto launch = [&](auto f32, auto rows, auto staged) -> cudaError_t {
+    const auto kernel = dw_assemble_kernel<f32.value, rows.value, staged.value>;
+    const size_t smem = smem_of(rows.value, staged.value);
+    const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
+    if (e != cudaSuccess) return e;
+    launch_kernel(kernel, dim3((unsigned)((a.C + rows.value - 1) / rows.value)), dim3(256), smem, st, a, n_split, vec);
+    return cudaGetLastError();
+  };
+  auto pick = [&](auto f32) -> cudaError_t {
+    using std::integral_constant;
+    if (aligned && smem_of(kAsmRows, true) <= 110 * 1024) return launch(f32, integral_constant<int, kAsmRows>{}, integral_constant<bool, true>{});
+    if (aligned && smem_of(2, true) <= 200 * 1024) return launch(f32, integral_constant<int, 2>{}, integral_constant<bool, true>{});
+    return launch(f32, integral_constant<int, kAsmRows>{}, integral_constant<bool, false>{});
+  };
+  return a.dw_is_f32 ? pick(std::integral_constant<bool, true>{}) : pick(std::integral_constant<bool, false>{});
 }
 
 // The assembling pass keeps one source index per channel and kAsmRows sums per outlier channel in shared memory.
