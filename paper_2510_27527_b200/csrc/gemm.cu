@@ -1063,21 +1063,25 @@ gemm_nvfp4_block128_kernel(const __grid_constant__ CUtensorMap tmA, const __grid
 // each CTA loads 96 rows of B. A 192-wide tile starts at a multiple of 64 B rows, i.e. possibly in the middle of a 128-row
 // scale tile: the two scale tiles it touches are copied whole and the MMA's scale address starts two columns later (one
 // tensor-memory column holds the scales of 32 rows).
-template <int PN>
+// DENSE: operands in BF16 without block scales (the simulated FP6 x FP4 products): the same 128 bytes per row and stage are a 64-wide k
+// tile, and the tensor memory that the scales leave holds a second accumulator at either width.
+template <int PN, bool DENSE = false>
 struct Cfg2 {
-  static constexpr int STAGES = 5;
+  static constexpr int STAGES = DENSE ? 6 : 5;
   static constexpr uint32_t B_ROWS = PN / 2;                                   // this CTA's rows of the B tile
   static constexpr uint32_t B_BYTES = B_ROWS * 128;
-  static constexpr uint32_t SFB_BYTES = 4096;                                  // scales of the two 128-row scale tiles touched
-  static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES + SFA_BYTES + SFB_BYTES;  // 38 KB / 34 KB
+  static constexpr uint32_t SFA2_BYTES = DENSE ? 0 : SFA_BYTES;
+  static constexpr uint32_t SFB_BYTES = DENSE ? 0 : 4096;                      // scales of the two 128-row scale tiles touched
+  static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES + SFA2_BYTES + SFB_BYTES;  // 38 KB / 34 KB, DENSE 32 KB / 28 KB
   // staging buffers of 4 KB: one per epilogue warp; with 192-wide tiles (room for it) the four warps that own 128 columns
   // alternate between two, so that a chunk does not wait for the previous chunk's bulk store to have read the buffer
   static constexpr uint32_t STAGING_BYTES = (PN == 256 ? 8 : 12) * 4096;
   static constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + STAGING_BYTES + 1024 + 256;
-  static constexpr int ACC_BUFS = PN == 256 ? 1 : 2;
+  static constexpr int ACC_BUFS = PN == 256 && !DENSE ? 1 : 2;
   static constexpr uint32_t SF_COLS = 16 + 32;
   static constexpr uint32_t SF_SETS = PN == 256 ? 4 : 2;
   static constexpr uint32_t SF_TMEM_COL = ACC_BUFS * PN;                       // 256 / 384; + SF_SETS * 48 <= 512
+  static_assert(STAGE_BYTES % 1024 == 0 && SMEM_BYTES <= 227 * 1024, "shared memory budget");
 };
 constexpr int C2_THREADS = 64 + 256;
 
@@ -1132,6 +1136,17 @@ __device__ __forceinline__ void tc2_mma_nvf4(uint32_t d_tmem, uint64_t a_desc, u
       "setp.ne.b32 q, %7, 0;\n"
       "@q tcgen05.mma.cta_group::2.kind::mxf4nvf4.block_scale.scale_vec::4X [%0], %1, %2, %3, [%5], [%6], p;\n}" ::"r"(d_tmem),
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(sfa_tmem), "r"(sfb_tmem), "r"(leader)
+      : "memory");
+}
+
+__device__ __forceinline__ void tc2_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate,
+                                             uint32_t leader) {
+  asm volatile(
+      "{\n.reg .pred p, q;\n"
+      "setp.ne.b32 p, %4, 0;\n"
+      "setp.ne.b32 q, %5, 0;\n"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
       : "memory");
 }
 
@@ -1191,12 +1206,12 @@ __device__ __forceinline__ void stage_and_store(const Params& p, const CUtensorM
   }
 }
 
-template <int GS, int PN>
+template <int GS, int PN, bool DENSE = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
 gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                        const __grid_constant__ CUtensorMap tmSFA, const __grid_constant__ CUtensorMap tmSFB,
                        const __grid_constant__ CUtensorMap tmC, const Params p) {
-  using C2 = Cfg2<PN>;
+  using C2 = Cfg2<PN, DENSE>;
   constexpr int STAGES = C2::STAGES;
   constexpr uint32_t C2_STAGE_BYTES = C2::STAGE_BYTES, C2_B_BYTES = C2::B_BYTES, C2_SF_COLS = C2::SF_COLS;
   constexpr int ACC_BUFS = C2::ACC_BUFS;
@@ -1260,8 +1275,10 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         const uint32_t st = smem_base + s * C2_STAGE_BYTES;
         const uint32_t full0 = map_to_cta(full_bar(s), 0);
         if (rank == 0) mbar_expect_tx(full_bar(s), 2 * C2_STAGE_BYTES + ((p.starve && it == 0) ? 16u : 0u), leader);
-        tma_load_2d_pair(st, &tmA, kt * (BK / 2), a_row, full0, leader);
-        tma_load_2d_pair(st + A_BYTES, &tmB, kt * (BK / 2), b_row, full0, leader);
+        constexpr int32_t KX = DENSE ? 64 : BK / 2;  // a k tile in elements of the maps: BF16, or bytes of codes
+        tma_load_2d_pair(st, &tmA, kt * KX, a_row, full0, leader);
+        tma_load_2d_pair(st + A_BYTES, &tmB, kt * KX, b_row, full0, leader);
+        if (DENSE) continue;
         tma_load_2d_pair(st + A_BYTES + C2_B_BYTES, &tmSFA, 0, sfa_row + kt * 16, full0, leader);
         tma_load_2d_pair(st + A_BYTES + C2_B_BYTES + SFA_BYTES, &tmSFB, 0, sfb_row0 + kt * 16, full0, leader);
         tma_load_2d_pair(st + A_BYTES + C2_B_BYTES + SFA_BYTES + 2048, &tmSFB, 0, sfb_row1 + kt * 16, full0, leader);
@@ -1278,7 +1295,8 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     // ===================================== MMA issuer (leader CTA only) ====================================
     if (rank == 0) {
       const uint32_t leader = elect_leader();
-      const uint32_t idesc = (1u << 7) | (1u << 10) | ((uint32_t)(PN >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+      // (DENSE: BF16 x BF16 -> FP32)
+      const uint32_t idesc = (DENSE ? 1u << 4 : 0u) | (1u << 7) | (1u << 10) | ((uint32_t)(PN >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
       // issue loop kept short as in the 128 x 128 kernel: running stage / phase counters, descriptors by addition to the low
       // word, the next stage's barrier tried before this stage's instructions
       uint32_t it = 0, tile_it = 0, stage = 0, phase = 0;
@@ -1308,17 +1326,24 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             phase ^= 1u;
           }
           const uint32_t next_try = mbar_test(full_bar(stage), phase);
-          const uint32_t sf_tmem = tmem_base + C2::SF_TMEM_COL + (it % C2::SF_SETS) * C2_SF_COLS;
+          if constexpr (DENSE) {
 #pragma unroll
-          for (int kk = 0; kk < BK / 64; ++kk) {
-            tc2_cp_sf(sf_tmem + kk * 4, ((uint64_t)SF_HI << 32) | (sfa_lo0 + st16 + kk * 32), leader);
-            tc2_cp_sf(sf_tmem + 16 + kk * 8, ((uint64_t)SF_HI << 32) | (sfa_lo0 + st16 + (SFA_BYTES >> 4) + kk * 32), leader);
-            tc2_cp_sf(sf_tmem + 16 + kk * 8 + 4, ((uint64_t)SF_HI << 32) | (sfa_lo0 + st16 + ((SFA_BYTES + 2048) >> 4) + kk * 32), leader);
+            for (int kk = 0; kk < 4; ++kk)  // 64 BF16 = four K = 16 steps of 32 bytes
+              tc2_mma_bf16(d_tmem, ((uint64_t)SW_HI << 32) | (a_lo0 + st16 + kk * 2), ((uint64_t)SW_HI << 32) | (a_lo0 + st16 + (A_BYTES >> 4) + kk * 2),
+                           idesc, (kt | kk) != 0, leader);
+          } else {
+            const uint32_t sf_tmem = tmem_base + C2::SF_TMEM_COL + (it % C2::SF_SETS) * C2_SF_COLS;
+#pragma unroll
+            for (int kk = 0; kk < BK / 64; ++kk) {
+              tc2_cp_sf(sf_tmem + kk * 4, ((uint64_t)SF_HI << 32) | (sfa_lo0 + st16 + kk * 32), leader);
+              tc2_cp_sf(sf_tmem + 16 + kk * 8, ((uint64_t)SF_HI << 32) | (sfa_lo0 + st16 + (SFA_BYTES >> 4) + kk * 32), leader);
+              tc2_cp_sf(sf_tmem + 16 + kk * 8 + 4, ((uint64_t)SF_HI << 32) | (sfa_lo0 + st16 + ((SFA_BYTES + 2048) >> 4) + kk * 32), leader);
+            }
+#pragma unroll
+            for (int kk = 0; kk < BK / 64; ++kk)
+              tc2_mma_nvf4(d_tmem, ((uint64_t)SW_HI << 32) | (a_lo0 + st16 + kk * 2), ((uint64_t)SW_HI << 32) | (a_lo0 + st16 + (A_BYTES >> 4) + kk * 2),
+                           idesc, sf_tmem + kk * 4, sf_tmem + 16 + kk * 8 + sfb_col, (kt | kk) != 0, leader);
           }
-#pragma unroll
-          for (int kk = 0; kk < BK / 64; ++kk)
-            tc2_mma_nvf4(d_tmem, ((uint64_t)SW_HI << 32) | (a_lo0 + st16 + kk * 2), ((uint64_t)SW_HI << 32) | (a_lo0 + st16 + (A_BYTES >> 4) + kk * 2),
-                         idesc, sf_tmem + kk * 4, sf_tmem + 16 + kk * 8 + sfb_col, (kt | kk) != 0, leader);
           tc2_commit_both(this_empty, leader);
           ready = __all_sync(0xFFFFFFFFu, next_try);
         }
@@ -1780,35 +1805,63 @@ cudaError_t launch_hp_dw_mma(const uint16_t* dY, int64_t lddy, const uint16_t* X
 }
 
 // Dense BF16 product (the simulated FP6 x FP4 layer): C = (SgA SgB) * A B^T with A [M, ld], B [N, ld] BF16 row-major, ld a
-// multiple of 64 and the same for both. It is the 128 x 128 kernel with no FP4 k tiles at all: only its BF16 side-product path
-// runs (64-wide k tiles, kind::f16, FP32 accumulation in the side accumulator) and the epilogue scales that accumulator.
-cudaError_t launch_dense_gemm(const void* A, const void* B, int64_t M, int64_t N, int64_t ld, const float* a_gscale,
-                              const float* b_gscale, void* Cp, int c_is_f32, int64_t ldc, int32_t* dev_status, cudaStream_t st) {
-  using C = Cfg;
-  if (M == 0 || N == 0) return cudaSuccess;
+// multiple of 64 and the same for both. On CTA pairs (PN > 0: the pair kernel's DENSE form, 256 x PN tiles), or on the 128 x 128 kernel
+// with no FP4 k tiles at all: only its BF16 side-product path runs (64-wide k tiles, FP32 accumulation in the side accumulator)
+// and the epilogue scales that accumulator.
+template <int PN>
+cudaError_t launch_dense(const void* A, const void* B, int64_t M, int64_t N, int64_t ld, const float* a_gscale, const float* b_gscale, void* Cp,
+                         int c_is_f32, int64_t ldc, int32_t* dev_status, cudaStream_t st) {
+  constexpr int TM = PN ? 256 : BM, TN = PN ? PN : BN;
   CUtensorMap tmAh, tmBh, tmC;
-  if (!make_hp_map(&tmAh, A, M, ld) || !make_hp_map(&tmBh, B, N, ld) || !make_c_map(&tmC, Cp, M, N, ldc, c_is_f32 != 0))
+  if (!make_hp_map(&tmAh, A, M, ld) || !make_hp_map(&tmBh, B, N, ld, PN ? PN / 2 : BN) || !make_c_map(&tmC, Cp, M, N, ldc, c_is_f32 != 0))
     return cudaErrorInvalidValue;
   Params p{};
   p.wait_limit = DEFAULT_WAIT_LIMIT_CYCLES;
-  p.hp_k_tiles = (int32_t)(ld / 64);
   p.a_gscale = a_gscale;
   p.b_gscale = b_gscale;
   p.C = Cp;
   p.ldc = ldc;
   p.M = M;
   p.N = N;
-  p.k_tiles = 0;
-  p.m_tiles = (int32_t)((M + BM - 1) / BM);
-  p.n_tiles = (int32_t)((N + BN - 1) / BN);
+  p.m_tiles = (int32_t)((M + TM - 1) / TM);
+  p.n_tiles = (int32_t)((N + TN - 1) / TN);
   p.c_is_f32 = c_is_f32;
   p.dev_status = dev_status;
-  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_nvfp4_kernel<kGsTensor>), C::SMEM_BYTES);
-  if (e != cudaSuccess) return e;
   const int64_t tiles = (int64_t)p.m_tiles * p.n_tiles;
-  const unsigned grid = (unsigned)std::min<int64_t>(tiles, sm_count());
-  launch_kernel(gemm_nvfp4_kernel<kGsTensor>, dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, tmAh, tmBh, tmC, tmAh, tmBh, p);
+  cudaError_t e;
+  if constexpr (PN > 0) {
+    p.k_tiles = (int32_t)(ld / 64);
+    const auto kernel = gemm_nvfp4_2cta_kernel<kGsTensor, PN, true>;
+    constexpr uint32_t smem = Cfg2<PN, true>::SMEM_BYTES;
+    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem)) != cudaSuccess) return e;
+    const unsigned pairs = (unsigned)std::min<int64_t>(tiles, sm_count() / 2);
+    launch_kernel(kernel, dim3(2 * pairs), dim3(C2_THREADS), smem, st, tmAh, tmBh, tmAh, tmBh, tmC, p);
+  } else {
+    p.hp_k_tiles = (int32_t)(ld / 64);
+    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_nvfp4_kernel<kGsTensor>), Cfg::SMEM_BYTES)) != cudaSuccess) return e;
+    const unsigned grid = (unsigned)std::min<int64_t>(tiles, sm_count());
+    launch_kernel(gemm_nvfp4_kernel<kGsTensor>, dim3(grid), dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, tmAh, tmBh, tmC, tmAh, tmBh, p);
+  }
   return cudaGetLastError();
+}
+
+// Variant by a cost model, as launch_gemm: rounds of the tiles x (fixed + per 64-wide k tile). The pairs win where the operands' way from
+// L2 to the SMs bounds the product (32 KB per k tile and SM for 256 x 256, as the 128 x 128 kernel takes for a quarter of that), and their
+// epilogue runs under the next tile; the small tiles where there are few. us, 128 x 128 / 256 x 256 / 256 x 192: 4096 x 3072 x 1024
+// 26.8 / 20.6 / 21.6, 4096 x 1024 x 3072 25.1 / 19.7 / 26.0, 3072 x 1024 x 4096 (FP32) 32.5 / 25.4 / 21.5, 2048^3 17.4 / 14.7 / 18.7,
+// 8192^3 1260 / 862 / 899, 1000 x 1416 x 1000 (FP32) 6.8 / 9.6 / 8.1, 2048 x 512 x 4000 (FP32) 17.7 / 23.2 / 18.5, 64 x 2048 x 2048 8.1 /
+// 12.5 / 9.9.
+cudaError_t launch_dense_gemm(const void* A, const void* B, int64_t M, int64_t N, int64_t ld, const float* a_gscale,
+                              const float* b_gscale, void* Cp, int c_is_f32, int64_t ldc, int32_t* dev_status, cudaStream_t st) {
+  if (M == 0 || N == 0) return cudaSuccess;
+  auto cost = [&](int64_t tm, int64_t tn, int64_t units, double fixed, double per_k_tile) {
+    const int64_t tiles = ((M + tm - 1) / tm) * ((N + tn - 1) / tn);
+    return (double)((tiles + units - 1) / units) * (fixed + per_k_tile * (double)(ld / 64));
+  };
+  const int64_t sms = sm_count();
+  const double c128 = cost(128, 128, sms, 0.6, 0.23), c256 = cost(256, 256, sms / 2, 1.2, 0.345), c192 = cost(256, 192, sms / 2, 0.9, 0.28);
+  const auto launch = c128 <= c256 && c128 <= c192 ? launch_dense<0> : c256 <= c192 ? launch_dense<256> : launch_dense<192>;
+  return launch(A, B, M, N, ld, a_gscale, b_gscale, Cp, c_is_f32, ldc, dev_status, st);
 }
 
 size_t gemm_workspace_bytes(int64_t, int64_t, int64_t) { return 0; }
