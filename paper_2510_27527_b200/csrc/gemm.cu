@@ -1367,6 +1367,11 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     const int half = (warp - 2) >> 2;
     // columns of the tile this warp owns: [half * 128, half * 128 + 32 * nq): the first four warps 128, the others the rest
     const int nq = half == 0 ? 4 : (PN - 128) / 32;
+    // The staging buffers: a warp with two takes them in turn by the bulk stores that it has issued, not by the chunk, as ragged chunks
+    // issue none: the buffer that is written next is then never the one of the last store, which may still be reading it.
+    const bool two_bufs = PN == 192 && half == 0;
+    const uint32_t my_stage = staging_base + (PN == 256 ? (uint32_t)(warp - 2) : (half == 0 ? 2u * (uint32_t)(warp - 2) : 4u + (uint32_t)(warp - 2))) * 4096u;
+    uint32_t buf_at = 0;
     uint32_t tile_it = 0;
     bool ok = true;
     float alpha = 1.0f;
@@ -1389,8 +1394,6 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(acc_empty_leader);
       // The accumulator is free again (the pair's next tile may start); scale, stage and store from the registers.
-      const bool two_bufs = PN == 192 && half == 0;
-      const uint32_t my_stage = staging_base + (PN == 256 ? (uint32_t)(warp - 2) : (half == 0 ? 2u * (uint32_t)(warp - 2) : 4u + (uint32_t)(warp - 2))) * 4096u;
       const int64_t m0 = (int64_t)mt * 256 + rank * 128 + quad * 32;
       if (m0 >= p.M) continue;
       if (p.c_is_f32) {
@@ -1402,7 +1405,8 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
           if (GS == kGsRow) load_sgb32(p.b_gscale, n0, p.N, sgb);
 #pragma unroll
           for (int j = 0; j < 32; ++j) o[j] = __uint_as_float(v[q][j]) * (GS == kGsRow ? __fmul_rn(sa, sgb[j]) : alpha);
-          stage_and_store<32>(p, &tmC, my_stage + (two_bufs ? (uint32_t)(q & 1) * 4096u : 0u), lane, m, m0, n0, o, two_bufs ? 1 : 0);
+          stage_and_store<32>(p, &tmC, my_stage + buf_at, lane, m, m0, n0, o, two_bufs ? 1 : 0);
+          if (two_bufs && n0 + 32 <= p.N) buf_at ^= 4096u;
         }
       } else {
 #pragma unroll
@@ -1416,7 +1420,8 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
           if (GS == kGsRow) load_sgb32(p.b_gscale, n0 + 32, p.N, sgb);
 #pragma unroll
           for (int j = 0; j < 32; ++j) o[32 + j] = __uint_as_float(v[2 * qq + 1][j]) * (GS == kGsRow ? __fmul_rn(sa, sgb[j]) : alpha);
-          stage_and_store<64>(p, &tmC, my_stage + (two_bufs ? (uint32_t)(qq & 1) * 4096u : 0u), lane, m, m0, n0, o, two_bufs ? 1 : 0);
+          stage_and_store<64>(p, &tmC, my_stage + buf_at, lane, m, m0, n0, o, two_bufs ? 1 : 0);
+          if (two_bufs && n0 + 64 <= p.N) buf_at ^= 4096u;
         }
       }
     }
