@@ -498,7 +498,7 @@ nvfp4_status nvfp4_fp6_quantize(const void* src_bf16, int64_t rows, int64_t cols
   if (!workspace || !aligned16(workspace) || ws_bytes < nvfp4_fp6_workspace_bytes()) return NVFP4_ERR_WORKSPACE;
   if ((s = check_arch()) != NVFP4_OK) return s;
   return launch_fp6_quantize_rows(static_cast<const uint16_t*>(src_bf16), rows, cols, ld, rounding == NVFP4_ROUND_SR, seed, stream_id,
-                                  static_cast<uint32_t*>(workspace), static_cast<uint16_t*>(out->vals), out->ld, out->gscale,
+                                  static_cast<uint32_t*>(workspace), ws_bytes, static_cast<uint16_t*>(out->vals), out->ld, out->gscale,
                                   static_cast<cudaStream_t>(stream)) == cudaSuccess
              ? NVFP4_OK
              : NVFP4_ERR_CUDA;

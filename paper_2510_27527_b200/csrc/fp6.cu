@@ -18,12 +18,11 @@ namespace nvfp4 {
 namespace {
 
 // Round 16 scaled values to E2M3 and return them times the block scale as packed BF16 pairs (8 words).
-// Stochastic rounding, exactly as for E2M1 with three mantissa bits instead of one: for a >= 1 the cell index and the
-// position inside the cell are the exponent / top three mantissa bits and the low 20 mantissa bits of a itself; the cells
-// below 1 (width 1/8) are mapped onto [0.5, 1) by z = 0.5 + a / 2 computed with round-up (an integer n is < x iff
-// n < ceil(x)); adding 2^20 - 1 - ((2u + 1) << 3) to the bits carries into the cell index iff position > (2u + 1) << 3,
-// i.e. iff (u + 0.5) / 65536 < position / 2^20; clearing the low 20 bits then leaves the rounded magnitude as a float (the
-// carry moves through the exponent like the value does), mapped back by 2 z - 1 below 1.
+// Stochastic rounding, as for E2M1 (e2m1x8_sr) with three mantissa bits instead of one: w = a * 2^-126, rounded up, has E2M3's own
+// spacing, its cell is bits(w) >> 20 and the low 20 bits the position inside it; adding 2^20 - 1 - ((2u + 1) << 3) to the bits
+// carries into the cell iff position > (2u + 1) << 3, i.e. iff (u + 0.5) / 65536 < position / 2^20 (an integer n is < x iff
+// n < ceil(x)); clearing the low 20 bits then leaves the rounded magnitude times 2^-126
+// (4096 x 3072 rows with the amax pass 24.6 -> 21.5 us against cells below 1 mapped onto [0.5, 1) and back).
 template <bool SR>
 __device__ __forceinline__ void fp6_block16(const float (&x)[16], float rcp, float Sbf, const PhiloxKeys& pk, uint32_t stream_id,
                                             uint64_t idx8, uint32_t (&out)[8]) {
@@ -32,28 +31,18 @@ __device__ __forceinline__ void fp6_block16(const float (&x)[16], float rcp, flo
     w[0] = sr_words(pk, stream_id, idx8);
     w[1] = sr_words(pk, stream_id, idx8 + 1);
   }
-  float v[16];
 #pragma unroll
   for (int i = 0; i < 16; i += 2) {
-    const float y0 = __fmul_rn(x[i], rcp), y1 = __fmul_rn(x[i + 1], rcp);
-    float p0, p1;
+    float y0, y1, p0, p1;
+    mul2_rn(x[i], x[i + 1], rcp, y0, y1);
     if (SR) {
       const uint4& ww = w[i >> 3];
-      const uint32_t word = ((i >> 1) & 3) == 0 ? ww.x : ((i >> 1) & 3) == 1 ? ww.y : ((i >> 1) & 3) == 2 ? ww.z : ww.w;
-      const uint32_t u[2] = {word & 0xFFFFu, word >> 16};
-      const float ys[2] = {y0, y1};
-      float ps[2];
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const float a = fminf(fabsf(ys[e]), 7.5f);
-        const float z = fmaxf(a, __fmaf_ru(a, 0.5f, 0.5f));
-        const uint32_t bits = __float_as_uint(z) + (((~u[e] & 0xFFFFu) << 4) | 0x7u);
-        const float zq = __uint_as_float(bits & 0xFFF00000u);
-        const float mag = a >= 1.0f ? zq : __fmaf_rn(zq, 2.0f, -1.0f);
-        ps[e] = __uint_as_float(__float_as_uint(mag) | (__float_as_uint(ys[e]) & 0x80000000u));
-      }
-      p0 = ps[0];
-      p1 = ps[1];
+      const uint32_t word = ~(((i >> 1) & 3) == 0 ? ww.x : ((i >> 1) & 3) == 1 ? ww.y : ((i >> 1) & 3) == 2 ? ww.z : ww.w);
+      float w0, w1;
+      mul2_up(fminf(fabsf(y0), 7.5f), fminf(fabsf(y1), 7.5f), 0x1p-126f, w0, w1);
+      const uint32_t b0 = __float_as_uint(w0) + ((word & 0xFFFFu) * 16u + 7u), b1 = __float_as_uint(w1) + ((word >> 16) * 16u + 7u);
+      mul2_rn(__uint_as_float((b0 & 0x7FF00000u) | (__float_as_uint(y0) & 0x80000000u)),
+              __uint_as_float((b1 & 0x7FF00000u) | (__float_as_uint(y1) & 0x80000000u)), 0x1p126f, p0, p1);
     } else {
       // hardware conversion: round to nearest even, saturating at 7.5; then back to FP16 (exact)
       uint16_t packed;
@@ -64,11 +53,10 @@ __device__ __forceinline__ void fp6_block16(const float (&x)[16], float rcp, flo
       p0 = f.x;
       p1 = f.y;
     }
-    v[i] = __fmul_rn(p0, Sbf);  // exact: at most 4 + 4 significant bits
-    v[i + 1] = __fmul_rn(p1, Sbf);
+    float v0, v1;  // exact, in BF16 too: at most 4 + 4 significant bits
+    mul2_rn(p0, p1, Sbf, v0, v1);
+    out[i >> 1] = __byte_perm(__float_as_uint(v0), __float_as_uint(v1), 0x7632);
   }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) out[i] = (uint32_t)f32_to_bf16_bits(v[2 * i]) | ((uint32_t)f32_to_bf16_bits(v[2 * i + 1]) << 16);
 }
 
 // The scale pair of a block: E4M3 block scale as a float and the reciprocal that maps x onto the E2M3 grid.
@@ -82,50 +70,69 @@ __device__ __forceinline__ float fp6_block_scale(float amax_b, float Sg, float& 
 }
 __device__ __forceinline__ float fp6_global_scale(float amax) { return amax == 0.0f ? 1.0f : __fdiv_rn(amax, 3360.0f); }
 
-// Row-axis FP6 quantize from BF16 [rows, cols] (leading dimension ld): one thread per 16-element block of the padded output
-// row (ld_out / 16 blocks: those past K are written as zeros). cell[0] = bits of max |x| over the tensor.
-template <bool SR>
+// n / d for n < total: a 32-bit division where that is enough (a 64-bit one is a hundred instructions).
+__device__ __forceinline__ int64_t quotient(int64_t n, int64_t d, int64_t total) {
+  return total < ((int64_t)1 << 32) ? (int64_t)((uint32_t)n / (uint32_t)d) : n / d;
+}
+
+// Row-axis FP6 quantize from BF16 [rows, cols] (leading dimension ld): NB 16-element blocks of the padded output rows (ld_out / 16 blocks
+// each: those past K are written as zeros) per thread, at a stride, all loads first. cells: bits of max |x| over the tensor, in `words`
+// words. Bound by the chain from the maximum to the scales of a block, which NB = 4 shares.
+template <bool SR, int NB>
 __global__ void __launch_bounds__(256)
 fp6_quantize_rows_kernel(const uint16_t* __restrict__ src, int64_t rows, int64_t K, int64_t ld, uint32_t stream_id,
-                         const uint32_t* __restrict__ cell, uint16_t* __restrict__ out, int64_t ld_out, float* __restrict__ gscale,
+                         const uint32_t* __restrict__ cells, int words, uint16_t* __restrict__ out, int64_t ld_out, float* __restrict__ gscale,
                          const __grid_constant__ PhiloxKeys pk) {
   pdl_prologue();
-  const int64_t nb = ld_out >> 4;
-  const int64_t gid = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (gid >= rows * nb) return;
-  const int64_t r = gid / nb, b = gid - r * nb;
-  const int64_t k0 = b << 4;
+  const int64_t nb = ld_out >> 4, total = rows * nb;
   const int64_t K16 = (K + 15) & ~(int64_t)15;
-  const float Sg = fp6_global_scale(__uint_as_float(cell[0]));
-  if (gid == 0) gscale[0] = Sg;
-  uint4* dst = reinterpret_cast<uint4*>(out + r * ld_out + k0);
-  if (k0 >= K) {
-    dst[0] = dst[1] = make_uint4(0, 0, 0, 0);
-    return;
+  const bool vec = (ld & 7) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0;
+  uint32_t w[NB][8];
+  int64_t row[NB], k0[NB];  // (row -1: none)
+#pragma unroll
+  for (int j = 0; j < NB; ++j) {
+    const int64_t gid = ((int64_t)blockIdx.x * NB + j) * 256 + threadIdx.x;
+    row[j] = gid < total ? quotient(gid, nb, total) : -1;
+    k0[j] = (gid - row[j] * nb) << 4;
+    const uint16_t* p = src + row[j] * ld + k0[j];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[j][i] = 0u;
+    if (row[j] < 0 || k0[j] >= K) continue;
+    if (vec && k0[j] + 16 <= K) {
+      const uint4 a = *reinterpret_cast<const uint4*>(p), c = *reinterpret_cast<const uint4*>(p + 8);
+      w[j][0] = a.x; w[j][1] = a.y; w[j][2] = a.z; w[j][3] = a.w;
+      w[j][4] = c.x; w[j][5] = c.y; w[j][6] = c.z; w[j][7] = c.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (k0[j] + i < K) w[j][i >> 1] |= (uint32_t)p[i] << (16 * (i & 1));
+    }
   }
-  float x[16];
-  const uint16_t* p = src + r * ld + k0;
-  if (k0 + 16 <= K && (ld & 7) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
-    const uint4 a = *reinterpret_cast<const uint4*>(p), c = *reinterpret_cast<const uint4*>(p + 8);
-    const uint32_t w[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
+  const float Sg = fp6_global_scale(__uint_as_float(tensor_amax_bits(cells, words)));
+  if (blockIdx.x == 0 && threadIdx.x == 0) gscale[0] = Sg;
+#pragma unroll
+  for (int j = 0; j < NB; ++j) {
+    if (row[j] < 0) break;
+    uint4* dst = reinterpret_cast<uint4*>(out + row[j] * ld_out + k0[j]);
+    if (k0[j] >= K) {
+      dst[0] = dst[1] = make_uint4(0, 0, 0, 0);
+      continue;
+    }
+    uint32_t m2 = 0;
+    float x[16];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      x[2 * i] = bf16_lo(w[i]);
-      x[2 * i + 1] = bf16_hi(w[i]);
+      m2 = amax16x2(m2, w[j][i]);
+      x[2 * i] = bf16_lo(w[j][i]);
+      x[2 * i + 1] = bf16_hi(w[j][i]);
     }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 16; ++i) x[i] = k0 + i < K ? bf16_bits_to_float(p[i]) : 0.0f;
+    float rcp;
+    const float Sbf = fp6_block_scale(__uint_as_float(hmax_of_pair(bf16x2_abs_bits(m2)) << 16), Sg, rcp);
+    uint32_t o[8];
+    fp6_block16<SR>(x, rcp, Sbf, pk, stream_id, (uint64_t)(row[j] * K16 + k0[j]) >> 3, o);
+    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
   }
-  float m = 0.0f;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) m = fmaxf(m, fabsf(x[i]));
-  float rcp;
-  const float Sbf = fp6_block_scale(m, Sg, rcp);
-  uint32_t o[8];
-  fp6_block16<SR>(x, rcp, Sbf, pk, stream_id, (uint64_t)(r * K16 + k0) >> 3, o);
-  dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-  dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
 }
 
 // Transposing FP6 re-quantize of a dense operand: in [rowsK, D] (values v, global scale Sg_in) -> out [D, rowsK] with blocks
@@ -140,15 +147,16 @@ fp6_requantize_t_kernel(const uint16_t* __restrict__ in, int64_t rowsK, int64_t 
   pdl_prologue();
   const int64_t d0 = ((int64_t)blockIdx.y * 32 + (threadIdx.x & 31)) * 4;
   const int64_t k0 = ((int64_t)blockIdx.x * 4 + (threadIdx.x >> 5)) * 16;
-  const float sg_in = in_gscale[0];
-  const float Sg = fp6_global_scale(__fmul_rn(__uint_as_float(cell[0]), sg_in));
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) gscale[0] = Sg;
-  if (d0 >= D || k0 >= ld_out) return;
+  const bool live = d0 < D && k0 < ld_out;
   const int64_t K16 = (rowsK + 15) & ~(int64_t)15;
   uint2 w[16];
 #pragma unroll
   for (int t = 0; t < 16; ++t)
-    w[t] = k0 + t < rowsK ? *reinterpret_cast<const uint2*>(in + (k0 + t) * ld_in + d0) : make_uint2(0u, 0u);  // ld_in, d0: multiples of 4
+    w[t] = live && k0 + t < rowsK ? *reinterpret_cast<const uint2*>(in + (k0 + t) * ld_in + d0) : make_uint2(0u, 0u);  // ld_in, d0: multiples of 4
+  const float sg_in = in_gscale[0];
+  const float Sg = fp6_global_scale(__fmul_rn(__uint_as_float(cell[0]), sg_in));
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) gscale[0] = Sg;
+  if (!live) return;
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     if (d0 + c >= D) break;
@@ -182,7 +190,7 @@ expand_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restri
   const int64_t gid = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (gid == 0) gscale[0] = in_gscale[0];
   if (gid >= R * n8) return;
-  const int64_t r = gid / n8, k0 = (gid - r * n8) << 3;
+  const int64_t r = quotient(gid, n8, R * n8), k0 = (gid - r * n8) << 3;
   const int64_t Kp = (K + 127) & ~(int64_t)127;
   uint4 o = make_uint4(0, 0, 0, 0);
   if (k0 < Kp) {
@@ -195,7 +203,7 @@ expand_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restri
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h[i]));
-      q[i] = (uint32_t)f32_to_bf16_bits(f.x) | ((uint32_t)f32_to_bf16_bits(f.y) << 16);  // exact: 2 + 4 significant bits
+      q[i] = __byte_perm(__float_as_uint(f.x), __float_as_uint(f.y), 0x7632);  // exact in BF16: 2 + 4 significant bits
     }
     o = make_uint4(q[0], q[1], q[2], q[3]);
   }
@@ -205,19 +213,33 @@ expand_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restri
 }  // namespace
 
 cudaError_t launch_fp6_quantize_rows(const uint16_t* src, int64_t rows, int64_t K, int64_t ld, int sr, uint64_t seed, uint32_t stream_id,
-                                     uint32_t* cell, uint16_t* out, int64_t ld_out, float* gscale, cudaStream_t st) {
+                                     uint32_t* cells, size_t cells_bytes, uint16_t* out, int64_t ld_out, float* gscale, cudaStream_t st) {
   if (rows == 0) return cudaSuccess;
+  // The maximum as words that need no clearing (a launch less: 3 us of host time) up to 2^20 blocks, if the workspace holds them, else
+  // folded into one cleared word: from there on what each warp spends on reading the words is more than the launch. Four blocks per
+  // thread from 4 CTAs of single ones per SM on, from 8 with the longer chain of stochastic rounding: then the threads that wait for the
+  // words are what is too many. us with the amax pass, words and NB = 1 / words and NB = 4 / one word and NB = 1, before: to nearest
+  // 64 x 256 3.4 / 4.6 / -, 3.8; 1000 x 1416 5.9 / 6.6 / -, 7.1; 4096 x 1024 9.3 / 7.4 / -, 8.1; 4096 x 3072 19.1 / 15.9 / 14.6, 15.7;
+  // 16384 x 4096 91 / 79.7 / 67.4, 74.5; stochastic 1000 x 1416 6.7 / 9.6 / -, 9.0; 4096 x 1024 9.0 / 12.2 / -, 10.8; 4096 x 3072 21.4 /
+  // 22.2 / 21.5, 24.6; 16384 x 4096 105 / 102 / 104, 121.
+  const int64_t blocks = rows * (ld_out >> 4);
+  const int words = blocks <= ((int64_t)1 << 20) && cells_bytes >= kTensorAmaxWords * sizeof(uint32_t) ? kTensorAmaxWords : 1;
   cudaError_t e;
-  if ((e = launch_zero_words(cell, 1, st)) != cudaSuccess) return e;
-  if ((e = launch_amax_tensor(src, rows, K, ld, cell, st)) != cudaSuccess) return e;
-  const unsigned grid = (unsigned)((rows * (ld_out >> 4) + 255) / 256);
-  const uint32_t* ccell = cell;
-  if (sr)
-    launch_kernel(fp6_quantize_rows_kernel<true>, dim3(grid), dim3(256), 0, st, src, rows, K, ld, stream_id, ccell, out, ld_out, gscale,
-                  make_philox_keys(seed));
+  if (words > 1) {
+    if ((e = launch_amax_tensor_words(src, rows, K, ld, cells, st)) != cudaSuccess) return e;
+  } else {
+    if ((e = launch_zero_words(cells, 1, st)) != cudaSuccess) return e;
+    if ((e = launch_amax_tensor(src, rows, K, ld, cells, st)) != cudaSuccess) return e;
+  }
+  const uint32_t* ccells = cells;
+  auto go = [&](auto kernel, int nb) {
+    launch_kernel(kernel, dim3((unsigned)((blocks + 256 * nb - 1) / (256 * nb))), dim3(256), 0, st, src, rows, K, ld, stream_id, ccells, words,
+                  out, ld_out, gscale, make_philox_keys(seed));
+  };
+  if (words > 1 && blocks > (int64_t)148 * (sr ? 8 : 4) * 256)
+    sr ? go(fp6_quantize_rows_kernel<true, 4>, 4) : go(fp6_quantize_rows_kernel<false, 4>, 4);
   else
-    launch_kernel(fp6_quantize_rows_kernel<false>, dim3(grid), dim3(256), 0, st, src, rows, K, ld, stream_id, ccell, out, ld_out, gscale,
-                  make_philox_keys(seed));
+    sr ? go(fp6_quantize_rows_kernel<true, 1>, 1) : go(fp6_quantize_rows_kernel<false, 1>, 1);
   return cudaGetLastError();
 }
 

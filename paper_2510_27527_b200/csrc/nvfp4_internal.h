@@ -185,9 +185,9 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st);
 cudaError_t launch_dense_gemm(const void* A, const void* B, int64_t M, int64_t N, int64_t ld, const float* a_gscale,
                               const float* b_gscale, void* C, int c_is_f32, int64_t ldc, int32_t* dev_status, cudaStream_t st);
 
-// Simulated FP6 (E2M3) quantizers and the FP4 -> dense expansion (fp6.cu). cell: one workspace word.
+// Simulated FP6 (E2M3) quantizers and the FP4 -> dense expansion (fp6.cu). cells: workspace of at least one word.
 cudaError_t launch_fp6_quantize_rows(const uint16_t* src, int64_t rows, int64_t K, int64_t ld, int sr, uint64_t seed, uint32_t stream_id,
-                                     uint32_t* cell, uint16_t* out, int64_t ld_out, float* gscale, cudaStream_t st);
+                                     uint32_t* cells, size_t cells_bytes, uint16_t* out, int64_t ld_out, float* gscale, cudaStream_t st);
 cudaError_t launch_fp6_requantize_t(const uint16_t* in, int64_t rowsK, int64_t D, int64_t ld_in, const float* in_gscale, int sr,
                                     uint64_t seed, uint32_t stream_id, uint32_t* cell, uint16_t* out, int64_t ld_out, float* gscale,
                                     cudaStream_t st);
