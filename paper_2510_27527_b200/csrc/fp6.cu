@@ -57,6 +57,10 @@ __device__ __forceinline__ void fp6_block16(const float (&x)[16], float rcp, flo
     mul2_rn(p0, p1, Sbf, v0, v1);
     out[i >> 1] = __byte_perm(__float_as_uint(v0), __float_as_uint(v1), 0x7632);
   }
+  if (Sbf != Sbf) {  // an infinity in the block: its values are written as -0 (the global scale is infinite)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) out[i] = 0x80008000u;
+  }
 }
 
 // The scale pair of a block: E4M3 block scale as a float and the reciprocal that maps x onto the E2M3 grid.
@@ -198,7 +202,8 @@ expand_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restri
     const int64_t nb = Kp >> 4;
     const size_t sfo = sf_tiled ? sf_tiled_offset(r, k0 >> 4, (nb + 15) & ~(int64_t)15) : (size_t)(r * nb + (k0 >> 4));
     uint32_t h[4];
-    decode8_h2(word, sf[sfo], h);
+    const uint8_t scale = sf[sfo];
+    decode8_h2(word, scale, h);
     uint32_t q[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -206,6 +211,7 @@ expand_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restri
       q[i] = __byte_perm(__float_as_uint(f.x), __float_as_uint(f.y), 0x7632);  // exact in BF16: 2 + 4 significant bits
     }
     o = make_uint4(q[0], q[1], q[2], q[3]);
+    if ((scale & 0x7Fu) == 0x7Fu) o = make_uint4(0x80008000u, 0x80008000u, 0x80008000u, 0x80008000u);  // a NaN scale, as in fp6_block16
   }
   *reinterpret_cast<uint4*>(out + r * ld_out + k0) = o;
 }
