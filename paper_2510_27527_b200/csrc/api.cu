@@ -772,14 +772,14 @@ static nvfp4_status bwd_dx_impl(const void* dY, int64_t lddy, const nvfp4_saved*
     } else {
       qa.compute_amax = 1;  // ROW: per-row cells, each pass fills the rows it owns; BLOCK128: no pre-pass
     }
+    QuantTransposeArgs qo = qa;
     qa.from_codes = 1;
     qa.D = D - n_out;
     qa.src = ts;
-    if (launch_quantize_transpose(qa, st) != cudaSuccess) return NVFP4_ERR_CUDA;
-    qa.from_codes = 0;
-    qa.D = n_out;
-    qa.src = th;
-    if (launch_quantize_transpose(qa, st) != cudaSuccess) return NVFP4_ERR_CUDA;
+    qo.from_codes = 0;
+    qo.D = n_out;
+    qo.src = th;
+    if (launch_requantize_outliers(qa, qo, st) != cudaSuccess) return NVFP4_ERR_CUDA;
   }
   return do_gemm(&q3, &q4, dX, cfg->dx_dtype, lddx, 0, cfg->dev_status, st);
 }

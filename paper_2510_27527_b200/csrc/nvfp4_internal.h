@@ -75,6 +75,7 @@ struct QuantTransposeArgs {
   int compute_amax;
   int cells_zeroed;        // the caller has already cleared gs_cells on this stream
   int tensor_closed_form;  // set by the launcher
+  int amax_only;           // the maxima of ROW's rows and no operand
   uint32_t* gs_cells;  // gs_words cells (TENSOR) or D cells (ROW)
   int gs_words;        // as in QuantRowsArgs
   uint8_t* codes;
@@ -131,6 +132,7 @@ inline AmaxGrid amax_grid(int64_t wanted_ctas, int n_words) {
 }
 
 cudaError_t launch_quantize_rows(const QuantRowsArgs& a, cudaStream_t st);
+cudaError_t launch_requantize_outliers(const QuantTransposeArgs& kept, const QuantTransposeArgs& outl, cudaStream_t st);
 cudaError_t launch_quantize_transpose(const QuantTransposeArgs& a, cudaStream_t st);
 // Q1 and Q2 in one launch (round to nearest, no column lists, tiled scales; TENSOR: the cells hold the maxima already). The
 // padding of the tiled scales is cleared as well.

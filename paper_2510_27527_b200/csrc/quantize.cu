@@ -1806,6 +1806,24 @@ quantize_bwd_kernel(const __grid_constant__ RowsJob q3, const __grid_constant__ 
   clear_scale_padding(q.sf, (uint32_t)q.D, (((uint32_t)q.rowsK + 127u) & ~127u) >> 4, bx, q.blocks);
 }
 
+// Q4 with outlier channels: the kept channels from the forward operand and the outlier channels from their BF16 copy, which fill disjoint
+// rows of one operand (in the TENSOR mode both write the same global scale). Latency of one tile: the outlier channels alone are a few
+// dozen CTAs that take as long as the kept ones (2816 x 1024 weights, 8.3 and 7.4 us; dX of 256 tokens 25.4 -> 19.8 us, kOutlierCtas).
+template <int GS, bool RHT>
+__global__ void __launch_bounds__(256, 3)
+requantize_outliers_kernel(const __grid_constant__ TransposeJob kept, const __grid_constant__ TransposeJob outl, uint64_t seed,
+                           const __grid_constant__ PhiloxKeys pk) {
+  pdl_prologue();
+  if (blockIdx.x < outl.blocks) {
+    quantize_transpose_body<0, GS, 1, true, RHT, false>(outl.s, outl.rowsK, outl.D, seed, outl.stream_id, outl.gs_cells, outl.gs_words, 0, outl.codes,
+                                                        outl.sf, outl.gscale, outl.rht_stream, pk, blockIdx.x % outl.grid_x, blockIdx.x / outl.grid_x);
+    return;
+  }
+  const uint32_t bx = blockIdx.x - outl.blocks;
+  quantize_transpose_body<1, GS, 1, true, RHT, false>(kept.s, kept.rowsK, kept.D, seed, kept.stream_id, kept.gs_cells, kept.gs_words, 0, kept.codes,
+                                                      kept.sf, kept.gscale, kept.rht_stream, pk, bx % kept.grid_x, bx / kept.grid_x);
+}
+
 // =========================================================================================================
 // Host-side launchers
 // =========================================================================================================
@@ -2121,6 +2139,7 @@ static cudaError_t launch_tr_amax_rht(const TransposeSrc& src, int64_t rowsK, in
 
 template <int SRC, int GS>
 static cudaError_t launch_tr_r(const QuantTransposeArgs& a, cudaStream_t st) {
+  if (a.amax_only) return cudaSuccess;
   return a.sr == 2 ? launch_tr_t<SRC, GS, 2>(a, st) : a.sr ? launch_tr_t<SRC, GS, 1>(a, st) : launch_tr_t<SRC, GS, 0>(a, st);
 }
 
@@ -2297,6 +2316,37 @@ cudaError_t launch_quantize_rows_pair(const QuantRowsArgs& a, const QuantRowsArg
     launch_kernel(quantize_rows_pair_kernel<kGsRow>, grid, dim3(256), 0, st, ja, jb);
   else
     launch_kernel(quantize_rows_pair_kernel<kGsBlock128>, grid, dim3(256), 0, st, ja, jb);
+  return cudaGetLastError();
+}
+
+// Both passes of Q4 with outlier channels (stochastic rounding): one launch while it is the outlier channels' latency that counts. us, dX
+// with 10 % outlier channels, 256 tokens, two launches / one, TENSOR, ROW, BLOCK128 with the Hadamard transformation: weights 512 x 512
+// 20.8 / 17.1, 25.3 / 21.2, 19.4 / 14.2; 1024 x 2816 24.1 / 19.9, 30.0 / 25.5, 25.4 / 19.8; 4096 x 4096 (12 CTAs per SM) 41.7 / 37.8,
+// 47.5 / 44.4; 8192 x 8192 (50) 108.2 / 105.8, 137.1 / 137.9; 28672 x 8192 325 / 327, 444 / 449. From 4 per SM on the outer block has a
+// variant of the transposing kernel with more of its CTAs on an SM.
+constexpr int kOutlierCtas = 32;
+cudaError_t launch_requantize_outliers(const QuantTransposeArgs& kept, const QuantTransposeArgs& outl, cudaStream_t st) {
+  auto ok = [](const QuantTransposeArgs& q) {
+    return q.sr == 1 && q.sf_tiled && small_index(q.rowsK) && small_index(q.D) && transpose_fast_path(q.src, q.from_codes);
+  };
+  const TransposeJob jk = transpose_job(kept), jo = transpose_job(outl);
+  const bool one = ok(kept) && ok(outl) &&
+                   (int64_t)jk.blocks <= (kept.gs_mode == kGsBlock128 ? 4 : kOutlierCtas) * (int64_t)device_sm_count();
+  if (!one || kept.gs_mode == kGsRow) {  // (ROW: the passes over the rows' maxima first)
+    QuantTransposeArgs k = kept, o = outl;
+    k.amax_only = o.amax_only = one;
+    cudaError_t e = launch_quantize_transpose(k, st);
+    if (e == cudaSuccess) e = launch_quantize_transpose(o, st);
+    if (e != cudaSuccess || !one) return e;
+  }
+  const dim3 grid(jk.blocks + jo.blocks);
+  auto go = [&](auto kernel) { launch_kernel(kernel, grid, dim3(256), 0, st, jk, jo, kept.seed, make_philox_keys(kept.seed)); };
+  if (kept.gs_mode == kGsTensor)
+    kept.rht_stream ? go(requantize_outliers_kernel<kGsTensor, true>) : go(requantize_outliers_kernel<kGsTensor, false>);
+  else if (kept.gs_mode == kGsRow)
+    kept.rht_stream ? go(requantize_outliers_kernel<kGsRow, true>) : go(requantize_outliers_kernel<kGsRow, false>);
+  else
+    kept.rht_stream ? go(requantize_outliers_kernel<kGsBlock128, true>) : go(requantize_outliers_kernel<kGsBlock128, false>);
   return cudaGetLastError();
 }
 
