@@ -455,9 +455,9 @@ class IndexArrays(tuple):
     streams: set | None = None  # streams that the allocator knows to read them; None: not on a CUDA device
 
     def here(self) -> "IndexArrays":
-        """The arrays, for kernels on the current stream: given back, their memory waits for that stream too."""
-        if self.streams is not None and (s := _stream_ptr()) not in self.streams:
-            self[0].record_stream(torch.cuda.current_stream())  # (the three are pieces of one allocation)
+        """The arrays, for kernels on their device's current stream: given back, their memory waits for that stream too."""
+        if self.streams is not None and (s := torch._C._cuda_getCurrentRawStream(self[0].device.index)) not in self.streams:
+            self[0].record_stream(torch.cuda.current_stream(self[0].device))  # (the three are pieces of one allocation)
             self.streams.add(s)
         return self
 

@@ -34,3 +34,30 @@ def test_index_arrays_go_by_value_and_are_bounded():
     again = cfg.index(16, "cpu")
     assert again is not first and all(np.array_equal(a, f) for a, f in zip(again, first))
     assert copy.deepcopy(cfg)._arrays._of == {}  # no device memory goes into a copy or a file
+
+
+def test_index_arrays_are_recorded_on_a_stream_of_their_own_device(monkeypatch):
+    """A module whose input lies on another device than the current one launches there (no second device is needed to see which
+    stream is asked for)."""
+    import torch
+
+    from paper_2510_27527_b200 import binding as b
+
+    class Piece:
+        device = torch.device("cuda", 1)
+        recorded = []
+
+        def record_stream(self, stream):
+            self.recorded.append(stream)
+
+    streams = {0: 10, 1: 21}
+    monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 0, raising=False)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda index: streams[index], raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device=None: ("stream", 0 if device is None else torch.device(device).index))
+    arrays = b.IndexArrays([Piece()] * 3)
+    arrays.streams = {21}  # uploaded there
+    arrays.here()
+    assert Piece.recorded == [] and arrays.streams == {21}
+    streams[1] = 22
+    arrays.here().here()
+    assert Piece.recorded == [("stream", 1)] and arrays.streams == {21, 22}
