@@ -39,13 +39,28 @@ def _compile(lib, sources, verbose):
     os.replace(tmp, lib)
 
 
+def node_tag() -> str:
+    """What the autograd node is compiled against, beside its sources: torch's and Python's binary interfaces have no file to compare."""
+    import torch
+
+    return f"torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
+def _node_stale(lib, sources) -> bool:
+    if _stale(lib, sources):
+        return True
+    with open(lib, "rb") as f:
+        return node_tag().encode() + b"\0" not in f.read()  # (the module holds it as `built_for`)
+
+
 def _compile_node(lib, sources):
     import torch
 
     at, cuda = os.path.dirname(torch.__file__), os.environ.get("CUDA_HOME", "/usr/local/cuda")
     tmp = lib + f".{os.getpid()}.tmp"
     subprocess.check_call(
-        [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+        [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+         f'-DNODE_TAG="{node_tag()}"']
         + ["-isystem" + d for d in (f"{at}/include", f"{at}/include/torch/csrc/api/include", f"{cuda}/include", sysconfig.get_paths()["include"])]
         + [os.path.join(CSRC, f) for f in sources] + ["-o", tmp, f"-L{at}/lib", "-ltorch", "-ltorch_cpu", "-ltorch_python", "-lc10", "-lc10_cuda",
                                                       f"-L{cuda}/lib64", "-lcudart", f"-L{HERE}", "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"])
@@ -56,7 +71,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     for lib, sources in ((LIB, SOURCES), (MEASURE_LIB, MEASURE_SOURCES)):
         if force or _stale(lib, sources):
             _compile(lib, sources, verbose)
-    if force or _stale(NODE_LIB, NODE_SOURCES):
+    if force or _node_stale(NODE_LIB, NODE_SOURCES):
         _compile_node(NODE_LIB, NODE_SOURCES)
     return LIB
 

@@ -253,5 +253,10 @@ PyMODINIT_FUNC PyInit__node() {
   names = {PyUnicode_InternFromString("gs_mode"),    PyUnicode_InternFromString("rounding"),   PyUnicode_InternFromString("rht"),
            PyUnicode_InternFromString("outlier_fp8"), PyUnicode_InternFromString("w_block16"), PyUnicode_InternFromString("concurrent"),
            PyUnicode_InternFromString("dev_status")};
-  return PyModule_Create(&module_def);
+  PyObject* module = PyModule_Create(&module_def);
+  if (module && PyModule_AddStringConstant(module, "built_for", NODE_TAG) < 0) {
+    Py_DECREF(module);
+    return nullptr;
+  }
+  return module;
 }

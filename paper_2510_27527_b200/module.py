@@ -14,9 +14,12 @@ import torch
 from torch.autograd import forward_ad
 
 from . import binding as B
+from .build import node_tag
 
 try:
     from . import _node
+    if getattr(_node, "built_for", None) != node_tag():  # (it may load all the same)
+        raise ImportError(f"{_node.__file__} is not for {node_tag()}")
 except ImportError as e:
     raise ImportError(f"{e}: build it with `python -m paper_2510_27527_b200.build`") from e
 
