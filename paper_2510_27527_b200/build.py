@@ -62,7 +62,9 @@ def _compile_node(lib, sources):
         [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
          f'-DNODE_TAG="{node_tag()}"']
         + ["-isystem" + d for d in (f"{at}/include", f"{at}/include/torch/csrc/api/include", f"{cuda}/include", sysconfig.get_paths()["include"])]
-        + [os.path.join(CSRC, f) for f in sources] + ["-o", tmp, f"-L{at}/lib", "-ltorch", "-ltorch_cpu", "-ltorch_python", "-lc10", "-lc10_cuda",
+        # (the C++ library that torch uses, by name: a compiler that has only the archive would put a second one into the node, whose
+        # streams, empty of locale facets, end the process when a message with a number in it is put together)
+        + [os.path.join(CSRC, f) for f in sources] + ["-o", tmp, "-l:libstdc++.so.6", f"-L{at}/lib", "-ltorch", "-ltorch_cpu", "-ltorch_python", "-lc10", "-lc10_cuda",
                                                       f"-L{cuda}/lib64", "-lcudart", f"-L{HERE}", "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"])
     os.replace(tmp, lib)
 

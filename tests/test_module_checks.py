@@ -12,3 +12,15 @@ def test_inputs_of_another_width_are_refused(shape, grad):
     with torch.set_grad_enabled(grad), pytest.raises(RuntimeError, match="256 input features"):
         layer(torch.zeros(shape, dtype=torch.bfloat16))
     assert layer._calls == 0  # no key of the layer's sequence is used up
+
+
+def _call(**opts):
+    from paper_2510_27527_b200 import binding as b
+    from paper_2510_27527_b200.module import NVFP4Linear
+
+    NVFP4Linear(256, 64, device="cpu", cfg=b.LayerConfig(**opts))(torch.zeros(4, 256, dtype=torch.bfloat16))
+
+
+def test_a_message_with_a_number_is_an_exception():
+    with pytest.raises((TypeError, IndexError), match="has 7 entries"):  # (it ended the process where the node had a C++ library of its own)
+        _call(rounding=(0, 0, 1, 1, 1, 1, 1))
