@@ -170,17 +170,24 @@ struct NVFP4LinearBackward : torch::autograd::Node {
   }
 };
 
-// An attribute of the configuration; as int() gives it.
+// An attribute of the configuration.
 pybind11::object attribute(PyObject* cfg, PyObject* name) {
   pybind11::object v = pybind11::reinterpret_steal<pybind11::object>(PyObject_GetAttr(cfg, name));
   if (!v) throw python_error();
   return v;
 }
-int64_t number(pybind11::handle v) {
+// A 32-bit field from it, as ctypes fills one: whole numbers only (a float or a text is a TypeError), the low bits of larger ones.
+int32_t field(pybind11::handle v) {
+  const pybind11::object i = pybind11::reinterpret_steal<pybind11::object>(PyNumber_Index(v.ptr()));
+  const unsigned long long n = i ? PyLong_AsUnsignedLongLongMask(i.ptr()) : ~0ull;
+  if (n == ~0ull && PyErr_Occurred()) throw python_error();
+  return (int32_t)(uint32_t)n;
+}
+// The same of int(v), for the switches.
+int32_t switch_field(pybind11::handle v) {
   const pybind11::object i = pybind11::reinterpret_steal<pybind11::object>(PyNumber_Long(v.ptr()));
-  const int64_t n = i ? PyLong_AsLongLong(i.ptr()) : -1;
-  if (n == -1 && PyErr_Occurred()) throw python_error();
-  return n;
+  if (!i) throw python_error();
+  return field(i);
 }
 
 struct Names {
@@ -204,16 +211,16 @@ PyObject* linear(PyObject*, PyObject* const* args, Py_ssize_t n) {
   // the configuration as it is now: what the caller changes later belongs to later calls
   nvfp4_layer_cfg& c = call.cfg;
   PyObject* cfg = args[2];
-  c.gs_mode = (int32_t)number(attribute(cfg, names.gs_mode));
-  c.rht = (int32_t)number(attribute(cfg, names.rht));
-  c.outlier_format = (int32_t)number(attribute(cfg, names.outlier_fp8));
-  c.weight_block = (int32_t)number(attribute(cfg, names.w_block16));
+  c.gs_mode = field(attribute(cfg, names.gs_mode));
+  c.rht = switch_field(attribute(cfg, names.rht));
+  c.outlier_format = switch_field(attribute(cfg, names.outlier_fp8));
+  c.weight_block = switch_field(attribute(cfg, names.w_block16));
   call.concurrent = PyObject_IsTrue(attribute(cfg, names.concurrent).ptr()) == 1;
   c.seed = PyLong_AsUnsignedLongLong(args[4]);
   if (PyErr_Occurred()) throw python_error();
   const pybind11::tuple rounding(attribute(cfg, names.rounding));
-  TORCH_CHECK_TYPE(rounding.size() == 6, "LayerConfig.rounding has ", rounding.size(), " entries instead of 6");
-  for (int i = 0; i < 6; ++i) c.rounding[i] = (int32_t)number(rounding[i]);
+  TORCH_CHECK_INDEX(rounding.size() <= 6, "LayerConfig.rounding has ", rounding.size(), " entries instead of 6");
+  for (size_t i = 0; i < rounding.size(); ++i) c.rounding[i] = field(rounding[i]);  // what is not given is to nearest
   const pybind11::object status = attribute(cfg, names.dev_status);
   if (!status.is_none()) {
     TORCH_CHECK_TYPE(THPVariable_Check(status.ptr()), "LayerConfig.dev_status is not a tensor");

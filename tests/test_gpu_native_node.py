@@ -47,6 +47,19 @@ def test_same_bytes_as_through_the_binding(shape, D, C, opts, monkeypatch):
             assert len(got) == len(want) and all(torch.equal(a, r) and a.stride() == r.stride() for a, r in zip(got, want))
 
 
+@pytest.mark.parametrize("rounding", [(0, 0, 1), (), (0, 0, 2, 1, 1)])
+def test_roundings_that_are_not_given_are_to_nearest(rounding, monkeypatch):
+    from paper_2510_27527_b200 import binding as b
+    from paper_2510_27527_b200.module import NVFP4Linear
+
+    layer = NVFP4Linear(256, 64, cfg=b.LayerConfig(seed=11, rounding=rounding))
+    layer.layer_id = 0
+    x, dy = mk(96, 256), mk(96, 64)
+    got, want = (run(layer, x, dy, native, monkeypatch) for native in (True, False))
+    layer.cfg.rounding = (*rounding, 0, 0, 0, 0, 0, 0)[:6]
+    assert all(torch.equal(a, r) and torch.equal(a, f) for a, r, f in zip(got, want, run(layer, x, dy, True, monkeypatch)))
+
+
 def test_rows_of_an_odd_width_are_padded(monkeypatch):
     from paper_2510_27527_b200 import module as m
 
