@@ -17,8 +17,10 @@ constexpr int kHpDwSplit = 16;
 // product, an outlier channel the sum of the high-precision side product's token splits. One coalesced pass over dW
 // instead of a column scatter plus a scattered reduce. A CTA takes kAsmRows rows. It builds, in shared memory, where every channel comes
 // from: src_of[d] = position in the compact product (>= 0) or -(1 + rank among the outliers); sums the splits of its outlier channels
-// there (four channels per thread, fixed order); and (STAGED) copies its rows of the compact product there as they are. All three start
-// at once and meet at one barrier, after which the rows are put together from shared memory and stored.
+// there (four channels per thread, fixed order); and (STAGED) copies its rows of the compact product there as they are. All of it is under
+// way together; the rows are then put together from shared memory and stored. An outlier's entry is its own, whatever the map holds there:
+// the map comes first, and a barrier. That barrier stands before the sums (us of dW alone, 8192 x 2816 -> 1024 with 282 outlier channels,
+// 128 x 8192 -> 8192 with 820: 83.3, 253 here; after the sums 84.7, 248; the map by plain loads 83.4, 265; no order at all 83.0, 258).
 // What bounds it is the latency of those loads: the rows of one CTA take a microsecond, a wave of CTAs is one or two of them. Reading the
 // compact product only once src_of is known, and the sums a channel per thread, was a second round of latency: us of a layer's backward with it,
 // before / now: 8192 x 1024 -> 2816 with 102 outlier channels 155 / 149, 8192 x 2816 -> 1024 with 282 161 / 150, 4095 x 1024 -> 2816 with
@@ -34,12 +36,26 @@ __global__ void __launch_bounds__(256) dw_assemble_kernel(const __grid_constant_
   int32_t* const src_of = reinterpret_cast<int32_t*>(rows + (STAGED ? ROWS * ldc : 0u));  // [D]
   const int64_t c0 = (int64_t)blockIdx.x * ROWS;
   const uint32_t nr = (uint32_t)min((int64_t)ROWS, a.C - c0);
+  // (the map need not stand on a 16-byte boundary)
+  const uint32_t map = (uint32_t)__cvta_generic_to_shared(src_of);
+  for (uint32_t d = threadIdx.x; d < D; d += 256)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(map + d * 4u), "l"(a.col_map + d) : "memory");
+  asm volatile("cp.async.commit_group;" ::: "memory");
   if (STAGED) {  // (rows of 16-byte pieces, one after another)
     const float* p = a.compact + c0 * ldc;
     const uint32_t dst = (uint32_t)__cvta_generic_to_shared(rows), pieces = nr * (ldc >> 2);
     for (uint32_t e = threadIdx.x; e < pieces; e += 256)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + e * 16u), "l"(p + (size_t)e * 4u) : "memory");
   }
+  int32_t own[2];  // the first 512 outlier channels, loaded beside the map
+#pragma unroll
+  for (uint32_t i = 0; i < 2; ++i) own[i] = threadIdx.x + i * 256u < n_out ? __ldg(a.outl + threadIdx.x + i * 256u) : -1;
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 1;" ::: "memory");  // the map's copies, not the rows'
+  __syncthreads();
+#pragma unroll
+  for (uint32_t i = 0; i < 2; ++i)
+    if (own[i] >= 0) src_of[own[i]] = -(int32_t)(1 + threadIdx.x + i * 256u);
+  for (uint32_t j = threadIdx.x + 512u; j < n_out; j += 256) src_of[__ldg(a.outl + j)] = -(int32_t)(1 + j);
   const int64_t split_stride = a.C * a.Kh;
   for (uint32_t e = threadIdx.x; e < nr * n_out4; e += 256) {
     const uint32_t rr = e / n_out4, j = (e - rr * n_out4) * 4u;  // (Kh is a multiple of 64: the columns past n_out exist)
@@ -56,12 +72,7 @@ __global__ void __launch_bounds__(256) dw_assemble_kernel(const __grid_constant_
     }
     *reinterpret_cast<float4*>(osum + rr * n_out4 * 4u + j) = v;
   }
-  for (uint32_t d = threadIdx.x; d < D; d += 256) {
-    const int32_t m = __ldg(a.col_map + d);
-    if (m >= 0) src_of[d] = m;
-  }
-  for (uint32_t j = threadIdx.x; j < n_out; j += 256) src_of[__ldg(a.outl + j)] = -(int32_t)(1 + j);
-  if (STAGED) asm volatile("cp.async.wait_all;" ::: "memory");
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   for (uint32_t rr = 0; rr < nr; ++rr) {
     const float* const kept = STAGED ? rows + rr * ldc : a.compact + (c0 + rr) * ldc;

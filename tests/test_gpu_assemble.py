@@ -37,3 +37,20 @@ def test_weight_gradient_of_kept_and_outlier_channels(T, D, C, n_out, f32):
     tol = T * 2.0 ** -24 * absdot + (0.0 if f32 else 2.0 ** -8 * want.abs())
     assert bool(((dw[:, idx].double() - want).abs() <= tol).all())
     assert bool((buf[:, D:] == 77.0).all())
+
+
+@pytest.mark.parametrize("D,n_out", [(264, 5), (1000, 300), (8200, 66), (20000, 1)])
+def test_an_outlier_takes_its_sums_whatever_the_channel_map_holds_for_it(D, n_out):
+    from paper_2510_27527_b200 import binding as b
+
+    g = torch.Generator(device="cuda").manual_seed(D)
+    mk = lambda r, c: torch.randn(r, c, device="cuda", generator=g).to(torch.bfloat16)  # noqa: E731
+    x, w, dy = mk(128, D), mk(16, D), mk(128, 16)
+    cfg = b.LayerConfig(gs_mode=b.GS_TENSOR, seed=5, outliers=synth.outlier_channels(D, n_out, 9))
+    _, saved = b.nvfp4_linear_fwd(x, w, cfg)
+    want = b.nvfp4_linear_bwd_dw(dy, saved, cfg)
+    outl, _, cmap = saved.index
+    for value in (0, D - n_out - 1):  # positions of kept channels
+        cmap[outl.long()] = value
+        for _ in range(5):
+            assert torch.equal(b.nvfp4_linear_bwd_dw(dy, saved, cfg), want)
