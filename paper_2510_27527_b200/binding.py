@@ -571,6 +571,7 @@ def _device_of(device) -> torch.device:
     return torch.device("cuda", torch.cuda.current_device()) if dev.type == "cuda" and dev.index is None else dev
 
 
+@torch.compiler.disable  # (a stream that is made while a function is compiled has no handle)
 def _make_side(dev: torch.device) -> tuple:
     """(stream, fork, join, aux, their four handles) on `dev`."""
     with torch.cuda.device(dev):

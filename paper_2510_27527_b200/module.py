@@ -103,8 +103,8 @@ class _Call:
 def _plain(x: torch.Tensor, weight: torch.Tensor) -> bool:
     """Whether a call can go to the native node. Not while a trace is recorded or compiled (it would not see what the library writes), under
     forward-mode differentiation or a function transform (which the autograd function refuses), or with tensor subclasses."""
-    return (type(x) is torch.Tensor and type(weight) is torch.nn.Parameter and forward_ad._current_level < 0 and not torch._C._is_tracing()
-            and not torch._C._are_functorch_transforms_active() and not torch.compiler.is_compiling())
+    return (not torch.compiler.is_compiling() and type(x) is torch.Tensor and type(weight) is torch.nn.Parameter and forward_ad._current_level < 0
+            and not torch._C._is_tracing() and not torch._C._are_functorch_transforms_active())
 
 
 class _NVFP4LinearFn(torch.autograd.Function):
