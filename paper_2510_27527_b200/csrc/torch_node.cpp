@@ -10,6 +10,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/function.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/dynamo/compiled_autograd.h>
 
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDACachingAllocator.h>
@@ -17,6 +18,7 @@
 #include <c10/cuda/CUDAStream.h>
 
 #include <array>
+#include <cstring>
 #include <list>
 
 #include "../../include/nvfp4.h"
@@ -84,14 +86,19 @@ at::Tensor matrix(int64_t rows, int64_t cols, const at::TensorOptions& opt) {
   throw e;
 }
 
-struct Call {
+// What a call is beside its tensors.
+struct Fixed {
+  nvfp4_saved saved{};                     // (into Call::buf)
+  nvfp4_layer_cfg cfg{};
+  cudaStream_t stream = nullptr;           // of forward
+  bool concurrent = false;
+};
+static_assert(std::is_trivially_copyable_v<Fixed>);
+
+struct Call : Fixed {
   at::Tensor buf;                          // what forward leaves for backward, in one piece, and forward's workspace
   std::array<at::Tensor, 3> index;         // outlier channels, kept channels, channel map
   at::Tensor dev_status;
-  cudaStream_t stream = nullptr;           // of forward
-  nvfp4_saved saved{};
-  nvfp4_layer_cfg cfg{};
-  bool concurrent = false;
 
   at::Tensor forward(const at::Tensor& x, const at::Tensor& w) {
     TORCH_CHECK(x.is_cuda() && w.device() == x.device(), "NVFP4Linear: input on ", x.device(), ", weight on ", w.device());
@@ -167,6 +174,43 @@ struct NVFP4LinearBackward : torch::autograd::Node {
   std::string name() const override { return "NVFP4LinearBackward"; }
   variable_list apply(variable_list&& grads) override {
     return call.backward(grads[0].defined() ? std::move(grads[0]) : input_metadata(0).zeros_like());
+  }
+
+  // Compiled autograd records a graph of the whole backward and runs it again on other calls of the same form: the node becomes one call of
+  // a function that is not looked into, and all that belongs to this call goes in as tensors.
+  mutable at::Tensor fixed;  // the bytes of call's Fixed
+  void compiled_args(torch::dynamo::autograd::CompiledNodeArgs& args) const override {
+    if (!fixed.defined()) {
+      fixed = at::empty({(int64_t)sizeof(Fixed)}, at::kByte);
+      std::memcpy(fixed.data_ptr(), static_cast<const Fixed*>(&call), sizeof(Fixed));
+    }
+    for (const at::Tensor* t : {&std::as_const(fixed), &call.buf, &call.index[0], &call.dev_status}) args.collect(*t);
+  }
+  variable_list apply_with_saved(const variable_list& grads, torch::dynamo::autograd::SwapSavedVariables& saved) override {
+    namespace dynamo = torch::dynamo::autograd;
+    const std::array<at::Tensor*, 4> all{&fixed, &call.buf, &call.index[0], &call.dev_status};
+    for (at::Tensor* t : all) saved.before(*t);
+    std::vector<c10::IValue> args;
+    std::vector<at::TypePtr> schema;
+    for (const at::Tensor* t : all)
+      if (t->defined()) {
+        args.emplace_back(*t);
+        schema.emplace_back(at::TensorType::get());
+      }
+    const auto& py = dynamo::getPyCompilerInterface();
+    const std::string function = py->bind_function(saved.get_py_compiler(), name(), replay, schema, /*is_custom_function=*/true, /*is_traceable=*/false);
+    variable_list out = py->call_function(saved.get_py_compiler(), "apply_functional", function, grads, args,
+                                          dynamo::IValuePacker<std::vector<std::optional<torch::autograd::InputMetadata>>>::pack(
+                                              dynamo::get_input_metadata(next_edges())));
+    for (at::Tensor* t : all) saved.after(*t);
+    return out;
+  }
+  static variable_list replay(const variable_list& grads, const std::vector<c10::IValue>& args) {
+    Call c;
+    std::memcpy(static_cast<Fixed*>(&c), args.at(0).toTensor().data_ptr(), sizeof(Fixed));
+    c.buf = args.at(1).toTensor();
+    if (c.cfg.n_out > 0) c.index[0] = args.at(2).toTensor();
+    return c.backward(grads[0].defined() ? grads[0] : at::zeros({c.saved.N_tok, c.saved.C}, c.buf.options().dtype(at::kBFloat16)));
   }
 };
 

@@ -52,3 +52,55 @@ def test_compiled(data, backend, warm):
     y = torch.compile(made, backend=backend)(xi)
     assert same((y, *torch.autograd.grad(y, (xi, made.weight), dy)), want)
     torch._dynamo.reset()
+
+
+@pytest.mark.parametrize("backend", ["eager", "inductor"])
+@pytest.mark.parametrize("opts", [dict(), dict(gs_mode=2, rht=True, outliers=[3, 40, 100]), dict(concurrent=False)])
+def test_compiled_autograd_over_ordinary_calls(opts, backend):
+    """A recorded backward, run again on later calls with other keys, inputs and weights: each has its own draws and saved operands."""
+    from torch._dynamo import compiled_autograd
+
+    first, second = mk(D, D), mk(C, D)
+    torch._dynamo.reset()
+    for step in range(3):
+        x, dy = mk(T + 8 * (step == 2), D), mk(T + 8 * (step == 2), C)
+        got = []
+        for compiled in (False, True):
+            from paper_2510_27527_b200 import binding as b
+            from paper_2510_27527_b200.module import NVFP4Linear
+
+            model = torch.nn.Sequential(NVFP4Linear(D, D, cfg=b.LayerConfig(seed=3, **opts)), torch.nn.ReLU(), layer(second, **opts))
+            model[0].layer_id = 1
+            with torch.no_grad():
+                model[0].weight.copy_(first)
+            for m in (model[0], model[2]):
+                m._calls = step
+            xi = x.clone().requires_grad_(step > 0)
+            y = model(xi)
+            if compiled:
+                with compiled_autograd._enable(torch.compile(backend=backend)):
+                    y.backward(dy)
+            else:
+                y.backward(dy)
+            got.append((y.detach(), model[0].weight.grad, model[2].weight.grad, *([xi.grad] if step else [])))
+        assert same(*got)
+    torch._dynamo.reset()
+
+
+def test_compiled_autograd_over_an_excluded_layer(data):
+    import torch._dynamo.config
+
+    x, w, dy, want = data
+    torch._dynamo.reset()
+    made, xi = layer(w), x.clone().requires_grad_()
+    apart = torch.compiler.disable(made)
+
+    @torch.compile(backend="eager")
+    def step(xi):
+        y = apart(xi)
+        y.backward(dy)
+        return y
+
+    with torch._dynamo.config.patch(compiled_autograd=True):
+        assert same((step(xi), xi.grad, made.weight.grad), want)
+    torch._dynamo.reset()
