@@ -107,6 +107,14 @@ def _plain(x: torch.Tensor, weight: torch.Tensor) -> bool:
             and not torch._C._is_tracing() and not torch._C._are_functorch_transforms_active())
 
 
+def _needs_function(x: torch.Tensor, weight: torch.Tensor) -> bool:
+    """Whether a call that the native node does not serve has to go through the autograd function: a gradient can be asked for, an input may
+    carry a forward-mode tangent or be a transform's (which the function refuses), or a trace is being recorded (which sees the function, but
+    not what the library writes). Else it goes to the library at once (48 instead of 55 us on 77 tokens)."""
+    return ((torch.is_grad_enabled() and (x.requires_grad or weight.requires_grad)) or forward_ad._current_level >= 0 or torch.jit.is_tracing()
+            or torch._C._are_functorch_transforms_active())
+
+
 class _NVFP4LinearFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x2d: torch.Tensor, weight: torch.Tensor, cfg: B.LayerConfig, seed: int):
@@ -153,8 +161,10 @@ class NVFP4Linear(torch.nn.Module):
             cfg = self.cfg
             index = None if cfg.outliers is None else cfg.index(self.in_features, x2d.device)
             y = _node.linear(x2d, weight, cfg, index, seed, torch.is_grad_enabled() and (x2d.requires_grad or weight.requires_grad))
-        else:
+        elif _needs_function(x2d, weight):
             y = _NVFP4LinearFn.apply(x2d, weight, self.cfg, seed)
+        else:
+            y = _Call().forward(x2d, weight, self.cfg, seed)
         if self.bias is not None:
             y = y + self.bias
         return y if len(shape) == 2 else y.reshape(*shape[:-1], self.out_features)

@@ -104,3 +104,50 @@ def test_compiled_autograd_over_an_excluded_layer(data):
     with torch._dynamo.config.patch(compiled_autograd=True):
         assert same((step(xi), xi.grad, made.weight.grad), want)
     torch._dynamo.reset()
+
+
+class Marked(torch.Tensor):
+    pass
+
+
+@pytest.mark.parametrize("which", ["weight", "input"])
+def test_calls_without_gradients_pass_the_autograd_function_by(data, which, monkeypatch):
+    from paper_2510_27527_b200 import module
+
+    x, w, _, want = data
+    monkeypatch.setattr(module._NVFP4LinearFn, "apply", lambda *a: pytest.fail("autograd function"))
+    with torch.no_grad():
+        y = torch.func.functional_call(layer(w), {"weight": w}, (x,)) if which == "weight" else layer(w)(x.as_subclass(Marked))
+    assert same((y,), want)
+    y = torch.func.functional_call(layer(w), {"weight": w}, (x,))  # with gradients on, but none asked for
+    assert same((y,), want) and not y.requires_grad
+
+
+@pytest.mark.parametrize("grad", [False, True])
+def test_transforms_are_refused(data, grad):
+    x, w, _, _ = data
+    with torch.set_grad_enabled(grad):
+        for call in (lambda m: torch.func.grad(lambda t: m(t).float().sum())(x), lambda m: torch.func.vmap(m)(x[None])):
+            with pytest.raises(RuntimeError, match="setup_context"):
+                call(layer(w))
+
+
+def test_other_weights_and_inputs_with_gradients(data):
+    import torch.nn.utils.parametrize as parametrize
+
+    class Same(torch.nn.Module):
+        def forward(self, w):
+            return w * 1
+
+    x, w, dy, want = data
+    xi, wi = x.clone().requires_grad_(), w.clone().requires_grad_()
+    y = torch.func.functional_call(layer(w), {"weight": wi}, (xi,))
+    assert same((y, *torch.autograd.grad(y, (xi, wi), dy)), want)
+    made = layer(w)
+    parametrize.register_parametrization(made, "weight", Same())
+    y = made(xi)
+    assert same((y, *torch.autograd.grad(y, (xi, made.parametrizations.weight.original), dy)), want)
+    made, xi = layer(w), x.clone().as_subclass(Marked).requires_grad_()
+    y = made(xi)
+    y.backward(dy)
+    assert same((y, xi.grad, made.weight.grad), want)
