@@ -150,6 +150,9 @@ struct Call : Fixed {
   }
 
   variable_list backward(at::Tensor dy) const {
+    // (the engine has seen to that; a node can also be called by hand)
+    TORCH_CHECK(dy.dim() == 2 && dy.size(0) == saved.N_tok && dy.size(1) == saved.C && dy.device() == buf.device(), "NVFP4LinearBackward: gradient of shape ",
+                dy.sizes(), " on ", dy.device(), " for an output of shape [", saved.N_tok, ", ", saved.C, "] on ", buf.device());
     dy = dy.contiguous();
     if (dy.scalar_type() != at::kBFloat16) dy = dy.to(at::kBFloat16);
     const c10::cuda::CUDAGuard guard(dy.device());

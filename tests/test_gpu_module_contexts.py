@@ -151,3 +151,14 @@ def test_other_weights_and_inputs_with_gradients(data):
     y = made(xi)
     y.backward(dy)
     assert same((y, xi.grad, made.weight.grad), want)
+
+
+def test_the_node_called_by_hand(data):
+    x, w, dy, want = data
+    y = layer(w)(x.clone().requires_grad_())
+    assert same((y, *y.grad_fn(dy)), want)
+    assert same((y, *y.grad_fn(dy.float())), want)
+    for bad in (dy[:-1], dy[:, :-1], dy[0], dy[None], mk(T + 1, C), dy.cpu(), mk(C, T)):
+        with pytest.raises(RuntimeError, match=r"gradient of shape .* for an output of shape \[96, 128\]"):
+            y.grad_fn(bad)
+    assert same((y, *y.grad_fn(dy)), want)
