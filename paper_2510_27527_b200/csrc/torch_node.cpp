@@ -163,8 +163,9 @@ struct Call : Fixed {
     at::Tensor ws = at::empty({(int64_t)ws_bytes}, dy.options().dtype(at::kByte));
     nvfp4_layer_cfg c = cfg;
     if (concurrent) set_side(c, main);  // (the engine's thread has its own)
-    if (index[0].defined() && main.stream() != stream)  // given back, their memory waits for this stream too
-      c10::cuda::CUDACachingAllocator::recordStream(index[0].storage().data_ptr(), main);  // (the three are pieces of one allocation)
+    if (main.stream() != stream)  // (by hand, or compiled autograd: the engine keeps to forward's) given back, their memory waits for this stream too
+      for (const at::Tensor* t : {&buf, &index[0], &dev_status})  // (the three index arrays are pieces of one allocation)
+        if (t->defined()) c10::cuda::CUDACachingAllocator::recordStream(t->storage().data_ptr(), main);
     const nvfp4_status st = nvfp4_linear_bwd(dy.data_ptr(), dy.stride(0), &saved, &c, dx.data_ptr(), dx.stride(0), dw.data_ptr(), dw.stride(0),
                                              ws.data_ptr(), ws_bytes, main.stream());
     if (st != NVFP4_OK) raise_status(st, "nvfp4_linear_bwd");
@@ -213,6 +214,7 @@ struct NVFP4LinearBackward : torch::autograd::Node {
     std::memcpy(static_cast<Fixed*>(&c), args.at(0).toTensor().data_ptr(), sizeof(Fixed));
     c.buf = args.at(1).toTensor();
     if (c.cfg.n_out > 0) c.index[0] = args.at(2).toTensor();
+    if (c.cfg.dev_status) c.dev_status = args.back().toTensor();
     return c.backward(grads[0].defined() ? grads[0] : at::zeros({c.saved.N_tok, c.saved.C}, c.buf.options().dtype(at::kBFloat16)));
   }
 };

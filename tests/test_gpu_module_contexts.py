@@ -162,3 +162,28 @@ def test_the_node_called_by_hand(data):
         with pytest.raises(RuntimeError, match=r"gradient of shape .* for an output of shape \[96, 128\]"):
             y.grad_fn(bad)
     assert same((y, *y.grad_fn(dy)), want)
+
+
+@pytest.mark.parametrize("opts", [dict(), dict(outliers=[3, 40, 100])])
+def test_what_backward_reads_on_another_stream_outlives_it(data, opts):
+    """The node called on a stream that has yet to get there, and dropped meanwhile: its buffer is not given to anyone before that."""
+    x, w, dy, _ = data
+    made = layer(w, **opts)
+    xi = x.clone().requires_grad_()
+    made(xi).backward(dy)
+    want = (xi.grad, made.weight.grad)
+    made._calls = 0
+    torch.cuda.synchronize()
+    before = torch.cuda.memory_allocated()
+    y = made(xi)
+    held = torch.cuda.memory_allocated() - before - y.untyped_storage().nbytes()  # the buffer, as the allocator rounds it
+    other = torch.cuda.Stream()
+    other.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(other):
+        torch.cuda._sleep(100_000_000)  # (about 50 ms)
+        got = y.grad_fn(dy)
+    del y
+    pending = sum(block["size"] for s in torch.cuda.memory_snapshot() for block in s["blocks"] if block["state"] == "active_pending_free")
+    filled = [torch.zeros(n, dtype=torch.uint8, device="cuda") for n in (held,) * 8]
+    torch.cuda.synchronize()
+    assert held > 0 and pending >= held and len(filled) == 8 and same(got, want)
