@@ -22,7 +22,7 @@ namespace {
 // spacing, its cell is bits(w) >> 20 and the low 20 bits the position inside it; adding 2^20 - 1 - ((2u + 1) << 3) to the bits
 // carries into the cell iff position > (2u + 1) << 3, i.e. iff (u + 0.5) / 65536 < position / 2^20 (an integer n is < x iff
 // n < ceil(x)); clearing the low 20 bits then leaves the rounded magnitude times 2^-126
-// (4096 x 3072 rows with the amax pass 24.6 -> 21.5 us against cells below 1 mapped onto [0.5, 1) and back).
+// (against cells below 1 mapped onto [0.5, 1) and back, 4096 x 3072 rows with the amax pass 24.6 -> 21.5 us).
 template <bool SR>
 __device__ __forceinline__ void fp6_block16(const float (&x)[16], float rcp, float Sbf, const PhiloxKeys& pk, uint32_t stream_id,
                                             uint64_t idx8, uint32_t (&out)[8]) {
@@ -221,15 +221,16 @@ expand_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restri
 cudaError_t launch_fp6_quantize_rows(const uint16_t* src, int64_t rows, int64_t K, int64_t ld, int sr, uint64_t seed, uint32_t stream_id,
                                      uint32_t* cells, size_t cells_bytes, uint16_t* out, int64_t ld_out, float* gscale, cudaStream_t st) {
   if (rows == 0) return cudaSuccess;
-  // The maximum as words that need no clearing (a launch less: 3 us of host time) up to 2^20 blocks, if the workspace holds them, else
-  // folded into one cleared word: from there on what each warp spends on reading the words is more than the launch. Four blocks per
-  // thread from 4 CTAs of single ones per SM on, from 8 with the longer chain of stochastic rounding: then the threads that wait for the
-  // words are what is too many. us with the amax pass, words and NB = 1 / words and NB = 4 / one word and NB = 1, before: to nearest
-  // 64 x 256 3.4 / 4.6 / -, 3.8; 1000 x 1416 5.9 / 6.6 / -, 7.1; 4096 x 1024 9.3 / 7.4 / -, 8.1; 4096 x 3072 19.1 / 15.9 / 14.6, 15.7;
-  // 16384 x 4096 91 / 79.7 / 67.4, 74.5; stochastic 1000 x 1416 6.7 / 9.6 / -, 9.0; 4096 x 1024 9.0 / 12.2 / -, 10.8; 4096 x 3072 21.4 /
-  // 22.2 / 21.5, 24.6; 16384 x 4096 105 / 102 / 104, 121.
-  const int64_t blocks = rows * (ld_out >> 4);
-  const int words = blocks <= ((int64_t)1 << 20) && cells_bytes >= kTensorAmaxWords * sizeof(uint32_t) ? kTensorAmaxWords : 1;
+  // The maximum as words that need no clearing (a launch less: 2 us of host time), or folded into one cleared word: every thread waits for the
+  // words, so that more threads make them dearer. To nearest, four blocks per thread share that wait from 4 CTAs of single ones per SM on, and
+  // from 8 on one word is better. With the longer chain of stochastic rounding the two are within 4 % of one another from 4 CTAs on (the line at 2^20
+  // blocks is where a launch less no longer shows), and four blocks per thread lose below it. us with the amax pass from a graph, words and NB = 1 /
+  // words and NB = 4 / one word; in brackets issued by the host: to nearest 64 x 256 3.4 / 4.8 / 3.8; 2400 x 1024 7.4 / 7.4 / 6.4 (8.0 / 7.9 / 10.2);
+  // 4096 x 1024 10.5 / 7.2 / 7.4 (10.0 / 8.0 / 10.1); 4096 x 1536 11.2 / 9.7 / 8.4 (11.6 / 10.3 / 10.1); 4096 x 3072 18.1 / 14.3 / 12.0;
+  // 16384 x 4096 93.1 / 80.3 / 67.9; stochastic 1000 x 1416 6.6 / 10.2 / 7.9; 4096 x 1024 8.9 / 12.1 / 9.3; 4096 x 3072 19.1 / 20.4 / 19.2;
+  // 8192 x 2048 (2^20 blocks) 23.9 / 23.8 / 24.8; 16384 x 4096 103 / 101 / 104.
+  const int64_t blocks = rows * (ld_out >> 4), per_sm = (int64_t)device_sm_count() * 256;
+  const int words = blocks <= (sr ? (int64_t)1 << 20 : 8 * per_sm) && cells_bytes >= kTensorAmaxWords * sizeof(uint32_t) ? kTensorAmaxWords : 1;
   cudaError_t e;
   if (words > 1) {
     if ((e = launch_amax_tensor_words(src, rows, K, ld, cells, st)) != cudaSuccess) return e;
@@ -242,10 +243,12 @@ cudaError_t launch_fp6_quantize_rows(const uint16_t* src, int64_t rows, int64_t 
     launch_kernel(kernel, dim3((unsigned)((blocks + 256 * nb - 1) / (256 * nb))), dim3(256), 0, st, src, rows, K, ld, stream_id, ccells, words,
                   out, ld_out, gscale, make_philox_keys(seed));
   };
-  if (words > 1 && blocks > (int64_t)148 * (sr ? 8 : 4) * 256)
-    sr ? go(fp6_quantize_rows_kernel<true, 4>, 4) : go(fp6_quantize_rows_kernel<false, 4>, 4);
+  if (sr)
+    go(fp6_quantize_rows_kernel<true, 1>, 1);
+  else if (words > 1 && blocks > 4 * per_sm)
+    go(fp6_quantize_rows_kernel<false, 4>, 4);
   else
-    sr ? go(fp6_quantize_rows_kernel<true, 1>, 1) : go(fp6_quantize_rows_kernel<false, 1>, 1);
+    go(fp6_quantize_rows_kernel<false, 1>, 1);
   return cudaGetLastError();
 }
 

@@ -9,8 +9,8 @@ from paper_2510_27527_b200 import binding as b
 
 pytestmark = pytest.mark.gpu
 
-# Blocks of the padded output around the lines: 148 * 4 * 256 = 151552 and 148 * 8 * 256 = 303104 (one or four per thread), 2^20 (words or
-# one word); rows that end inside a block, a row of one block, and a tensor smaller than one CTA.
+# Blocks of the padded output around the lines: 148 * 4 * 256 = 151552 (one or four per thread, to nearest), 148 * 8 * 256 = 303104 and
+# 2^20 (words or one word, to nearest and stochastic); rows that end inside a block, a row of one block, and a tensor smaller than one CTA.
 SHAPES = [(1, 8), (3, 24), (77, 1000), (2368, 1024), (2369, 1024), (4736, 1024), (4737, 1016), (8192, 2048), (8193, 2048), (151553, 16)]
 
 
