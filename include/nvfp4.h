@@ -345,9 +345,10 @@ nvfp4_status nvfp4_linear_bwd(const void* dY, int64_t lddy, const nvfp4_saved* s
  *   nvfp4_expand_operand    an ordinary FP4 operand (TENSOR mode, either scale layout) as a dense operand: no arithmetic
  *                           beyond P * S_block.
  *   nvfp4_dense_gemm        C [A.R, B.R] = (A.gscale B.gscale) A.vals B.vals^T, A.K == B.K: BF16 tensor-core product with
- *                           FP32 accumulation (the BF16 path of the 128 x 128 GEMM kernel), C BF16 or FP32 with leading
+ *                           FP32 accumulation (CTA pairs, or the BF16 path of the 128 x 128 GEMM kernel), C BF16 or FP32 with leading
  *                           dimension ldc, 16-byte aligned rows; dev_status as for nvfp4_gemm.
- * workspace (the two quantizers): at least nvfp4_fp6_workspace_bytes() bytes, 16-byte aligned. All pointers device.
+ * workspace (the two quantizers): nvfp4_fp6_workspace_bytes() bytes, 16-byte aligned; with less, down to 16, the row quantizer
+ * clears a word first (a launch more, the same results). All pointers device.
  * Errors: NULL / SHAPE / ALIGN / ENUM (rounding, c_dtype, an operand that is not TENSOR mode) / WORKSPACE / ARCH; nothing is
  * launched on an error.
  * --------------------------------------------------------------------------------------------------------- */

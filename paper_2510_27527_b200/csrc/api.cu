@@ -478,7 +478,8 @@ nvfp4_status nvfp4_gemm_ex(const nvfp4_operand* A, const nvfp4_operand* B, void*
 }
 
 int64_t nvfp4_dense_ld(int64_t K) { return (K + 63) & ~(int64_t)63; }
-size_t nvfp4_fp6_workspace_bytes(void) { return 16; }
+size_t nvfp4_fp6_workspace_bytes(void) { return kTensorAmaxWords * sizeof(uint32_t); }
+constexpr size_t kFp6LeastWorkspace = 16;  // one word does, at the price of a launch that clears it
 
 static nvfp4_status check_dense(const nvfp4_dense_operand* o) {
   if (!o || !o->vals || !o->gscale) return NVFP4_ERR_NULL;
@@ -495,7 +496,7 @@ nvfp4_status nvfp4_fp6_quantize(const void* src_bf16, int64_t rows, int64_t cols
   if (rows <= 0 || cols <= 0 || ld < cols || out->R != rows || out->K != cols) return NVFP4_ERR_SHAPE;
   if (rounding != NVFP4_ROUND_RTN && rounding != NVFP4_ROUND_SR) return NVFP4_ERR_ENUM;
   if (bad_matrix(src_bf16, ld, cols, 2)) return NVFP4_ERR_ALIGN;  // 16-byte aligned rows, as for nvfp4_quantize
-  if (!workspace || !aligned16(workspace) || ws_bytes < nvfp4_fp6_workspace_bytes()) return NVFP4_ERR_WORKSPACE;
+  if (!workspace || !aligned16(workspace) || ws_bytes < kFp6LeastWorkspace) return NVFP4_ERR_WORKSPACE;
   if ((s = check_arch()) != NVFP4_OK) return s;
   return launch_fp6_quantize_rows(static_cast<const uint16_t*>(src_bf16), rows, cols, ld, rounding == NVFP4_ROUND_SR, seed, stream_id,
                                   static_cast<uint32_t*>(workspace), ws_bytes, static_cast<uint16_t*>(out->vals), out->ld, out->gscale,
@@ -511,7 +512,7 @@ nvfp4_status nvfp4_fp6_requantize_t(const nvfp4_dense_operand* in, int32_t round
   if ((s = check_dense(out)) != NVFP4_OK) return s;
   if (out->R != in->K || out->K != in->R) return NVFP4_ERR_SHAPE;
   if (rounding != NVFP4_ROUND_RTN && rounding != NVFP4_ROUND_SR) return NVFP4_ERR_ENUM;
-  if (!workspace || !aligned16(workspace) || ws_bytes < nvfp4_fp6_workspace_bytes()) return NVFP4_ERR_WORKSPACE;
+  if (!workspace || !aligned16(workspace) || ws_bytes < kFp6LeastWorkspace) return NVFP4_ERR_WORKSPACE;
   if ((s = check_arch()) != NVFP4_OK) return s;
   return launch_fp6_requantize_t(static_cast<const uint16_t*>(in->vals), in->R, in->K, in->ld, in->gscale, rounding == NVFP4_ROUND_SR, seed,
                                  stream_id, static_cast<uint32_t*>(workspace), static_cast<uint16_t*>(out->vals), out->ld, out->gscale,

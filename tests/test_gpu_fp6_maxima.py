@@ -37,3 +37,19 @@ def test_every_form_gives_the_same_operand(shape, rounding):
     y = got[0].vals[:, :cols].float() * got[0].gscale
     pad = torch.nn.functional.pad(x.abs(), (0, -cols % 16)).reshape(rows, -1, 16).amax(2).repeat_interleave(16, 1)[:, :cols]
     assert bool(((y - x).abs() <= x.abs() * 0.1875 + pad * (0.25 / 7)).all())
+
+
+@pytest.mark.parametrize("rounding", [0, 1])
+def test_the_librarys_own_workspace_size_saves_the_clearing_launch(rounding):
+    x = torch.randn(64, 256, device="cuda").to(torch.bfloat16)
+    out = b.alloc_dense(64, 256)
+
+    def launches(nbytes):
+        ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        before = b.lib.nvfp4_launch_count()
+        b.nvfp4_fp6_quantize(x, rounding, 1, 1, out=out, workspace=ws)
+        return b.lib.nvfp4_launch_count() - before
+
+    assert launches(b.lib.nvfp4_fp6_workspace_bytes()) == 2 and launches(16) == 3
+    with pytest.raises(b.Nvfp4Error, match="workspace"):
+        launches(15)
