@@ -6,8 +6,8 @@
 // the even code) or the 16-bit stochastic rounding of the FP4 quantizer with the same Philox addressing.
 // No tensor-core instruction multiplies E2M3 by E2M1 under E4M3 block scales, and the paper itself simulates: the operands
 // of the simulated products are "dense": P * S_block as BF16, which is exact for both formats (at most 4 + 4 significant
-// bits), plus the FP32 global scale; the product runs on the BF16 tensor-core path of the 128 x 128 GEMM kernel with FP32
-// accumulation and the two global scales in the epilogue.
+// bits), plus the FP32 global scale; the product runs on BF16 tensor cores (CTA pairs, or the side-product path of the 128 x 128 GEMM
+// kernel) with FP32 accumulation and the two global scales in the epilogue.
 #include <algorithm>
 
 #include "nvfp4_device.cuh"

@@ -342,12 +342,14 @@ __device__ __forceinline__ uint32_t e2m1x8_rtn(const float (&y)[8]) {
 //         v = 4 * bits + ((~u & 0xFFFF) << 8) + 127 = 4 * bits - c,   c = (u << 8) + 129 - 2^24,
 //     has the magnitude index of the result as its top byte, and c is the draw's two bytes between two constant ones: one byte
 //     permutation per element.
-// The codes' bytes are then collected by byte permutations, even and odd elements apart, and the signs likewise. 13.0 instructions per
-// element with the draws. An earlier form (a second mapping for a < 1, the draw brought to bits 12 .. 27 by multiply-adds, sign and
-// code moved into place element by element) took 17.3. us, 16384 x 8192, before / after: rows 114.6 / 100.1, columns 129.2 / 108.6, from
-// codes 162.5 / 141.5 (1x128 outer scales), and 16384 x 2816 with one scale and the amax pass 63.0 / 57.4, 62.7 / 58.0, 48.2 / 42.1.
-// What bounds it is the ALU pipe (16 lanes a cycle): the generator's logic operations, the permutations, the clamp, and the two cycles
-// of that pipe which each widening multiply takes beside its four of the multiply pipe. Measured and not better: packing by dp4a, the
+// The codes' bytes are then collected by byte permutations, even and odd elements apart, and the signs likewise. Instructions executed per
+// element (counters): the whole row kernel 18.0, columns 19.3, from codes 21.0, against 22.1, 23.3 and 25.4 of an earlier form (a second
+// mapping for a < 1, the draw brought to bits 12 .. 27 by multiply-adds, sign and code moved into place element by element); rows to nearest
+// 9.7. us, 16384 x 8192, before / after: rows 114.6 / 100.1, columns 129.2 / 108.6, from codes 162.5 / 141.5 (1x128 outer scales), and
+// 16384 x 2816 with one scale and the amax pass 63.0 / 57.4, 62.7 / 58.0, 48.2 / 42.1.
+// The busiest pipe is the ALU's (16 lanes a cycle; 63 - 64 % of the cycles, as many as the issue slots; what keeps both from more is not
+// known): the generator's logic operations, the permutations, the clamp, and the two cycles of that pipe which each widening multiply takes
+// beside its four of the multiply pipe. Measured and not better: packing by dp4a, the
 // generator's high halves by FP64 FMAs, its first two rounds folded.
 //
 // Stochastic rounding of 8 scaled values with the draws packed in w (two 16-bit draws per word), packed low nibble first. The
