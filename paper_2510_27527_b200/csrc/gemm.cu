@@ -498,9 +498,10 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 // instructions) into one of two or three tensor-memory buffers; promotion warps pull it out, 32 rows x CW columns each, and promote it
 // into FP32 register accumulators with the rank-1 scale SgA[m, kc] * SgB[n, kc] (packed f32x2 multiply + FMA).
 //
-// What bounds it: the promotion. A packed operation issues every 2.8 cycles at best (timed in a loop from registers, two or more
-// warps per scheduler), which is 540 cycles per partial of 192 columns against 200 of its MMAs; the kernel takes 790 to 840 there at long
-// K, about 620 with 128 columns and 380 with 64.
+// What bounds it: no pipe, but the chain of a partial. A packed operation issues every 2.8 cycles at best (timed in a loop from registers,
+// two or more warps per scheduler), which is 540 cycles per partial of 192 columns against 200 of its MMAs; the kernel takes 790 to 840
+// there at long K, about 620 with 128 columns and 380 with 64. Without the promotion's arithmetic 8192 x 1024 x 3072 still takes 26.5 of
+// 36.8 us: bringing the operands, handing partials over and loading them from tensor memory is the larger part.
 //   - Two or three promotion warps per scheduler: a warp's barrier, tensor-memory load and hand-over latencies (about 400 cycles per
 //     partial) run under the others' arithmetic. With one (a 128 x 128 tile, four warps with 128 columns each) they add up:
 //     760 cycles per 128 columns. 192 columns are what a register file of 128 a thread on average holds (setmaxnreg: 80 for the

@@ -187,3 +187,16 @@ def test_what_backward_reads_on_another_stream_outlives_it(data, opts):
     filled = [torch.zeros(n, dtype=torch.uint8, device="cuda") for n in (held,) * 8]
     torch.cuda.synchronize()
     assert held > 0 and pending >= held and len(filled) == 8 and same(got, want)
+
+
+def test_what_the_node_holds_is_no_saved_variable(data):
+    """As with the autograd function: hooks see nothing of it, and a second backward runs."""
+    x, w, dy, want = data
+    made, xi, seen = layer(w), x.clone().requires_grad_(), []
+    with torch.autograd.graph.saved_tensors_hooks(lambda t: seen.append(t) or t, lambda t: t):
+        y = made(xi)
+    for _ in range(2):
+        xi.grad = made.weight.grad = None
+        y.backward(dy)
+        assert same((y, xi.grad, made.weight.grad), want)
+    assert seen == []
